@@ -38,8 +38,10 @@
  *     pass (the softmax is shift invariant).
  *   - sar_dtype is the STORAGE type of feat / out / gout / dfeat.  el, er, m, d, D, del, der, the
  *     running numerator `acc` and every accumulation are float32.
- *   - The fast kernels need 16-byte aligned feature arrays and F * sizeof(element) a multiple of
- *     16 bytes; other shapes run on slower scalar kernels with the same results.
+ *   - Feature arrays whose F elements are a multiple of 16 bytes should be 16-byte aligned (they are read as they
+ *     are).  For any other F the aggregation calls copy the arrays they gather from into a padded layout in the
+ *     workspace; the *_workspace_bytes functions account for it.  A call that gets neither (misaligned arrays, or a
+ *     ragged F without that much workspace) runs on slower scalar kernels with the same results.
  */
 #ifndef SAR_H_
 #define SAR_H_

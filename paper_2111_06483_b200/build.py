@@ -18,16 +18,15 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(CSRC, "build")
 LIB = os.path.join(PKG, "libsar.so")
-SOURCES = ["sar_gat.cu", "sar_lean_fwd_f32.cu", "sar_lean_fwd_bf16.cu", "sar_lean_bwd_dst_f32.cu", "sar_lean_bwd_dst_bf16.cu", "sar_lean_bwd_src_f32.cu", "sar_lean_bwd_src_bf16.cu",
-           "sar_graph.cu", "sar_host.cu", "sar_noalloc.cu", "sar_storing.cu",
-           "sar_glue.cu", "sar_norm.cu", "sar_linear.cu", "sar_rgcn.cu"]
+ROW_PASSES = ["fwd", "fwd_part", "dst", "dst_part", "src", "sum"]   # one translation unit per pass and storage type
+SOURCES = ["sar_linear.cu"] + [f"sar_lean_{p}_{t}.cu" for p in ("fwd", "bwd_dst", "bwd_src") for t in ("f32", "bf16")] + [f"sar_rows_{p}_{t}.cu" for p in ROW_PASSES for t in ("f32", "bf16")] + [
+    "sar_gat.cu", "sar_span.cu", "sar_rows_merge.cu", "sar_graph.cu", "sar_host.cu", "sar_noalloc.cu", "sar_storing.cu",
+    "sar_glue.cu", "sar_norm.cu", "sar_rgcn.cu"]
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
     "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "--expt-relaxed-constexpr",
     "-DSAR_BUILT_FOR_SM=100", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
 ]
-# extra flags for the lean-kernel translation units only (tuning experiments), e.g. SAR_LEAN_NVCC_EXTRA="-DSAR_LEAN_EXPERIMENT"
-LEAN_EXTRA = os.environ.get("SAR_LEAN_NVCC_EXTRA", "").split()
 
 
 def _nvcc() -> str:
@@ -74,7 +73,7 @@ def _fingerprint(src: str) -> str:
     for path in sorted(_deps(os.path.join(CSRC, src))):
         h.update(os.path.basename(path).encode())
         h.update(open(path, "rb").read())
-    h.update(" ".join(NVCC_FLAGS + (LEAN_EXTRA if src.startswith("sar_lean_") else [])).encode())
+    h.update(" ".join(NVCC_FLAGS).encode())
     return h.hexdigest()
 
 
@@ -92,8 +91,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if not force and os.path.exists(obj) and os.path.exists(stamp) and open(stamp).read() == fp:
             return obj, False
         inc = _cutlass_includes() if src == "sar_linear.cu" else []
-        lean = LEAN_EXTRA if src.startswith("sar_lean_") else []
-        cmd = [nvcc, *NVCC_FLAGS, *lean, *inc, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [nvcc, *NVCC_FLAGS, *inc, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}\n{r.stderr}")

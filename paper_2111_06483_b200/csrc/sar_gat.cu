@@ -1,10 +1,11 @@
 // C-ABI entry points of the fused GAT aggregation and of the sum aggregation: argument checks,
 // kernel selection and launches.  Declarations and contracts are in include/sar.h.
-#include "sar_gat_kernels.cuh"
-#include "sar_span_kernels.cuh"
-#include "sar_lean.cuh"
 #include "sar_dispatch.cuh"
+#include "sar_gat_kernels.cuh"
 #include "sar_generic_kernels.cuh"
+#include "sar_lean.cuh"
+#include "sar_rows.cuh"
+#include "sar_span.cuh"
 
 namespace sar {
 
@@ -41,17 +42,89 @@ sar_status make_shape(int32_t H, int32_t F, sar_dtype t, bool ptrs_16B_aligned, 
     return SAR_OK;
 }
 
-// ---- workspace layout ---------------------------------------------------------------------------
-// [ destination records: n_dst*H float4 ][ long-row partials of the CSR ][ long-row partials of the CSC ]
-static size_t rec_bytes(long long n_dst, int H) { return sar_round_up((size_t)n_dst * H * 16, 256); }
-static long long part_stride(int H, int F) {  // floats per segment, a multiple of 4 (float4 rows)
-    return (2LL * H * F + 2LL * H + 3) & ~3LL;
-}
-static size_t part_bytes(const sar_split *sp, int H, int F) {
-    return sp ? sar_round_up((size_t)sp->n_seg * part_stride(H, F) * 4, 256) : 0;
+// ---- what the row kernels work on -------------------------------------------------------------------------------
+// Heads are made of whole 16-byte vectors.  Where F elements are no multiple of 16 bytes (as wide as there are classes,
+// say) the rows that are gathered are copied into a padded array in the workspace first: the copy is one pass over
+// [n,H,F] against a gather of every edge's row, and an aligned row touches fewer sectors than one that starts anywhere.
+struct RowShape {
+    bool ok;           // H and F within what the kernels cover
+    bool ragged;       // F elements are no whole number of vectors
+    int vph;           // vectors per head
+    unsigned row_bytes;
+    RowGeo geo;
+};
+
+static int pow2_at_least(int x, int lo) {
+    const int p = sar_pow2_ceil(x);
+    return p < lo ? lo : p;
 }
 
-static SplitArgs split_args(const sar_split *sp, float *part, int H, int F, bool fast) {
+static RowShape row_shape(int H, int F, sar_dtype t) {
+    RowShape r{};
+    const int epv = t == SAR_BF16 ? 8 : 4;
+    r.ragged = F % epv != 0;
+    r.vph = (F + epv - 1) / epv;
+    r.row_bytes = (unsigned)H * (unsigned)r.vph * 16u;
+    r.ok = H <= SAR_MAX_HEADS && (long long)H * r.vph * 16 <= (1LL << 24) && sar_pow2_ceil(r.vph) <= 256;
+    const int vphp = sar_pow2_ceil(r.vph);
+    int HP = sar_pow2_ceil(H) < 8 ? sar_pow2_ceil(H) : 8;
+    while (HP > 1 && HP * vphp > 64) HP /= 2;
+    r.geo = RowGeo{pow2_at_least(HP * vphp, HP == 8 ? 8 : 4), HP, (H + HP - 1) / HP};
+    return r;
+}
+
+static RowShape sum_shape(int F, sar_dtype t) {
+    RowShape r{};
+    const int epv = t == SAR_BF16 ? 8 : 4;
+    r.ragged = F % epv != 0;
+    r.vph = (F + epv - 1) / epv;
+    r.row_bytes = (unsigned)r.vph * 16u;
+    r.ok = true;
+    const int NV = pow2_at_least(r.vph, 4) < 64 ? pow2_at_least(r.vph, 4) : 64;
+    r.geo = RowGeo{NV, 1, (r.vph + NV - 1) / NV};
+    return r;
+}
+
+// [n,H,F] -> [n,H,vph*EPV], zeros behind the F elements of a head; one 16-byte vector per thread
+template <typename T>
+__global__ void __launch_bounds__(256) pad_rows_kernel(long long vecs, int F, int vph, const T *__restrict__ in, uint4 *__restrict__ out) {
+    constexpr int EPV = Elem<T>::EPV;
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (i >= vecs) return;
+    const long long nh = i / vph;
+    const int f0 = (int)(i - nh * vph) * EPV;
+    const T *p = in + nh * F + f0;
+    float x[EPV];
+#pragma unroll
+    for (int k = 0; k < EPV; ++k) x[k] = f0 + k < F ? Elem<T>::load1(p + k) : 0.f;
+    out[i] = Elem<T>::pack(x);
+}
+
+static sar_status pad_rows(long long n, int H, int F, const RowShape &r, sar_dtype t, const void *in, void *out, cudaStream_t st) {
+    const long long vecs = n * H * r.vph;
+    if (vecs == 0) return SAR_OK;
+    const unsigned blocks = (unsigned)((vecs + 255) / 256);
+    if (t == SAR_F32)
+        SAR_LAUNCH("pad_rows", st, (pad_rows_kernel<float><<<blocks, 256, 0, st>>>(vecs, F, r.vph, static_cast<const float *>(in), static_cast<uint4 *>(out))));
+    else
+        SAR_LAUNCH("pad_rows", st, (pad_rows_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(vecs, F, r.vph, static_cast<const __nv_bfloat16 *>(in), static_cast<uint4 *>(out))));
+    return sar_after_launch();
+}
+
+// ---- workspace layout ---------------------------------------------------------------------------
+// [ destination records: n_dst*H float4 ][ padded gout ][ segments of the CSR ][ segments of the CSC ][ padded feat ]
+// (the padded arrays for ragged shapes only).  The first two do not depend on the partition: the steps of a call-by-call
+// backward pass share them.
+static size_t rec_bytes(long long n_dst, int H) { return sar_round_up((size_t)n_dst * H * 16, 256); }
+static long long part_stride(int H, const RowShape &r, sar_dtype t) {  // floats per segment, a multiple of 4 (float4 rows)
+    return ((long long)H * r.vph * (t == SAR_BF16 ? 8 : 4) + 3LL * H + 3) & ~3LL;
+}
+static size_t part_bytes(const sar_split *sp, int H, const RowShape &r, sar_dtype t) {
+    return sp ? sar_round_up((size_t)sp->n_seg * part_stride(H, r, t) * 4, 256) : 0;
+}
+static size_t pad_bytes(long long n, const RowShape &r) { return r.ragged ? sar_round_up((size_t)n * r.row_bytes, 256) : 0; }
+
+static SplitArgs split_args(const sar_split *sp, float *part, int H, const RowShape &r, sar_dtype t) {
     SplitArgs a;
     a.threshold = 0;
     a.n_long = 0;
@@ -59,8 +132,8 @@ static SplitArgs split_args(const sar_split *sp, float *part, int H, int F, bool
     a.long_row = nullptr;
     a.long_seg = nullptr;
     a.part = part;
-    a.pstride = part_stride(H, F);
-    if (sp && fast && sp->n_long > 0 && sp->threshold > 0) {
+    a.pstride = part_stride(H, r, t);
+    if (sp && sp->n_long > 0 && sp->threshold > 0) {
         a.threshold = sp->threshold;
         a.n_long = sp->n_long;
         a.n_seg = sp->n_seg;
@@ -93,91 +166,29 @@ static sar_status check_part(const sar_part *g, bool need_csc) {
 }
 
 
-// ---- span kernels ---------------------------------------------------------------------------------
-constexpr int kCapFwd = 256, kCapDst = 256, kCapSrc = 192, kCapSum = 256;
-constexpr int kCapSeg = 128;  // capacity of the segment launches (segments hold at most the plan threshold)
-constexpr int kMinBlocksFwd = 24, kMinBlocksBwd = 20;  // resident blocks per SM the register budget is cut for
-constexpr size_t kStageBytes = 16 * 1024;              // shared memory a partition step may spend on the rows' own data
-
-static int rows_per_span(long long n_rows, long long nnz, int cap) {
-    const double avg = n_rows > 0 ? (double)nnz / (double)n_rows : 0.0;
-    int R = avg > 0.5 ? (int)(1.0 * cap / avg + 0.5) : kMaxSpanRows;  // about cap edges per span (the long rows counted in avg are skipped)
-    if (R < 1) R = 1;
-    if (R > kMaxSpanRows) R = kMaxSpanRows;
-    return R;
+// The row kernels, or the span kernels?  Out of the L2 (126 MB) the row kernels are the faster ones, for arrays that do
+// not fit it the span kernels, whose ring keeps more bytes in flight.  Forward + backward, row against span kernels:
+// 100,000 nodes of 256 bytes 0.39 against 0.50 ms, 233,000 (forward alone) 0.41 against 0.57 ms, 400,000 1.43 against
+// 1.55 ms, 1 million of 576 bytes 12.0 against 10.3 ms.  A sum has nothing between its ids and its rows, and there the
+// ring is ahead much earlier: 100,000 nodes of 128 bytes 0.175 against 0.172 ms, 500,000 of 192 bytes 0.72 against
+// 0.67 ms, 2.45 million of 1 KB 15.0 against 12.5 ms; below that the row kernels' single launch counts.
+constexpr unsigned long long kSpanBytes = 128ull << 20, kSpanSumBytes = 12ull << 20;
+static bool use_span(const Shape &s, long long n_gathered, unsigned long long bytes = kSpanBytes) {
+    return s.fast && (unsigned long long)n_gathered * s.row_bytes > bytes;
 }
 
-// Launches span_kernel<MODE> over the rows (mode 0) and, with a long-row plan, over the segments
-// (mode 1).  The merge launch is the caller's.
-template <typename T, int G, int V, int S, int MODE, int CAP, int MINB>
-static sar_status launch_span(SpanArgs a, long long nnz, const char *name, const char *seg_name, cudaStream_t st) {
-    // The segment launch never stages more than `threshold` edges at a time: when that fits the small
-    // capacity it runs the instantiation with the smaller shared-memory footprint (more resident warps).
-    constexpr int CAP_SEG = CAP < kCapSeg ? CAP : kCapSeg;
-    auto kern = span_kernel<T, G, V, S, MODE, CAP, MINB>;
-    const size_t smem = (size_t)kSpanWarps * span_layout<MODE>(a.g.Hp, V, CAP, S, 32 / G).total;
-    SAR_TRY(ensure_smem(kern, smem));
-    a.mode = 0;
-    constexpr bool kIsSum = MODE == kSum || MODE == kSumW;
-    constexpr int kGeo = (kIsSum || G * V >= 4) ? 1 : 0;
-    const bool geo = kGeo && a.g.n_vec == G * V && (kIsSum ? a.g.H == 1 : (a.g.H == 4 && a.g.Hp == 4 && a.hvec));
-    a.R = rows_per_span(a.n_rows, nnz, CAP);
-    const bool whole = (a.flags & SAR_FIRST) && (a.flags & SAR_LAST);
-    // A partition step of the destination-major pass stages the rows' output-gradient rows per chunk when that fits
-    // kStageBytes of shared memory, with fewer rows per span if need be.
-    size_t stage_bytes = 0;
-    a.stage_rows = 0;
-    if (!whole && (MODE == kBwdDst || MODE == kBwdDstGivenD)) {
-        const size_t rsb = (size_t)a.g.n_vec * 16;
-        if (rsb <= kStageBytes) {
-            if ((size_t)a.R * rsb > kStageBytes) a.R = (int)(kStageBytes / rsb);
-            a.stage_rows = a.R;
-            stage_bytes = (size_t)a.R * rsb;
-        }
-    }
-    const long long spans = (a.n_rows + a.R - 1) / a.R;
-    if (spans > 0) {
-        const unsigned blocks = (unsigned)((spans + kSpanWarps - 1) / kSpanWarps);
-        if (whole && !(a.flags & (SAR_KEEP_NUMERATOR | SAR_RELU_OUT))) {  // the epilogue's flag tests decided at compile time
-            if (geo) {
-                auto wk = span_kernel<T, G, V, S, MODE, CAP, MINB, 1, kGeo>;
-                SAR_TRY(ensure_smem(wk, smem));
-                SAR_LAUNCH(name, st, wk<<<blocks, kSpanThreads, smem, st>>>(a));
-            } else {
-                auto wk = span_kernel<T, G, V, S, MODE, CAP, MINB, 1>;
-                SAR_TRY(ensure_smem(wk, smem));
-                SAR_LAUNCH(name, st, wk<<<blocks, kSpanThreads, smem, st>>>(a));
-            }
-        } else {
-            const size_t smem_st = (size_t)kSpanWarps * span_layout<MODE>(a.g.Hp, V, CAP, S, 32 / G, stage_bytes).total;
-            SAR_TRY(ensure_smem(kern, smem_st));
-            SAR_LAUNCH(name, st, kern<<<blocks, kSpanThreads, smem_st, st>>>(a));
-        }
-        SAR_TRY(sar_after_launch());
-    }
-    if (a.sp.threshold > 0 && a.sp.n_seg > 0) {
-        a.mode = 1;
-        const unsigned blocks = (unsigned)((a.sp.n_seg + kSpanWarps - 1) / kSpanWarps);
-        if (a.sp.threshold <= CAP_SEG) {
-            const size_t seg_smem = (size_t)kSpanWarps * span_layout<MODE>(a.g.Hp, V, CAP_SEG, S, 32 / G).total;
-            auto seg_kern = geo ? span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2, kGeo> : span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2>;
-            SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2, kGeo>, seg_smem));
-            SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2>, seg_smem));
-            SAR_LAUNCH(seg_name, st, seg_kern<<<blocks, kSpanThreads, seg_smem, st>>>(a));
-        } else {
-            auto seg_kern = geo ? span_kernel<T, G, V, S, MODE, CAP, MINB, 2, kGeo> : span_kernel<T, G, V, S, MODE, CAP, MINB, 2>;
-            SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP, MINB, 2, kGeo>, smem));
-            SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP, MINB, 2>, smem));
-            SAR_LAUNCH(seg_name, st, seg_kern<<<blocks, kSpanThreads, smem, st>>>(a));
-        }
-        SAR_TRY(sar_after_launch());
-    }
-    return SAR_OK;
+static sar_status check_shape(int32_t H, int32_t F, sar_dtype t) {
+    Shape s;
+    return make_shape(H, F, t, false, &s);
 }
 
-// stages of the gather ring: 8 x 512 bytes in flight per warp for one-vector rows
-template <int V> struct UFwd { static constexpr int u = V == 1 ? 8 : (V == 2 ? 4 : 2); };
-template <int V> struct UBwd { static constexpr int u = V == 1 ? 8 : (V == 2 ? 4 : 2); };
+// the per-head scalars of a tile's row can be read as one or two float4 (float2 for two heads)
+static int heads_aligned(int H, int HP, std::initializer_list<const void *> ps) {
+    if (H % HP != 0) return 0;
+    for (const void *p : ps)
+        if (p && !sar_aligned(p, HP >= 4 ? 16 : (size_t)HP * 4)) return 0;
+    return 1;
+}
 
 }  // namespace sar
 
@@ -211,16 +222,30 @@ int32_t sar_built_for_sm(void) {
 #endif
 }
 
+// Offsets of the workspace's parts, and what a call that needs all of them (`full`) or no padded copies asks for.
+struct WsLayout {
+    size_t gout, csr, csc, feat, full, plain;
+};
+static WsLayout ws_layout(const sar_part *g, int H, const RowShape &r, sar_dtype t) {
+    WsLayout w;
+    w.gout = rec_bytes(g->n_dst, H);
+    w.csr = w.gout + pad_bytes(g->n_dst, r);
+    w.csc = w.csr + part_bytes(g->split, H, r, t);
+    w.feat = w.csc + part_bytes(g->t_split, H, r, t);
+    w.full = w.feat + pad_bytes(g->n_src, r);
+    w.plain = w.gout;
+    return w;
+}
+
 size_t sar_gat_workspace_bytes(const sar_part *g, int32_t H, int32_t F, sar_dtype t) {
-    (void)t;
     if (!g || H < 1 || F < 1) return 0;
-    return rec_bytes(g->n_dst, H) + part_bytes(g->split, H, F) + part_bytes(g->t_split, H, F) + 256;
+    return ws_layout(g, H, row_shape(H, F, t), t).full + 256;
 }
 
 size_t sar_spmm_workspace_bytes(const sar_part *g, int32_t F, sar_dtype t) {
-    (void)t;
     if (!g || F < 1) return 0;
-    return part_bytes(g->split, 1, F) + 256;
+    const RowShape r = sum_shape(F, t);
+    return part_bytes(g->split, 1, r, t) + pad_bytes(g->n_src, r) + 256;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -234,15 +259,21 @@ sar_status sar_gat_fwd(const sar_part *g, const void *feat_q, const float *el, c
     if (!el || !m || !d) return SAR_ERR_INVALID_ARG;
     if (g->n_src > 0 && (!feat_q || !er_q)) return SAR_ERR_INVALID_ARG;
     if (last && !out) return SAR_ERR_INVALID_ARG;
-    if ((!(first && last) || (flags & SAR_KEEP_NUMERATOR)) && !acc) return SAR_ERR_INVALID_ARG;
+    const bool part = !(first && last) || (flags & SAR_KEEP_NUMERATOR);
+    if (part && !acc) return SAR_ERR_INVALID_ARG;
     SAR_TRY(check_elem_align({el, er_q, m, d, acc}, 4));
     SAR_TRY(check_elem_align({feat_q, out}, sar_elem_size(t)));
-    Shape s;
-    SAR_TRY(make_shape(H, F, t, all16({feat_q, out, acc}), &s));
+    SAR_TRY(check_shape(H, F, t));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (g->n_dst == 0) return SAR_OK;
 
-    if (!s.fast) {
+    const RowShape r = row_shape(H, F, t);
+    const WsLayout w = ws_layout(g, H, r, t);
+    const bool use_split = g->split && g->split->n_long > 0;
+    const bool have_ws = workspace && sar_aligned(workspace, 16);
+    char *wsb = static_cast<char *>(workspace);
+    const bool rows = r.ok && (r.ragged ? have_ws && workspace_bytes >= w.full : all16({feat_q, out, acc}));
+    if (!rows) {
         GenericArgs a{};
         a.n_dst = g->n_dst;
         a.indptr = g->indptr;
@@ -267,53 +298,39 @@ sar_status sar_gat_fwd(const sar_part *g, const void *feat_q, const float *el, c
         return sar_after_launch();
     }
 
-    const bool use_split = g->split && g->split->n_long > 0;
-    float *part = nullptr;
-    if (use_split) {
-        const size_t need = rec_bytes(g->n_dst, H) + part_bytes(g->split, H, F);
-        if (!workspace || workspace_bytes < need || !sar_aligned(workspace, 16)) return SAR_ERR_WORKSPACE;
-        part = reinterpret_cast<float *>(static_cast<char *>(workspace) + rec_bytes(g->n_dst, H));
-    }
-    FwdArgs ma;  // arguments of the merge launch
-    ma.n_dst = g->n_dst;
-    ma.indptr = g->indptr;
-    ma.indices = g->indices;
-    ma.feat = feat_q;
-    ma.el = el;
-    ma.er = er_q;
-    ma.acc = acc;
-    ma.m = m;
-    ma.d = d;
-    ma.out = out;
-    ma.slope = slope;
-    ma.flags = flags;
-    ma.g = s.geom;
-    ma.sp = split_args(g->split, part, H, F, true);
-    ma.mode = 0;
-    SpanArgs a{};
+    if (use_split && (!have_ws || workspace_bytes < w.csc)) return SAR_ERR_WORKSPACE;
+    RowArgs a{};
     a.n_rows = g->n_dst;
     a.indptr = g->indptr;
     a.indices = g->indices;
+    a.last_col = (unsigned)(g->n_src > 0 ? g->n_src - 1 : 0);
     a.gather = feat_q;
+    a.row_bytes = r.row_bytes;
     a.el = el;
     a.er = er_q;
-    a.acc_state = acc;
-    a.m_state = m;
-    a.d_state = d;
+    a.acc = acc;
+    a.m_io = m;
+    a.d_io = d;
     a.out = out;
     a.slope = slope;
     a.flags = flags;
-    a.g = s.geom;
-    a.sp = ma.sp;
-    a.hvec = (H % 4 == 0) && sar_aligned(er_q, 16);
-    const bool lean = lean_applies(s, flags, slope, g->split, g->n_src) && sar_aligned(er_q, 16);
-    // A partition step of a call-by-call pass.  The last one folds like the others and leaves the division to a
-    // launch of its own over all rows (most rows have no edge in a given partition, and every row has to be divided).
-    const bool lean_part = !(first && last) && lean_shape_applies(s, slope, g->split, g->n_src) && sar_aligned(er_q, 16) &&
-                           (g->nnz < (long long)kLeanPartMaxDegree * g->n_dst ||
-                            (g->nnz >= (long long)kLeanPartMinDenseDegree * g->n_dst && !first));
-    LeanArgs la{};
+    a.H = H;
+    a.F = F;
+    a.vph = r.vph;
+    a.ragged = r.ragged;
+    a.hvec = heads_aligned(H, r.geo.HP, {el, er_q});
+    a.sp = split_args(g->split, use_split ? reinterpret_cast<float *>(wsb + w.csr) : nullptr, H, r, t);
+    if (r.ragged) {
+        SAR_TRY(pad_rows(g->n_src, H, F, r, t, feat_q, wsb + w.feat, st));
+        a.gather = wsb + w.feat;
+    }
+    Shape s;
+    SAR_TRY(make_shape(H, F, t, !r.ragged, &s));
+    const bool lean_shape = lean_shape_applies(s, slope, g->split, g->n_src) && sar_aligned(er_q, 16);
+    const bool lean = lean_shape && !part;
+    const bool lean_part = lean_shape && part && !(first && last);
     if (lean || lean_part) {
+        LeanArgs la{};
         la.n_rows = g->n_dst;
         la.indptr = g->indptr;
         la.indices = g->indices;
@@ -327,32 +344,29 @@ sar_status sar_gat_fwd(const sar_part *g, const void *feat_q, const float *el, c
         la.out = out;
         la.relu = (flags & SAR_RELU_OUT) ? 1 : 0;
         la.slope = slope;
-        la.sp = ma.sp;
+        la.sp = a.sp;
         la.sp.threshold = g->split->threshold;
-    }
-    return dispatch(s, [&](auto cfg) -> sar_status {
-        using C = decltype(cfg);
-        using T = typename C::type;
-        if (lean)
-            SAR_TRY(s.t == SAR_F32 ? lean_fwd_f32(s, la, g->nnz, st) : lean_fwd_bf16(s, la, g->nnz, st));
-        else if (lean_part)
-            SAR_TRY(s.t == SAR_F32 ? lean_fwd_part_f32(s, la, g->nnz, st) : lean_fwd_part_bf16(s, la, g->nnz, st));
-        else
-            SAR_TRY((launch_span<T, C::g, C::v, UFwd<C::v>::u, kFwd, kCapFwd, kMinBlocksFwd>(a, g->nnz, "gat_fwd", "gat_fwd_seg", st)));
-        const bool divide_after = lean_part && last;
-        if (ma.sp.threshold > 0) {
-            FwdArgs mm = ma;
-            if (divide_after) mm.flags = 0;   // the long rows' state is folded like the others'
-            SAR_LAUNCH("gat_fwd_merge", st, gat_fwd_merge_kernel<T, C::g, C::v><<<blocks_for(mm.sp.n_long, C::g), kThreads, 0, st>>>(mm));
-            SAR_TRY(sar_after_launch());
+        if (lean) {
+            SAR_TRY(t == SAR_F32 ? lean_fwd_f32(s, la, g->nnz, st) : lean_fwd_bf16(s, la, g->nnz, st));
+            return use_split ? rows_fwd_merge(a, t, st) : SAR_OK;
         }
-        if (divide_after) {
-            const long long nv = g->n_dst * (long long)s.geom.n_vec;
-            SAR_LAUNCH("gat_fwd_finalize", st, gat_fwd_finalize_kernel<T><<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(ma));
-            SAR_TRY(sar_after_launch());
+        SAR_TRY(t == SAR_F32 ? lean_fwd_part_f32(s, la, g->nnz, st) : lean_fwd_part_bf16(s, la, g->nnz, st));
+        // The last step folds like the others; a launch of its own divides all rows (most have no edge in a given partition).
+        if (last) a.flags = first ? SAR_FIRST : 0;
+        if (use_split) SAR_TRY(rows_fwd_merge(a, t, st));
+        if (last) {
+            a.flags = flags;
+            SAR_TRY(rows_fwd_finalize(a, t, st));
         }
         return SAR_OK;
-    });
+    }
+    if (use_span(s, g->n_src))
+        SAR_TRY(span_fwd(s, a, g->nnz, st));
+    else if (part)
+        SAR_TRY(t == SAR_F32 ? rows_fwd_part_f32(a, r.geo, g->nnz, st) : rows_fwd_part_bf16(a, r.geo, g->nnz, st));
+    else
+        SAR_TRY(t == SAR_F32 ? rows_fwd_f32(a, r.geo, g->nnz, st) : rows_fwd_bf16(a, r.geo, g->nnz, st));
+    return use_split ? rows_fwd_merge(a, t, st) : SAR_OK;
 }
 
 static sar_status check_fused(const sar_part *g, int32_t k, const int64_t *bounds) {
@@ -440,18 +454,21 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
     if (g->n_src > 0 && (!feat_q || !er_q || !dfeat_q || !der_q)) return SAR_ERR_INVALID_ARG;
     SAR_TRY(check_elem_align({el, er_q, m, d, del, der_q}, 4));
     SAR_TRY(check_elem_align({feat_q, gout, dfeat_q}, sar_elem_size(t)));
-    Shape s;
-    SAR_TRY(make_shape(H, F, t, all16({feat_q, gout, dfeat_q}), &s));
-    const size_t need = rec_bytes(g->n_dst, H) + (s.fast ? part_bytes(g->split, H, F) + part_bytes(g->t_split, H, F) : 0);
-    if (!workspace || !sar_aligned(workspace, 16) || workspace_bytes < need) return SAR_ERR_WORKSPACE;
+    SAR_TRY(check_shape(H, F, t));
+    const RowShape r = row_shape(H, F, t);
+    const WsLayout w = ws_layout(g, H, r, t);
+    const bool rows = r.ok && (r.ragged ? workspace_bytes >= w.full : all16({feat_q, gout, dfeat_q}));
+    if (!workspace || !sar_aligned(workspace, 16) || workspace_bytes < (rows ? w.feat : w.plain)) return SAR_ERR_WORKSPACE;
     const bool whole = (flags & SAR_FIRST) && (flags & SAR_LAST);  // D rebuilt from the edges
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    float4 *rec = static_cast<float4 *>(workspace);
     char *wsb = static_cast<char *>(workspace);
-    float *part_csr = reinterpret_cast<float *>(wsb + rec_bytes(g->n_dst, H));
-    float *part_csc = reinterpret_cast<float *>(wsb + rec_bytes(g->n_dst, H) + part_bytes(g->split, H, F));
+    float4 *rec = reinterpret_cast<float4 *>(wsb);
+    // The padded copy of gout serves every step of a call-by-call pass: the first step makes it, whichever kernels it
+    // runs itself (its place does not depend on the partition).
+    if (r.ok && r.ragged && (flags & SAR_FIRST) && workspace_bytes >= w.csr)
+        SAR_TRY(pad_rows(g->n_dst, H, F, r, t, gout, wsb + w.gout, st));
 
-    if (!s.fast) {
+    if (!rows) {
         GenericArgs a{};
         a.n_dst = g->n_dst;
         a.n_src = g->n_src;
@@ -492,155 +509,110 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
         }
         return SAR_OK;
     }
-
-    BwdDstArgs da;  // merge launches
-    da.n_dst = g->n_dst;
-    da.indptr = g->indptr;
-    da.indices = g->indices;
-    da.feat = feat_q;
-    da.gout = gout;
-    da.el = el;
-    da.er = er_q;
-    da.m = m;
-    da.d = d;
-    da.rec = rec;
-    da.del = del;
-    da.slope = slope;
-    da.flags = flags;
-    da.g = s.geom;
-    da.sp = split_args(g->split, part_csr, H, F, true);
-    da.mode = 0;
-    BwdSrcArgs sa;
-    sa.n_src = g->n_src;
-    sa.t_indptr = g->t_indptr;
-    sa.t_indices = g->t_indices;
-    sa.gout = gout;
-    sa.feat = feat_q;
-    sa.er = er_q;
-    sa.rec = rec;
-    sa.dfeat = dfeat_q;
-    sa.der = der_q;
-    sa.slope = slope;
-    sa.g = s.geom;
-    sa.sp = split_args(g->t_split, part_csc, H, F, true);
-    sa.mode = 0;
-    SpanArgs d1{};  // destination-major pass over the CSR
-    d1.n_rows = g->n_dst;
-    d1.indptr = g->indptr;
-    d1.indices = g->indices;
-    d1.gather = feat_q;
-    d1.rowvec = gout;
-    d1.el = el;
-    d1.er = er_q;
-    d1.m = m;
-    d1.d = d;
-    d1.rec_in = rec;
-    d1.rec_out = rec;
-    d1.del = del;
-    d1.slope = slope;
-    d1.flags = flags;
-    d1.g = s.geom;
-    d1.sp = da.sp;
-    d1.hvec = (H % 4 == 0) && sar_aligned(er_q, 16);
-    SpanArgs s1{};  // source-major pass over the CSC
-    s1.n_rows = g->n_src;
-    s1.indptr = g->t_indptr;
-    s1.indices = g->t_indices;
-    s1.gather = gout;
-    s1.rowvec = feat_q;
-    s1.er = er_q;
-    s1.rec_in = rec;
-    s1.out = dfeat_q;
-    s1.der = der_q;
-    s1.slope = slope;
-    s1.flags = flags;
-    s1.g = s.geom;
-    s1.sp = sa.sp;
-    s1.hvec = (H % 4 == 0);
-
-    const bool lean_dst_shape = lean_shape_applies(s, slope, g->split, g->n_src) && sar_aligned(er_q, 16);
-    const bool lean_dst = whole && lean_dst_shape;
-    const bool lean_dst_part = !whole && lean_dst_shape;   // a partition step: D given, del collects
-    const bool lean_src = lean_shape_applies(s, slope, g->t_split, g->n_dst);   // whole graph or partition step alike
-    LeanArgs ld{};
-    LeanSrcArgs ls{};
-    if (lean_src) {
-        ls.n_rows = g->n_src;
-        ls.indptr = g->t_indptr;
-        ls.indices = g->t_indices;
-        ls.gather = gout;
-        ls.rowvec = feat_q;
-        ls.er = er_q;
-        ls.rec_in = rec;
-        ls.out = dfeat_q;
-        ls.der = der_q;
-        ls.slope = slope;
-        ls.sp = sa.sp;
-        ls.sp.threshold = g->t_split->threshold;
+    const void *feat_g = feat_q, *gout_g = gout;
+    if (r.ragged) {
+        SAR_TRY(pad_rows(g->n_src, H, F, r, t, feat_q, wsb + w.feat, st));
+        feat_g = wsb + w.feat;
+        gout_g = wsb + w.gout;
     }
-    if (lean_dst || lean_dst_part) {
-        ld.n_rows = g->n_dst;
-        ld.indptr = g->indptr;
-        ld.indices = g->indices;
-        ld.gather = feat_q;
-        ld.rowvec = gout;
-        ld.el = el;
-        ld.er = er_q;
-        ld.m = m;
-        ld.d = d;
-        ld.rec_out = rec;
-        ld.rec_in = rec;
-        ld.first = (flags & SAR_FIRST) ? 1 : 0;
-        ld.del = del;
-        ld.slope = slope;
-        ld.sp = da.sp;
-        ld.sp.threshold = g->split->threshold;
-    }
-
-    return dispatch(s, [&](auto cfg) -> sar_status {
-        using C = decltype(cfg);
-        using T = typename C::type;
-        constexpr int U = UBwd<C::v>::u;
-        const size_t msmem = (size_t)kWarpsPerBlock * warp_smem_floats(s.geom.Hp, C::v, 4) * 4;
-        if (g->n_dst > 0) {
-            if (whole) {
-                if (lean_dst)
-                    SAR_TRY(s.t == SAR_F32 ? lean_bwd_dst_f32(s, ld, g->nnz, st) : lean_bwd_dst_bf16(s, ld, g->nnz, st));
-                else
-                    SAR_TRY((launch_span<T, C::g, C::v, U, kBwdDst, kCapDst, kMinBlocksBwd>(d1, g->nnz, "gat_bwd_dst", "gat_bwd_dst_seg", st)));
-                if (da.sp.threshold > 0) {
-                    auto merge = gat_bwd_dst_merge_kernel<T, C::g, C::v, false>;
-                    SAR_TRY(ensure_smem(merge, msmem));
-                    SAR_LAUNCH("gat_bwd_dst_merge", st, merge<<<blocks_for(da.sp.n_long, C::g), kThreads, msmem, st>>>(da));
-                    SAR_TRY(sar_after_launch());
-                }
-            } else {
-                if (lean_dst_part)
-                    SAR_TRY(s.t == SAR_F32 ? lean_bwd_dst_part_f32(s, ld, g->nnz, st) : lean_bwd_dst_part_bf16(s, ld, g->nnz, st));
-                else
-                    SAR_TRY((launch_span<T, C::g, C::v, U, kBwdDstGivenD, kCapDst, kMinBlocksBwd>(d1, g->nnz, "gat_bwd_dst", "gat_bwd_dst_seg", st)));
-                if (da.sp.threshold > 0) {
-                    auto merge = gat_bwd_dst_merge_kernel<T, C::g, C::v, true>;
-                    SAR_TRY(ensure_smem(merge, msmem));
-                    SAR_LAUNCH("gat_bwd_dst_merge", st, merge<<<blocks_for(da.sp.n_long, C::g), kThreads, msmem, st>>>(da));
-                    SAR_TRY(sar_after_launch());
-                }
-            }
-        }
-        if (g->n_src > 0) {
-            if (lean_src)
-                SAR_TRY(s.t == SAR_F32 ? lean_bwd_src_f32(s, ls, g->nnz, st) : lean_bwd_src_bf16(s, ls, g->nnz, st));
+    RowArgs a{};
+    a.row_bytes = r.row_bytes;
+    a.el = el;
+    a.er = er_q;
+    a.m = m;
+    a.d = d;
+    a.rec = rec;
+    a.slope = slope;
+    a.flags = flags;
+    a.H = H;
+    a.F = F;
+    a.vph = r.vph;
+    a.ragged = r.ragged;
+    a.hvec = heads_aligned(H, r.geo.HP, {el, er_q, m, d});
+    Shape s;
+    SAR_TRY(make_shape(H, F, t, !r.ragged, &s));
+    if (g->n_dst > 0) {   // destination-major pass over the CSR
+        a.n_rows = g->n_dst;
+        a.indptr = g->indptr;
+        a.indices = g->indices;
+        a.last_col = (unsigned)(g->n_src > 0 ? g->n_src - 1 : 0);
+        a.gather = feat_g;
+        a.rowvec = gout_g;
+        a.dscal = del;
+        a.sp = split_args(g->split, reinterpret_cast<float *>(wsb + w.csr), H, r, t);
+        if (lean_shape_applies(s, slope, g->split, g->n_src) && sar_aligned(er_q, 16)) {
+            LeanArgs la{};
+            la.n_rows = g->n_dst;
+            la.indptr = g->indptr;
+            la.indices = g->indices;
+            la.gather = feat_q;
+            la.rowvec = gout;
+            la.el = el;
+            la.er = er_q;
+            la.m = m;
+            la.d = d;
+            la.rec_out = rec;
+            la.rec_in = rec;
+            la.first = (flags & SAR_FIRST) ? 1 : 0;
+            la.del = del;
+            la.slope = slope;
+            la.sp = a.sp;
+            la.sp.threshold = g->split->threshold;
+            if (whole)
+                SAR_TRY(t == SAR_F32 ? lean_bwd_dst_f32(s, la, g->nnz, st) : lean_bwd_dst_bf16(s, la, g->nnz, st));
             else
-                SAR_TRY((launch_span<T, C::g, C::v, U, kBwdSrc, kCapSrc, kMinBlocksBwd>(s1, g->nnz, "gat_bwd_src", "gat_bwd_src_seg", st)));
-            if (sa.sp.threshold > 0) {
-                auto merge = gat_bwd_src_merge_kernel<T, C::g, C::v>;
-                SAR_TRY(ensure_smem(merge, msmem));
-                SAR_LAUNCH("gat_bwd_src_merge", st, merge<<<blocks_for(sa.sp.n_long, C::g), kThreads, msmem, st>>>(sa));
-                SAR_TRY(sar_after_launch());
+                SAR_TRY(t == SAR_F32 ? lean_bwd_dst_part_f32(s, la, g->nnz, st) : lean_bwd_dst_part_bf16(s, la, g->nnz, st));
+        } else if (use_span(s, g->n_src)) {
+            SAR_TRY(span_dst(s, a, g->nnz, !whole, st));
+            a.n_rows = 0;   // the segments
+            if (a.sp.n_seg > 0) {
+                if (whole)
+                    SAR_TRY(t == SAR_F32 ? rows_dst_f32(a, r.geo, g->nnz, st) : rows_dst_bf16(a, r.geo, g->nnz, st));
+                else
+                    SAR_TRY(t == SAR_F32 ? rows_dst_part_f32(a, r.geo, g->nnz, st) : rows_dst_part_bf16(a, r.geo, g->nnz, st));
             }
+            a.n_rows = g->n_dst;
+        } else if (whole)
+            SAR_TRY(t == SAR_F32 ? rows_dst_f32(a, r.geo, g->nnz, st) : rows_dst_bf16(a, r.geo, g->nnz, st));
+        else
+            SAR_TRY(t == SAR_F32 ? rows_dst_part_f32(a, r.geo, g->nnz, st) : rows_dst_part_bf16(a, r.geo, g->nnz, st));
+        if (a.sp.n_long > 0) SAR_TRY(rows_dst_merge(a, !whole, st));
+    }
+    if (g->n_src > 0) {   // source-major pass over the CSC
+        a.n_rows = g->n_src;
+        a.indptr = g->t_indptr;
+        a.indices = g->t_indices;
+        a.last_col = (unsigned)(g->n_dst - 1);
+        a.gather = gout_g;
+        a.rowvec = feat_g;
+        a.out = dfeat_q;
+        a.dscal = der_q;
+        a.sp = split_args(g->t_split, reinterpret_cast<float *>(wsb + w.csc), H, r, t);
+        if (lean_shape_applies(s, slope, g->t_split, g->n_dst)) {
+            LeanSrcArgs la{};
+            la.n_rows = g->n_src;
+            la.indptr = g->t_indptr;
+            la.indices = g->t_indices;
+            la.gather = gout;
+            la.rowvec = feat_q;
+            la.er = er_q;
+            la.rec_in = rec;
+            la.out = dfeat_q;
+            la.der = der_q;
+            la.slope = slope;
+            la.sp = a.sp;
+            la.sp.threshold = g->t_split->threshold;
+            SAR_TRY(t == SAR_F32 ? lean_bwd_src_f32(s, la, g->nnz, st) : lean_bwd_src_bf16(s, la, g->nnz, st));
+        } else {
+            if (use_span(s, g->n_dst)) {
+                SAR_TRY(span_src(s, a, g->nnz, st));
+                a.n_rows = 0;   // the segments
+            }
+            SAR_TRY(t == SAR_F32 ? rows_src_f32(a, r.geo, g->nnz, st) : rows_src_bf16(a, r.geo, g->nnz, st));
         }
-        return SAR_OK;
-    });
+        if (a.sp.n_long > 0) SAR_TRY(rows_src_merge(a, t, st));
+    }
+    return SAR_OK;
 }
 
 sar_status sar_gat_bwd_fused(const sar_part *g, int32_t k, const int64_t *bounds, const void *feat, const float *el,
@@ -663,12 +635,14 @@ static sar_status spmm_impl(const sar_part *g, const void *feat_q, int32_t F, sa
     SAR_TRY(check_elem_align({feat_q, out}, sar_elem_size(t)));
     SAR_TRY(check_elem_align({deg_total}, 8));
     SAR_TRY(check_elem_align({src_scale, dst_scale}, 4));
-    const bool weighted = src_scale || dst_scale;
-    Shape s;
-    SAR_TRY(make_shape(1, F, t, all16({feat_q, out}), &s));
+    SAR_TRY(check_shape(1, F, t));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (g->n_dst == 0) return SAR_OK;
-    if (!s.fast) {
+    const RowShape r = sum_shape(F, t);
+    const size_t parts = part_bytes(g->split, 1, r, t);
+    const bool have_ws = workspace && sar_aligned(workspace, 16);
+    const bool rows = r.ragged ? have_ws && workspace_bytes >= parts + pad_bytes(g->n_src, r) : all16({feat_q, out});
+    if (!rows) {
         GenericArgs a{};
         a.n_dst = g->n_dst;
         a.indptr = g->indptr;
@@ -689,45 +663,36 @@ static sar_status spmm_impl(const sar_part *g, const void *feat_q, int32_t F, sa
         return sar_after_launch();
     }
     const bool use_split = g->split && g->split->n_long > 0;
-    if (use_split && (!workspace || !sar_aligned(workspace, 16) || workspace_bytes < part_bytes(g->split, 1, F)))
-        return SAR_ERR_WORKSPACE;
-    SumArgs ma;  // merge launch
-    ma.n_dst = g->n_dst;
-    ma.indptr = g->indptr;
-    ma.indices = g->indices;
-    ma.feat = feat_q;
-    ma.out = out;
-    ma.deg_total = deg_total;
-    ma.dst_scale = dst_scale;
-    ma.flags = flags;
-    ma.g = s.geom;
-    ma.sp = split_args(g->split, static_cast<float *>(workspace), 1, F, true);
-    ma.mode = 0;
-    SpanArgs a{};
+    if (use_split && (!have_ws || workspace_bytes < parts)) return SAR_ERR_WORKSPACE;
+    RowArgs a{};
     a.n_rows = g->n_dst;
     a.indptr = g->indptr;
     a.indices = g->indices;
+    a.last_col = (unsigned)(g->n_src > 0 ? g->n_src - 1 : 0);
     a.gather = feat_q;
+    a.row_bytes = r.row_bytes;
     a.out = out;
-    a.deg_total = deg_total;
+    a.deg = deg_total;
     a.src_scale = src_scale;
     a.dst_scale = dst_scale;
     a.flags = flags;
-    a.g = s.geom;
-    a.sp = ma.sp;
-    return dispatch(s, [&](auto cfg) -> sar_status {
-        using C = decltype(cfg);
-        using T = typename C::type;
-        if (weighted)
-            SAR_TRY((launch_span<T, C::g, C::v, UFwd<C::v>::u, kSumW, kCapSum, kMinBlocksFwd>(a, g->nnz, "spmm", "spmm_seg", st)));
-        else
-            SAR_TRY((launch_span<T, C::g, C::v, UFwd<C::v>::u, kSum, kCapSum, kMinBlocksFwd>(a, g->nnz, "spmm", "spmm_seg", st)));
-        if (ma.sp.threshold > 0) {
-            SAR_LAUNCH("spmm_merge", st, spmm_merge_kernel<T, C::g, C::v><<<blocks_for(ma.sp.n_long, C::g), kThreads, 0, st>>>(ma));
-            SAR_TRY(sar_after_launch());
-        }
-        return SAR_OK;
-    });
+    a.H = 1;
+    a.F = F;
+    a.vph = r.vph;
+    a.ragged = r.ragged;
+    a.sp = split_args(g->split, static_cast<float *>(workspace), 1, r, t);
+    if (r.ragged) {
+        SAR_TRY(pad_rows(g->n_src, 1, F, r, t, feat_q, static_cast<char *>(workspace) + parts, st));
+        a.gather = static_cast<char *>(workspace) + parts;
+    }
+    const bool weighted = src_scale != nullptr;
+    Shape s;
+    SAR_TRY(make_shape(1, F, t, !r.ragged, &s));
+    if (use_span(s, g->n_src, kSpanSumBytes))
+        SAR_TRY(span_sum(s, a, g->nnz, weighted, st));
+    else
+        SAR_TRY(t == SAR_F32 ? rows_sum_f32(a, r.geo, g->nnz, weighted, st) : rows_sum_bf16(a, r.geo, g->nnz, weighted, st));
+    return use_split ? rows_sum_merge(a, t, st) : SAR_OK;
 }
 
 sar_status sar_spmm_agg(const sar_part *g, const void *feat_q, int32_t F, sar_dtype t, uint32_t flags,

@@ -44,15 +44,11 @@ struct LeanSrcArgs {
 };
 
 constexpr int kLeanCap = 256;   // edges a chunk stages; rows and segments must not exceed it
-// A forward partition step takes the lean partition-step kernel when the partition holds fewer than kLeanPartMaxDegree
-// edges per row (mostly empty rows: what the kernel is laid out for) or at least kLeanPartMinDenseDegree (a span then
-// holds few rows, all or most of them with their numerator staged).  In between - short rows, nearly all with edges,
-// 31 of them per span but room for the numerators of 8 - span_kernel is faster.  Per step, partition-step kernel
-// against span_kernel: large workload (0.94 edges per row and partition) 3.0 against 6.1 ms, first step 3.1 against
-// 5.8 ms, last step 5.1 against 11.1 ms; dense workload (25 edges) 2.38 against 2.64 ms; medium workload (6.3 edges)
-// 2.05 against 1.93 ms, last step 2.59 against 2.01 ms.
-constexpr int kLeanPartMaxDegree = 2;
-constexpr int kLeanPartMinDenseDegree = 16;
+// Where the lean kernels cover a shape they take every pass of it; the row kernels (sar_rows_kernel.cuh) take the others.
+// Both cover these shapes; measured on them, lean against row kernels, bf16, 4 heads of 32, forward / destination-major /
+// source-major: large workload 15.2 / 15.2 / 16.8 against 20.2 / 20.1 / 32.7 ms, 100,000 nodes and 2 million edges
+// 117 / 116 / 120 against 115 / 111 / 181 us; a partition step of the large workload 3.0 / 2.2 / 1.0 against
+// 3.9 / 2.8 / 2.1 ms.
 
 // Do the lean kernels cover this shape?  Slope >= 0, heads in groups of four, rows of
 // exactly G*V vectors with V <= 2, the vectors of a head a power of two within one lane group, and a long-row

@@ -3,8 +3,8 @@
 // pass for the common shapes (heads in groups of four, rows of exactly G*V 16-byte vectors), written for the fewest
 // issued instructions per edge.
 //
-// Same plan as span_kernel (sar_span_kernels.cuh) - a warp owns a span of consecutive rows, stages a chunk of whole
-// rows in shared memory slot-major and streams the gathered rows through a cp.async ring - with these differences:
+// The plan: a warp owns a span of consecutive rows, stages a chunk of whole
+// rows in shared memory slot-major and streams the gathered rows through a cp.async ring:
 //   * The ring works in STAGES of 2 or 4 KB (SPS slots): one commit group and one wait per stage, the slots of a
 //     stage walked with compile-time offsets (fully unrolled), the stage refilled as a whole.  The staged column ids
 //     are pre-scaled row offsets in 16-byte units, stored per stage with the slot index fastest, so that one
@@ -21,12 +21,12 @@
 //     (slope >= 0) and runs online, stage by stage.
 //   * Dot products of the backward epilogues are taken on the un-folded accumulators and reduced with three shuffles
 //     per quantity; per-(row, head) scalars leave through shared memory, coalesced, once per chunk.
-// Preconditions (checked by the host, which otherwise launches span_kernel): SAR_FIRST|SAR_LAST, slope >= 0, every row of
+// Preconditions (checked by the host, which otherwise launches the row kernels): SAR_FIRST|SAR_LAST, slope >= 0, every row of
 // the rows launch at most CAP edges (a long-row plan with threshold <= CAP), segments of at most CAP edges, fewer
 // than 2^32 16-byte vectors in the gathered array.
 #pragma once
 
-#include "sar_span_kernels.cuh"
+#include "sar_device.cuh"
 #include "sar_lean.cuh"
 #include "sar_dispatch.cuh"
 
@@ -84,12 +84,19 @@ constexpr int kLeanMinBlocksBwdRows = 24;
 // Resident blocks per SM the rows launch of a partition step is compiled for.
 constexpr int kLeanMinBlocksPart = 16;
 
+constexpr int kMaxSpanRows = 16;   // rows a span holds at most
+
+// Rows per span: about `cap` edges (the long rows counted in the average are skipped), but no more than leaves every SM
+// kLeanFill spans: a graph with fewer is done when its longest span is.
+constexpr int kLeanSMs = 148, kLeanFill = 24;
 static inline int lean_rows_per_span(long long n_rows, long long nnz, int cap, int max_rows = kMaxSpanRows) {
     const double avg = n_rows > 0 ? (double)nnz / (double)n_rows : 0.0;
-    int R = avg > 0.5 ? (int)(1.0 * cap / avg + 0.5) : max_rows;
+    long long R = avg > 0.5 ? (long long)(1.0 * cap / avg + 0.5) : max_rows;
+    const long long fill = n_rows / (kLeanSMs * kLeanFill);
+    if (R > fill) R = fill;
     if (R < 1) R = 1;
     if (R > max_rows) R = max_rows;
-    return R;
+    return (int)R;
 }
 
 }  // namespace sar

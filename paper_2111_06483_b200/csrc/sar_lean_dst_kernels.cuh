@@ -129,14 +129,17 @@ __global__ void __launch_bounds__(32, MINB) lean_dst_kernel(const LeanArgs a) {
     // the (position, head) pairs this lane copies the record of and scores: it = lane (+ 32)
     constexpr int NIT = (ITEMS + 31) / 32;
 
-    f32x2 pacc0[V][NP], pacc1[V][NP];
+    // D and del are linear in the dot products <gout_i, feat_j>: a lane adds up alpha (and alpha g') times its own 16
+    // bytes' share of them, and the lanes of a head meet once per row.
+    f32x2 go[V][NP], d2[V], b2[V];   // the row's gout; sum alpha <.,.>; sum alpha g' <.,.>
     float sv[V];
     uint4 rvq[V], rvq_next[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         sv[v] = 0.f;
+        d2[v] = b2[v] = zero2();
 #pragma unroll
-        for (int k = 0; k < NP; ++k) pacc0[v][k] = pacc1[v][k] = zero2();
+        for (int k = 0; k < NP; ++k) go[v][k] = zero2();
         rvq[v] = rvq_next[v] = make_uint4(0u, 0u, 0u, 0u);
     }
     auto request_rowvec = [&](long long row_, uint4 (&dst)[V]) {
@@ -332,8 +335,8 @@ __global__ void __launch_bounds__(32, MINB) lean_dst_kernel(const LeanArgs a) {
             cp_async_commit();
         }
 
-        if constexpr (!SEG && !PART) {
-            if (nslots > 0) request_rowvec(row0 + r + (__ffs(nemask) - 1), rvq_next);
+        if constexpr (!PART) {
+            if (nslots > 0) request_rowvec(row0 + r + (SEG ? 0 : __ffs(nemask) - 1), rvq_next);
         }
 
         // ---- the stages ------------------------------------------------------------------------------------------
@@ -342,6 +345,29 @@ __global__ void __launch_bounds__(32, MINB) lean_dst_kernel(const LeanArgs a) {
             int ri = SEG ? 0 : (__ffs(nemask) - 1);
             unsigned staged_row = rowst_s + (unsigned)(gl * 16);   // partition step: gout of the row in progress
             int staged_left = kLeanPartStaged;                     // ... and how many more rows found room
+            // row `ri` begins: its gout, asked for one row ahead (a partition step: staged with the chunk, or loaded here when
+            // the chunk has more rows with edges than there was room for)
+            auto open_row = [&]() {
+                if constexpr (PART) {
+                    if (staged_left > 0) {
+#pragma unroll
+                        for (int v = 0; v < V; ++v) rvq[v] = lds128(staged_row + (unsigned)(v * G * 16));
+                        staged_row += ROWB;
+                        --staged_left;
+                    } else {
+                        request_rowvec(row0 + r + ri, rvq);
+                    }
+                } else {
+#pragma unroll
+                    for (int v = 0; v < V; ++v) rvq[v] = rvq_next[v];
+                    if constexpr (!SEG) {
+                        const unsigned rest = nemask & ~((2u << ri) - 1u);
+                        if (rest) request_rowvec(row0 + r + (__ffs(rest) - 1), rvq_next);
+                    }
+                }
+#pragma unroll
+                for (int v = 0; v < V; ++v) Pairs<T>::get(rvq[v], go[v]);
+            };
             for (int j = 0; j < nstages; ++j) {
                 cp_async_wait<NS - 1>();
                 __syncwarp();   // the records of this stage were copied by other lanes; the previous weights are consumed
@@ -365,6 +391,7 @@ __global__ void __launch_bounds__(32, MINB) lean_dst_kernel(const LeanArgs a) {
                     }
                 }
                 __syncwarp();
+                if (j == 0) open_row();
                 const unsigned ring_a = ring_l + (unsigned)((j % NS) * STAGE);
                 const int cnt = nslots - s;
                 unsigned ends;
@@ -393,79 +420,20 @@ __global__ void __launch_bounds__(32, MINB) lean_dst_kernel(const LeanArgs a) {
                         const float al = fabsf(wk);
                         const float wg = wk < 0.f ? al * a.slope : al;   // alpha * LeakyReLU'
                         sv[v] += wg;
-                        const f32x2 a2 = pack2(al, al), g2 = pack2(wg, wg);
+                        f32x2 dot = fma2(x[0], go[v][0], zero2());
 #pragma unroll
-                        for (int t = 0; t < NP; ++t) {
-                            if constexpr (!PART) pacc0[v][t] = fma2(a2, x[t], pacc0[v][t]);   // A is for D, given to a partition step
-                            pacc1[v][t] = fma2(g2, x[t], pacc1[v][t]);
-                        }
+                        for (int t = 1; t < NP; ++t) dot = fma2(x[t], go[v][t], dot);
+                        if constexpr (!PART) d2[v] = fma2(pack2(al, al), dot, d2[v]);   // for D, given to a partition step
+                        b2[v] = fma2(pack2(wg, wg), dot, b2[v]);
                     }
                     if (ends & (1u << k)) {
                         // ---- the row is complete -------------------------------------------------------------
-                        const long long row = row0 + r + ri;
-                        if constexpr (PART) {
-                            if (staged_left > 0) {
-#pragma unroll
-                                for (int v = 0; v < V; ++v) rvq[v] = lds128(staged_row + (unsigned)(v * G * 16));
-                                staged_row += ROWB;
-                                --staged_left;
-                            } else {   // more rows with edges in this chunk than there was room for
-                                request_rowvec(row, rvq);
-                            }
-                        } else if constexpr (!SEG) {
-#pragma unroll
-                            for (int v = 0; v < V; ++v) rvq[v] = rvq_next[v];
-                            const unsigned rest = nemask & ~((2u << ri) - 1u);
-                            if (rest) request_rowvec(row0 + r + (__ffs(rest) - 1), rvq_next);
-                        }
-                        if constexpr (SEG) {
-                            float acc0[V][EPV], acc1[V][EPV];
-#pragma unroll
-                            for (int v = 0; v < V; ++v)
-#pragma unroll
-                                for (int t = 0; t < NP; ++t) {
-                                    unpack2(pacc0[v][t], acc0[v][2 * t], acc0[v][2 * t + 1]);
-                                    unpack2(pacc1[v][t], acc1[v][2 * t], acc1[v][2 * t + 1]);
-                                }
-#pragma unroll
-                            for (int off = G; off < 32; off <<= 1)
-#pragma unroll
-                                for (int v = 0; v < V; ++v) {
-                                    sv[v] += __shfl_xor_sync(0xffffffffu, sv[v], off);
-#pragma unroll
-                                    for (int e = 0; e < EPV; ++e) {
-                                        acc0[v][e] += __shfl_xor_sync(0xffffffffu, acc0[v][e], off);
-                                        acc1[v][e] += __shfl_xor_sync(0xffffffffu, acc1[v][e], off);
-                                    }
-                                }
-                            if (half == 0) {
-                                constexpr long long rowf = (long long)NVEC * EPV;
-                                float *rec = a.sp.part + seg * a.sp.pstride;
-                                bool vok[V];
-#pragma unroll
-                                for (int v = 0; v < V; ++v) vok[v] = true;
-                                store_acc_row<G, V, EPV>(rec, gl, vok, acc1);
-                                store_acc_row<G, V, EPV>(rec + rowf, gl, vok, acc0);
-#pragma unroll
-                                for (int v = 0; v < V; ++v)
-                                    if ((gl % VPH) == 0) rec[2 * rowf + hv[v]] = sv[v];
-                            }
-                        } else {
-                            // <gout_i, A> and <gout_i, B> on the un-folded accumulators, reduced over the lanes of each
-                            // head and over the edge lanes
-                            float pA[V], pB[V];
+                        {
+                            float pA[V], pB[V];   // reduced over the lanes of each head and over the edge lanes
 #pragma unroll
                             for (int v = 0; v < V; ++v) {
-                                f32x2 rv[NP];
-                                Pairs<T>::get(rvq[v], rv);
-                                f32x2 qa = zero2(), qb = zero2();
-#pragma unroll
-                                for (int t = 0; t < NP; ++t) {
-                                    if constexpr (!PART) qa = fma2(rv[t], pacc0[v][t], qa);
-                                    qb = fma2(rv[t], pacc1[v][t], qb);
-                                }
-                                pA[v] = qa.x + qa.y;
-                                pB[v] = qb.x + qb.y;
+                                pA[v] = d2[v].x + d2[v].y;
+                                pB[v] = b2[v].x + b2[v].y;
                             }
 #pragma unroll
                             for (int off = 1; off < 32; off <<= 1) {
@@ -478,6 +446,17 @@ __global__ void __launch_bounds__(32, MINB) lean_dst_kernel(const LeanArgs a) {
                                     }
                                 }
                             }
+                            if constexpr (SEG) {   // the segment's D, B and S per head, for the merge launch
+                                if ((gl % VPH) == 0 && half == 0) {
+                                    float *rec = a.sp.part + seg * a.sp.pstride;
+#pragma unroll
+                                    for (int v = 0; v < V; ++v) {
+                                        rec[hv[v]] = pA[v];
+                                        rec[H + hv[v]] = pB[v];
+                                        rec[2 * H + hv[v]] = sv[v];
+                                    }
+                                }
+                            } else
                             if ((gl % VPH) == 0 && half == 0) {
 #pragma unroll
                                 for (int v = 0; v < V; ++v) {
@@ -494,12 +473,12 @@ __global__ void __launch_bounds__(32, MINB) lean_dst_kernel(const LeanArgs a) {
 #pragma unroll
                         for (int v = 0; v < V; ++v) {
                             sv[v] = 0.f;
-#pragma unroll
-                            for (int t = 0; t < NP; ++t) pacc0[v][t] = pacc1[v][t] = zero2();
+                            d2[v] = b2[v] = zero2();
                         }
                         if constexpr (!SEG) {
                             const unsigned rest = nemask & ~((2u << ri) - 1u);
                             ri = rest ? __ffs(rest) - 1 : nr;
+                            if (rest) open_row();
                         }
                         if (k + 1 >= cnt) goto chunk_done;
                     }

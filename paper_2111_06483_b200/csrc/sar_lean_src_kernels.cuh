@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(32, MINB) lean_src_kernel(const LeanSrcArgs a)
                 uint4 *rp = reinterpret_cast<uint4 *>(a.out) + (row0 + r + i) * NVEC;
                 for (int x = lane; x < NVEC; x += 32) rp[x] = make_uint4(0u, 0u, 0u, 0u);
             }
-            if (nslots > 0) request_rowvec(row0 + r + (__ffs(nemask) - 1), rvq_next);
         }
+        if (nslots > 0) request_rowvec(row0 + r + (SEG ? 0 : __ffs(nemask) - 1), rvq_next);
 
         // ---- the stages ------------------------------------------------------------------------------------------
         {
@@ -346,9 +346,9 @@ __global__ void __launch_bounds__(32, MINB) lean_src_kernel(const LeanSrcArgs a)
                     if (ends & (1u << k)) {
                         // ---- the row is complete -------------------------------------------------------------
                         const long long row = row0 + r + ri;
-                        if constexpr (!SEG) {
 #pragma unroll
-                            for (int v = 0; v < V; ++v) rvq[v] = rvq_next[v];
+                        for (int v = 0; v < V; ++v) rvq[v] = rvq_next[v];
+                        if constexpr (!SEG) {
                             const unsigned rest = nemask & ~((2u << ri) - 1u);
                             if (rest) request_rowvec(row0 + r + (__ffs(rest) - 1), rvq_next);
                         }
@@ -357,36 +357,7 @@ __global__ void __launch_bounds__(32, MINB) lean_src_kernel(const LeanSrcArgs a)
                         for (int v = 0; v < V; ++v)
 #pragma unroll
                             for (int t = 0; t < NP; ++t) unpack2(pacc0[v][t], acc0[v][2 * t], acc0[v][2 * t + 1]);
-                        if constexpr (SEG) {
-                            float acc1[V][EPV];
-#pragma unroll
-                            for (int v = 0; v < V; ++v)
-#pragma unroll
-                                for (int t = 0; t < NP; ++t) unpack2(pacc1[v][t], acc1[v][2 * t], acc1[v][2 * t + 1]);
-#pragma unroll
-                            for (int off = G; off < 32; off <<= 1)
-#pragma unroll
-                                for (int v = 0; v < V; ++v) {
-                                    sv[v] += __shfl_xor_sync(0xffffffffu, sv[v], off);
-#pragma unroll
-                                    for (int e = 0; e < EPV; ++e) {
-                                        acc0[v][e] += __shfl_xor_sync(0xffffffffu, acc0[v][e], off);
-                                        acc1[v][e] += __shfl_xor_sync(0xffffffffu, acc1[v][e], off);
-                                    }
-                                }
-                            if (half == 0) {
-                                constexpr long long rowf = (long long)NVEC * EPV;
-                                float *rec = a.sp.part + seg * a.sp.pstride;
-                                bool vok[V];
-#pragma unroll
-                                for (int v = 0; v < V; ++v) vok[v] = true;
-                                store_acc_row<G, V, EPV>(rec, gl, vok, acc0);
-                                store_acc_row<G, V, EPV>(rec + rowf, gl, vok, acc1);
-#pragma unroll
-                                for (int v = 0; v < V; ++v)
-                                    if ((gl % VPH) == 0) rec[2 * rowf + hv[v]] = sv[v];
-                            }
-                        } else {
+                        {
                             // <feat_j, C> on the un-folded accumulator, reduced over the lanes of each head and the edge lanes
                             float pC[V];
 #pragma unroll
@@ -414,6 +385,19 @@ __global__ void __launch_bounds__(32, MINB) lean_src_kernel(const LeanSrcArgs a)
                                 for (int v = 0; v < V; ++v)
 #pragma unroll
                                     for (int e = 0; e < EPV; ++e) acc0[v][e] += __shfl_xor_sync(0xffffffffu, acc0[v][e], off);
+                            if constexpr (SEG) {   // the segment's share of dfeat (float32) and of der, for the merge launch
+                                if (half == 0) {
+                                    constexpr long long rowf = (long long)NVEC * EPV;
+                                    float *rec = a.sp.part + seg * a.sp.pstride;
+                                    bool vok[V];
+#pragma unroll
+                                    for (int v = 0; v < V; ++v) vok[v] = true;
+                                    store_acc_row<G, V, EPV>(rec, gl, vok, acc0);
+#pragma unroll
+                                    for (int v = 0; v < V; ++v)
+                                        if ((gl % VPH) == 0) rec[rowf + hv[v]] = pC[v] - sv[v];
+                                }
+                            } else
                             if (half == 0) {
                                 uint4 *rp = reinterpret_cast<uint4 *>(a.out) + row * NVEC + gl;
 #pragma unroll

@@ -44,10 +44,7 @@ sar_status sar_gat_bwd_noalloc(const sar_part *g, const void *feat, const float 
                                const float *d, const void *gout, int32_t H, int32_t F, sar_dtype t, float slope,
                                void *dfeat, float *del, float *der, void *stream) {
     if (!g || H < 1 || F < 1) return SAR_ERR_INVALID_ARG;
-    // what the ordinary entry point would ask its caller for; it must fit the fixed array
-    const size_t need = sar_gat_workspace_bytes(g, H, F, t);
-    if (need == 0) return SAR_ERR_INVALID_ARG;
-    if (need > SAR_NOALLOC_SCRATCH_BYTES) return SAR_ERR_WORKSPACE;
+    // A problem that needs more than the fixed array is refused by the entry point below.
     void *scratch = nullptr;
     SAR_TRY(scratch_for_current_device(&scratch));
     // Whole graph in one call: the destination-major pass writes every record and every long-row

@@ -1,0 +1,49 @@
+// Launch of the row kernels (internal): grid, rows per warp, and the instantiation that fits a geometry.
+#pragma once
+
+#include "sar_dispatch.cuh"
+#include "sar_rows_kernel.cuh"
+
+namespace sar {
+
+constexpr int kRowSMs = 148;
+
+// Rows a warp takes: several, so that their row pointers are one load and the next row's column ids can be asked for a
+// row ahead, but no more than leaves every SM kRowFill warps.
+constexpr int kRowMax = 8, kRowFill = 64;
+static inline int rows_per_warp(long long n_rows) {
+    const long long R = n_rows / (kRowSMs * kRowFill);
+    return R < 1 ? 1 : R > kRowMax ? kRowMax : (int)R;
+}
+
+template <typename T, int NV, int HP, int MODE>
+static sar_status launch_row_kernel(RowArgs a, RowGeo g, long long nnz, const char *name, cudaStream_t st) {
+    constexpr int MINB = NV >= 256 ? 2 : NV == 128 ? 4 : (NV == 64 || HP == 8) ? 7 : 8;   // 32 warps per SM at 64 registers (7 and 10 blocks: 2 and 10 % slower)
+    a.nnz = nnz;
+    a.R = rows_per_warp(a.n_rows);
+    const long long items = a.sp.n_seg + (a.n_rows + a.R - 1) / a.R;
+    if (items <= 0) return SAR_OK;
+    constexpr size_t smem = (size_t)kRowWarps * RowSmem<HP, MODE>::total * 4;
+    auto kern = row_kernel<T, NV, HP, MODE, MINB>;
+    SAR_TRY(ensure_smem(kern, smem));
+    const dim3 grid((unsigned)((items + kRowWarps - 1) / kRowWarps), (unsigned)g.tiles);
+    SAR_LAUNCH(name, st, (kern<<<grid, kRowWarps * 32, smem, st>>>(a)));
+    return sar_after_launch();
+}
+
+template <typename T, int MODE>
+static sar_status dispatch_rows(const RowArgs &a, RowGeo g, long long nnz, const char *name, cudaStream_t st) {
+#define SAR_ROW_CASE(NV_, HP_) \
+    if (g.NV == NV_ && g.HP == HP_) return launch_row_kernel<T, NV_, HP_, MODE>(a, g, nnz, name, st);
+    SAR_ROW_CASE(4, 1) SAR_ROW_CASE(8, 1) SAR_ROW_CASE(16, 1) SAR_ROW_CASE(32, 1) SAR_ROW_CASE(64, 1)
+    SAR_ROW_CASE(128, 1) SAR_ROW_CASE(256, 1)
+    if constexpr (MODE != kRowSum && MODE != kRowSumW) {
+        SAR_ROW_CASE(4, 2) SAR_ROW_CASE(8, 2) SAR_ROW_CASE(16, 2) SAR_ROW_CASE(32, 2) SAR_ROW_CASE(64, 2)
+        SAR_ROW_CASE(4, 4) SAR_ROW_CASE(8, 4) SAR_ROW_CASE(16, 4) SAR_ROW_CASE(32, 4) SAR_ROW_CASE(64, 4)
+        SAR_ROW_CASE(8, 8) SAR_ROW_CASE(16, 8) SAR_ROW_CASE(32, 8) SAR_ROW_CASE(64, 8)
+    }
+#undef SAR_ROW_CASE
+    return SAR_ERR_UNSUPPORTED;
+}
+
+}  // namespace sar

@@ -1,0 +1,241 @@
+// Long rows, from their segments' records (see sar_rows_kernel.cuh): one block per long row.  The records of a hub row
+// (hundreds) are read by several streams of threads at once - a thread holds one float4 column of every kStreams-th
+// record - and the streams are added up in shared memory in a fixed order, so a result does not depend on the schedule.
+// Large workload, three merges of a layer (0.28-0.30 ms each with one lane group per long row walking all its records).
+#include "sar_dispatch.cuh"
+#include "sar_rows.cuh"
+
+namespace sar {
+
+constexpr int kMergeThreads = 128;
+
+__device__ __forceinline__ void add4(float4 &a, const float4 &b, float f) {
+    a.x = fmaf(b.x, f, a.x);
+    a.y = fmaf(b.y, f, a.y);
+    a.z = fmaf(b.z, f, a.z);
+    a.w = fmaf(b.w, f, a.w);
+}
+
+// Elements of a finished row.  `c` = first float of the column in the padded row (heads of vph*EPV floats).
+template <typename T, typename Fn>
+__device__ __forceinline__ void merge_store(const RowArgs &a, long long row, int c, const float4 &x, Fn &&finish) {
+    const int fp = a.vph * Elem<T>::EPV;
+    const float v[4] = {x.x, x.y, x.z, x.w};
+    const int head = c / fp, f0 = c - head * fp;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (f0 + k < a.F) finish(row * (long long)a.H * a.F + (long long)head * a.F + f0 + k, head, v[k]);
+}
+
+// Sum over a row's records of (column of the record) x (factor of (record, head)); valid in the threads of stream 0.
+template <typename Fn>
+__device__ __forceinline__ float4 merge_columns(const RowArgs &a, long long s0, long long s1, int c, int stream, int streams,
+                                                float4 *red, int cols_pad, int col, Fn &&factor) {
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    long long s = s0 + stream;
+    for (; s + 3LL * streams < s1; s += 4LL * streams) {
+        float4 r[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) r[u] = *reinterpret_cast<const float4 *>(a.sp.part + (s + (long long)u * streams) * a.sp.pstride + c);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) add4(x, r[u], factor(s + (long long)u * streams));
+    }
+    for (; s < s1; s += streams) add4(x, *reinterpret_cast<const float4 *>(a.sp.part + s * a.sp.pstride + c), factor(s));
+    if (streams > 1) {
+        if (stream < streams) red[stream * cols_pad + col] = x;
+        __syncthreads();
+        if (stream == 0)
+            for (int k = 1; k < streams; ++k) add4(x, red[k * cols_pad + col], 1.f);
+        __syncthreads();
+    }
+    return x;
+}
+
+// MODE: kRowFwd / kRowFwdPart, kRowSrc, kRowSum
+template <typename T, int MODE>
+__global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs a) {
+    constexpr int EPV = Elem<T>::EPV;
+    constexpr bool kF = MODE == kRowFwd;
+    __shared__ float4 red[kMergeThreads];
+    __shared__ float sM[SAR_MAX_HEADS], sD[SAR_MAX_HEADS], sOld[SAR_MAX_HEADS];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long row = a.sp.long_row[blockIdx.x];
+    const long long s0 = a.sp.long_seg[blockIdx.x], s1 = a.sp.long_seg[blockIdx.x + 1];
+    const int rowf = a.H * a.vph * EPV;
+    const bool first = a.flags & SAR_FIRST, last = a.flags & SAR_LAST;
+
+    if constexpr (kF) {   // statistics of the row: a warp per head
+        for (int h = warp; h < a.H; h += kMergeThreads / 32) {
+            float M = SAR_NEG_INF;
+            for (long long s = s0 + lane; s < s1; s += 32) M = fmaxf(M, a.sp.part[s * a.sp.pstride + rowf + h]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+            const float m_old = first ? SAR_NEG_INF : a.m_io[row * a.H + h], d_old = first ? 0.f : a.d_io[row * a.H + h];
+            const float mn = fmaxf(M, m_old);
+            float d = 0.f;
+            for (long long s = s0 + lane; s < s1; s += 32) {
+                const float *rec = a.sp.part + s * a.sp.pstride + rowf;
+                d += rec[a.H + h] * fast_exp(rec[h] - mn);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            const float fo = m_old == mn ? 1.f : fast_exp(m_old - mn);
+            d += d_old * fo;
+            if (lane == 0) {
+                sM[h] = mn;
+                sD[h] = d;
+                sOld[h] = fo;
+            }
+        }
+        __syncthreads();
+        if (tid < a.H) {
+            a.m_io[row * a.H + tid] = sM[tid];
+            a.d_io[row * a.H + tid] = sD[tid];
+        }
+    }
+    if constexpr (MODE == kRowSrc) {
+        for (int h = warp; h < a.H; h += kMergeThreads / 32) {
+            float d = 0.f;
+            for (long long s = s0 + lane; s < s1; s += 32) d += a.sp.part[s * a.sp.pstride + rowf + h];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (lane == 0) a.dscal[row * a.H + h] = d;
+        }
+    }
+
+    const int cols = rowf / 4;
+    const int cols_pad = cols < kMergeThreads ? cols : kMergeThreads;
+    const int streams = (kMergeThreads / cols_pad) < (int)(s1 - s0) ? kMergeThreads / cols_pad : (int)(s1 - s0);
+    const int col = tid % cols_pad, stream = tid / cols_pad;
+    for (int c0 = 0; c0 < cols; c0 += cols_pad) {
+        const bool in = c0 + col < cols && stream < streams;
+        const int c = in ? (c0 + col) * 4 : 0;
+        const int head = c / (a.vph * EPV);
+        const float4 x = merge_columns(a, in ? s0 : s1, s1, c, stream, streams, red, cols_pad, col, [&](long long s) {
+            if constexpr (kF) return fast_exp(a.sp.part[s * a.sp.pstride + rowf + head] - sM[head]);
+            else return 1.f;
+        });
+        if (!in || stream != 0) continue;
+        T *out = reinterpret_cast<T *>(a.out);
+        if constexpr (kF) {
+            merge_store<T>(a, row, c, x, [&](long long o, int h, float y) {
+                if (!first) y += a.acc[o] * sOld[h];
+                if (!last || (a.flags & SAR_KEEP_NUMERATOR)) a.acc[o] = y;
+                if (last) {
+                    y *= sD[h] > 0.f ? 1.f / sD[h] : 0.f;
+                    Elem<T>::store1(out + o, (a.flags & SAR_RELU_OUT) ? fmaxf(y, 0.f) : y);
+                }
+            });
+        } else if constexpr (MODE == kRowSrc) {
+            merge_store<T>(a, row, c, x, [&](long long o, int, float y) { Elem<T>::store1(out + o, y); });
+        } else {
+            const float ds = a.dst_scale ? a.dst_scale[row] : 1.f;
+            float inv = 1.f;
+            if ((a.flags & SAR_MEAN) && last) inv = a.deg[row] > 0 ? 1.f / (float)a.deg[row] : 0.f;
+            merge_store<T>(a, row, c, x, [&](long long o, int, float y) {
+                y *= ds;
+                if (!first) {
+                    if constexpr (sizeof(T) == 4) y += out[o];
+                    else y += __bfloat162float(out[o]);
+                }
+                Elem<T>::store1(out + o, y * inv);
+            });
+        }
+    }
+}
+
+// Destination-major: D, B and S of the segments are numbers; a warp per long row and head.
+template <bool PART>
+__global__ void __launch_bounds__(kMergeThreads) rows_dst_merge_kernel(const RowArgs a) {
+    const int lane = threadIdx.x & 31;
+    const long long item = (long long)blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5);
+    const int lr = (int)(item / a.H), h = (int)(item % a.H);
+    if (lr >= a.sp.n_long) return;
+    const long long row = a.sp.long_row[lr], s1 = a.sp.long_seg[lr + 1];
+    float D = 0.f, Bs = 0.f, S = 0.f;
+    for (long long s = a.sp.long_seg[lr] + lane; s < s1; s += 32) {
+        const float *rec = a.sp.part + s * a.sp.pstride;
+        if (!PART) D += rec[h];
+        Bs += rec[a.H + h];
+        S += rec[2 * a.H + h];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (!PART) D += __shfl_xor_sync(0xffffffffu, D, o);
+        Bs += __shfl_xor_sync(0xffffffffu, Bs, o);
+        S += __shfl_xor_sync(0xffffffffu, S, o);
+    }
+    if (lane == 0) {
+        const long long o = row * a.H + h;
+        if (PART) {
+            const float x = Bs - a.rec[o].w * S;
+            a.dscal[o] = (a.flags & SAR_FIRST) ? x : a.dscal[o] + x;
+        } else {
+            const float dd = a.d[o];
+            a.dscal[o] = Bs - D * S;
+            a.rec[o] = make_float4(a.el[o], a.m[o], dd > 0.f ? __fdividef(1.f, dd) : 0.f, D);
+        }
+    }
+}
+
+// The end of Algorithm 1: out = numerator / d for every row (0 where d = 0), one thread per 16-byte vector of `out`.
+// Follows a last partition step that left the complete state behind (aligned shapes).
+template <typename T>
+__global__ void __launch_bounds__(256) rows_finalize_kernel(const RowArgs a) {
+    constexpr int EPV = Elem<T>::EPV;
+    const long long vi = (long long)blockIdx.x * 256 + threadIdx.x;
+    const int n_vec = a.H * a.vph;
+    if (vi >= a.n_rows * n_vec) return;
+    const long long row = vi / n_vec;
+    const float dd = a.d_io[row * a.H + (int)(vi - row * n_vec) / a.vph];
+    const float inv = dd > 0.f ? __fdividef(1.f, dd) : 0.f;
+    const float4 *src = reinterpret_cast<const float4 *>(a.acc) + vi * (EPV / 4);
+    float x[EPV];
+#pragma unroll
+    for (int q = 0; q < EPV / 4; ++q) {
+        const float4 t = src[q];
+        x[4 * q] = t.x * inv;
+        x[4 * q + 1] = t.y * inv;
+        x[4 * q + 2] = t.z * inv;
+        x[4 * q + 3] = t.w * inv;
+    }
+    if (a.flags & SAR_RELU_OUT) {
+#pragma unroll
+        for (int e = 0; e < EPV; ++e) x[e] = fmaxf(x[e], 0.f);
+    }
+    reinterpret_cast<uint4 *>(a.out)[vi] = Elem<T>::pack(x);
+}
+
+template <int MODE>
+static sar_status launch_merge(const RowArgs &a, sar_dtype t, const char *name, cudaStream_t st) {
+    if (t == SAR_F32)
+        SAR_LAUNCH(name, st, (rows_merge_kernel<float, MODE><<<a.sp.n_long, kMergeThreads, 0, st>>>(a)));
+    else
+        SAR_LAUNCH(name, st, (rows_merge_kernel<__nv_bfloat16, MODE><<<a.sp.n_long, kMergeThreads, 0, st>>>(a)));
+    return sar_after_launch();
+}
+
+sar_status rows_fwd_merge(const RowArgs &a, sar_dtype t, cudaStream_t st) { return launch_merge<kRowFwd>(a, t, "gat_fwd_merge", st); }
+sar_status rows_src_merge(const RowArgs &a, sar_dtype t, cudaStream_t st) { return launch_merge<kRowSrc>(a, t, "gat_bwd_src_merge", st); }
+sar_status rows_sum_merge(const RowArgs &a, sar_dtype t, cudaStream_t st) { return launch_merge<kRowSum>(a, t, "spmm_merge", st); }
+
+sar_status rows_fwd_finalize(const RowArgs &a, sar_dtype t, cudaStream_t st) {
+    const unsigned blocks = (unsigned)((a.n_rows * a.H * a.vph + 255) / 256);
+    if (t == SAR_F32)
+        SAR_LAUNCH("gat_fwd_finalize", st, (rows_finalize_kernel<float><<<blocks, 256, 0, st>>>(a)));
+    else
+        SAR_LAUNCH("gat_fwd_finalize", st, (rows_finalize_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(a)));
+    return sar_after_launch();
+}
+
+sar_status rows_dst_merge(const RowArgs &a, bool part, cudaStream_t st) {
+    const long long warps = (long long)a.sp.n_long * a.H;
+    const unsigned blocks = (unsigned)((warps + kMergeThreads / 32 - 1) / (kMergeThreads / 32));
+    if (part)
+        SAR_LAUNCH("gat_bwd_dst_merge", st, (rows_dst_merge_kernel<true><<<blocks, kMergeThreads, 0, st>>>(a)));
+    else
+        SAR_LAUNCH("gat_bwd_dst_merge", st, (rows_dst_merge_kernel<false><<<blocks, kMergeThreads, 0, st>>>(a)));
+    return sar_after_launch();
+}
+
+}  // namespace sar

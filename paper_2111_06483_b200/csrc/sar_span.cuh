@@ -1,0 +1,14 @@
+// Host-side interface of the span kernels (internal): sar_span.cu.
+#pragma once
+
+#include "sar_rows.cuh"
+
+namespace sar {
+
+// Rows launch, in the forward pass and the sums the segment launch too.
+sar_status span_fwd(const Shape &s, const RowArgs &r, long long nnz, cudaStream_t st);
+sar_status span_dst(const Shape &s, const RowArgs &r, long long nnz, bool part, cudaStream_t st);
+sar_status span_src(const Shape &s, const RowArgs &r, long long nnz, cudaStream_t st);
+sar_status span_sum(const Shape &s, const RowArgs &r, long long nnz, bool weighted, cudaStream_t st);
+
+}  // namespace sar

@@ -19,13 +19,29 @@
 // Nothing per edge is written to global memory.  No floating-point atomics: every output element
 // has one writer (the per-(row, head) max of the forward pass is a shared-memory atomicMax on an
 // order-preserving integer key, whose result does not depend on the order).
-// Rows above the plan's threshold are skipped here and processed as independent segments by a second
-// launch (mode 1) that writes partial accumulators; the merge kernels of sar_gat_kernels.cuh fold them.
+// Rows above the plan's threshold are skipped here and processed as independent segments by a second launch that writes
+// partial results - mode 1 of this kernel in the forward pass and the sums, the row kernels in the backward passes - which
+// the merge kernels of sar_rows_merge.cu fold.
+//
+// Where it runs: gathered arrays larger than the L2 (span_applies in sar_span.cuh).  What bounds a gather there is bytes
+// in flight, and the ring holds them without registers; out of the L2 the row kernels (sar_rows_kernel.cuh) are faster.
 #pragma once
 
+#include "sar_device.cuh"
 #include "sar_rowkernels.cuh"
 
 namespace sar {
+
+enum GatherMode { kFwd = 0, kBwdDst = 1, kBwdDstGivenD = 2, kBwdSrc = 3, kSum = 4, kSumW = 5 };
+
+template <int MODE>
+struct WeightOf {
+    using type = float;
+};
+template <>
+struct WeightOf<kBwdSrc> {
+    using type = float2;
+};
 
 constexpr int kSpanWarps = 1;             // warps per block
 constexpr int kSpanThreads = kSpanWarps * 32;
@@ -57,38 +73,12 @@ struct SpanArgs {
     int stage_rows;          // mode 0: rows whose own data is staged in shared memory per chunk (R, or 0: none)
 };
 
-// order-preserving float -> unsigned key (for shared-memory atomicMax)
-__device__ __forceinline__ unsigned fkey(float x) {
-    const unsigned b = __float_as_uint(x);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float fkey_inv(unsigned k) {
-    return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
-constexpr unsigned kKeyNegInf = 0x007fffffu;  // fkey(-inf)
-
 // 16-byte asynchronous copy global -> shared that bypasses L1; src_bytes = 0 writes zeros.
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc, int src_bytes) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gsrc), "r"(src_bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
 // shared-memory accesses through 32-bit shared-window addresses (no 64-bit pointer arithmetic)
-__device__ __forceinline__ uint4 lds128(unsigned addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ float lds_f32(unsigned addr) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(addr));
-    return v;
-}
 __device__ __forceinline__ float2 lds_f32x2(unsigned addr) {
     float2 v;
     asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(addr));
@@ -102,35 +92,6 @@ __device__ __forceinline__ int lds_s32(unsigned addr) {
 __device__ __forceinline__ void cp_async16_s(unsigned smem_addr, const void *gsrc, int src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_addr), "l"(gsrc), "r"(src_bytes) : "memory");
 }
-
-// packed pairs of float32 (Blackwell's two-wide FP32 pipe: one instruction, two fused multiply-adds)
-typedef float2 f32x2;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) { return make_float2(lo, hi); }
-__device__ __forceinline__ void unpack2(f32x2 p, float &lo, float &hi) {
-    lo = p.x;
-    hi = p.y;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { return __ffma2_rn(a, b, c); }  // a*b + c, element-wise
-__device__ __forceinline__ f32x2 zero2() { return make_float2(0.f, 0.f); }
-// 16 bytes of storage type T -> EPV/2 packed float32 pairs
-template <typename T>
-struct Pairs;
-template <>
-struct Pairs<float> {
-    __device__ __forceinline__ static void get(const uint4 &d, f32x2 (&p)[2]) {
-        p[0] = pack2(__uint_as_float(d.x), __uint_as_float(d.y));
-        p[1] = pack2(__uint_as_float(d.z), __uint_as_float(d.w));
-    }
-};
-template <>
-struct Pairs<__nv_bfloat16> {
-    __device__ __forceinline__ static void get(const uint4 &d, f32x2 (&p)[4]) {
-        p[0] = pack2(__uint_as_float(d.x << 16), __uint_as_float(d.x & 0xffff0000u));
-        p[1] = pack2(__uint_as_float(d.y << 16), __uint_as_float(d.y & 0xffff0000u));
-        p[2] = pack2(__uint_as_float(d.z << 16), __uint_as_float(d.z & 0xffff0000u));
-        p[3] = pack2(__uint_as_float(d.w << 16), __uint_as_float(d.w & 0xffff0000u));
-    }
-};
 
 // Shared-memory layout of one warp (byte offsets).
 struct SpanSmem {
@@ -161,7 +122,7 @@ __host__ __device__ inline SpanSmem span_layout(int Hp, int V, int cap, int stag
 }
 
 // STATIC decides the launch mode at compile time, so that the flag tests of the row epilogue fold away:
-// 1 = rows (mode 0) of a partition that holds all sources (SAR_FIRST | SAR_LAST), the benchmarked configuration;
+// 1 = rows (mode 0) of a partition that holds all sources (SAR_FIRST | SAR_LAST), in the sums of any partition;
 // 2 = long-row segments (mode 1); 0 = whatever SpanArgs says.
 // GEO = 1 fixes the row geometry at compile time as well: rows of exactly G*V vectors and, for the attention modes,
 // 4 heads scored four at a time (SpanArgs::hvec set; the paper's GAT: 4 heads, hidden size 128), for the sums one
@@ -171,7 +132,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
     constexpr int EPV = Elem<T>::EPV;
     constexpr int EPW = 32 / G;  // edges per slot
     const int mode_ = STATIC == 1 ? 0 : (STATIC == 2 ? 1 : a.mode);
-    const unsigned flags_ = STATIC == 1 ? ((unsigned)(SAR_FIRST | SAR_LAST) | (a.flags & (unsigned)SAR_MEAN)) : a.flags;
+    const unsigned flags_ = STATIC == 1 && MODE != kSum && MODE != kSumW ? (unsigned)(SAR_FIRST | SAR_LAST) : a.flags;
     using W = typename WeightOf<MODE>::type;
     constexpr bool kFwdMode = MODE == kFwd;
     constexpr bool kDst = MODE == kBwdDst || MODE == kBwdDstGivenD;
@@ -890,16 +851,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
                     }
                 }
             } else if constexpr (kDst) {
-                if (mode_ == 1) {
-                    if (writer) {
-                        float *rec = a.sp.part + seg * a.sp.pstride;
-                        store_acc_row<G, V, EPV>(rec, gl, vok, acc1);
-                        if constexpr (MODE == kBwdDst) store_acc_row<G, V, EPV>(rec + rowf, gl, vok, acc0);
-#pragma unroll
-                        for (int v = 0; v < V; ++v)
-                            if (lead[v]) rec[2 * rowf + hv[v]] = sv[v];
-                    }
-                } else {
+                {
                     float pA[V], pB[V], rv[V][EPV];
                     if (staged_now) {
 #pragma unroll
@@ -944,16 +896,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
                     __syncwarp();
                 }
             } else if constexpr (kSrc) {
-                if (mode_ == 1) {
-                    if (writer) {
-                        float *rec = a.sp.part + seg * a.sp.pstride;
-                        store_acc_row<G, V, EPV>(rec, gl, vok, acc0);
-                        store_acc_row<G, V, EPV>(rec + rowf, gl, vok, acc1);
-#pragma unroll
-                        for (int v = 0; v < V; ++v)
-                            if (lead[v]) rec[2 * rowf + hv[v]] = sv[v];
-                    }
-                } else {
+                {
                     float pC[V], rv[V][EPV];
 #pragma unroll
                     for (int v = 0; v < V; ++v) {

@@ -1,0 +1,68 @@
+"""The kernels behind the shapes that the lean kernels do not cover, at the sizes where they can go wrong: heads that are no
+power of two or no whole number of 16-byte words, rows wider than one lane group, arrays on either side of the size where
+the dispatch changes from the row kernels to the span kernels, and calls that get no room for padded copies."""
+import numpy as np
+import pytest
+import torch
+
+import workloads
+from helpers import allclose_report
+from test_gpu_parity import DEV, Problem, _full_check, check_out, hub_graph
+
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    from paper_2111_06483_b200 import api, binding as B
+
+
+@pytest.mark.parametrize("H,F,dtype", [(1, 47, "bf16"), (3, 33, "f32"), (6, 24, "bf16"), (2, 64, "bf16"), (7, 9, "f32"), (1, 300, "f32"),
+                                       (2, 260, "f32"), (1, 520, "bf16"), (12, 8, "f32"), (1, 1030, "bf16")])
+@pytest.mark.parametrize("threshold", [0, 24])
+def test_attention_on_general_shapes(H, F, dtype, threshold):
+    n, src, dst = hub_graph(n=2000, e=24000, d_max=400.0, seed=19)
+    p = Problem(n, src, dst, H, F, 70 + H + F, dtype=dtype, k=3, threshold=threshold, build_parts=True)
+    # the dot products that cancel in del and der grow with F at worst
+    _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=max(1.0, F / 64))
+
+
+@pytest.mark.parametrize("H,F,dtype,n", [(2, 64, "bf16", 540_000), (1, 60, "f32", 600_000)])
+def test_attention_on_arrays_larger_than_the_l2(H, F, dtype, n):
+    spec = workloads.ChungLuSpec(n=n, e=1_500_000, gamma=2.1, d_max=3000.0, seed=5)
+    src, dst = workloads.chung_lu_edges(spec)
+    p = Problem(n, src, dst, H, F, 7, dtype=dtype, k=2, build_parts=True)
+    # a million sums of up to 3000 terms that cancel
+    _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
+
+
+@pytest.mark.parametrize("F", [1, 3, 47, 48, 127, 180, 260, 1030])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("n", [1500, 40_000])
+def test_sums_of_ragged_rows(F, dtype, n):
+    """Sums of small whole numbers are exact in float32 and, below 256, in bf16."""
+    spec = workloads.ChungLuSpec(n=n, e=6 * n, gamma=2.1, d_max=300.0, seed=8)
+    src, dst = (x.to(DEV) for x in workloads.chung_lu_edges(spec))
+    g = api.Graph.from_coo(n, src, dst, threshold=64)
+    x = (torch.arange(n * F, device=DEV).view(n, F) % 3 == 0).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    want = torch.zeros(n, F, device=DEV).index_add_(0, dst.long(), x.float()[src.long()])
+    got = api.spmm_sum(g.whole, x)
+    assert torch.equal(got, want.to(x.dtype))
+    scale = torch.full((n,), 2.0, device=DEV)
+    out = x.clone()
+    api.spmm_scaled(g.whole, x, src_scale=scale, dst_scale=scale, out=out, first=False)   # += 4 * sum
+    assert torch.equal(out, (x.float() + 4.0 * want).to(x.dtype))
+
+
+def test_ragged_shape_without_room_for_padded_copies():
+    """No workspace in the forward call, one that holds the records alone in the backward call: the scalar kernels."""
+    n, src, dst = hub_graph(n=500, e=6000, d_max=100.0, seed=3)
+    p = Problem(n, src, dst, 2, 7, 4, threshold=512)
+    d, f = p.dev, p.oracle_fwd()
+    out, m, dd = torch.empty_like(d["feat"]), torch.empty_like(d["el"]), torch.empty_like(d["el"])
+    B.sar_gat_fwd(p.graph.whole, d["feat"], d["el"], d["er"], 2, 7, 0.2, B.SAR_FIRST | B.SAR_LAST, None, m, dd, out, None)
+    check_out(out, f.out, "f32", "out")
+    b = p.oracle_bwd(f)
+    dfeat, del_, der = torch.empty_like(d["feat"]), torch.empty_like(m), torch.empty_like(m)
+    ws = torch.empty((n * 2 * 16 + 255) // 256 * 256, dtype=torch.uint8, device=DEV)
+    B.sar_gat_bwd(p.graph.whole, d["feat"], d["el"], d["er"], m, dd, d["gout"], 2, 7, 0.2, B.SAR_FIRST | B.SAR_LAST, dfeat, del_, der, ws)
+    for got, want in ((dfeat, b.dfeat), (del_, b.del_), (der, b.der)):
+        allclose_report(got.cpu().numpy(), np.asarray(want), 1e-4, 1e-5, "gradients")
