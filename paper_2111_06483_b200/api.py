@@ -1,4 +1,5 @@
-"""Convenience layer over the binding: allocates device tensors with torch and calls libsar.
+"""Convenience layer over the library: allocates device tensors with torch and calls libsar.  The calls of a training step
+do both in native code (csrc/sar_torch.cpp, through binding.native()); the others go through the ctypes binding.
 
 Nothing is computed here; every step (graph build, transpose, split, long-row plan, forward,
 backward, sum aggregation) is a call into the C-ABI library.
@@ -193,30 +194,11 @@ def gat_forward(g: Graph, feat: torch.Tensor, el: torch.Tensor, er: torch.Tensor
     keep_numerator (stateful mode): returns (out, m, d, acc) with the complete float32 numerator in acc,
     which gat_backward can take in place of `out` for the row dot.
     relu_out: out = max(out, 0), the ReLU that closes the layer, applied where the aggregate is finalised."""
-    n, H, F = feat.shape
-    dev = feat.device
-    m = torch.empty((g.n, H), dtype=torch.float32, device=dev)
-    d = torch.empty((g.n, H), dtype=torch.float32, device=dev)
-    out = torch.empty((g.n, H, F), dtype=feat.dtype, device=dev)
     if mode == "fused":
-        ws = workspace if workspace is not None else gat_workspace(g.whole, H, F, feat.dtype)
-        if relu_out:   # the un-split graph as one partition holding all sources
-            B.sar_gat_fwd(g.whole, feat, el, er, H, F, slope, B.SAR_FIRST | B.SAR_LAST | B.SAR_RELU_OUT, None, m, d, out, ws)
-        else:
-            B.sar_gat_fwd_fused(g.whole, g.bounds, feat, el, er, H, F, slope, m, d, out, ws)
-        return out, m, d
+        return B.native().gat_forward(g.whole.addr, g.bounds, feat, el, er, slope, workspace, relu_out)
     assert g.parts, "stateful mode needs Graph.from_coo(..., build_parts=True)"
-    acc = torch.empty((g.n, H, F), dtype=torch.float32, device=dev) if (g.k > 1 or keep_numerator) else None
-    for q, part in enumerate(g.parts):
-        flags = (B.SAR_FIRST if q == 0 else 0) | (B.SAR_LAST if q == g.k - 1 else 0)
-        if keep_numerator and q == g.k - 1:
-            flags |= B.SAR_KEEP_NUMERATOR
-        if relu_out and q == g.k - 1:
-            flags |= B.SAR_RELU_OUT
-        ws = gat_workspace(part, H, F, feat.dtype)
-        s0, s1 = g.bounds[q], g.bounds[q + 1]
-        B.sar_gat_fwd(part, feat[s0:s1], el, er[s0:s1], H, F, slope, flags, acc, m, d, out, ws)
-    return (out, m, d, acc) if keep_numerator else (out, m, d)
+    r = B.native().gat_forward_parts([p.addr for p in g.parts], g.bounds, g.n, feat, el, er, slope, keep_numerator, relu_out)
+    return r if keep_numerator else r[:3]
 
 
 def gat_backward(g: Graph, feat: torch.Tensor, el: torch.Tensor, er: torch.Tensor, m: torch.Tensor,
@@ -224,38 +206,16 @@ def gat_backward(g: Graph, feat: torch.Tensor, el: torch.Tensor, er: torch.Tenso
                  workspace: Optional[torch.Tensor] = None, mode: str = "fused", acc: Optional[torch.Tensor] = None):
     """Backward over the K partitions; returns (dfeat, del, der).  "stateful" needs `out` or the complete
     float32 numerator `acc` (for the row dot) and runs sar_gat_bwd_prepare followed by K calls of sar_gat_bwd."""
-    n, H, F = feat.shape
-    dev = feat.device
-    dfeat = torch.empty_like(feat)
-    del_ = torch.empty((g.n, H), dtype=torch.float32, device=dev)
-    der = torch.empty((g.n, H), dtype=torch.float32, device=dev)
     if mode == "fused":
-        ws = workspace if workspace is not None else gat_workspace(g.whole, H, F, feat.dtype)
-        B.sar_gat_bwd_fused(g.whole, g.bounds, feat, el, er, m, d, gout, H, F, slope, dfeat, del_, der, ws)
-        return dfeat, del_, der
+        return B.native().gat_backward(g.whole.addr, g.bounds, feat, el, er, m, d, gout, slope, workspace)
     assert g.parts and (out is not None or acc is not None)
-    nbytes = max(B.sar_gat_workspace_bytes(p, H, F, B._dtype(feat)) for p in g.parts)
-    ws = _workspace(nbytes, dev)
-    if acc is not None:
-        B.sar_gat_bwd_prepare(g.n, H, F, acc, True, gout, el, m, d, None, ws)
-    else:
-        B.sar_gat_bwd_prepare(g.n, H, F, out, False, gout, el, m, d, None, ws)
-    for q, part in enumerate(g.parts):
-        flags = (B.SAR_FIRST if q == 0 else 0) | (B.SAR_LAST if q == g.k - 1 else 0)
-        s0, s1 = g.bounds[q], g.bounds[q + 1]
-        B.sar_gat_bwd(part, feat[s0:s1], el, er[s0:s1], m, d, gout, H, F, slope, flags, dfeat[s0:s1], del_,
-                      der[s0:s1], ws)
-    return dfeat, del_, der
+    return B.native().gat_backward_parts([p.addr for p in g.parts], g.bounds, g.n, feat, el, er, m, d, gout, slope,
+                                         out if acc is None else acc, acc is not None)
 
 
 def spmm_sum(part: B.Part, feat: torch.Tensor, mean: bool = False, deg_total: Optional[torch.Tensor] = None):
     """out[i,:] = sum (or mean) of feat over the in-edges of i for one partition holding all sources."""
-    F = feat.shape[1]
-    out = torch.empty((part.n_dst, F), dtype=feat.dtype, device=feat.device)
-    ws = _workspace(B.sar_spmm_workspace_bytes(part, F, B._dtype(feat)), feat.device)
-    flags = B.SAR_FIRST | B.SAR_LAST | (B.SAR_MEAN if mean else 0)
-    B.sar_spmm_agg(part, feat, F, flags, deg_total, out, ws)
-    return out
+    return B.native().spmm(part.addr, feat, B.SAR_FIRST | B.SAR_LAST | (B.SAR_MEAN if mean else 0), deg_total)
 
 
 # ----------------------------------------------------------------------------------------------
@@ -293,12 +253,7 @@ def gat_layer_backward(g: Graph, z: torch.Tensor, a_l: torch.Tensor, a_r: torch.
 def spmm_scaled(part: B.Part, feat: torch.Tensor, src_scale: Optional[torch.Tensor] = None,
                 dst_scale: Optional[torch.Tensor] = None, out: Optional[torch.Tensor] = None, first: bool = True):
     """out[i,:] (+)= dst_scale[i] * sum over the in-edges of i of src_scale[j] * feat[j,:] (one partition)."""
-    F = feat.shape[1]
-    if out is None:
-        out = torch.empty((part.n_dst, F), dtype=feat.dtype, device=feat.device)
-    ws = _workspace(B.sar_spmm_workspace_bytes(part, F, B._dtype(feat)), feat.device)
-    B.sar_spmm_agg_scaled(part, feat, F, (B.SAR_FIRST if first else 0) | B.SAR_LAST, src_scale, dst_scale, out, ws)
-    return out
+    return B.native().spmm_scaled(part.addr, feat, (B.SAR_FIRST if first else 0) | B.SAR_LAST, src_scale, dst_scale, out)
 
 
 # ----------------------------------------------------------------------------------------------
@@ -343,6 +298,9 @@ def bn_forward(x: torch.Tensor, eps: float = 1e-5, gamma: Optional[torch.Tensor]
                beta: Optional[torch.Tensor] = None, group=None):
     """Returns (y, saved) with saved = (mean, rstd, n_all) for bn_backward.  x is [n_local, C]."""
     n, C = x.shape
+    if group is None:
+        y, mean, rstd = B.native().bn_forward(x, eps, gamma, beta)
+        return y, (mean, rstd, n)
     dev = x.device
     ws = _workspace(B.sar_bn_workspace_bytes(C), dev)
     mean = torch.empty(C, dtype=torch.float32, device=dev)
@@ -361,6 +319,8 @@ def bn_backward(x: torch.Tensor, gy: torch.Tensor, saved, gamma: Optional[torch.
     n, C = x.shape
     dev = x.device
     mean, rstd, n_all = saved
+    if group is None:
+        return B.native().bn_backward(x, gy, mean, rstd, gamma, n_all)
     ws = _workspace(B.sar_bn_workspace_bytes(C), dev)
     s0 = torch.empty(C, dtype=torch.float32, device=dev)
     s1 = torch.empty(C, dtype=torch.float32, device=dev)
@@ -379,43 +339,15 @@ def full_layer_forward(g: Graph, h: torch.Tensor, W: torch.Tensor, a_l: torch.Te
                        relu_input: bool = False):
     """h [n, D_in], W [D_in, H*F] (bf16), a_l / a_r [H, F] float32.  Returns (out [n,H,F], saved).
     relu_input=True first applies h = max(h, 0) in place (the activation that closes the previous layer)."""
-    n = h.shape[0]
-    H, F = a_l.shape
-    if relu_input:
-        B.sar_relu(h)
-    z = torch.empty((n, H, F), dtype=h.dtype, device=h.device)
-    ws = _workspace(B.sar_linear_workspace_bytes(n, h.shape[1], H * F), h.device)
-    el = torch.empty((n, H), dtype=torch.float32, device=h.device)
-    er = torch.empty_like(el)
-    if F % 8 == 0 and 128 % F == 0:   # the scores leave the projection's epilogue
-        B.sar_linear_project(h, W, a_l, a_r, z.view(n, H * F), el, er, ws)
-    else:
-        B.sar_linear(h, W, z.view(n, H * F), ws)
-        B.sar_gat_project(z, a_l, a_r, el, er, 0)
-    out, m, d = gat_forward(g, z, el, er, slope)
-    return out, (z, el, er, m, d)
+    out, *saved = B.native().layer_forward(g.whole.addr, g.bounds, h, W, a_l, a_r, slope, relu_input)
+    return out, tuple(saved)
 
 
 def full_layer_backward(g: Graph, h: torch.Tensor, W: torch.Tensor, a_l: torch.Tensor, a_r: torch.Tensor, saved,
                         gout: torch.Tensor, slope: float, relu_input: bool = False):
     """Returns (dh [n, D_in], dW [D_in, H*F] float32, da_l, da_r); with relu_input=True dh is the gradient
     before the input's ReLU (h must be the array full_layer_forward left, i.e. already max(h, 0))."""
-    n, d_in = h.shape
-    H, F = a_l.shape
-    z, el, er, m, d = saved
-    dz, del_, der = gat_backward(g, z, el, er, m, d, gout, slope)
-    da_l = torch.empty((H, F), dtype=torch.float32, device=h.device)
-    da_r = torch.empty_like(da_l)
-    B.sar_gat_project_bwd(z, a_l, a_r, del_, der, dz, da_l, da_r, _workspace(B.sar_gat_project_workspace_bytes(H, F), h.device), 0)
-    ws = _workspace(B.sar_linear_workspace_bytes(n, d_in, H * F), h.device)
-    dW = torch.empty((d_in, H * F), dtype=torch.float32, device=h.device)
-    B.sar_linear_bwd_weight(h, dz.view(n, H * F), dW, ws)
-    dh = torch.empty_like(h)
-    if relu_input:   # the mask of the input's ReLU is applied in the GEMM's epilogue
-        B.sar_linear_bwd_input_relu(dz.view(n, H * F), W, h, dh, ws)
-    else:
-        B.sar_linear_bwd_input(dz.view(n, H * F), W, dh, ws)
-    return dh, dW, da_l, da_r
+    return B.native().layer_backward(g.whole.addr, g.bounds, h, W, a_l, a_r, *saved, gout, slope, relu_input)
 
 
 # ----------------------------------------------------------------------------------------------
@@ -504,39 +436,18 @@ def rgcn_basis_backward(a: torch.Tensor, V: torch.Tensor, dW: torch.Tensor):
 
 def sage_layer_forward(g: Graph, h: torch.Tensor, W: torch.Tensor, W_res: torch.Tensor, inv: Optional[torch.Tensor] = None):
     """h [n, d_in], W and W_res [d_in, d_out] (bf16).  Returns (pre [n, d_out] before the activation, saved)."""
-    n, d_in = h.shape
-    d_out = W.shape[1]
     if inv is None:
         inv = rgcn_inv_degrees([g])[0]
-    agg = torch.empty_like(h)
-    _rgcn_aggregate(g, h, inv, agg)
-    pre = torch.empty((n, d_out), dtype=h.dtype, device=h.device)
-    ws = _workspace(B.sar_linear_workspace_bytes(n, d_in, d_out), h.device)
-    B.sar_linear(h, W_res, pre, ws)
-    B.sar_linear_accumulate(agg, W, pre, ws)
+    parts, bounds = _pieces(g)
+    pre, agg = B.native().sage_forward([p.addr for p in parts], bounds, h, W, W_res, inv)
     return pre, (agg, inv)
 
 
 def sage_layer_backward(g: Graph, h: torch.Tensor, W: torch.Tensor, W_res: torch.Tensor, saved, gpre: torch.Tensor):
     """Returns (dh [n, d_in], dW, dW_res [d_in, d_out] float32) for the upstream gradient gpre [n, d_out]."""
-    n, d_in = h.shape
-    d_out = W.shape[1]
     agg, inv = saved
-    ws = _workspace(B.sar_linear_workspace_bytes(n, d_in, d_out), h.device)
-    dW = torch.empty((d_in, d_out), dtype=torch.float32, device=h.device)
-    dW_res = torch.empty_like(dW)
-    B.sar_linear_bwd_weight(agg, gpre, dW, ws)
-    B.sar_linear_bwd_weight(h, gpre, dW_res, ws)
-    dh = torch.empty_like(h)
-    B.sar_linear_bwd_input(gpre, W_res, dh, ws)       # the residual path
-    dagg = torch.empty_like(h)
-    B.sar_linear_bwd_input(gpre, W, dagg, ws)
     parts, bounds = _pieces(g)
-    for q, part in enumerate(parts):                  # plus what every out-edge hands back: dagg_i / |N(i)|
-        tp = part.transposed()
-        sws = _workspace(B.sar_spmm_workspace_bytes(tp, d_in, B._dtype(h)), h.device)
-        B.sar_spmm_agg_scaled(tp, dagg, d_in, B.SAR_LAST, inv, None, dh[bounds[q]:bounds[q + 1]], sws)
-    return dh, dW, dW_res
+    return B.native().sage_backward([p.addr for p in parts], bounds, h, W, W_res, agg, inv, gpre)
 
 
 # ----------------------------------------------------------------------------------------------
@@ -556,16 +467,5 @@ def sym_norm_scales(g: Graph):
 def propagate(g: Graph, x0: torch.Tensor, alpha: float, iters: int, src_scale: Optional[torch.Tensor] = None,
               dst_scale: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Returns X_iters with X_0 = x0 and X_{t+1} = (1 - alpha) x0 + alpha S X_t; x0 [n, F]."""
-    x = x0.clone()
-    nxt = torch.empty_like(x0)
     parts, bounds = _pieces(g)
-    F = x0.shape[1]
-    for _ in range(iters):
-        for q, part in enumerate(parts):
-            flags = (B.SAR_FIRST if q == 0 else 0) | (B.SAR_LAST if q == len(parts) - 1 else 0)
-            ws = _workspace(B.sar_spmm_workspace_bytes(part, F, B._dtype(x0)), x0.device)
-            sq = None if src_scale is None else src_scale[bounds[q]:bounds[q + 1]]
-            B.sar_spmm_agg_scaled(part, x[bounds[q]:bounds[q + 1]], F, flags, sq, dst_scale, nxt, ws)
-        B.sar_axpby(1.0 - alpha, x0, alpha, nxt)
-        x, nxt = nxt, x
-    return x
+    return B.native().propagate([p.addr for p in parts], bounds, x0, alpha, iters, src_scale, dst_scale)

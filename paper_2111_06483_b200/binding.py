@@ -80,6 +80,25 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_native = None
+
+
+def native():
+    """The native side of api.py (csrc/sar_torch.cpp), working on the loaded library.  Raises if it is missing."""
+    global _native
+    if _native is None:
+        from importlib import machinery, util
+        path = os.path.join(_PKG, "_sar_torch.so")
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} not found: run `python -m paper_2111_06483_b200.build`")
+        loader = machinery.ExtensionFileLoader("_sar_torch", path)
+        mod = util.module_from_spec(util.spec_from_loader("_sar_torch", loader))
+        loader.exec_module(mod)
+        mod.init(lib()._handle, SarError, torch.OutOfMemoryError)
+        _native = mod
+    return _native
+
+
 def _check(fn: str, code: int) -> None:
     if code != SAR_OK:
         raise SarError(fn, code, lib().sar_status_string(code).decode())
@@ -135,6 +154,7 @@ class Part:
                           t_indices.data_ptr() if t_indices is not None else None,
                           ctypes.pointer(split.c) if split is not None else None,
                           ctypes.pointer(t_split.c) if t_split is not None else None)
+        self.addr = ctypes.addressof(self.c)   # for the native side
 
     def transposed(self) -> "Part":
         """The same edges with the roles of rows and columns swapped (for the backward of the sum)."""

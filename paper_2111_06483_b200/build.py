@@ -1,4 +1,5 @@
-"""Builds libsar.so (the C-ABI library of include/sar.h) in-tree with nvcc for sm_100a.
+"""Builds libsar.so (the C-ABI library of include/sar.h) in-tree with nvcc for sm_100a, and _sar_torch.so (the native
+side of api.py: allocation with torch's allocator and the calls into libsar) with g++.
 
     python -m paper_2111_06483_b200.build [--force] [--verbose]
 
@@ -18,6 +19,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(CSRC, "build")
 LIB = os.path.join(PKG, "libsar.so")
+TORCH_EXT = os.path.join(PKG, "_sar_torch.so")
 ROW_PASSES = ["fwd", "fwd_part", "dst", "dst_part", "src", "sum"]   # one translation unit per pass and storage type
 SOURCES = ["sar_linear.cu"] + [f"sar_lean_{p}_{t}.cu" for p in ("fwd", "bwd_dst", "bwd_src") for t in ("f32", "bf16")] + [f"sar_rows_{p}_{t}.cu" for p in ROW_PASSES for t in ("f32", "bf16")] + [
     "sar_gat.cu", "sar_span.cu", "sar_rows_merge.cu", "sar_graph.cu", "sar_host.cu", "sar_noalloc.cu", "sar_storing.cu",
@@ -77,6 +79,31 @@ def _fingerprint(src: str) -> str:
     return h.hexdigest()
 
 
+def build_torch_ext(force: bool = False) -> str:
+    """_sar_torch.so, when its source, sar.h or torch changed.  It links against nothing of libsar: the entry points are
+    looked up in the library that the process has loaded."""
+    import sysconfig
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    src, stamp = os.path.join(CSRC, "sar_torch.cpp"), os.path.join(OBJ, "sar_torch.fingerprint")
+    fp = hashlib.sha256((_fingerprint("sar_torch.cpp") + torch.__version__ + sys.version).encode()).hexdigest()
+    if not force and os.path.exists(TORCH_EXT) and os.path.exists(stamp) and open(stamp).read() == fp:
+        return TORCH_EXT
+    inc = [f"-I{p}" for p in include_paths() + [sysconfig.get_paths()["include"], os.path.join(ROOT, "include"),
+                                                os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")]]
+    libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = TORCH_EXT + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *inc, src, "-o", tmp, f"-L{libdir}",
+           f"-Wl,-rpath,{libdir}", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch", "-ltorch_python", "-ldl"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on sar_torch.cpp:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, TORCH_EXT)
+    open(stamp, "w").write(fp)
+    return TORCH_EXT
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compiles the sources whose contents (or headers, or flags) changed since their object was built, in
     parallel, and links libsar.so when any object is new."""
@@ -101,7 +128,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return obj, True
 
     with ThreadPoolExecutor(min(len(SOURCES), os.cpu_count() or 4)) as ex:
+        ext = ex.submit(build_torch_ext, force)
         results = list(ex.map(compile_one, SOURCES))
+        ext.result()
     objs = [o for o, _ in results]
     if not force and os.path.exists(LIB) and not any(new for _, new in results):
         return LIB
