@@ -2,11 +2,12 @@
 // per head, their backward pass (chain-rule add into dz, gradients of a), and the element-wise ReLU
 // between layers.  Streaming kernels; contracts are in include/sar.h.
 #include "sar_dispatch.cuh"
+#include "sar_reduce.cuh"
 #include "sar_rowkernels.cuh"
 
 namespace sar {
 
-constexpr int kGlueBlocks = 148 * 8;  // fixed grid of the reducing kernel: a fixed summation order
+constexpr int kGlueBlocks = 148 * 8;  // largest grid of the reducing kernel (it depends on the sizes alone: a fixed summation order)
 
 struct ProjArgs {
     long long n;
@@ -169,15 +170,6 @@ __global__ void __launch_bounds__(kThreads) project_bwd_kernel(const ProjArgs a)
         for (int gq = 0; gq < GPB; ++gq) acc += smem[(size_t)gq * 2 * rowf + which * rowf + o];
         a.partial[(size_t)blockIdx.x * 2 * HF + x] = acc;
     }
-}
-
-__global__ void project_reduce_kernel(int blocks, int HF, const float *__restrict__ partial, float *__restrict__ da_l,
-                                      float *__restrict__ da_r) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= 2 * HF) return;
-    float acc = 0.f;
-    for (int b = 0; b < blocks; ++b) acc += partial[(size_t)b * 2 * HF + x];
-    if (x < HF) da_l[x] = acc; else da_r[x - HF] = acc;
 }
 
 __device__ __forceinline__ float as_float(float x) { return x; }
@@ -428,11 +420,11 @@ sar_status sar_gat_project_bwd(int64_t n, int32_t H, int32_t F, sar_dtype t, con
         auto kern = mask ? project_bwd_kernel<T, C::g, C::v, true> : project_bwd_kernel<T, C::g, C::v, false>;
         SAR_TRY(ensure_smem(project_bwd_kernel<T, C::g, C::v, true>, smem));
         SAR_TRY(ensure_smem(project_bwd_kernel<T, C::g, C::v, false>, smem));
-        SAR_LAUNCH("gat_project_bwd", st, kern<<<kGlueBlocks, kThreads, smem, st>>>(a));
+        const unsigned want = blocks_for((a.n + 3) / 4, C::g);
+        const unsigned blocks = want < 1 ? 1 : want < (unsigned)kGlueBlocks ? want : (unsigned)kGlueBlocks;
+        SAR_LAUNCH("gat_project_bwd", st, kern<<<blocks, kThreads, smem, st>>>(a));
         SAR_TRY(sar_after_launch());
-        SAR_LAUNCH("gat_project_reduce", st,
-                   project_reduce_kernel<<<(2 * HF + 255) / 256, 256, 0, st>>>(kGlueBlocks, HF, a.partial, da_l, da_r));
-        return sar_after_launch();
+        return reduce_partials("gat_project_reduce", (int)blocks, 2 * HF, HF, a.partial, 1.0, da_l, da_r, st);
     });
 }
 

@@ -3,11 +3,12 @@
 // of the rows can combine its statistics with the other workers' before applying them.  Streaming kernels;
 // contracts are in include/sar.h.
 #include "sar_dispatch.cuh"
+#include "sar_reduce.cuh"
 #include "sar_rowkernels.cuh"
 
 namespace sar {
 
-constexpr int kNormBlocks = 148 * 8;  // fixed grid of the reducing kernels: a fixed summation order
+constexpr int kNormBlocks = 148 * 8;  // largest grid of the reducing kernels (it depends on the sizes alone: a fixed summation order)
 
 struct NormArgs {
     long long n;
@@ -139,21 +140,6 @@ __global__ void __launch_bounds__(kThreads) norm_sums_kernel(const NormArgs a) {
     }
 }
 
-// block partials -> totals, accumulated in float64; out0 / out1 may be null.  scale multiplies both.
-__global__ void norm_reduce_kernel(int blocks, int C, const float *__restrict__ partial, double scale,
-                                   float *__restrict__ out0, float *__restrict__ out1) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= 2 * C) return;
-    double acc = 0.0;
-    for (int b = 0; b < blocks; ++b) acc += (double)partial[(size_t)b * 2 * C + x];
-    acc *= scale;
-    if (x < C) {
-        if (out0) out0[x] = (float)acc;
-    } else if (out1) {
-        out1[x - C] = (float)acc;
-    }
-}
-
 // y = (x - mean) * rstd * gamma + beta             (BWD = false)
 // gx = gamma * rstd * (gy - s0/N - xhat * s1/N)    (BWD = true; inv_count = 1/N)
 template <typename T, int G, int V, bool BWD, int ACT = 0>
@@ -273,8 +259,7 @@ static sar_status norm_sums(const Shape &s, NormArgs a, double scale, float *out
         else
             SAR_LAUNCH(name, st, (norm_sums_generic<__nv_bfloat16, WHAT><<<blocks, 256, 0, st>>>(a, (int)slices)));
         SAR_TRY(sar_after_launch());
-        SAR_LAUNCH("bn_reduce", st, norm_reduce_kernel<<<(2 * a.C + 255) / 256, 256, 0, st>>>((int)slices, a.C, a.partial, scale, out0, out1));
-        return sar_after_launch();
+        return reduce_partials("bn_reduce", (int)slices, 2 * a.C, a.C, a.partial, scale, out0, out1, st);
     }
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
@@ -285,10 +270,12 @@ static sar_status norm_sums(const Shape &s, NormArgs a, double scale, float *out
                     : (a.act == 3 ? norm_sums_kernel<T, C::g, C::v, WHAT, (WHAT == kSumGrad ? 3 : 0)>
                                   : norm_sums_kernel<T, C::g, C::v, WHAT, (WHAT == kSumGrad ? 1 : 0)>);
         SAR_TRY(ensure_smem(kern, smem));
-        SAR_LAUNCH(name, st, kern<<<kNormBlocks, kThreads, smem, st>>>(a));
+        // a few rows per lane group before a block pays for its record; the grid depends on n alone
+        const unsigned want = blocks_for((a.n + 3) / 4, C::g);
+        const unsigned blocks = want < 1 ? 1 : want < (unsigned)kNormBlocks ? want : (unsigned)kNormBlocks;
+        SAR_LAUNCH(name, st, kern<<<blocks, kThreads, smem, st>>>(a));
         SAR_TRY(sar_after_launch());
-        SAR_LAUNCH("bn_reduce", st, norm_reduce_kernel<<<(2 * a.C + 255) / 256, 256, 0, st>>>(kNormBlocks, a.C, a.partial, scale, out0, out1));
-        return sar_after_launch();
+        return reduce_partials("bn_reduce", (int)blocks, 2 * a.C, a.C, a.partial, scale, out0, out1, st);
     });
 }
 
