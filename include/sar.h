@@ -138,6 +138,12 @@ SAR_API sar_status sar_csr_from_coo(int64_t n_rows, int64_t n_cols, int64_t nnz,
                             const int32_t *col, int64_t *indptr, int32_t *indices, void *workspace,
                             size_t workspace_bytes, void *stream);
 
+/* Both orientations of a graph of n nodes in one call: the CSR by destination and the CSC of the edges src[t] -> dst[t],
+ * the same arrays that the two calls of sar_csr_from_coo would give (the CSC costs one sort of the CSR's edges). */
+SAR_API sar_status sar_graph_from_coo(int64_t n, int64_t nnz, const int32_t *src, const int32_t *dst, int64_t *indptr,
+                                      int32_t *indices, int64_t *t_indptr, int32_t *t_indices, void *workspace,
+                                      size_t workspace_bytes, void *stream);
+
 /* CSR (n_rows x n_cols) -> its transpose (n_cols x n_rows), same ordering rule. */
 SAR_API sar_status sar_csr_transpose(int64_t n_rows, int64_t n_cols, const int64_t *indptr, const int32_t *indices,
                              int64_t *t_indptr, int32_t *t_indices, void *workspace, size_t workspace_bytes,
@@ -223,6 +229,28 @@ SAR_API sar_status sar_plan_count(int64_t n_rows, const int64_t *indptr, int32_t
 SAR_API sar_status sar_plan_fill(int64_t n_rows, const int64_t *indptr, int32_t threshold, int32_t n_long,
                          int32_t *long_row, int64_t *long_seg, void *workspace, size_t workspace_bytes,
                          void *stream);
+
+/* The plans of several CSRs together (the whole graph's two and its partitions'), with no synchronisation inside: jobs is
+ * a HOST array (count <= 2 * SAR_MAX_PARTS + 2), its indptr arrays DEVICE.  sar_plan_count_many writes n_long and n_seg
+ * of job j to the DEVICE array counts[2j], counts[2j + 1]; the caller reads them, sizes the arrays, enters them as
+ * long_row / long_seg (DEVICE; long_row may be any pointer where n_long = 0) and calls sar_plan_fill_many with the
+ * same jobs and the same, untouched workspace of sar_plan_many_workspace_bytes. */
+typedef struct {
+    int64_t n_rows;
+    const int64_t *indptr;
+    int32_t threshold;
+    int32_t *long_row;
+    int64_t *long_seg;
+} sar_plan_job;
+SAR_API size_t sar_plan_many_workspace_bytes(int32_t count, const sar_plan_job *jobs);
+SAR_API sar_status sar_plan_count_many(int32_t count, const sar_plan_job *jobs, int64_t *counts, void *workspace,
+                                       size_t workspace_bytes, void *stream);
+SAR_API sar_status sar_plan_fill_many(int32_t count, const sar_plan_job *jobs, void *workspace, size_t workspace_bytes,
+                                      void *stream);
+
+/* out[i] = *from[i]: single values of several DEVICE arrays side by side, so that one copy brings them to the host.
+ * from: HOST array of count DEVICE pointers (count <= 2 * SAR_MAX_PARTS + 2), out: DEVICE. */
+SAR_API sar_status sar_gather_i64(int32_t count, const int64_t *const *from, int64_t *out, void *stream);
 
 /* ---------------------------------------------------------------------------------------------
  * Fused GAT aggregation, forward (Eq. 3; Algorithm 1; Sec. 3.3; running max of Sec. 3.4).

@@ -87,21 +87,20 @@ class Graph:
             src, dst = src2, dst2
         elif reorder is not None:
             raise ValueError(f"unknown reorder {reorder!r}")
-        ws = _workspace(B.sar_graph_workspace_bytes(nnz, n), dev)
-        indptr = torch.empty(n + 1, dtype=torch.int64, device=dev)
-        indices = torch.empty(nnz, dtype=torch.int32, device=dev)
-        B.sar_csr_from_coo(n, n, dst, src, indptr, indices, ws)
-        t_indptr = torch.empty(n + 1, dtype=torch.int64, device=dev)
-        t_indices = torch.empty(nnz, dtype=torch.int32, device=dev)
-        B.sar_csr_from_coo(n, n, src, dst, t_indptr, t_indices, ws)
         if t_threshold is None:   # the CSC's plan has its own threshold
             t_threshold = DEFAULT_T_THRESHOLD if threshold == DEFAULT_THRESHOLD else threshold
-        split = build_plan(n, indptr, threshold) if threshold else None
-        t_split = build_plan(n, t_indptr, t_threshold) if t_threshold else None
-        whole = B.Part(n, n, indptr, indices, t_indptr, t_indices, split, t_split)
-        g = Graph(n=n, nnz=nnz, whole=whole, k=k, bounds=B.sar_partition_bounds(n, k), order=order, rank=rank)
-        if build_parts:
-            g.parts = split_parts(whole, g.bounds, threshold, ws)
+        assert src.dtype == torch.int32 and dst.dtype == torch.int32 and nnz == dst.numel()
+        bounds = B.sar_partition_bounds(n, k)
+        arrays, plans, parts = B.native().from_coo(n, src, dst, bounds, threshold or 0, t_threshold or 0, build_parts)
+        plans = iter(plans)
+
+        def plan(thr):
+            return B.Split(thr, *next(plans)) if thr else None
+
+        whole = B.Part(n, n, *arrays, plan(threshold), plan(t_threshold))
+        g = Graph(n=n, nnz=nnz, whole=whole, k=k, bounds=bounds, order=order, rank=rank)
+        g.parts = [B.Part(n, bounds[q + 1] - bounds[q], ip, idx, t_ip, t_idx, plan(threshold), plan(threshold), nnz=nnz_q)
+                   for q, (ip, idx, t_ip, t_idx, nnz_q) in enumerate(parts)]
         return g
 
 

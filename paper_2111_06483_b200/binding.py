@@ -36,6 +36,7 @@ EXPORTS = [
     "sar_bn_bwd_stats_act", "sar_bn_bwd_apply_act", "sar_csc_slice_indptr",
     "sar_gat_storing_workspace_bytes", "sar_gat_fwd_storing", "sar_gat_bwd_storing", "sar_bn_combine_moments",
     "sar_bn_combine_sums", "sar_degree_order_workspace_bytes", "sar_degree_order", "sar_relabel", "sar_permute_rows", "sar_linear_project", "sar_linear_bwd_input_relu",
+    "sar_graph_from_coo", "sar_plan_many_workspace_bytes", "sar_plan_count_many", "sar_plan_fill_many", "sar_gather_i64",
 ]
 
 
@@ -47,6 +48,11 @@ class SarError(RuntimeError):
 
 class sar_split(Structure):
     _fields_ = [("threshold", c_int32), ("n_long", c_int32), ("n_seg", c_int64), ("long_row", c_void_p),
+                ("long_seg", c_void_p)]
+
+
+class sar_plan_job(Structure):
+    _fields_ = [("n_rows", c_int64), ("indptr", c_void_p), ("threshold", c_int32), ("long_row", c_void_p),
                 ("long_seg", c_void_p)]
 
 
@@ -74,7 +80,7 @@ def lib() -> ctypes.CDLL:
         for name in ("sar_graph_workspace_bytes", "sar_gat_workspace_bytes", "sar_spmm_workspace_bytes",
                      "sar_gat_stack_arena_bytes", "sar_gat_bwd_noalloc_limit", "sar_gat_project_workspace_bytes",
                      "sar_bn_workspace_bytes", "sar_linear_workspace_bytes", "sar_gat_storing_workspace_bytes",
-                     "sar_degree_order_workspace_bytes"):
+                     "sar_degree_order_workspace_bytes", "sar_plan_many_workspace_bytes"):
             getattr(L, name).restype = c_size_t
         _lib = L
     return _lib
@@ -239,6 +245,15 @@ def sar_csr_from_coo(n_rows: int, n_cols: int, row: torch.Tensor, col: torch.Ten
                                                       _stream()))
 
 
+def sar_graph_from_coo(n: int, src: torch.Tensor, dst: torch.Tensor, indptr: torch.Tensor, indices: torch.Tensor,
+                       t_indptr: torch.Tensor, t_indices: torch.Tensor, workspace: torch.Tensor) -> None:
+    assert src.dtype == torch.int32 and dst.dtype == torch.int32 and src.numel() == dst.numel()
+    w, wb = _ws(workspace)
+    _check("sar_graph_from_coo", lib().sar_graph_from_coo(c_int64(n), c_int64(src.numel()), _ptr(src), _ptr(dst),
+                                                          _ptr(indptr), _ptr(indices), _ptr(t_indptr), _ptr(t_indices),
+                                                          w, wb, _stream()))
+
+
 def sar_csr_transpose(n_rows: int, n_cols: int, indptr: torch.Tensor, indices: torch.Tensor,
                       t_indptr: torch.Tensor, t_indices: torch.Tensor, workspace: torch.Tensor) -> None:
     w, wb = _ws(workspace)
@@ -345,6 +360,35 @@ def sar_plan_fill(n_rows: int, indptr: torch.Tensor, threshold: int, n_long: int
     w, wb = _ws(workspace)
     _check("sar_plan_fill", lib().sar_plan_fill(c_int64(n_rows), _ptr(indptr), c_int32(threshold), c_int32(n_long),
                                                 _ptr(long_row), _ptr(long_seg), w, wb, _stream()))
+
+
+def _plan_jobs(jobs):
+    """jobs: (n_rows, indptr, threshold, long_row or None, long_seg or None) of each CSR"""
+    arr = (sar_plan_job * max(len(jobs), 1))()
+    for a, (n_rows, indptr, threshold, row, seg) in zip(arr, jobs):
+        a.n_rows, a.threshold, a.indptr = n_rows, threshold, indptr.data_ptr()
+        a.long_row, a.long_seg = (row.data_ptr() or seg.data_ptr(), seg.data_ptr()) if seg is not None else (None, None)
+    return arr
+
+
+def sar_plan_many_workspace_bytes(jobs) -> int:
+    return int(lib().sar_plan_many_workspace_bytes(c_int32(len(jobs)), _plan_jobs(jobs)))
+
+
+def sar_plan_count_many(jobs, counts: torch.Tensor, workspace: torch.Tensor) -> None:
+    w, wb = _ws(workspace)
+    _check("sar_plan_count_many", lib().sar_plan_count_many(c_int32(len(jobs)), _plan_jobs(jobs), _ptr(counts), w, wb, _stream()))
+
+
+def sar_plan_fill_many(jobs, workspace: torch.Tensor) -> None:
+    w, wb = _ws(workspace)
+    _check("sar_plan_fill_many", lib().sar_plan_fill_many(c_int32(len(jobs)), _plan_jobs(jobs), w, wb, _stream()))
+
+
+def sar_gather_i64(arrays_and_offsets, out: torch.Tensor) -> None:
+    """out[i] = array[offset] for each (array, offset), int64"""
+    ptrs = (c_void_p * max(len(arrays_and_offsets), 1))(*[t.data_ptr() + 8 * int(o) for t, o in arrays_and_offsets])
+    _check("sar_gather_i64", lib().sar_gather_i64(c_int32(len(arrays_and_offsets)), ptrs, _ptr(out), _stream()))
 
 
 # ----------------------------------------------------------------------------------------------

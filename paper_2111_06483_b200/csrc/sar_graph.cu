@@ -1,12 +1,13 @@
 // Graph preparation on the device: edge list -> CSR / CSC, split by source range, long-row plan,
 // validation.  Integer work whose results are unique.  Sorting and prefix sums are CUB device
-// primitives; everything else is small kernels in this file.  Contracts are in include/sar.h.
+// primitives or the passes of sar_radix.cuh; everything else is small kernels in this file.  Contracts are in include/sar.h.
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_scan.cuh>
 #include <cub/device/device_select.cuh>
 #include <thrust/iterator/counting_iterator.h>
 
 #include "sar_common.cuh"
+#include "sar_radix.cuh"
 
 namespace sar {
 
@@ -46,6 +47,43 @@ __global__ void keys_to_csr_kernel(long long nnz, long long n_rows, const unsign
     if (t < nnz) indices[t] = (int32_t)(unsigned)(keys[t] & 0xffffffffull);
 }
 
+// Sorted row ids of the edges -> indptr (first position of each row); four ids a thread (one a thread: 0.20 ms for 62
+// million edges, now 0.11).  row is 16-byte aligned.
+__global__ void rows_to_indptr_kernel(long long nnz, long long n_rows, const unsigned *__restrict__ row, int64_t *__restrict__ indptr) {
+    const long long t0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (t0 > nnz) return;
+    unsigned id[4];
+    if (t0 + 4 <= nnz) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(row + t0);
+        id[0] = v.x;
+        id[1] = v.y;
+        id[2] = v.z;
+        id[3] = v.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) id[i] = t0 + i < nnz ? row[t0 + i] : (unsigned)n_rows;
+    }
+    long long r = t0 > 0 ? (long long)row[t0 - 1] + 1 : 0;   // rows below r have their place
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const long long cur = t0 + i < nnz ? min((long long)id[i], n_rows) : n_rows;
+        if (t0 + i <= nnz)
+            for (; r <= cur; ++r) indptr[r] = t0 + i;
+    }
+}
+
+// row id of every edge of a CSR, found by bisection of indptr
+__global__ void edge_rows_kernel(long long nnz, long long n_rows, const int64_t *__restrict__ indptr, unsigned *__restrict__ row) {
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nnz) return;
+    long long lo = 0, hi = n_rows;  // last r with indptr[r] <= t
+    while (hi - lo > 1) {
+        const long long mid = (lo + hi) >> 1;
+        if (indptr[mid] <= t) lo = mid; else hi = mid;
+    }
+    row[t] = (unsigned)lo;
+}
+
 __device__ __forceinline__ long long lower_bound_row(const int32_t *__restrict__ idx, long long lo, long long hi,
                                                      long long key) {
     while (lo < hi) {
@@ -70,16 +108,76 @@ __global__ void split_count_kernel(long long n_dst, const int64_t *__restrict__ 
     }
 }
 
-__global__ void split_fill_kernel(long long n_dst, const int64_t *__restrict__ indptr,
-                                  const int32_t *__restrict__ indices, Bounds b, Bounds off,
-                                  const int64_t *__restrict__ indptr_all, int32_t *__restrict__ indices_all) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_dst) return;
-    const long long end = indptr[i + 1];
-    long long t = indptr[i];
-    for (int q = 0; q < b.k && t < end; ++q) {
-        long long w = off.s[q] + indptr_all[(long long)q * (n_dst + 1) + i];
-        while (t < end && indices[t] < b.s[q + 1]) indices_all[w++] = (int32_t)(indices[t++] - b.s[q]);
+// The edges of a block's rows, one partition after the other: a stable partition of a run of edges.  The block takes its
+// run 2048 edges at a time and writes every partition's share behind what it wrote before, starting where indptr_all says
+// its first row's edges go; within a tile, ballots over the partition's number rank the edges of a warp.  Rows are only
+// looked at for the run's ends, so long and short ones cost the same.  62 million edges in four partitions: 0.29 ms; a
+// warp per row took 0.87 ms (three loads in a chain for 25 edges) and a thread per row 1.92 ms.
+constexpr int kSplitItems = 8, kSplitWarps = 8;
+__global__ void __launch_bounds__(kSplitWarps * 32) split_fill_kernel(long long n_dst, int rows, int q_bits, const int64_t *__restrict__ indptr,
+                                                                      const int32_t *__restrict__ indices, const Bounds b, const Bounds off,
+                                                                      const int64_t *__restrict__ indptr_all, int32_t *__restrict__ indices_all) {
+    __shared__ long long next[SAR_MAX_PARTS];
+    __shared__ int bound[SAR_MAX_PARTS];
+    __shared__ unsigned short count[kSplitWarps][SAR_MAX_PARTS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long row0 = (long long)blockIdx.x * rows, row1 = row0 + rows < n_dst ? row0 + rows : n_dst;
+    const long long beg = indptr[row0], end = indptr[row1];
+    if ((int)threadIdx.x < b.k) {
+        bound[threadIdx.x] = (int)b.s[threadIdx.x];
+        next[threadIdx.x] = off.s[threadIdx.x] + indptr_all[(long long)threadIdx.x * (n_dst + 1) + row0];
+    }
+    __syncthreads();
+    const unsigned lt = (1u << lane) - 1u;
+    for (long long base = beg; base < end; base += kSplitWarps * 32 * kSplitItems) {
+        const int left = (int)(end - base < kSplitWarps * 32 * kSplitItems ? end - base : kSplitWarps * 32 * kSplitItems) - warp * (32 * kSplitItems) - lane;
+        const int32_t *from = indices + base + warp * (32 * kSplitItems) + lane;
+        int j[kSplitItems];
+        unsigned place[kSplitItems];   // partition in the upper half, rank among the warp's edges of it in the lower
+#pragma unroll
+        for (int i = 0; i < kSplitItems; ++i) j[i] = i * 32 < left ? from[i * 32] : 0;
+        for (int q = lane; q < b.k; q += 32) count[warp][q] = 0;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < kSplitItems; ++i) {
+            const bool in = i * 32 < left;
+            int lo = 0, hi = b.k;   // last q with bounds[q] <= j: empty partitions are skipped by taking the last
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (bound[mid] <= j[i]) lo = mid; else hi = mid;
+            }
+            unsigned same = __ballot_sync(0xffffffffu, in);
+            for (int bit = 0; bit < q_bits; ++bit) {
+                const bool set = (lo >> bit) & 1;
+                const unsigned m = __ballot_sync(0xffffffffu, set);
+                same &= set ? m : ~m;
+            }
+            const unsigned before = count[warp][lo];
+            place[i] = (unsigned)lo << 16 | (before + __popc(same & lt));
+            __syncwarp();
+            if (in && (same & lt) == 0u) count[warp][lo] = (unsigned short)(before + __popc(same));
+            __syncwarp();
+        }
+        __syncthreads();
+        unsigned total = 0;
+        if ((int)threadIdx.x < b.k) {
+#pragma unroll
+            for (int w = 0; w < kSplitWarps; ++w) {
+                const unsigned c = count[w][threadIdx.x];
+                count[w][threadIdx.x] = (unsigned short)total;
+                total += c;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kSplitItems; ++i) {
+            if (i * 32 < left) {
+                const unsigned q = place[i] >> 16;
+                indices_all[next[q] + count[warp][q] + (place[i] & 0xffffu)] = j[i] - bound[q];
+            }
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < b.k) next[threadIdx.x] += total;
     }
 }
 
@@ -120,6 +218,126 @@ __global__ void plan_segcount_kernel(int n_long, const int32_t *__restrict__ lon
     }
     const long long deg = indptr[long_row[lr] + 1] - indptr[long_row[lr]];
     segs[lr] = (deg + threshold - 1) / threshold;
+}
+
+// ---- long-row plans of several CSRs at once -----------------------------------------------------------------------------
+constexpr int kPlanThreads = 256, kPlanRows = 1024, kPlanMax = 2 * SAR_MAX_PARTS + 2;
+struct PlanJobs {
+    int count;
+    struct {
+        long long n_rows;
+        const int64_t *indptr;
+        long long first_block;   // of this job among all jobs' blocks
+        int32_t *long_row;
+        int64_t *long_seg;
+    } job[kPlanMax];
+    int threshold[kPlanMax];
+};
+static_assert(sizeof(PlanJobs) <= 4096 * 2, "kernel parameters");
+
+// (long rows, segments) of the block's rows; FILL: written out behind those of the blocks before
+template <bool FILL>
+__global__ void __launch_bounds__(kPlanThreads) plan_many_kernel(const __grid_constant__ PlanJobs jobs, unsigned long long *__restrict__ blocks) {
+    __shared__ unsigned long long warp_sum[kPlanThreads / 32];
+    const int j = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long n = jobs.job[j].n_rows, row0 = (long long)blockIdx.x * kPlanRows + threadIdx.x * (kPlanRows / kPlanThreads);
+    if ((long long)blockIdx.x * kPlanRows >= n) return;
+    const int64_t *indptr = jobs.job[j].indptr;
+    const long long threshold = jobs.threshold[j];
+    // rows in the low 16 bits (a block has 1024), segments above them
+    unsigned long long mine = 0;
+    long long segs[kPlanRows / kPlanThreads];
+    long long prev = row0 < n ? indptr[row0] : 0;
+#pragma unroll
+    for (int k = 0; k < kPlanRows / kPlanThreads; ++k) {
+        segs[k] = 0;
+        if (row0 + k < n) {
+            const long long next = indptr[row0 + k + 1], deg = next - prev;
+            prev = next;
+            if (deg > threshold) {
+                segs[k] = (deg + threshold - 1) / threshold;
+                mine += 1ull + ((unsigned long long)segs[k] << 16);
+            }
+        }
+    }
+    unsigned long long inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+    }
+    if (lane == 31) warp_sum[warp] = inc;
+    __syncthreads();
+    unsigned long long before = inc - mine, all = 0;
+#pragma unroll
+    for (int w = 0; w < kPlanThreads / 32; ++w) {
+        if (w < warp) before += warp_sum[w];
+        all += warp_sum[w];
+    }
+    unsigned long long *rec = blocks + 2 * (jobs.job[j].first_block + blockIdx.x);
+    if (!FILL) {
+        if (threadIdx.x == 0) {
+            rec[0] = all & 0xffffull;
+            rec[1] = all >> 16;
+        }
+    } else {
+        long long lr = (long long)(rec[0] + (before & 0xffffull)), sg = (long long)(rec[1] + (before >> 16));
+#pragma unroll
+        for (int k = 0; k < kPlanRows / kPlanThreads; ++k) {
+            if (segs[k] > 0) {
+                jobs.job[j].long_row[lr] = (int32_t)(row0 + k);
+                jobs.job[j].long_seg[lr] = sg;
+                ++lr;
+                sg += segs[k];
+                if ((long long)blockIdx.x * kPlanRows + kPlanRows >= n && lr == (long long)(rec[0] + (all & 0xffffull))) jobs.job[j].long_seg[lr] = sg;
+            }
+        }
+        // a last block without long rows of its own closes the list all the same
+        if (threadIdx.x == 0 && (long long)blockIdx.x * kPlanRows + kPlanRows >= n && (all & 0xffffull) == 0)
+            jobs.job[j].long_seg[rec[0]] = (int64_t)rec[1];
+    }
+}
+
+// blocks' records -> exclusive prefix sums, totals to counts[2 * job ..]; one block per job
+__global__ void __launch_bounds__(1024) plan_scan_kernel(const __grid_constant__ PlanJobs jobs, unsigned long long *__restrict__ blocks, int64_t *__restrict__ counts) {
+    __shared__ unsigned long long warp_sum[2][32], carry[2];
+    const int j = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long nb = (jobs.job[j].n_rows + kPlanRows - 1) / kPlanRows;
+    unsigned long long *rec = blocks + 2 * jobs.job[j].first_block;
+    if (threadIdx.x < 2) carry[threadIdx.x] = 0;
+    __syncthreads();
+    for (long long base = 0; base < nb; base += 1024) {
+        const long long at = base + threadIdx.x;
+        unsigned long long v[2], inc[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            v[c] = inc[c] = at < nb ? rec[2 * at + c] : 0ull;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long t = __shfl_up_sync(0xffffffffu, inc[c], o);
+                if (lane >= o) inc[c] += t;
+            }
+            if (lane == 31) warp_sum[c][warp] = inc[c];
+        }
+        __syncthreads();
+        if (warp < 2) {
+            unsigned long long w = warp_sum[warp][lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long t = __shfl_up_sync(0xffffffffu, w, o);
+                if (lane >= o) w += t;
+            }
+            warp_sum[warp][lane] = w;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            if (at < nb) rec[2 * at + c] = carry[c] + (warp ? warp_sum[c][warp - 1] : 0ull) + inc[c] - v[c];
+        __syncthreads();
+        if (threadIdx.x < 2) carry[threadIdx.x] += warp_sum[threadIdx.x][31];
+        __syncthreads();
+    }
+    if (threadIdx.x < 2) counts[2 * j + threadIdx.x] = (int64_t)carry[threadIdx.x];
 }
 
 __global__ void validate_kernel(long long n_rows, long long n_cols, long long nnz, const int64_t *__restrict__ indptr,
@@ -271,6 +489,125 @@ static int bits_for(long long n) {
     return b;
 }
 
+// ---- CSR and CSC from (row, column) pairs ---------------------------------------------------------------------------------
+constexpr long long kPairLimit = 1LL << 31;   // edges from which positions no longer fit 32 bits: 64-bit keys through CUB
+
+struct PairBuffers {
+    unsigned *b[4];   // nnz ids each
+    void *scratch;
+};
+static sar_status pair_buffers(long long nnz, void *ws, size_t ws_bytes, PairBuffers *p) {
+    const size_t kb = sar_round_up((size_t)nnz * 4, 256);
+    if (!ws || !sar_aligned(ws, 256) || ws_bytes < 4 * kb + radix_scratch_bytes(nnz)) return SAR_ERR_WORKSPACE;
+    for (int i = 0; i < 4; ++i) p->b[i] = reinterpret_cast<unsigned *>(static_cast<char *>(ws) + i * kb);
+    p->scratch = static_cast<char *>(ws) + 4 * kb;
+    return SAR_OK;
+}
+
+// Edges ordered by (row, column): a stable sort by column, then one by row.  *rows = the sorted row ids (one of b[0], b[2]).
+static sar_status csr_from_pairs(long long n_rows, long long n_cols, long long nnz, const int32_t *row, const int32_t *col, int64_t *indptr,
+                                 int32_t *indices, const PairBuffers &p, unsigned **rows, cudaStream_t st) {
+    *rows = p.b[0];
+    if (nnz > 0) {
+        unsigned *const *b = p.b;
+        SAR_TRY(radix_sort_pairs(nnz, bits_for(n_cols), reinterpret_cast<const unsigned *>(col), reinterpret_cast<const unsigned *>(row), b[0], b[1],
+                                 b[2], b[3], p.scratch, st));   // (column, row) in b[2], b[3]
+        // an odd number of passes writes its result first, when the input is still being read: it goes elsewhere
+        const bool even = radix_passes(bits_for(n_rows)) % 2 == 0;
+        unsigned *out = even ? b[2] : b[0], *kt = even ? b[0] : b[3], *vt = even ? b[1] : b[2];
+        SAR_TRY(radix_sort_pairs(nnz, bits_for(n_rows), b[3], b[2], kt, vt, out, reinterpret_cast<unsigned *>(indices), p.scratch, st));
+        *rows = out;
+    }
+    rows_to_indptr_kernel<<<nblk(nnz / 4 + 1), 256, 0, st>>>(nnz, n_rows, *rows, indptr);
+    return sar_after_launch();
+}
+
+// (row, column) pairs in row order (rows: b[0] or b[2]) -> the CSC
+static sar_status csc_from_rows(long long n_cols, long long nnz, const unsigned *rows, const int32_t *indices, int64_t *t_indptr, int32_t *t_indices,
+                                const PairBuffers &p, cudaStream_t st) {
+    unsigned *const *b = p.b;
+    unsigned *cols = rows == b[0] ? b[2] : b[0];
+    if (nnz > 0)
+        SAR_TRY(radix_sort_pairs(nnz, bits_for(n_cols), reinterpret_cast<const unsigned *>(indices), rows, b[1], b[3], cols,
+                                 reinterpret_cast<unsigned *>(t_indices), p.scratch, st));
+    rows_to_indptr_kernel<<<nblk(nnz / 4 + 1), 256, 0, st>>>(nnz, n_cols, cols, t_indptr);
+    return sar_after_launch();
+}
+
+// counts of one partition per block -> its indptr, in place (inclusive prefix sum of n values), for small graphs
+__global__ void __launch_bounds__(1024) split_scan_kernel(long long n, int64_t *__restrict__ indptr_all) {
+    __shared__ long long warp_sum[32], carry;
+    int64_t *p = indptr_all + (long long)blockIdx.x * n;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) carry = 0;
+    __syncthreads();
+    for (long long base = 0; base < n; base += 4096) {
+        long long v[4], s = 0;
+        const long long at = base + threadIdx.x * 4;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = at + k < n ? p[at + k] : 0;
+            s += v[k];
+        }
+        long long inc = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
+        }
+        if (lane == 31) warp_sum[warp] = inc;
+        __syncthreads();
+        if (warp == 0) {
+            long long w = warp_sum[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long t = __shfl_up_sync(0xffffffffu, w, o);
+                if (lane >= o) w += t;
+            }
+            warp_sum[lane] = w;
+        }
+        __syncthreads();
+        long long run = carry + (warp ? warp_sum[warp - 1] : 0) + inc - s;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            run += v[k];
+            if (at + k < n) p[at + k] = run;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) carry += warp_sum[31];
+        __syncthreads();
+    }
+}
+constexpr long long kSplitScanRows = 32 * 1024;   // rows up to which a block per partition beats a device-wide scan for each
+
+struct GatherList {
+    int count;
+    const int64_t *from[2 * SAR_MAX_PARTS + 2];
+};
+__global__ void gather_i64_kernel(const GatherList g, int64_t *__restrict__ out) {
+    if ((int)threadIdx.x < g.count) out[threadIdx.x] = *g.from[threadIdx.x];
+}
+
+static sar_status plan_jobs(int32_t count, const sar_plan_job *jobs, PlanJobs *out, long long *blocks, long long *widest) {
+    if (count < 0 || count > kPlanMax || (count > 0 && !jobs)) return SAR_ERR_INVALID_ARG;
+    out->count = count;
+    *blocks = *widest = 0;
+    for (int j = 0; j < count; ++j) {
+        if (jobs[j].n_rows < 0 || !jobs[j].indptr || jobs[j].threshold < 1) return SAR_ERR_INVALID_ARG;
+        if (jobs[j].n_rows > INT32_MAX) return SAR_ERR_UNSUPPORTED;
+        const long long nb = (jobs[j].n_rows + kPlanRows - 1) / kPlanRows;
+        out->job[j].n_rows = jobs[j].n_rows;
+        out->job[j].indptr = jobs[j].indptr;
+        out->job[j].first_block = *blocks;
+        out->job[j].long_row = jobs[j].long_row;
+        out->job[j].long_seg = jobs[j].long_seg;
+        out->threshold[j] = jobs[j].threshold;
+        *blocks += nb;
+        if (nb > *widest) *widest = nb;
+    }
+    return SAR_OK;
+}
+
 }  // namespace sar
 
 using namespace sar;
@@ -279,11 +616,11 @@ extern "C" {
 
 size_t sar_graph_workspace_bytes(int64_t nnz, int64_t n_rows) {
     if (nnz < 0 || n_rows < 0) return 0;
-    size_t temp = sort_temp_bytes(nnz);
+    size_t temp = nnz < kPairLimit ? radix_scratch_bytes(nnz) : sort_temp_bytes(nnz);
     const size_t a = scan_temp_bytes(n_rows + 1), b = select_temp_bytes(n_rows);
     if (a > temp) temp = a;
     if (b > temp) temp = b;
-    return 2 * sar_round_up((size_t)nnz * 8, 256) + sar_round_up(temp, 256) + sar_round_up((size_t)(n_rows + 1) * 8, 256) + 512;
+    return 2 * sar_round_up((size_t)nnz * 8, 256) + sar_round_up(temp, 256) + sar_round_up((size_t)(n_rows + 1) * 8, 256) + 1024;
 }
 
 sar_status sar_csr_from_coo(int64_t n_rows, int64_t n_cols, int64_t nnz, const int32_t *row, const int32_t *col,
@@ -294,18 +631,44 @@ sar_status sar_csr_from_coo(int64_t n_rows, int64_t n_cols, int64_t nnz, const i
     if (nnz > 0 && (!row || !col || !indices)) return SAR_ERR_INVALID_ARG;
     if (!sar_aligned(indptr, 8) || !sar_aligned(indices, 4) || !sar_aligned(row, 4) || !sar_aligned(col, 4))
         return SAR_ERR_ALIGNMENT;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (nnz < kPairLimit) {
+        PairBuffers p;
+        SAR_TRY(pair_buffers(nnz, workspace, workspace_bytes, &p));
+        unsigned *rows = nullptr;
+        return csr_from_pairs(n_rows, n_cols, nnz, row, col, indptr, indices, p, &rows, st);
+    }
     const size_t kb = sar_round_up((size_t)nnz * 8, 256);
     if (!workspace || !sar_aligned(workspace, 256) || workspace_bytes < 2 * kb) return SAR_ERR_WORKSPACE;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned long long *keys = static_cast<unsigned long long *>(workspace);
     unsigned long long *sorted = keys;
-    if (nnz > 0) {
-        make_keys_kernel<<<nblk(nnz), 256, 0, st>>>(nnz, row, col, keys);
-        SAR_TRY(sar_after_launch());
-        SAR_TRY(sort_keys(nnz, 32 + bits_for(n_rows), workspace, workspace_bytes, st, &sorted));
-    }
+    make_keys_kernel<<<nblk(nnz), 256, 0, st>>>(nnz, row, col, keys);
+    SAR_TRY(sar_after_launch());
+    SAR_TRY(sort_keys(nnz, 32 + bits_for(n_rows), workspace, workspace_bytes, st, &sorted));
     keys_to_csr_kernel<<<nblk(nnz + 1), 256, 0, st>>>(nnz, n_rows, sorted, indptr, indices);
     return sar_after_launch();
+}
+
+sar_status sar_graph_from_coo(int64_t n, int64_t nnz, const int32_t *src, const int32_t *dst, int64_t *indptr, int32_t *indices,
+                              int64_t *t_indptr, int32_t *t_indices, void *workspace, size_t workspace_bytes, void *stream) {
+    if (n < 0 || nnz < 0 || !indptr || !t_indptr) return SAR_ERR_INVALID_ARG;
+    if (n > INT32_MAX) return SAR_ERR_UNSUPPORTED;
+    if (nnz > 0 && (!src || !dst || !indices || !t_indices)) return SAR_ERR_INVALID_ARG;
+    for (const void *q : {(const void *)indptr, (const void *)t_indptr})
+        if (!sar_aligned(q, 8)) return SAR_ERR_ALIGNMENT;
+    for (const void *q : {(const void *)src, (const void *)dst, (const void *)indices, (const void *)t_indices})
+        if (!sar_aligned(q, 4)) return SAR_ERR_ALIGNMENT;
+    if (nnz >= kPairLimit) {
+        SAR_TRY(sar_csr_from_coo(n, n, nnz, dst, src, indptr, indices, workspace, workspace_bytes, stream));
+        return sar_csr_from_coo(n, n, nnz, src, dst, t_indptr, t_indices, workspace, workspace_bytes, stream);
+    }
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    PairBuffers p;
+    SAR_TRY(pair_buffers(nnz, workspace, workspace_bytes, &p));
+    unsigned *rows = nullptr;
+    SAR_TRY(csr_from_pairs(n, n, nnz, dst, src, indptr, indices, p, &rows, st));
+    // the CSR's edges, destinations ascending, brought into source order by a stable sort: the CSC
+    return csc_from_rows(n, nnz, rows, indices, t_indptr, t_indices, p, st);
 }
 
 sar_status sar_csr_transpose(int64_t n_rows, int64_t n_cols, const int64_t *indptr, const int32_t *indices,
@@ -322,15 +685,22 @@ sar_status sar_csr_transpose(int64_t n_rows, int64_t n_cols, const int64_t *indp
     SAR_CUDA_TRY(cudaStreamSynchronize(st));
     if (nnz < 0) return SAR_ERR_BAD_GRAPH;
     if (nnz > 0 && (!indices || !t_indices)) return SAR_ERR_INVALID_ARG;
+    if (nnz < kPairLimit) {
+        PairBuffers p;
+        SAR_TRY(pair_buffers(nnz, workspace, workspace_bytes, &p));
+        if (nnz > 0) {
+            edge_rows_kernel<<<nblk(nnz), 256, 0, st>>>(nnz, n_rows, indptr, p.b[0]);
+            SAR_TRY(sar_after_launch());
+        }
+        return csc_from_rows(n_cols, nnz, p.b[0], indices, t_indptr, t_indices, p, st);
+    }
     const size_t kb = sar_round_up((size_t)nnz * 8, 256);
     if (!workspace || !sar_aligned(workspace, 256) || workspace_bytes < 2 * kb) return SAR_ERR_WORKSPACE;
     unsigned long long *keys = static_cast<unsigned long long *>(workspace);
     unsigned long long *sorted = keys;
-    if (nnz > 0) {
-        make_transposed_keys_kernel<<<nblk(nnz), 256, 0, st>>>(nnz, n_rows, indptr, indices, keys);
-        SAR_TRY(sar_after_launch());
-        SAR_TRY(sort_keys(nnz, 32 + bits_for(n_cols), workspace, workspace_bytes, st, &sorted));
-    }
+    make_transposed_keys_kernel<<<nblk(nnz), 256, 0, st>>>(nnz, n_rows, indptr, indices, keys);
+    SAR_TRY(sar_after_launch());
+    SAR_TRY(sort_keys(nnz, 32 + bits_for(n_cols), workspace, workspace_bytes, st, &sorted));
     keys_to_csr_kernel<<<nblk(nnz + 1), 256, 0, st>>>(nnz, n_cols, sorted, t_indptr, t_indices);
     return sar_after_launch();
 }
@@ -365,6 +735,10 @@ sar_status sar_csr_split_indptr(int64_t n_dst, const int64_t *indptr, const int3
     }
     split_count_kernel<<<nblk(n_dst), 256, 0, st>>>(n_dst, indptr, indices, b, indptr_all);
     SAR_TRY(sar_after_launch());
+    if (n_dst <= kSplitScanRows) {
+        split_scan_kernel<<<k, 1024, 0, st>>>(n_dst + 1, indptr_all);
+        return sar_after_launch();
+    }
     size_t need = 0;
     SAR_CUDA_TRY(cub::DeviceScan::InclusiveSum(nullptr, need, indptr_all, indptr_all, n_dst + 1, st));
     if (!workspace || workspace_bytes < need) return SAR_ERR_WORKSPACE;
@@ -385,7 +759,11 @@ sar_status sar_csr_split_indices(int64_t n_dst, const int64_t *indptr, const int
     if (n_dst == 0 || nnz_off[k] == 0) return SAR_OK;
     if (!indices || !indices_all) return SAR_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    split_fill_kernel<<<nblk(n_dst), 256, 0, st>>>(n_dst, indptr, indices, b, off, indptr_all, indices_all);
+    // rows of a block: about a tile and a half of edges on average
+    const long long per = n_dst * 3072 / nnz_off[k];
+    const int rows = (int)(per < 1 ? 1 : per > 1024 ? 1024 : per);
+    split_fill_kernel<<<(unsigned)((n_dst + rows - 1) / rows), kSplitWarps * 32, 0, st>>>(n_dst, rows, bits_for(k), indptr, indices, b, off, indptr_all,
+                                                                                          indices_all);
     return sar_after_launch();
 }
 
@@ -502,6 +880,55 @@ sar_status sar_plan_fill(int64_t n_rows, const int64_t *indptr, int32_t threshol
     if (need > temp_bytes) return SAR_ERR_WORKSPACE;
     SAR_CUDA_TRY(cub::DeviceScan::ExclusiveSum(temp, need, long_seg, long_seg, n_long + 1, st));
     return SAR_OK;
+}
+
+size_t sar_plan_many_workspace_bytes(int32_t count, const sar_plan_job *jobs) {
+    PlanJobs p;
+    long long blocks = 0, widest = 0;
+    if (plan_jobs(count, jobs, &p, &blocks, &widest) != SAR_OK) return 0;
+    return (size_t)blocks * 16 + 256;
+}
+
+sar_status sar_plan_count_many(int32_t count, const sar_plan_job *jobs, int64_t *counts, void *workspace, size_t workspace_bytes, void *stream) {
+    PlanJobs p;
+    long long blocks = 0, widest = 0;
+    SAR_TRY(plan_jobs(count, jobs, &p, &blocks, &widest));
+    if (count == 0) return SAR_OK;
+    if (!counts) return SAR_ERR_INVALID_ARG;
+    if (!workspace || !sar_aligned(workspace, 16) || workspace_bytes < (size_t)blocks * 16) return SAR_ERR_WORKSPACE;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    unsigned long long *rec = static_cast<unsigned long long *>(workspace);
+    if (widest > 0) {
+        plan_many_kernel<false><<<dim3((unsigned)widest, (unsigned)count), kPlanThreads, 0, st>>>(p, rec);
+        SAR_TRY(sar_after_launch());
+    }
+    plan_scan_kernel<<<count, 1024, 0, st>>>(p, rec, counts);
+    return sar_after_launch();
+}
+
+sar_status sar_plan_fill_many(int32_t count, const sar_plan_job *jobs, void *workspace, size_t workspace_bytes, void *stream) {
+    PlanJobs p;
+    long long blocks = 0, widest = 0;
+    SAR_TRY(plan_jobs(count, jobs, &p, &blocks, &widest));
+    if (!workspace || !sar_aligned(workspace, 16) || workspace_bytes < (size_t)blocks * 16) return SAR_ERR_WORKSPACE;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    for (int j = 0; j < count; ++j) {
+        if (!jobs[j].long_seg || (jobs[j].n_rows > 0 && !jobs[j].long_row)) return SAR_ERR_INVALID_ARG;
+        if (jobs[j].n_rows == 0) SAR_CUDA_TRY(cudaMemsetAsync(jobs[j].long_seg, 0, 8, st));
+    }
+    if (widest == 0) return SAR_OK;
+    plan_many_kernel<true><<<dim3((unsigned)widest, (unsigned)count), kPlanThreads, 0, st>>>(p, static_cast<unsigned long long *>(workspace));
+    return sar_after_launch();
+}
+
+sar_status sar_gather_i64(int32_t count, const int64_t *const *from, int64_t *out, void *stream) {
+    if (count < 0 || count > (int32_t)(sizeof(GatherList::from) / sizeof(GatherList::from[0])) || (count > 0 && (!from || !out))) return SAR_ERR_INVALID_ARG;
+    if (count == 0) return SAR_OK;
+    GatherList g;
+    g.count = count;
+    for (int i = 0; i < count; ++i) g.from[i] = from[i];
+    gather_i64_kernel<<<1, 256, 0, static_cast<cudaStream_t>(stream)>>>(g, out);
+    return sar_after_launch();
 }
 
 size_t sar_degree_order_workspace_bytes(int64_t n) {

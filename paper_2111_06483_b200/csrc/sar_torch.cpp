@@ -24,7 +24,9 @@ namespace {
     X(sar_axpby) X(sar_relu) X(sar_gat_project) X(sar_gat_project_bwd) X(sar_gat_project_workspace_bytes)              \
     X(sar_linear_workspace_bytes) X(sar_linear) X(sar_linear_accumulate) X(sar_linear_project)                         \
     X(sar_linear_bwd_input) X(sar_linear_bwd_input_relu) X(sar_linear_bwd_weight) X(sar_bn_workspace_bytes)            \
-    X(sar_bn_stats) X(sar_bn_rstd) X(sar_bn_apply) X(sar_bn_bwd_stats) X(sar_bn_bwd_apply)
+    X(sar_bn_stats) X(sar_bn_rstd) X(sar_bn_apply) X(sar_bn_bwd_stats) X(sar_bn_bwd_apply)                             \
+    X(sar_graph_workspace_bytes) X(sar_graph_from_coo) X(sar_csr_split_indptr) X(sar_csr_split_indices)                \
+    X(sar_csc_slice_indptr) X(sar_plan_many_workspace_bytes) X(sar_plan_count_many) X(sar_plan_fill_many) X(sar_gather_i64)
 
 struct Lib {
 #define X(f) decltype(&::f) f;
@@ -134,6 +136,78 @@ PyObject *tuple(const Ts &...ts) {
     Py_ssize_t k = 0;
     ((PyTuple_SET_ITEM(r, k++, wrap(ts))), ...);
     return r;
+}
+
+// ---- graph preparation -----------------------------------------------------------------------------------------------------
+// The sizes that the host needs (edges of the partitions, long rows and segments of the plans) come over in ONE copy, so
+// that the stream is drained once: with a copy per plan and partition a small graph in 4 parts took 1.2 ms, nearly all of
+// it waiting.
+PyObject *from_coo(Args &a) {   // n, src, dst, bounds, threshold, t_threshold, parts -> ((4 arrays), plans, parts)
+    const int64_t n = a.integer();
+    const at::Tensor &src = a.tensor(), &dst = a.tensor();
+    const auto bounds = a.integers();
+    const int32_t threshold = (int32_t)a.integer(), t_threshold = (int32_t)a.integer();
+    const int64_t k = a.flag() ? (int64_t)bounds.size() - 1 : 0, nnz = src.numel();
+    const at::Tensor indptr = empty({n + 1}, at::kLong, src), t_indptr = empty({n + 1}, at::kLong, src);
+    const at::Tensor indices = empty({nnz}, at::kInt, src), t_indices = empty({nnz}, at::kInt, src);
+    auto i64 = [](const at::Tensor &t) { return static_cast<int64_t *>(t.mutable_data_ptr()); };
+    auto i32 = [](const at::Tensor &t) { return static_cast<int32_t *>(t.mutable_data_ptr()); };
+    const at::Tensor ws = bytes(L.sar_graph_workspace_bytes(nnz, n), src);
+    SAR(sar_graph_from_coo, n, nnz, i32(src), i32(dst), i64(indptr), i32(indices), i64(t_indptr), i32(t_indices), ptrm(ws), ws.nbytes(), stream());
+
+    at::Tensor indptr_all, indices_all;
+    std::vector<at::Tensor> t_ip;
+    if (k > 0) {
+        indptr_all = empty({k, n + 1}, at::kLong, src);
+        indices_all = empty({nnz > 0 ? nnz : 1}, at::kInt, src);
+        SAR(sar_csr_split_indptr, n, i64(indptr), i32(indices), (int32_t)k, bounds.data(), i64(indptr_all), ptrm(ws), ws.nbytes(), stream());
+        for (int64_t q = 0; q < k; ++q) {
+            t_ip.push_back(empty({bounds[q + 1] - bounds[q] + 1}, at::kLong, src));
+            SAR(sar_csc_slice_indptr, bounds[q], bounds[q + 1], i64(t_indptr), i64(t_ip.back()), stream());
+        }
+    }
+    std::vector<sar_plan_job> jobs;
+    if (threshold) jobs.push_back({n, i64(indptr), threshold, nullptr, nullptr});
+    if (t_threshold) jobs.push_back({n, i64(t_indptr), t_threshold, nullptr, nullptr});
+    for (int64_t q = 0; threshold && q < k; ++q) {
+        jobs.push_back({n, i64(indptr_all) + q * (n + 1), threshold, nullptr, nullptr});
+        jobs.push_back({bounds[q + 1] - bounds[q], i64(t_ip[q]), threshold, nullptr, nullptr});
+    }
+    const int32_t nj = (int32_t)jobs.size();
+    const at::Tensor sizes = empty({2 * nj + k + 1}, at::kLong, src), plan_ws = bytes(L.sar_plan_many_workspace_bytes(nj, jobs.data()), src);
+    SAR(sar_plan_count_many, nj, jobs.data(), i64(sizes), ptrm(plan_ws), plan_ws.nbytes(), stream());
+    std::vector<int64_t> host((size_t)(2 * nj + k + 1), 0);
+    if (k > 0) {   // a partition's edges are a run of the whole CSC: its first source's first edge to the next one's
+        std::vector<const int64_t *> from((size_t)k + 1);
+        for (int64_t q = 0; q <= k; ++q) from[q] = i64(t_indptr) + bounds[q];
+        SAR(sar_gather_i64, (int32_t)k + 1, from.data(), i64(sizes) + 2 * nj, stream());
+    }
+    if (nj > 0 || k > 0) {
+        cudaError_t e;
+        Py_BEGIN_ALLOW_THREADS
+        e = cudaMemcpyAsync(host.data(), i64(sizes), host.size() * 8, cudaMemcpyDeviceToHost, at::cuda::getCurrentCUDAStream());
+        if (e == cudaSuccess) e = cudaStreamSynchronize(at::cuda::getCurrentCUDAStream());
+        Py_END_ALLOW_THREADS
+        check("sar_plan_count_many", e == cudaSuccess ? SAR_OK : SAR_ERR_CUDA);
+    }
+    const int64_t *first = host.data() + 2 * nj;
+    if (k > 0)
+        SAR(sar_csr_split_indices, n, i64(indptr), i32(indices), (int32_t)k, bounds.data(), i64(indptr_all), first, i32(indices_all), stream());
+    PyObject *plans = PyTuple_New(nj);
+    for (int32_t j = 0; j < nj; ++j) {
+        const at::Tensor row = empty({host[2 * j]}, at::kInt, src), seg = empty({host[2 * j] + 1}, at::kLong, src);
+        jobs[j].long_row = host[2 * j] > 0 ? i32(row) : i32(ws);
+        jobs[j].long_seg = i64(seg);
+        PyTuple_SET_ITEM(plans, j, Py_BuildValue("(LLNN)", (long long)host[2 * j], (long long)host[2 * j + 1], wrap(row), wrap(seg)));
+    }
+    SAR(sar_plan_fill_many, nj, jobs.data(), ptrm(plan_ws), plan_ws.nbytes(), stream());
+    PyObject *parts = PyTuple_New(k);
+    for (int64_t q = 0; q < k; ++q) {
+        const int64_t cnt = first[q + 1] - first[q];
+        PyTuple_SET_ITEM(parts, q, Py_BuildValue("(NNNNL)", wrap(indptr_all.select(0, q)), wrap(indices_all.narrow(0, first[q], cnt)), wrap(t_ip[q]),
+                                                 wrap(t_indices.narrow(0, first[q], cnt)), (long long)cnt));
+    }
+    return Py_BuildValue("(NNN)", tuple(indptr, indices, t_indptr, t_indices), plans, parts);
 }
 
 // ---- aggregation -----------------------------------------------------------------------------------------------------------
@@ -498,7 +572,7 @@ PyObject *entry(PyObject *, PyObject *const *args, Py_ssize_t n) {
     }
 }
 #define M(f) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&entry<f>)), METH_FASTCALL, nullptr}
-PyMethodDef g_methods[] = {M(init), M(gat_forward), M(gat_backward), M(gat_forward_parts), M(gat_backward_parts), M(spmm), M(spmm_scaled),
+PyMethodDef g_methods[] = {M(init), M(from_coo), M(gat_forward), M(gat_backward), M(gat_forward_parts), M(gat_backward_parts), M(spmm), M(spmm_scaled),
                            M(propagate), M(layer_forward), M(layer_backward), M(sage_forward), M(sage_backward), M(bn_forward), M(bn_backward),
                            {nullptr, nullptr, 0, nullptr}};
 PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_sar_torch", nullptr, -1, g_methods, nullptr, nullptr, nullptr, nullptr};
