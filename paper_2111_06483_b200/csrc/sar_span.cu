@@ -50,27 +50,9 @@ static sar_status launch_span(SpanArgs a, long long nnz, const char *name, const
             stage_bytes = (size_t)a.R * rsb;
         }
     }
-    const long long spans = (a.n_rows + a.R - 1) / a.R;
-    if (spans > 0) {
-        const unsigned blocks = (unsigned)((spans + kSpanWarps - 1) / kSpanWarps);
-        if (kIsSum || (whole && !(a.flags & (SAR_KEEP_NUMERATOR | SAR_RELU_OUT)))) {  // the epilogue's flag tests decided at compile time
-            if (geo) {
-                auto wk = span_kernel<T, G, V, S, MODE, CAP, MINB, 1, kGeo>;
-                SAR_TRY(ensure_smem(wk, smem));
-                SAR_LAUNCH(name, st, wk<<<blocks, kSpanThreads, smem, st>>>(a));
-            } else {
-                auto wk = span_kernel<T, G, V, S, MODE, CAP, MINB, 1>;
-                SAR_TRY(ensure_smem(wk, smem));
-                SAR_LAUNCH(name, st, wk<<<blocks, kSpanThreads, smem, st>>>(a));
-            }
-        } else {
-            const size_t smem_st = (size_t)kSpanWarps * span_layout<MODE>(a.g.Hp, V, CAP, S, 32 / G, stage_bytes).total;
-            SAR_TRY(ensure_smem(kern, smem_st));
-            SAR_LAUNCH(name, st, kern<<<blocks, kSpanThreads, smem_st, st>>>(a));
-        }
-        SAR_TRY(sar_after_launch());
-    }
+    bool beside = false;
     if constexpr (MODE == kFwd || kIsSum) if (a.sp.threshold > 0 && a.sp.n_seg > 0) {
+        beside = true;
         a.mode = 1;
         const unsigned blocks = (unsigned)((a.sp.n_seg + kSpanWarps - 1) / kSpanWarps);
         if (a.sp.threshold <= CAP_SEG) {
@@ -84,6 +66,27 @@ static sar_status launch_span(SpanArgs a, long long nnz, const char *name, const
             SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP, MINB, 2, kGeo>, smem));
             SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP, MINB, 2>, smem));
             SAR_LAUNCH(seg_name, st, seg_kern<<<blocks, kSpanThreads, smem, st>>>(a));
+        }
+        SAR_TRY(sar_after_launch());
+    }
+    a.mode = 0;
+    const long long spans = (a.n_rows + a.R - 1) / a.R;
+    if (spans > 0) {
+        const unsigned blocks = (unsigned)((spans + kSpanWarps - 1) / kSpanWarps);
+        if (kIsSum || (whole && !(a.flags & (SAR_KEEP_NUMERATOR | SAR_RELU_OUT)))) {  // the epilogue's flag tests decided at compile time
+            if (geo) {
+                auto wk = span_kernel<T, G, V, S, MODE, CAP, MINB, 1, kGeo>;
+                SAR_TRY(ensure_smem(wk, smem));
+                SAR_LAUNCH(name, st, launch_beside_segments(wk, blocks, kSpanThreads, smem, beside, a, st));
+            } else {
+                auto wk = span_kernel<T, G, V, S, MODE, CAP, MINB, 1>;
+                SAR_TRY(ensure_smem(wk, smem));
+                SAR_LAUNCH(name, st, launch_beside_segments(wk, blocks, kSpanThreads, smem, beside, a, st));
+            }
+        } else {
+            const size_t smem_st = (size_t)kSpanWarps * span_layout<MODE>(a.g.Hp, V, CAP, S, 32 / G, stage_bytes).total;
+            SAR_TRY(ensure_smem(kern, smem_st));
+            SAR_LAUNCH(name, st, launch_beside_segments(kern, blocks, kSpanThreads, smem_st, beside, a, st));
         }
         SAR_TRY(sar_after_launch());
     }

@@ -139,6 +139,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
     constexpr bool kSrc = MODE == kBwdSrc;
     constexpr bool kAcc0 = MODE != kBwdDstGivenD;                  // accumulator 0 live
     constexpr bool kAcc1 = kDst || kSrc;                           // accumulator 1 live
+    if (mode_ == 1) let_rows_in();
     extern __shared__ __align__(16) unsigned char smem_raw[];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -977,6 +978,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
             r = r2;
         }
     }
+    if (mode_ == 0) rows_end();
 }
 
 }  // namespace sar
