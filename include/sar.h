@@ -378,6 +378,16 @@ SAR_API sar_status sar_spmm_agg_scaled(const sar_part *g, const void *feat_q, in
                                        const float *src_scale, const float *dst_scale, void *out, void *workspace,
                                        size_t workspace_bytes, void *stream);
 
+/* The iterated propagation of that post-processing: X_0 = x0, X_{i+1} = (1 - alpha) x0 + alpha S X_i, iters >= 1 times;
+ * out = X_iters.  parts: HOST array of k partitions (k <= SAR_MAX_PARTS) that together hold the graph, part q the sources
+ * bounds[q] .. bounds[q + 1] (HOST bounds, bounds[0] = 0, bounds[k] = n_dst of every part).  x0, out: [n, F] of type t,
+ * x0 != out; rows are accumulated in float32 and stored in type t between the steps, multiplied by src_scale (a source is
+ * scaled once, where its row is stored, not on every edge).  workspace: sar_propagate_workspace_bytes, 256-byte aligned. */
+SAR_API size_t sar_propagate_workspace_bytes(int32_t k, const sar_part *const *parts, int32_t F, sar_dtype t);
+SAR_API sar_status sar_propagate(int32_t k, const sar_part *const *parts, const int64_t *bounds, const void *x0, int32_t F,
+                                 sar_dtype t, float alpha, int64_t iters, const float *src_scale, const float *dst_scale,
+                                 void *out, void *workspace, size_t workspace_bytes, void *stream);
+
 /* ---------------------------------------------------------------------------------------------
  * The rest of a GAT layer around the aggregation (Eq. 3; Eq. 1's f_node reduced to a ReLU).
  *   sar_gat_project      el[i,h] = <z[i,h,:], a_l[h,:]>, er[i,h] = <z[i,h,:], a_r[h,:]>: the two halves of

@@ -37,6 +37,7 @@ EXPORTS = [
     "sar_gat_storing_workspace_bytes", "sar_gat_fwd_storing", "sar_gat_bwd_storing", "sar_bn_combine_moments",
     "sar_bn_combine_sums", "sar_degree_order_workspace_bytes", "sar_degree_order", "sar_relabel", "sar_permute_rows", "sar_linear_project", "sar_linear_bwd_input_relu",
     "sar_graph_from_coo", "sar_plan_many_workspace_bytes", "sar_plan_count_many", "sar_plan_fill_many", "sar_gather_i64",
+    "sar_propagate_workspace_bytes", "sar_propagate",
 ]
 
 
@@ -80,7 +81,7 @@ def lib() -> ctypes.CDLL:
         for name in ("sar_graph_workspace_bytes", "sar_gat_workspace_bytes", "sar_spmm_workspace_bytes",
                      "sar_gat_stack_arena_bytes", "sar_gat_bwd_noalloc_limit", "sar_gat_project_workspace_bytes",
                      "sar_bn_workspace_bytes", "sar_linear_workspace_bytes", "sar_gat_storing_workspace_bytes",
-                     "sar_degree_order_workspace_bytes", "sar_plan_many_workspace_bytes"):
+                     "sar_degree_order_workspace_bytes", "sar_plan_many_workspace_bytes", "sar_propagate_workspace_bytes"):
             getattr(L, name).restype = c_size_t
         _lib = L
     return _lib
@@ -782,6 +783,24 @@ def sar_linear_bwd_weight(h: torch.Tensor, dz: torch.Tensor, dw: torch.Tensor, w
 def sar_dropout(x: torch.Tensor, p: float, seed: int, y: torch.Tensor) -> None:
     _check("sar_dropout", lib().sar_dropout(c_int64(x.numel()), ctypes.c_int(_dtype(x)), _ptr(x), c_float(p),
                                             ctypes.c_uint64(seed & 0xFFFFFFFFFFFFFFFF), _ptr(y), _stream()))
+
+
+def _part_array(parts: Sequence[Part]):
+    return (c_void_p * max(len(parts), 1))(*[p.addr for p in parts])
+
+
+def sar_propagate_workspace_bytes(parts: Sequence[Part], F: int, dtype: int) -> int:
+    return int(lib().sar_propagate_workspace_bytes(c_int32(len(parts)), _part_array(parts), c_int32(F), ctypes.c_int(dtype)))
+
+
+def sar_propagate(parts: Sequence[Part], bounds: Sequence[int], x0: torch.Tensor, alpha: float, iters: int,
+                  src_scale: Optional[torch.Tensor], dst_scale: Optional[torch.Tensor], out: torch.Tensor,
+                  workspace: torch.Tensor) -> None:
+    w, wb = _ws(workspace)
+    _check("sar_propagate", lib().sar_propagate(c_int32(len(parts)), _part_array(parts), _host_i64(bounds), _ptr(x0),
+                                                c_int32(x0.shape[1]), ctypes.c_int(_dtype(x0)), c_float(alpha),
+                                                c_int64(iters), _ptr(src_scale), _ptr(dst_scale), _ptr(out), w, wb,
+                                                _stream()))
 
 
 def sar_axpby(a: float, x: torch.Tensor, b: float, y: torch.Tensor) -> None:

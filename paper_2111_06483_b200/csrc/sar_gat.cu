@@ -111,6 +111,56 @@ static sar_status pad_rows(long long n, int H, int F, const RowShape &r, sar_dty
     return sar_after_launch();
 }
 
+// The start of a propagation: x0 with padded rows and / or scaled row by row (either may be null); one 16-byte vector per thread
+template <typename T>
+__global__ void __launch_bounds__(256) propagate_start_kernel(long long vecs, int F, int vph, const T *__restrict__ in, const float *__restrict__ scale,
+                                                              uint4 *__restrict__ padded, uint4 *__restrict__ scaled) {
+    constexpr int EPV = Elem<T>::EPV;
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (i >= vecs) return;
+    const long long row = i / vph;
+    const int f0 = (int)(i - row * vph) * EPV;
+    const T *p = in + row * F + f0;
+    float x[EPV];
+#pragma unroll
+    for (int k = 0; k < EPV; ++k) x[k] = f0 + k < F ? Elem<T>::load1(p + k) : 0.f;
+    if (padded) padded[i] = Elem<T>::pack(x);
+    if (scaled) {
+        const float s = __ldg(scale + row);
+#pragma unroll
+        for (int k = 0; k < EPV; ++k) x[k] *= s;
+        scaled[i] = Elem<T>::pack(x);
+    }
+}
+static sar_status propagate_start(long long n, int F, const RowShape &r, sar_dtype t, const void *in, const float *scale, void *padded, void *scaled,
+                                  cudaStream_t st) {
+    const long long vecs = n * r.vph;
+    const unsigned blocks = (unsigned)((vecs + 255) / 256);
+    uint4 *p = static_cast<uint4 *>(padded), *s = static_cast<uint4 *>(scaled);
+    if (t == SAR_F32)
+        SAR_LAUNCH("propagate_start", st, (propagate_start_kernel<float><<<blocks, 256, 0, st>>>(vecs, F, r.vph, static_cast<const float *>(in), scale, p, s)));
+    else
+        SAR_LAUNCH("propagate_start", st, (propagate_start_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(vecs, F, r.vph, static_cast<const __nv_bfloat16 *>(in), scale, p, s)));
+    return sar_after_launch();
+}
+// padded rows -> rows of F elements; one element per thread
+template <typename T>
+__global__ void __launch_bounds__(256) strip_rows_kernel(long long elems, int F, int pitch, const T *__restrict__ in, T *__restrict__ out) {
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (i >= elems) return;
+    const long long row = i / F;
+    out[i] = in[row * pitch + (i - row * F)];
+}
+static sar_status strip_rows(long long n, int F, const RowShape &r, sar_dtype t, const void *in, void *out, cudaStream_t st) {
+    const unsigned blocks = (unsigned)((n * F + 255) / 256);
+    const int pitch = (int)(r.row_bytes / sar_elem_size(t));
+    if (t == SAR_F32)
+        SAR_LAUNCH("strip_rows", st, (strip_rows_kernel<float><<<blocks, 256, 0, st>>>(n * F, F, pitch, static_cast<const float *>(in), static_cast<float *>(out))));
+    else
+        SAR_LAUNCH("strip_rows", st, (strip_rows_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(n * F, F, pitch, static_cast<const __nv_bfloat16 *>(in), static_cast<__nv_bfloat16 *>(out))));
+    return sar_after_launch();
+}
+
 // ---- workspace layout ---------------------------------------------------------------------------
 // [ destination records: n_dst*H float4 ][ padded gout ][ segments of the CSR ][ segments of the CSC ][ padded feat ]
 // (the padded arrays for ragged shapes only).  The first two do not depend on the partition: the steps of a call-by-call
@@ -625,6 +675,37 @@ sar_status sar_gat_bwd_fused(const sar_part *g, int32_t k, const int64_t *bounds
 }
 
 // ---------------------------------------------------------------------------------------------
+// The sum on rows of whole vectors: gather and, unless r.ragged, out; part = room for the segments of the long rows
+static sar_status sum_rows(const sar_part *g, const RowShape &r, int32_t F, sar_dtype t, uint32_t flags, const void *gather, const int64_t *deg_total,
+                           const float *src_scale, const float *dst_scale, const SumMix &mix, void *out, float *part, cudaStream_t st) {
+    RowArgs a{};
+    a.n_rows = g->n_dst;
+    a.indptr = g->indptr;
+    a.indices = g->indices;
+    a.last_col = (unsigned)(g->n_src > 0 ? g->n_src - 1 : 0);
+    a.gather = gather;
+    a.row_bytes = r.row_bytes;
+    a.out = out;
+    a.deg = deg_total;
+    a.src_scale = src_scale;
+    a.dst_scale = dst_scale;
+    a.mix = mix;
+    a.flags = flags;
+    a.H = 1;
+    a.F = F;
+    a.vph = r.vph;
+    a.ragged = r.ragged;
+    a.sp = split_args(g->split, part, 1, r, t);
+    const bool weighted = src_scale != nullptr;
+    Shape s;
+    SAR_TRY(make_shape(1, F, t, !r.ragged, &s));
+    if (use_span(s, g->n_src, kSpanSumBytes))
+        SAR_TRY(span_sum(s, a, g->nnz, weighted, st));
+    else
+        SAR_TRY(t == SAR_F32 ? rows_sum_f32(a, r.geo, g->nnz, weighted, st) : rows_sum_bf16(a, r.geo, g->nnz, weighted, st));
+    return a.sp.n_long > 0 ? rows_sum_merge(a, t, st) : SAR_OK;
+}
+
 static sar_status spmm_impl(const sar_part *g, const void *feat_q, int32_t F, sar_dtype t, uint32_t flags,
                             const int64_t *deg_total, const float *src_scale, const float *dst_scale, void *out,
                             void *workspace, size_t workspace_bytes, void *stream) {
@@ -664,35 +745,11 @@ static sar_status spmm_impl(const sar_part *g, const void *feat_q, int32_t F, sa
     }
     const bool use_split = g->split && g->split->n_long > 0;
     if (use_split && (!have_ws || workspace_bytes < parts)) return SAR_ERR_WORKSPACE;
-    RowArgs a{};
-    a.n_rows = g->n_dst;
-    a.indptr = g->indptr;
-    a.indices = g->indices;
-    a.last_col = (unsigned)(g->n_src > 0 ? g->n_src - 1 : 0);
-    a.gather = feat_q;
-    a.row_bytes = r.row_bytes;
-    a.out = out;
-    a.deg = deg_total;
-    a.src_scale = src_scale;
-    a.dst_scale = dst_scale;
-    a.flags = flags;
-    a.H = 1;
-    a.F = F;
-    a.vph = r.vph;
-    a.ragged = r.ragged;
-    a.sp = split_args(g->split, static_cast<float *>(workspace), 1, r, t);
     if (r.ragged) {
         SAR_TRY(pad_rows(g->n_src, 1, F, r, t, feat_q, static_cast<char *>(workspace) + parts, st));
-        a.gather = static_cast<char *>(workspace) + parts;
+        feat_q = static_cast<char *>(workspace) + parts;
     }
-    const bool weighted = src_scale != nullptr;
-    Shape s;
-    SAR_TRY(make_shape(1, F, t, !r.ragged, &s));
-    if (use_span(s, g->n_src, kSpanSumBytes))
-        SAR_TRY(span_sum(s, a, g->nnz, weighted, st));
-    else
-        SAR_TRY(t == SAR_F32 ? rows_sum_f32(a, r.geo, g->nnz, weighted, st) : rows_sum_bf16(a, r.geo, g->nnz, weighted, st));
-    return use_split ? rows_sum_merge(a, t, st) : SAR_OK;
+    return sum_rows(g, r, F, t, flags, feat_q, deg_total, src_scale, dst_scale, SumMix{}, out, static_cast<float *>(workspace), st);
 }
 
 sar_status sar_spmm_agg(const sar_part *g, const void *feat_q, int32_t F, sar_dtype t, uint32_t flags,
@@ -706,6 +763,66 @@ sar_status sar_spmm_agg_scaled(const sar_part *g, const void *feat_q, int32_t F,
                                size_t workspace_bytes, void *stream) {
     if (flags & SAR_MEAN) return SAR_ERR_INVALID_ARG;
     return spmm_impl(g, feat_q, F, t, flags, nullptr, src_scale, dst_scale, out, workspace, workspace_bytes, stream);
+}
+
+// Workspace of a propagation: [ segments of the long rows ][ two arrays of padded rows ][ x0 with padded rows ]
+static size_t propagate_parts(int32_t k, const sar_part *const *parts, const RowShape &r, sar_dtype t) {
+    size_t b = 0;
+    for (int32_t q = 0; q < k; ++q) {
+        const size_t p = part_bytes(parts[q]->split, 1, r, t);
+        b = p > b ? p : b;
+    }
+    return b;
+}
+size_t sar_propagate_workspace_bytes(int32_t k, const sar_part *const *parts, int32_t F, sar_dtype t) {
+    if (k < 1 || !parts || F < 1) return 0;
+    for (int32_t q = 0; q < k; ++q)
+        if (!parts[q]) return 0;
+    const RowShape r = sum_shape(F, t);
+    return propagate_parts(k, parts, r, t) + 3 * sar_round_up((size_t)parts[0]->n_dst * r.row_bytes, 256) + 256;
+}
+
+sar_status sar_propagate(int32_t k, const sar_part *const *parts, const int64_t *bounds, const void *x0, int32_t F, sar_dtype t, float alpha,
+                         int64_t iters, const float *src_scale, const float *dst_scale, void *out, void *workspace, size_t workspace_bytes,
+                         void *stream) {
+    if (k < 1 || !parts || !bounds || iters < 1) return SAR_ERR_INVALID_ARG;
+    if (k > SAR_MAX_PARTS) return SAR_ERR_UNSUPPORTED;
+    for (int32_t q = 0; q < k; ++q) {
+        SAR_TRY(check_part(parts[q], false));
+        if (parts[q]->n_dst != parts[0]->n_dst || bounds[q] < 0 || bounds[q + 1] - bounds[q] != parts[q]->n_src) return SAR_ERR_INVALID_ARG;
+    }
+    const int64_t n = parts[0]->n_dst;
+    if (bounds[0] != 0 || bounds[k] != n || (n > 0 && (!x0 || !out)) || x0 == out) return SAR_ERR_INVALID_ARG;
+    SAR_TRY(check_elem_align({x0, out}, sar_elem_size(t)));
+    SAR_TRY(check_elem_align({src_scale, dst_scale}, 4));
+    SAR_TRY(check_shape(1, F, t));
+    if (n == 0) return SAR_OK;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const RowShape ragged = sum_shape(F, t);
+    const int32_t Fp = (int32_t)(ragged.row_bytes / sar_elem_size(t));
+    const RowShape r = sum_shape(Fp, t);   // the same rows, every vector of them whole
+    const size_t array = sar_round_up((size_t)n * r.row_bytes, 256), seg = propagate_parts(k, parts, r, t);
+    if (!workspace || !sar_aligned(workspace, 256) || workspace_bytes < seg + 3 * array) return SAR_ERR_WORKSPACE;
+    char *ws = static_cast<char *>(workspace), *y[2] = {ws + seg, ws + seg + array};
+    const bool in_place = !ragged.ragged && all16({x0});                  // x0 can be read as it lies
+    const bool out_direct = !ragged.ragged && all16({out});
+    const void *x0p = in_place ? x0 : ws + seg + 2 * array;
+    const void *cur = x0p;
+    if (!in_place || src_scale) {
+        if (src_scale) cur = y[0];
+        SAR_TRY(propagate_start(n, F, r, t, x0, src_scale, in_place ? nullptr : ws + seg + 2 * array, src_scale ? y[0] : nullptr, st));
+    }
+    for (int64_t i = 0; i < iters; ++i) {
+        const bool end = i + 1 == iters;
+        void *nxt = end && out_direct ? out : y[(i + 1) & 1];
+        const SumMix mix{x0p, 1.f - alpha, alpha, end ? nullptr : src_scale};
+        for (int32_t q = 0; q < k; ++q)
+            SAR_TRY(sum_rows(parts[q], r, Fp, t, (q == 0 ? SAR_FIRST : 0u) | (q + 1 == k ? SAR_LAST : 0u),
+                             static_cast<const char *>(cur) + (size_t)bounds[q] * r.row_bytes, nullptr, nullptr, dst_scale, mix, nxt,
+                             reinterpret_cast<float *>(ws), st));
+        cur = nxt;
+    }
+    return out_direct ? SAR_OK : strip_rows(n, F, r, t, cur, out, st);
 }
 
 }  // extern "C"

@@ -96,6 +96,13 @@ __device__ __forceinline__ void load_row_vec(const void *base, long long row, in
     }
 }
 
+// What a sum's last partition does to a row before it is stored: y = (keep * x0[row] + scale * y) * post[row]
+struct SumMix {
+    const void *x0;      // null: nothing
+    float keep, scale;
+    const float *post;   // may be null
+};
+
 template <typename T, int G, int V>
 __device__ __forceinline__ void store_row_vec(void *base, long long row, int n_vec, int gl,
                                               const bool (&vok)[V], const float (&r)[V][Elem<T>::EPV]) {

@@ -33,6 +33,7 @@ struct RowArgs {
     float *dscal;            // del / der
     const int64_t *deg;      // sum: total in-degree for the mean
     const float *src_scale, *dst_scale;
+    SumMix mix;              // sum
     float slope;
     unsigned flags;
     int H, F;                // heads and features per head as stored in out (F may be ragged)

@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, MINB) row_kernel(const RowArgs
         if (beg == end) {                   // nothing to add: only what a flag forces to be written
             if (MODE == kRowFwdPart && !first && !last) continue;
             if (MODE == kRowDstPart && !first) continue;
-            if (kAgg && !first && !((a.flags & SAR_MEAN) && last)) continue;
+            if (kAgg && !first && !(((a.flags & SAR_MEAN) || a.mix.x0) && last)) continue;
         }
         const long long row = row0 + r;
 
@@ -635,6 +635,12 @@ __global__ void __launch_bounds__(kRowWarps * 32, MINB) row_kernel(const RowArgs
                         }
 #pragma unroll
                         for (int k = 0; k < NE; ++k) y[v][k] = (y[v][k] * ds + old[k]) * inv;
+                        if (a.mix.x0 && last) {
+                            load_elems<T, NE>(reinterpret_cast<const T *>(a.mix.x0) + row * (long long)HF + oel[v], old, orem[v], a.ragged);
+                            const float post = a.mix.post ? __ldg(a.mix.post + row) : 1.f;
+#pragma unroll
+                            for (int k = 0; k < NE; ++k) y[v][k] = (a.mix.keep * old[k] + a.mix.scale * y[v][k]) * post;
+                        }
                         store_elems<T, NE>(outp + row * (long long)HF + oel[v], y[v], orem[v], a.ragged);
                     }
                 }

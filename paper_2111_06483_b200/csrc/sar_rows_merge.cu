@@ -138,7 +138,10 @@ __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs
                     if constexpr (sizeof(T) == 4) y += out[o];
                     else y += __bfloat162float(out[o]);
                 }
-                Elem<T>::store1(out + o, y * inv);
+                y *= inv;
+                if (a.mix.x0 && last)
+                    y = (a.mix.keep * Elem<T>::load1(reinterpret_cast<const T *>(a.mix.x0) + o) + a.mix.scale * y) * (a.mix.post ? a.mix.post[row] : 1.f);
+                Elem<T>::store1(out + o, y);
             });
         }
     }

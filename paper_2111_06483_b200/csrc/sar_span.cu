@@ -119,6 +119,7 @@ static SpanArgs span_args(const Shape &s, const RowArgs &r) {
     a.deg_total = r.deg;
     a.src_scale = r.src_scale;
     a.dst_scale = r.dst_scale;
+    a.mix = r.mix;
     a.slope = r.slope;
     a.flags = r.flags;
     a.g = s.geom;

@@ -62,6 +62,7 @@ struct SpanArgs {
     void *out;               // forward: out; bwd-src: dfeat; sum: out
     float *del, *der;
     const int64_t *deg_total;
+    SumMix mix;              // sum
     const float *src_scale, *dst_scale;  // weighted sum (kSumW): per-source factor, per-row factor (either may be null)
     float slope;
     unsigned flags;
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
     else if (MODE == kBwdDst) write_empty = true;
     else if (MODE == kBwdDstGivenD) write_empty = flags_ & SAR_FIRST;
     else if (kSrc) write_empty = true;
-    else write_empty = (flags_ & SAR_FIRST) || mean_now;
+    else write_empty = (flags_ & SAR_FIRST) || mean_now || (a.mix.x0 && (flags_ & SAR_LAST));
     if (mode_ == 1) write_empty = false;
 
     // ---- lane geometry ------------------------------------------------------------------------
@@ -949,6 +950,15 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
                         for (int v = 0; v < V; ++v)
 #pragma unroll
                             for (int e = 0; e < EPV; ++e) acc0[v][e] *= inv;
+                    }
+                    if (a.mix.x0 && (flags_ & SAR_LAST)) {
+                        float x0[V][EPV];
+                        load_row_vec<T, G, V, true>(a.mix.x0, row, n_vec, gl, vok, x0);
+                        const float post = a.mix.post ? __ldg(a.mix.post + row) : 1.f;
+#pragma unroll
+                        for (int v = 0; v < V; ++v)
+#pragma unroll
+                            for (int e = 0; e < EPV; ++e) acc0[v][e] = (a.mix.keep * x0[v][e] + a.mix.scale * acc0[v][e]) * post;
                     }
                     store_row_vec<T, G, V>(a.out, row, n_vec, gl, vok, acc0);
                 }

@@ -21,7 +21,7 @@ namespace {
 #define SAR_TABLE(X)                                                                                                   \
     X(sar_status_string) X(sar_gat_workspace_bytes) X(sar_gat_fwd) X(sar_gat_fwd_fused) X(sar_gat_bwd_prepare)         \
     X(sar_gat_bwd) X(sar_gat_bwd_fused) X(sar_spmm_agg) X(sar_spmm_workspace_bytes) X(sar_spmm_agg_scaled)             \
-    X(sar_axpby) X(sar_relu) X(sar_gat_project) X(sar_gat_project_bwd) X(sar_gat_project_workspace_bytes)              \
+    X(sar_propagate) X(sar_propagate_workspace_bytes) X(sar_relu) X(sar_gat_project) X(sar_gat_project_bwd) X(sar_gat_project_workspace_bytes)              \
     X(sar_linear_workspace_bytes) X(sar_linear) X(sar_linear_accumulate) X(sar_linear_project)                         \
     X(sar_linear_bwd_input) X(sar_linear_bwd_input_relu) X(sar_linear_bwd_weight) X(sar_bn_workspace_bytes)            \
     X(sar_bn_stats) X(sar_bn_rstd) X(sar_bn_apply) X(sar_bn_bwd_stats) X(sar_bn_bwd_apply)                             \
@@ -396,20 +396,15 @@ PyObject *propagate(Args &a) {   // parts, bounds, x0, alpha, iters, src_scale, 
     const double alpha = a.real();
     const int64_t iters = a.integer();
     const at::Tensor src = a.optional(), dst = a.optional();
-    const size_t k = parts.size();
     if (iters <= 0) return wrap(x0.clone());
-    at::Tensor x = x0, buf[2];   // the first step reads x0 itself
-    Scratch ws;
-    for (int64_t i = 0; i < iters; ++i) {
-        at::Tensor &nxt = buf[i & 1];
-        if (!nxt.defined()) nxt = empty(x0.sizes(), x0.scalar_type(), x0);
-        for (size_t q = 0; q < k; ++q)
-            sum_scaled(reinterpret_cast<const sar_part *>(parts[q]), rows(x, bounds[q]), x0, step_flags(q, k),
-                       src.defined() ? f32(src) + bounds[q] : nullptr, f32(dst), ptrm(nxt), ws);
-        SAR(sar_axpby, x0.numel(), code(x0), (float)(1.0 - alpha), ptr(x0), (float)alpha, ptrm(nxt), stream());
-        x = nxt;
-    }
-    return wrap(x);
+    std::vector<const sar_part *> ps;
+    for (int64_t p : parts) ps.push_back(reinterpret_cast<const sar_part *>(p));
+    const int32_t k = (int32_t)ps.size(), F = (int32_t)x0.size(1);
+    const at::Tensor out = empty(x0.sizes(), x0.scalar_type(), x0);
+    const at::Tensor ws = bytes(L.sar_propagate_workspace_bytes(k, ps.data(), F, code(x0)), x0);
+    SAR(sar_propagate, k, ps.data(), bounds.data(), ptr(x0), F, code(x0), (float)alpha, iters, f32(src), f32(dst), ptrm(out), ptrm(ws), ws.nbytes(),
+        stream());
+    return wrap(out);
 }
 
 // sum over the pieces of one graph of inv * A x

@@ -1,0 +1,40 @@
+"""The iterated propagation as one call: ragged and misaligned rows, one and several partitions, long rows, arrays below and
+above the size at which the span kernels take over, an odd and an even number of steps; against float64 sums."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2111_06483_b200 import api
+
+from helpers import allclose_report
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("n,F,dtype,k,iters,scaled,shift", [
+    (1, 1, "f32", 1, 1, True, 0), (900, 3, "f32", 1, 3, True, 0), (900, 47, "f32", 4, 2, False, 0), (900, 300, "f32", 1, 1, True, 0),
+    (900, 16, "f32", 1, 2, True, 1), (900, 16, "f32", 3, 1, False, 0), (900, 9, "bf16", 2, 2, True, 0), (70_000, 47, "f32", 1, 3, True, 0),
+    (70_000, 48, "f32", 3, 2, True, 0), (70_000, 100, "bf16", 1, 2, False, 0)])
+def test_propagation_in_one_call(n, F, dtype, k, iters, scaled, shift):
+    tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+    gen = torch.Generator().manual_seed(n + F)
+    e = n * 6
+    src, dst = (torch.randint(0, max(n - 1, 1), (e,), generator=gen, dtype=torch.int32) for _ in range(2))
+    dst[: e // 4] = 0                                     # a long row; the last node has no edge
+    g = api.Graph.from_coo(n, src.to(DEV), dst.to(DEV), k=k, build_parts=k > 1, threshold=64)
+    x0 = torch.randn((n, F), generator=gen).to(tdt)
+    s = torch.rand(n, generator=gen) + 0.5 if scaled else None
+    d = 1.0 / torch.bincount(dst.long(), minlength=n).clamp(min=1).float()
+    buf = torch.empty(n * F + shift, dtype=tdt, device=DEV)
+    x = buf[shift:].view(n, F)
+    x.copy_(x0)
+    got = api.propagate(g, x, 0.7, iters, s.to(DEV) if scaled else None, d.to(DEV))
+    adj = torch.sparse_coo_tensor(torch.stack([dst.long(), src.long()]), torch.ones(e, dtype=torch.float64), (n, n)).to_sparse_csr()
+    want, x64 = x0.double(), x0.double()
+    for _ in range(iters):
+        y = want * s.double()[:, None] if scaled else want
+        want = 0.3 * x64 + 0.7 * d.double()[:, None] * (adj @ y)
+    tol = dict(rtol=1e-5, atol=1e-5) if dtype == "f32" else dict(rtol=2e-2, atol=2e-2)
+    allclose_report(got.double().cpu().numpy(), want.numpy(), what="propagation", **tol)
+    assert np.isfinite(got.float().cpu().numpy()).all()
