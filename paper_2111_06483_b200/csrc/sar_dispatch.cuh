@@ -4,6 +4,7 @@
 #include <initializer_list>
 
 #include "sar_common.cuh"
+#include "sar_launch.cuh"
 
 namespace sar {
 
@@ -42,31 +43,6 @@ static inline sar_status ensure_smem(K kernel, size_t bytes) {
     if (bytes > 48 * 1024)
         SAR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
     return SAR_OK;
-}
-
-// The segments of the long rows and the other rows are independent launches of one pass.  The segments go first (a segment
-// is the longest chain of work in the pass); each of their blocks lets the next launch in as soon as it runs
-// (launch_beside_segments below sets the attribute, let_rows_in is the device side), so the rows fill whatever the segments
-// leave free.  The last block of the rows launch waits for the segments' end, so that whatever follows the rows launch
-// follows both.  Before, the segments came after the rows: a partition step over 100,000 rows and 250,000 edges spent
-// 20 us of 80 on a handful of segments with the rest of the chip idle.
-__device__ __forceinline__ void let_rows_in() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-__device__ __forceinline__ void rows_end() {
-    if (blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;\n" ::: "memory");
-}
-template <typename A>
-static inline void launch_beside_segments(void (*kernel)(A), unsigned blocks, unsigned threads, size_t smem, bool beside, const A &args, cudaStream_t st) {
-    cudaLaunchConfig_t c = {};
-    c.gridDim = dim3(blocks);
-    c.blockDim = dim3(threads);
-    c.dynamicSmemBytes = smem;
-    c.stream = st;
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    c.attrs = &at;
-    c.numAttrs = beside ? 1 : 0;
-    (void)cudaLaunchKernelEx(&c, kernel, args);   // reported by sar_after_launch
 }
 
 static inline bool all16(std::initializer_list<const void *> ps) {

@@ -88,6 +88,7 @@ static RowShape sum_shape(int F, sar_dtype t) {
 // [n,H,F] -> [n,H,vph*EPV], zeros behind the F elements of a head; one 16-byte vector per thread
 template <typename T>
 __global__ void __launch_bounds__(256) pad_rows_kernel(long long vecs, int F, int vph, const T *__restrict__ in, uint4 *__restrict__ out) {
+    after_predecessor();
     constexpr int EPV = Elem<T>::EPV;
     const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
     if (i >= vecs) return;
@@ -105,9 +106,9 @@ static sar_status pad_rows(long long n, int H, int F, const RowShape &r, sar_dty
     if (vecs == 0) return SAR_OK;
     const unsigned blocks = (unsigned)((vecs + 255) / 256);
     if (t == SAR_F32)
-        SAR_LAUNCH("pad_rows", st, (pad_rows_kernel<float><<<blocks, 256, 0, st>>>(vecs, F, r.vph, static_cast<const float *>(in), static_cast<uint4 *>(out))));
+        SAR_LAUNCH("pad_rows", st, launch(pad_rows_kernel<float>, blocks, 256, 0, st, vecs, F, r.vph, static_cast<const float *>(in), static_cast<uint4 *>(out)));
     else
-        SAR_LAUNCH("pad_rows", st, (pad_rows_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(vecs, F, r.vph, static_cast<const __nv_bfloat16 *>(in), static_cast<uint4 *>(out))));
+        SAR_LAUNCH("pad_rows", st, launch(pad_rows_kernel<__nv_bfloat16>, blocks, 256, 0, st, vecs, F, r.vph, static_cast<const __nv_bfloat16 *>(in), static_cast<uint4 *>(out)));
     return sar_after_launch();
 }
 
@@ -115,6 +116,7 @@ static sar_status pad_rows(long long n, int H, int F, const RowShape &r, sar_dty
 template <typename T>
 __global__ void __launch_bounds__(256) propagate_start_kernel(long long vecs, int F, int vph, const T *__restrict__ in, const float *__restrict__ scale,
                                                               uint4 *__restrict__ padded, uint4 *__restrict__ scaled) {
+    after_predecessor();
     constexpr int EPV = Elem<T>::EPV;
     const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
     if (i >= vecs) return;
@@ -138,14 +140,15 @@ static sar_status propagate_start(long long n, int F, const RowShape &r, sar_dty
     const unsigned blocks = (unsigned)((vecs + 255) / 256);
     uint4 *p = static_cast<uint4 *>(padded), *s = static_cast<uint4 *>(scaled);
     if (t == SAR_F32)
-        SAR_LAUNCH("propagate_start", st, (propagate_start_kernel<float><<<blocks, 256, 0, st>>>(vecs, F, r.vph, static_cast<const float *>(in), scale, p, s)));
+        SAR_LAUNCH("propagate_start", st, launch(propagate_start_kernel<float>, blocks, 256, 0, st, vecs, F, r.vph, static_cast<const float *>(in), scale, p, s));
     else
-        SAR_LAUNCH("propagate_start", st, (propagate_start_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(vecs, F, r.vph, static_cast<const __nv_bfloat16 *>(in), scale, p, s)));
+        SAR_LAUNCH("propagate_start", st, launch(propagate_start_kernel<__nv_bfloat16>, blocks, 256, 0, st, vecs, F, r.vph, static_cast<const __nv_bfloat16 *>(in), scale, p, s));
     return sar_after_launch();
 }
 // padded rows -> rows of F elements; one element per thread
 template <typename T>
 __global__ void __launch_bounds__(256) strip_rows_kernel(long long elems, int F, int pitch, const T *__restrict__ in, T *__restrict__ out) {
+    after_predecessor();
     const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
     if (i >= elems) return;
     const long long row = i / F;
@@ -155,9 +158,9 @@ static sar_status strip_rows(long long n, int F, const RowShape &r, sar_dtype t,
     const unsigned blocks = (unsigned)((n * F + 255) / 256);
     const int pitch = (int)(r.row_bytes / sar_elem_size(t));
     if (t == SAR_F32)
-        SAR_LAUNCH("strip_rows", st, (strip_rows_kernel<float><<<blocks, 256, 0, st>>>(n * F, F, pitch, static_cast<const float *>(in), static_cast<float *>(out))));
+        SAR_LAUNCH("strip_rows", st, launch(strip_rows_kernel<float>, blocks, 256, 0, st, n * F, F, pitch, static_cast<const float *>(in), static_cast<float *>(out)));
     else
-        SAR_LAUNCH("strip_rows", st, (strip_rows_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(n * F, F, pitch, static_cast<const __nv_bfloat16 *>(in), static_cast<__nv_bfloat16 *>(out))));
+        SAR_LAUNCH("strip_rows", st, launch(strip_rows_kernel<__nv_bfloat16>, blocks, 256, 0, st, n * F, F, pitch, static_cast<const __nv_bfloat16 *>(in), static_cast<__nv_bfloat16 *>(out)));
     return sar_after_launch();
 }
 
@@ -487,9 +490,9 @@ sar_status sar_gat_bwd_prepare(int64_t n_dst, int32_t H, int32_t F, sar_dtype t,
         const size_t smem = (size_t)kWarpsPerBlock * 32 * C::v * 4;
         const unsigned blocks = blocks_for((n_dst + PrepRows<C::v>::n - 1) / PrepRows<C::v>::n, C::g);
         if (acc_is_numerator)
-            SAR_LAUNCH("gat_bwd_prepare", st, gat_bwd_prepare_kernel<T, C::g, C::v, true><<<blocks, kThreads, smem, st>>>(a));
+            SAR_LAUNCH("gat_bwd_prepare", st, (launch(gat_bwd_prepare_kernel<T, C::g, C::v, true>, blocks, kThreads, smem, st, a)));
         else
-            SAR_LAUNCH("gat_bwd_prepare", st, gat_bwd_prepare_kernel<T, C::g, C::v, false><<<blocks, kThreads, smem, st>>>(a));
+            SAR_LAUNCH("gat_bwd_prepare", st, (launch(gat_bwd_prepare_kernel<T, C::g, C::v, false>, blocks, kThreads, smem, st, a)));
         return sar_after_launch();
     });
 }

@@ -2,6 +2,7 @@
 // the 16-byte vector v*G + gl of the row.
 #pragma once
 
+#include "sar_launch.cuh"
 #include "sar_rowkernels.cuh"
 
 namespace sar {
@@ -30,6 +31,7 @@ struct PrepRows {
 
 template <typename T, int G, int V, bool NUMERATOR>
 __global__ void __launch_bounds__(kThreads) gat_bwd_prepare_kernel(const PrepArgs a) {
+    after_predecessor();
     constexpr int EPV = Elem<T>::EPV;
     constexpr int RPW = 32 / G;
     constexpr int RPG = PrepRows<V>::n;

@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(32, MINB) lean_dst_kernel(const LeanArgs a) {
     static_assert((1 << LGNVEC) == NVEC, "row geometry");
     static_assert(P <= 32 && 32 % P == 0 && (SPS == 4 || SPS == 8), "stage geometry: four or eight slots per stage");
     static_assert(ITEMS <= 64, "at most two (position, head) pairs per lane");
-    if constexpr (SEG) let_rows_in();
+    if constexpr (SEG) after_predecessor();
+    else beside_segments(a.sp.n_seg > 0);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const unsigned sbase = (unsigned)__cvta_generic_to_shared(smem_raw);
     const unsigned ring_s = sbase + L::ring, rec_s = sbase + L::rec, w_s = sbase + L::w, offs_s = sbase + L::offs;
@@ -509,7 +510,7 @@ __global__ void __launch_bounds__(32, MINB) lean_dst_kernel(const LeanArgs a) {
         }
         r = r2;
     }
-    if constexpr (!SEG) rows_end();
+    if constexpr (!SEG) rows_end(a.sp.n_seg > 0);
 }
 
 // ---- launcher ------------------------------------------------------------------------------------------------------
@@ -524,13 +525,13 @@ static sar_status launch_lean_dst(LeanArgs a, long long nnz, cudaStream_t st) {
     if (a.sp.n_seg > 0) {
         auto kern = lean_dst_kernel<T, G, V, H, true, kLeanCap, P, NS, kLeanMinBlocks>;
         SAR_TRY(ensure_smem(kern, LS::total));
-        SAR_LAUNCH("gat_bwd_dst_seg", st, kern<<<(unsigned)a.sp.n_seg, 32, LS::total, st>>>(a));
+        SAR_LAUNCH("gat_bwd_dst_seg", st, launch(kern, (unsigned)a.sp.n_seg, 32, LS::total, st, a));
         SAR_TRY(sar_after_launch());
     }
     if (spans > 0) {
         auto kern = lean_dst_kernel<T, G, V, H, false, kLeanCap, P, NS, kLeanMinBlocksBwdRows>;
         SAR_TRY(ensure_smem(kern, LR::total));
-        SAR_LAUNCH("gat_bwd_dst", st, launch_beside_segments(kern, (unsigned)spans, 32, LR::total, a.sp.n_seg > 0, a, st));
+        SAR_LAUNCH("gat_bwd_dst", st, launch(kern, (unsigned)spans, 32, LR::total, st, a));
         SAR_TRY(sar_after_launch());
     }
     return SAR_OK;
@@ -549,13 +550,13 @@ static sar_status launch_lean_dst_part(LeanArgs a, long long nnz, cudaStream_t s
     if (a.sp.n_seg > 0) {
         auto kern = lean_dst_kernel<T, G, V, H, true, kLeanCap, P, NS, kLeanMinBlocks>;
         SAR_TRY(ensure_smem(kern, LS::total));
-        SAR_LAUNCH("gat_bwd_dst_seg", st, kern<<<(unsigned)a.sp.n_seg, 32, LS::total, st>>>(a));
+        SAR_LAUNCH("gat_bwd_dst_seg", st, launch(kern, (unsigned)a.sp.n_seg, 32, LS::total, st, a));
         SAR_TRY(sar_after_launch());
     }
     if (spans > 0) {
         auto kern = lean_dst_kernel<T, G, V, H, false, kLeanCap, P, NS, kLeanMinBlocksPart, true>;
         SAR_TRY(ensure_smem(kern, LR::total));
-        SAR_LAUNCH("gat_bwd_dst", st, launch_beside_segments(kern, (unsigned)spans, 32, LR::total, a.sp.n_seg > 0, a, st));
+        SAR_LAUNCH("gat_bwd_dst", st, launch(kern, (unsigned)spans, 32, LR::total, st, a));
         SAR_TRY(sar_after_launch());
     }
     return SAR_OK;

@@ -27,6 +27,7 @@
 #pragma once
 
 #include "sar_device.cuh"
+#include "sar_launch.cuh"
 #include "sar_rows.cuh"
 
 namespace sar {
@@ -189,6 +190,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, MINB) row_kernel(const RowArgs
     constexpr bool kAcc = kF || kS || kAgg;                        // a vector is accumulated
     constexpr bool kDot = kD || kS;                                // dot products with the row-stationary vector
     constexpr int WN = RowW<MODE>::n;
+    after_predecessor();
     extern __shared__ __align__(16) float smem_f[];
     const int lane = threadIdx.x & 31;
     float *sw = smem_f + (threadIdx.x >> 5) * RowSmem<HP, MODE>::total;

@@ -27,7 +27,7 @@ static sar_status launch_row_kernel(RowArgs a, RowGeo g, long long nnz, const ch
     auto kern = row_kernel<T, NV, HP, MODE, MINB>;
     SAR_TRY(ensure_smem(kern, smem));
     const dim3 grid((unsigned)((items + kRowWarps - 1) / kRowWarps), (unsigned)g.tiles);
-    SAR_LAUNCH(name, st, (kern<<<grid, kRowWarps * 32, smem, st>>>(a)));
+    SAR_LAUNCH(name, st, launch(kern, grid, kRowWarps * 32, smem, st, a));
     return sar_after_launch();
 }
 

@@ -56,6 +56,7 @@ template <typename T, int MODE>
 __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs a) {
     constexpr int EPV = Elem<T>::EPV;
     constexpr bool kF = MODE == kRowFwd;
+    after_predecessor();
     __shared__ float4 red[kMergeThreads];
     __shared__ float sM[SAR_MAX_HEADS], sD[SAR_MAX_HEADS], sOld[SAR_MAX_HEADS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -150,6 +151,7 @@ __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs
 // Destination-major: D, B and S of the segments are numbers; a warp per long row and head.
 template <bool PART>
 __global__ void __launch_bounds__(kMergeThreads) rows_dst_merge_kernel(const RowArgs a) {
+    after_predecessor();
     const int lane = threadIdx.x & 31;
     const long long item = (long long)blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5);
     const int lr = (int)(item / a.H), h = (int)(item % a.H);
@@ -185,6 +187,7 @@ __global__ void __launch_bounds__(kMergeThreads) rows_dst_merge_kernel(const Row
 // Follows a last partition step that left the complete state behind (aligned shapes).
 template <typename T>
 __global__ void __launch_bounds__(256) rows_finalize_kernel(const RowArgs a) {
+    after_predecessor();
     constexpr int EPV = Elem<T>::EPV;
     const long long vi = (long long)blockIdx.x * 256 + threadIdx.x;
     const int n_vec = a.H * a.vph;
@@ -212,9 +215,9 @@ __global__ void __launch_bounds__(256) rows_finalize_kernel(const RowArgs a) {
 template <int MODE>
 static sar_status launch_merge(const RowArgs &a, sar_dtype t, const char *name, cudaStream_t st) {
     if (t == SAR_F32)
-        SAR_LAUNCH(name, st, (rows_merge_kernel<float, MODE><<<a.sp.n_long, kMergeThreads, 0, st>>>(a)));
+        SAR_LAUNCH(name, st, launch(rows_merge_kernel<float, MODE>, (unsigned)a.sp.n_long, kMergeThreads, 0, st, a));
     else
-        SAR_LAUNCH(name, st, (rows_merge_kernel<__nv_bfloat16, MODE><<<a.sp.n_long, kMergeThreads, 0, st>>>(a)));
+        SAR_LAUNCH(name, st, launch(rows_merge_kernel<__nv_bfloat16, MODE>, (unsigned)a.sp.n_long, kMergeThreads, 0, st, a));
     return sar_after_launch();
 }
 
@@ -225,9 +228,9 @@ sar_status rows_sum_merge(const RowArgs &a, sar_dtype t, cudaStream_t st) { retu
 sar_status rows_fwd_finalize(const RowArgs &a, sar_dtype t, cudaStream_t st) {
     const unsigned blocks = (unsigned)((a.n_rows * a.H * a.vph + 255) / 256);
     if (t == SAR_F32)
-        SAR_LAUNCH("gat_fwd_finalize", st, (rows_finalize_kernel<float><<<blocks, 256, 0, st>>>(a)));
+        SAR_LAUNCH("gat_fwd_finalize", st, launch(rows_finalize_kernel<float>, blocks, 256, 0, st, a));
     else
-        SAR_LAUNCH("gat_fwd_finalize", st, (rows_finalize_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(a)));
+        SAR_LAUNCH("gat_fwd_finalize", st, launch(rows_finalize_kernel<__nv_bfloat16>, blocks, 256, 0, st, a));
     return sar_after_launch();
 }
 
@@ -235,9 +238,9 @@ sar_status rows_dst_merge(const RowArgs &a, bool part, cudaStream_t st) {
     const long long warps = (long long)a.sp.n_long * a.H;
     const unsigned blocks = (unsigned)((warps + kMergeThreads / 32 - 1) / (kMergeThreads / 32));
     if (part)
-        SAR_LAUNCH("gat_bwd_dst_merge", st, (rows_dst_merge_kernel<true><<<blocks, kMergeThreads, 0, st>>>(a)));
+        SAR_LAUNCH("gat_bwd_dst_merge", st, launch(rows_dst_merge_kernel<true>, blocks, kMergeThreads, 0, st, a));
     else
-        SAR_LAUNCH("gat_bwd_dst_merge", st, (rows_dst_merge_kernel<false><<<blocks, kMergeThreads, 0, st>>>(a)));
+        SAR_LAUNCH("gat_bwd_dst_merge", st, launch(rows_dst_merge_kernel<false>, blocks, kMergeThreads, 0, st, a));
     return sar_after_launch();
 }
 

@@ -50,9 +50,7 @@ static sar_status launch_span(SpanArgs a, long long nnz, const char *name, const
             stage_bytes = (size_t)a.R * rsb;
         }
     }
-    bool beside = false;
     if constexpr (MODE == kFwd || kIsSum) if (a.sp.threshold > 0 && a.sp.n_seg > 0) {
-        beside = true;
         a.mode = 1;
         const unsigned blocks = (unsigned)((a.sp.n_seg + kSpanWarps - 1) / kSpanWarps);
         if (a.sp.threshold <= CAP_SEG) {
@@ -60,12 +58,12 @@ static sar_status launch_span(SpanArgs a, long long nnz, const char *name, const
             auto seg_kern = geo ? span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2, kGeo> : span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2>;
             SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2, kGeo>, seg_smem));
             SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2>, seg_smem));
-            SAR_LAUNCH(seg_name, st, seg_kern<<<blocks, kSpanThreads, seg_smem, st>>>(a));
+            SAR_LAUNCH(seg_name, st, launch(seg_kern, blocks, kSpanThreads, seg_smem, st, a));
         } else {
             auto seg_kern = geo ? span_kernel<T, G, V, S, MODE, CAP, MINB, 2, kGeo> : span_kernel<T, G, V, S, MODE, CAP, MINB, 2>;
             SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP, MINB, 2, kGeo>, smem));
             SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP, MINB, 2>, smem));
-            SAR_LAUNCH(seg_name, st, seg_kern<<<blocks, kSpanThreads, smem, st>>>(a));
+            SAR_LAUNCH(seg_name, st, launch(seg_kern, blocks, kSpanThreads, smem, st, a));
         }
         SAR_TRY(sar_after_launch());
     }
@@ -77,16 +75,16 @@ static sar_status launch_span(SpanArgs a, long long nnz, const char *name, const
             if (geo) {
                 auto wk = span_kernel<T, G, V, S, MODE, CAP, MINB, 1, kGeo>;
                 SAR_TRY(ensure_smem(wk, smem));
-                SAR_LAUNCH(name, st, launch_beside_segments(wk, blocks, kSpanThreads, smem, beside, a, st));
+                SAR_LAUNCH(name, st, launch(wk, blocks, kSpanThreads, smem, st, a));
             } else {
                 auto wk = span_kernel<T, G, V, S, MODE, CAP, MINB, 1>;
                 SAR_TRY(ensure_smem(wk, smem));
-                SAR_LAUNCH(name, st, launch_beside_segments(wk, blocks, kSpanThreads, smem, beside, a, st));
+                SAR_LAUNCH(name, st, launch(wk, blocks, kSpanThreads, smem, st, a));
             }
         } else {
             const size_t smem_st = (size_t)kSpanWarps * span_layout<MODE>(a.g.Hp, V, CAP, S, 32 / G, stage_bytes).total;
             SAR_TRY(ensure_smem(kern, smem_st));
-            SAR_LAUNCH(name, st, launch_beside_segments(kern, blocks, kSpanThreads, smem_st, beside, a, st));
+            SAR_LAUNCH(name, st, launch(kern, blocks, kSpanThreads, smem_st, st, a));
         }
         SAR_TRY(sar_after_launch());
     }

@@ -28,6 +28,7 @@
 #pragma once
 
 #include "sar_device.cuh"
+#include "sar_launch.cuh"
 #include "sar_rowkernels.cuh"
 
 namespace sar {
@@ -140,7 +141,9 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
     constexpr bool kSrc = MODE == kBwdSrc;
     constexpr bool kAcc0 = MODE != kBwdDstGivenD;                  // accumulator 0 live
     constexpr bool kAcc1 = kDst || kSrc;                           // accumulator 1 live
-    if (mode_ == 1) let_rows_in();
+    const bool beside = (MODE == kFwd || MODE == kSum || MODE == kSumW) && a.sp.threshold > 0 && a.sp.n_seg > 0;
+    if (mode_ == 1) after_predecessor();
+    else beside_segments(beside);
     extern __shared__ __align__(16) unsigned char smem_raw[];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -988,7 +991,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
             r = r2;
         }
     }
-    if (mode_ == 0) rows_end();
+    if (mode_ == 0) rows_end(beside);
 }
 
 }  // namespace sar
