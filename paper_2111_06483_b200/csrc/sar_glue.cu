@@ -41,6 +41,7 @@ __device__ __forceinline__ void load_coeffs(const float *__restrict__ a, const R
 // RELU: z = max(z, 0) is written back before it is projected (the ReLU that closes the previous layer).
 template <typename T, int G, int V, bool RELU>
 __global__ void __launch_bounds__(kThreads) project_kernel(const ProjArgs a) {
+    after_predecessor();
     constexpr int EPV = Elem<T>::EPV;
     constexpr int RPW = 32 / G;
     constexpr int U = V <= 2 ? 2 : 1;  // rows in flight per group
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(kThreads) project_kernel(const ProjArgs a) {
 // ReLU's backward pass).
 template <typename T, int G, int V, bool MASK>
 __global__ void __launch_bounds__(kThreads) project_bwd_kernel(const ProjArgs a) {
+    after_predecessor();
     constexpr int EPV = Elem<T>::EPV;
     constexpr int RPW = 32 / G;
     constexpr int GPB = kWarpsPerBlock * RPW;  // groups per block
@@ -226,6 +228,7 @@ __global__ void project_bwd_generic(const ProjArgs a, float *da_l, float *da_r, 
 // element at a time.
 template <typename T, bool BWD>
 __global__ void relu_kernel(long long n, const T *y, T *x, long long n_vec16) {
+    after_predecessor();
     constexpr int EPV = Elem<T>::EPV;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nthreads = (long long)gridDim.x * blockDim.x;
@@ -254,7 +257,7 @@ static sar_status launch_relu(const char *name, int64_t n, const void *y, void *
     const long long work = n_vec16 > 0 ? n_vec16 : n;
     long long blocks = (work + 255) / 256;
     if (blocks > 148 * 64) blocks = 148 * 64;
-    SAR_LAUNCH(name, st, (relu_kernel<T, BWD><<<(unsigned)blocks, 256, 0, st>>>(n, static_cast<const T *>(y), static_cast<T *>(x), n_vec16)));
+    SAR_LAUNCH(name, st, launch(relu_kernel<T, BWD>, (unsigned)blocks, 256, 0, st, n, static_cast<const T *>(y), static_cast<T *>(x), n_vec16));
     return sar_after_launch();
 }
 
@@ -371,9 +374,9 @@ sar_status sar_gat_project(int64_t n, int32_t H, int32_t F, sar_dtype t, void *f
         unsigned blocks = blocks_for(n, C::g);
         if (blocks > (unsigned)kGlueBlocks * 4) blocks = kGlueBlocks * 4;
         if (relu)
-            SAR_LAUNCH("gat_project", st, (project_kernel<T, C::g, C::v, true><<<blocks, kThreads, smem, st>>>(a)));
+            SAR_LAUNCH("gat_project", st, launch(project_kernel<T, C::g, C::v, true>, blocks, kThreads, smem, st, a));
         else
-            SAR_LAUNCH("gat_project", st, (project_kernel<T, C::g, C::v, false><<<blocks, kThreads, smem, st>>>(a)));
+            SAR_LAUNCH("gat_project", st, launch(project_kernel<T, C::g, C::v, false>, blocks, kThreads, smem, st, a));
         return sar_after_launch();
     });
 }
@@ -422,7 +425,7 @@ sar_status sar_gat_project_bwd(int64_t n, int32_t H, int32_t F, sar_dtype t, con
         SAR_TRY(ensure_smem(project_bwd_kernel<T, C::g, C::v, false>, smem));
         const unsigned want = blocks_for((a.n + 3) / 4, C::g);
         const unsigned blocks = want < 1 ? 1 : want < (unsigned)kGlueBlocks ? want : (unsigned)kGlueBlocks;
-        SAR_LAUNCH("gat_project_bwd", st, kern<<<blocks, kThreads, smem, st>>>(a));
+        SAR_LAUNCH("gat_project_bwd", st, launch(kern, blocks, kThreads, smem, st, a));
         SAR_TRY(sar_after_launch());
         return reduce_partials("gat_project_reduce", (int)blocks, 2 * HF, HF, a.partial, 1.0, da_l, da_r, st);
     });

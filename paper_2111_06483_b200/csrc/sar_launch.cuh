@@ -1,7 +1,7 @@
 // Launches that overlap the end of the launch before them (internal).
 //
 // A pass over a small graph is a chain of kernels of 3 to 5 us, and between two of them lies 1.5 us in which the second is
-// only being set up.  So every kernel of the aggregation is launched with programmatic stream serialisation and begins
+// only being set up.  So every kernel of the aggregation and of the streaming steps around it is launched with programmatic stream serialisation and begins
 // with after_predecessor(): its blocks may be placed as soon as all blocks of the launch before run, wait there until that
 // launch has ended and its writes are visible, and then let the next launch be placed in turn.  Nothing is read or
 // written before the wait, so the order of the stream holds for every pair of launches, whoever issued them; a launch that
@@ -36,10 +36,10 @@ __device__ __forceinline__ void rows_end(bool segments) {
 }
 
 template <typename... K, typename... A>
-static inline void launch(void (*kernel)(K...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, const A &...args) {
+static inline void launch(void (*kernel)(K...), dim3 grid, dim3 threads, size_t smem, cudaStream_t st, const A &...args) {
     cudaLaunchConfig_t c = {};
     c.gridDim = grid;
-    c.blockDim = dim3(threads);
+    c.blockDim = threads;
     c.dynamicSmemBytes = smem;
     c.stream = st;
     cudaLaunchAttribute at = {};

@@ -73,6 +73,7 @@ __device__ __forceinline__ void load_cols(const float *__restrict__ p, float fil
 // sum gy * xhat with xhat = (x - mean) * rstd.  Per-block partials, no atomics.
 template <typename T, int G, int V, int WHAT, int ACT = 0>
 __global__ void __launch_bounds__(kThreads) norm_sums_kernel(const NormArgs a) {
+    after_predecessor();
     constexpr int EPV = Elem<T>::EPV;
     constexpr int RPW = 32 / G;
     constexpr int GPB = kWarpsPerBlock * RPW;
@@ -144,6 +145,7 @@ __global__ void __launch_bounds__(kThreads) norm_sums_kernel(const NormArgs a) {
 // gx = gamma * rstd * (gy - s0/N - xhat * s1/N)    (BWD = true; inv_count = 1/N)
 template <typename T, int G, int V, bool BWD, int ACT = 0>
 __global__ void __launch_bounds__(kThreads) norm_apply_kernel(const NormArgs a) {
+    after_predecessor();
     constexpr int EPV = Elem<T>::EPV;
     constexpr int RPW = 32 / G;
     const LaneId<G> id;
@@ -273,7 +275,7 @@ static sar_status norm_sums(const Shape &s, NormArgs a, double scale, float *out
         // a few rows per lane group before a block pays for its record; the grid depends on n alone
         const unsigned want = blocks_for((a.n + 3) / 4, C::g);
         const unsigned blocks = want < 1 ? 1 : want < (unsigned)kNormBlocks ? want : (unsigned)kNormBlocks;
-        SAR_LAUNCH(name, st, kern<<<blocks, kThreads, smem, st>>>(a));
+        SAR_LAUNCH(name, st, launch(kern, blocks, kThreads, smem, st, a));
         SAR_TRY(sar_after_launch());
         return reduce_partials("bn_reduce", (int)blocks, 2 * a.C, a.C, a.partial, scale, out0, out1, st);
     });
@@ -297,7 +299,7 @@ static sar_status norm_apply(const Shape &s, const NormArgs &a, cudaStream_t st,
         if (blocks > (unsigned)kNormBlocks * 4) blocks = kNormBlocks * 4;
         auto kern = a.act == 0 ? norm_apply_kernel<T, C::g, C::v, BWD, 0>
                                : (a.act == 3 ? norm_apply_kernel<T, C::g, C::v, BWD, 3> : norm_apply_kernel<T, C::g, C::v, BWD, 1>);
-        SAR_LAUNCH(name, st, (kern<<<blocks, kThreads, 0, st>>>(a)));
+        SAR_LAUNCH(name, st, launch(kern, blocks, kThreads, 0, st, a));
         return sar_after_launch();
     });
 }
@@ -309,6 +311,7 @@ using namespace sar;
 namespace sar {
 // rstd[c] = 1 / sqrt(m2[c] / count + eps): the last step of the statistics, on C floats
 __global__ void norm_rstd_kernel(int C, const float *__restrict__ m2, double inv_count, float eps, float *__restrict__ rstd) {
+    after_predecessor();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c < C) rstd[c] = (float)(1.0 / sqrt((double)m2[c] * inv_count + (double)eps));
 }
@@ -400,7 +403,7 @@ sar_status sar_bn_stats(int64_t n, int32_t C, sar_dtype t, const void *x, float 
 sar_status sar_bn_rstd(int32_t C, const float *m2, int64_t count, float eps, float *rstd, void *stream) {
     if (C < 1 || count < 1 || !m2 || !rstd || !(eps >= 0.f)) return SAR_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    SAR_LAUNCH("bn_rstd", st, (sar::norm_rstd_kernel<<<(unsigned)((C + 127) / 128), 128, 0, st>>>(C, m2, 1.0 / (double)count, eps, rstd)));
+    SAR_LAUNCH("bn_rstd", st, (sar::launch(sar::norm_rstd_kernel, (unsigned)((C + 127) / 128), 128, 0, st, C, m2, 1.0 / (double)count, eps, rstd)));
     return sar_after_launch();
 }
 

@@ -2,6 +2,7 @@
 #pragma once
 
 #include "sar_common.cuh"
+#include "sar_launch.cuh"
 
 namespace sar {
 
@@ -11,6 +12,7 @@ namespace sar {
 constexpr int kReduceSlices = 16;
 static __global__ void __launch_bounds__(32 * kReduceSlices) reduce_partials_kernel(int blocks, int cols, int split, const float *__restrict__ partial,
                                                                                     double scale, float *__restrict__ out0, float *__restrict__ out1) {
+    after_predecessor();
     __shared__ double red[kReduceSlices][32];
     const int x = blockIdx.x * 32 + threadIdx.x;
     double acc = 0.0;
@@ -33,7 +35,7 @@ static __global__ void __launch_bounds__(32 * kReduceSlices) reduce_partials_ker
 
 static inline sar_status reduce_partials(const char *name, int blocks, int cols, int split, const float *partial, double scale, float *out0, float *out1,
                                          cudaStream_t st) {
-    SAR_LAUNCH(name, st, (reduce_partials_kernel<<<(cols + 31) / 32, dim3(32, kReduceSlices), 0, st>>>(blocks, cols, split, partial, scale, out0, out1)));
+    SAR_LAUNCH(name, st, launch(reduce_partials_kernel, (cols + 31) / 32, dim3(32, kReduceSlices), 0, st, blocks, cols, split, partial, scale, out0, out1));
     return sar_after_launch();
 }
 
