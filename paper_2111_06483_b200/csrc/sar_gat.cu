@@ -229,6 +229,23 @@ constexpr unsigned long long kSpanBytes = 128ull << 20, kSpanSumBytes = 12ull <<
 static bool use_span(const Shape &s, long long n_gathered, unsigned long long bytes = kSpanBytes) {
     return s.fast && (unsigned long long)n_gathered * s.row_bytes > bytes;
 }
+// Short rows: a row kernel's warp spends its time on the starts and ends of rows, a span kernel's gathers across them, so
+// the latter take over below some edges per row, once there are rows enough to fill the chip with spans.  Where the lines
+// lie, from 2 to 32 edges per row and 4,000 to 1.2 million rows, time of the span kernels over that of the row kernels:
+//   forward, 2 / 4 / 8 / 16 edges, 300,000 rows: 4 heads of 8, float32 0.72 / 0.78 / 0.91 / 1.19; 2 of 64, float32 0.76 /
+//     0.83 / 0.95 / 1.17; 3 of 32, bf16 0.82 / 0.87 / 0.99 / 1.25; 6 of 48, bf16 0.59 / 0.66 / 0.81 / 0.95; 1 of 16, bf16
+//     0.98 / 1.00 / 1.09 / 1.33; with 20,000 rows 1.1 to 1.7 but for 6 of 48 (0.88 / 0.89 / 1.02 / 1.26).
+//   backward: 4 of 8 0.64 / 0.67 / 0.72 / 0.85 (32 edges 0.93); 2 of 64 0.89 / 0.90 / 0.99 / 1.04; 3 of 32 0.81 / 0.84 /
+//     0.90 / 1.02; 6 of 48 0.43 / 0.49 / 0.61 / 0.73 (tiles of eight heads spill), 0.5 to 0.9 in partition steps of any
+//     size; 1 of 16 1.13 to 1.32; partition steps of the other shapes 0.93 to 1.26.
+static bool short_rows(const Shape &s, long long n_rows, long long nnz, bool backward, bool part) {
+    const int H = s.geom.H;
+    if (!s.fast || s.row_bytes < 128) return false;
+    if (H > 4) return backward ? part || n_rows >= 10000 : n_rows >= 20000 && nnz <= 10 * n_rows;
+    if (!backward) return n_rows >= 60000 && nnz <= (part ? 4 : 6) * n_rows;
+    if (part) return H == 3 && n_rows >= 60000 && nnz <= 5 * n_rows;
+    return H == 4 ? n_rows >= 20000 && nnz <= 32 * n_rows : H == 3 ? n_rows >= 20000 && nnz <= 10 * n_rows : n_rows >= 60000 && nnz <= 5 * n_rows;
+}
 
 static sar_status check_shape(int32_t H, int32_t F, sar_dtype t) {
     Shape s;
@@ -413,7 +430,7 @@ sar_status sar_gat_fwd(const sar_part *g, const void *feat_q, const float *el, c
         }
         return SAR_OK;
     }
-    if (use_span(s, g->n_src))
+    if (use_span(s, g->n_src) || short_rows(s, g->n_dst, g->nnz, false, part))
         SAR_TRY(span_fwd(s, a, g->nnz, st));
     else if (part)
         SAR_TRY(t == SAR_F32 ? rows_fwd_part_f32(a, r.geo, g->nnz, st) : rows_fwd_part_bf16(a, r.geo, g->nnz, st));
@@ -615,9 +632,8 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
                 SAR_TRY(t == SAR_F32 ? lean_bwd_dst_f32(s, la, g->nnz, st) : lean_bwd_dst_bf16(s, la, g->nnz, st));
             else
                 SAR_TRY(t == SAR_F32 ? lean_bwd_dst_part_f32(s, la, g->nnz, st) : lean_bwd_dst_part_bf16(s, la, g->nnz, st));
-        } else if (use_span(s, g->n_src)) {
-            SAR_TRY(span_dst(s, a, g->nnz, !whole, st));
-            a.n_rows = 0;   // the segments
+        } else if (use_span(s, g->n_src) || short_rows(s, g->n_dst, g->nnz, true, !whole)) {
+            a.n_rows = 0;   // the segments first, the rows beside them
             if (a.sp.n_seg > 0) {
                 if (whole)
                     SAR_TRY(t == SAR_F32 ? rows_dst_f32(a, r.geo, g->nnz, st) : rows_dst_bf16(a, r.geo, g->nnz, st));
@@ -625,6 +641,7 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
                     SAR_TRY(t == SAR_F32 ? rows_dst_part_f32(a, r.geo, g->nnz, st) : rows_dst_part_bf16(a, r.geo, g->nnz, st));
             }
             a.n_rows = g->n_dst;
+            SAR_TRY(span_dst(s, a, g->nnz, !whole, st));
         } else if (whole)
             SAR_TRY(t == SAR_F32 ? rows_dst_f32(a, r.geo, g->nnz, st) : rows_dst_bf16(a, r.geo, g->nnz, st));
         else
@@ -657,11 +674,11 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
             la.sp.threshold = g->t_split->threshold;
             SAR_TRY(t == SAR_F32 ? lean_bwd_src_f32(s, la, g->nnz, st) : lean_bwd_src_bf16(s, la, g->nnz, st));
         } else {
-            if (use_span(s, g->n_dst)) {
-                SAR_TRY(span_src(s, a, g->nnz, st));
-                a.n_rows = 0;   // the segments
-            }
+            const bool span = use_span(s, g->n_dst) || short_rows(s, g->n_src, g->nnz, true, !whole);
+            if (span) a.n_rows = 0;   // the segments first, the rows beside them
             SAR_TRY(t == SAR_F32 ? rows_src_f32(a, r.geo, g->nnz, st) : rows_src_bf16(a, r.geo, g->nnz, st));
+            a.n_rows = g->n_src;
+            if (span) SAR_TRY(span_src(s, a, g->nnz, st));
         }
         if (a.sp.n_long > 0) SAR_TRY(rows_src_merge(a, t, st));
     }

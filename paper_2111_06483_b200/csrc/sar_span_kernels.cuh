@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
     constexpr bool kSrc = MODE == kBwdSrc;
     constexpr bool kAcc0 = MODE != kBwdDstGivenD;                  // accumulator 0 live
     constexpr bool kAcc1 = kDst || kSrc;                           // accumulator 1 live
-    const bool beside = (MODE == kFwd || MODE == kSum || MODE == kSumW) && a.sp.threshold > 0 && a.sp.n_seg > 0;
+    const bool beside = a.sp.threshold > 0 && a.sp.n_seg > 0;   // the segments (of the backward passes: the row kernel's) go first
     if (mode_ == 1) after_predecessor();
     else beside_segments(beside);
     extern __shared__ __align__(16) unsigned char smem_raw[];

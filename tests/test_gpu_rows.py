@@ -34,6 +34,15 @@ def test_attention_on_arrays_larger_than_the_l2(H, F, dtype, n):
     _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
 
 
+@pytest.mark.parametrize("H,F,dtype,n,deg,d_max", [(4, 8, "f32", 61_000, 3, 200.0), (2, 64, "bf16", 61_000, 2, 400.0), (3, 32, "bf16", 61_000, 4, 900.0),
+                                                   (6, 48, "bf16", 21_000, 9, 300.0), (12, 16, "f32", 10_100, 2, 500.0)])
+def test_attention_on_short_rows(H, F, dtype, n, deg, d_max):
+    """Few edges per row: the span kernels on small arrays, whole and step by step, with long rows among them."""
+    n, src, dst = hub_graph(n=n, e=deg * n, d_max=d_max, seed=H + F)
+    p = Problem(n, src, dst, H, F, 31, dtype=dtype, k=2, threshold=100, build_parts=True)
+    _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
+
+
 @pytest.mark.parametrize("F", [1, 3, 47, 48, 127, 180, 260, 1030])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("n", [1500, 40_000])
