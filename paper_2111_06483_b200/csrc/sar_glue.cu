@@ -257,7 +257,7 @@ static sar_status launch_relu(const char *name, int64_t n, const void *y, void *
     const long long work = n_vec16 > 0 ? n_vec16 : n;
     long long blocks = (work + 255) / 256;
     if (blocks > 148 * 64) blocks = 148 * 64;
-    SAR_LAUNCH(name, st, launch(relu_kernel<T, BWD>, (unsigned)blocks, 256, 0, st, n, static_cast<const T *>(y), static_cast<T *>(x), n_vec16));
+    SAR_LAUNCH(name, st, launch_if(n <= kOverlapElems, relu_kernel<T, BWD>, (unsigned)blocks, 256, 0, st, n, static_cast<const T *>(y), static_cast<T *>(x), n_vec16));
     return sar_after_launch();
 }
 
@@ -374,9 +374,9 @@ sar_status sar_gat_project(int64_t n, int32_t H, int32_t F, sar_dtype t, void *f
         unsigned blocks = blocks_for(n, C::g);
         if (blocks > (unsigned)kGlueBlocks * 4) blocks = kGlueBlocks * 4;
         if (relu)
-            SAR_LAUNCH("gat_project", st, launch(project_kernel<T, C::g, C::v, true>, blocks, kThreads, smem, st, a));
+            SAR_LAUNCH("gat_project", st, launch_if(n * H * F <= kOverlapElems, project_kernel<T, C::g, C::v, true>, blocks, kThreads, smem, st, a));
         else
-            SAR_LAUNCH("gat_project", st, launch(project_kernel<T, C::g, C::v, false>, blocks, kThreads, smem, st, a));
+            SAR_LAUNCH("gat_project", st, launch_if(n * H * F <= kOverlapElems, project_kernel<T, C::g, C::v, false>, blocks, kThreads, smem, st, a));
         return sar_after_launch();
     });
 }
@@ -425,7 +425,7 @@ sar_status sar_gat_project_bwd(int64_t n, int32_t H, int32_t F, sar_dtype t, con
         SAR_TRY(ensure_smem(project_bwd_kernel<T, C::g, C::v, false>, smem));
         const unsigned want = blocks_for((a.n + 3) / 4, C::g);
         const unsigned blocks = want < 1 ? 1 : want < (unsigned)kGlueBlocks ? want : (unsigned)kGlueBlocks;
-        SAR_LAUNCH("gat_project_bwd", st, launch(kern, blocks, kThreads, smem, st, a));
+        SAR_LAUNCH("gat_project_bwd", st, launch_if(n * HF <= kOverlapElems, kern, blocks, kThreads, smem, st, a));
         SAR_TRY(sar_after_launch());
         return reduce_partials("gat_project_reduce", (int)blocks, 2 * HF, HF, a.partial, 1.0, da_l, da_r, st);
     });

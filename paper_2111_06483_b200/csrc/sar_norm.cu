@@ -275,7 +275,7 @@ static sar_status norm_sums(const Shape &s, NormArgs a, double scale, float *out
         // a few rows per lane group before a block pays for its record; the grid depends on n alone
         const unsigned want = blocks_for((a.n + 3) / 4, C::g);
         const unsigned blocks = want < 1 ? 1 : want < (unsigned)kNormBlocks ? want : (unsigned)kNormBlocks;
-        SAR_LAUNCH(name, st, launch(kern, blocks, kThreads, smem, st, a));
+        SAR_LAUNCH(name, st, launch_if(a.n * a.C <= kOverlapElems, kern, blocks, kThreads, smem, st, a));
         SAR_TRY(sar_after_launch());
         return reduce_partials("bn_reduce", (int)blocks, 2 * a.C, a.C, a.partial, scale, out0, out1, st);
     });
@@ -299,7 +299,7 @@ static sar_status norm_apply(const Shape &s, const NormArgs &a, cudaStream_t st,
         if (blocks > (unsigned)kNormBlocks * 4) blocks = kNormBlocks * 4;
         auto kern = a.act == 0 ? norm_apply_kernel<T, C::g, C::v, BWD, 0>
                                : (a.act == 3 ? norm_apply_kernel<T, C::g, C::v, BWD, 3> : norm_apply_kernel<T, C::g, C::v, BWD, 1>);
-        SAR_LAUNCH(name, st, launch(kern, blocks, kThreads, 0, st, a));
+        SAR_LAUNCH(name, st, launch_if(a.n * a.C <= kOverlapElems, kern, blocks, kThreads, 0, st, a));
         return sar_after_launch();
     });
 }
