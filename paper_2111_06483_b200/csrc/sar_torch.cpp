@@ -109,7 +109,33 @@ sar_dtype code(const at::Tensor &t) {
     if (t.scalar_type() == at::kBFloat16) return SAR_BF16;
     fail(PyExc_TypeError, "unsupported storage dtype");
 }
-const float *f32(const at::Tensor &t) { return t.defined() ? static_cast<const float *>(t.const_data_ptr()) : nullptr; }
+void require(bool ok, const char *text) {
+    if (!ok) fail(PyExc_AssertionError, text);
+}
+// The library sees a pointer, so what it will read behind it is checked here: the type and at least n elements.
+const float *f32(const at::Tensor &t, int64_t n) {
+    if (!t.defined()) return nullptr;
+    require(t.scalar_type() == at::kFloat, "expected a float32 tensor");
+    require(t.numel() >= n, "a float32 tensor is smaller than its use");
+    return static_cast<const float *>(t.const_data_ptr());
+}
+void require_like(const at::Tensor &t, const at::Tensor &like, int64_t n) {
+    require(t.scalar_type() == like.scalar_type(), "tensors of one storage type expected");
+    require(t.numel() >= n, "a tensor is smaller than its use");
+}
+void require_matrix(const at::Tensor &t, const at::Tensor &like, int64_t rows, int64_t cols) {
+    require(t.dim() == 2 && t.size(0) == rows && t.size(1) == cols, "a weight matrix of another shape");
+    require(t.scalar_type() == like.scalar_type(), "tensors of one storage type expected");
+}
+void require_rows(const at::Tensor &t, int64_t n) { require(t.dim() > 0 && t.size(0) >= n, "a node array has fewer rows than the graph"); }
+// ... of every piece of a graph: its destinations and its slice of the sources
+void require_pieces(const std::vector<int64_t> &parts, const std::vector<int64_t> &bounds, int64_t n_src, int64_t n_dst) {
+    require(!parts.empty() && bounds.size() == parts.size() + 1, "one more bound than partitions expected");
+    for (size_t q = 0; q < parts.size(); ++q) {
+        const sar_part *g = reinterpret_cast<const sar_part *>(parts[q]);
+        require(g->n_dst <= n_dst && bounds[q] >= 0 && bounds[q] + g->n_src <= n_src, "a node array has fewer rows than the graph");
+    }
+}
 float *f32m(const at::Tensor &t) { return t.defined() ? static_cast<float *>(t.mutable_data_ptr()) : nullptr; }
 const void *ptr(const at::Tensor &t) { return t.const_data_ptr(); }
 void *ptrm(const at::Tensor &t) { return t.mutable_data_ptr(); }
@@ -235,6 +261,8 @@ struct Forward {
 Forward forward_fused(const sar_part *g, const std::vector<int64_t> &bounds, const at::Tensor &feat, const at::Tensor &el,
                       const at::Tensor &er, double slope, at::Tensor ws, bool relu) {
     const Dims d(feat);
+    require_rows(feat, g->n_src);
+    const float *pl = f32(el, g->n_dst * d.H), *pr = f32(er, g->n_src * d.H);
     Forward r;
     r.m = empty({g->n_dst, d.H}, at::kFloat, feat);
     r.d = empty({g->n_dst, d.H}, at::kFloat, feat);
@@ -243,10 +271,10 @@ Forward forward_fused(const sar_part *g, const std::vector<int64_t> &bounds, con
     void *w = ws.defined() ? ptrm(ws) : nullptr;
     const size_t wb = ws.defined() ? ws.nbytes() : 0;
     if (relu)   // the un-split graph as one partition holding all sources
-        SAR(sar_gat_fwd, g, ptr(feat), f32(el), f32(er), d.H, d.F, d.t, (float)slope, SAR_FIRST | SAR_LAST | SAR_RELU_OUT, nullptr,
+        SAR(sar_gat_fwd, g, ptr(feat), pl, pr, d.H, d.F, d.t, (float)slope, SAR_FIRST | SAR_LAST | SAR_RELU_OUT, nullptr,
             f32m(r.m), f32m(r.d), ptrm(r.out), w, wb, stream());
     else
-        SAR(sar_gat_fwd_fused, g, (int32_t)bounds.size() - 1, bounds.data(), ptr(feat), f32(el), f32(er), d.H, d.F, d.t, (float)slope,
+        SAR(sar_gat_fwd_fused, g, (int32_t)bounds.size() - 1, bounds.data(), ptr(feat), pl, pr, d.H, d.F, d.t, (float)slope,
             f32m(r.m), f32m(r.d), ptrm(r.out), w, wb, stream());
     return r;
 }
@@ -264,10 +292,14 @@ Backward backward_outputs(const at::Tensor &feat, const Dims &d, int64_t n_dst) 
 Backward backward_fused(const sar_part *g, const std::vector<int64_t> &bounds, const at::Tensor &feat, const at::Tensor &el,
                         const at::Tensor &er, const at::Tensor &m, const at::Tensor &dd, const at::Tensor &gout, double slope, at::Tensor ws) {
     const Dims d(feat);
+    const int64_t nh = g->n_dst * d.H;
+    require_rows(feat, g->n_src);
+    require_like(gout, feat, nh * d.F);
+    const float *pl = f32(el, nh), *pr = f32(er, g->n_src * d.H), *pm = f32(m, nh), *pd = f32(dd, nh);
     Backward r = backward_outputs(feat, d, g->n_dst);
     if (!ws.defined()) ws = bytes(L.sar_gat_workspace_bytes(g, d.H, d.F, d.t), feat);
-    SAR(sar_gat_bwd_fused, g, (int32_t)bounds.size() - 1, bounds.data(), ptr(feat), f32(el), f32(er), f32(m), f32(dd), ptr(gout), d.H, d.F,
-        code(gout), (float)slope, ptrm(r.dfeat), f32m(r.del), f32m(r.der), ptrm(ws), ws.nbytes(), stream());
+    SAR(sar_gat_bwd_fused, g, (int32_t)bounds.size() - 1, bounds.data(), ptr(feat), pl, pr, pm, pd, ptr(gout), d.H, d.F,
+        d.t, (float)slope, ptrm(r.dfeat), f32m(r.del), f32m(r.der), ptrm(ws), ws.nbytes(), stream());
     return r;
 }
 
@@ -308,6 +340,9 @@ PyObject *gat_forward_parts(Args &a) {   // parts, bounds, n_dst, feat, el, er, 
     const bool keep = a.flag(), relu = a.flag();
     const Dims d(feat);
     const size_t k = parts.size();
+    require_pieces(parts, bounds, d.n, n_dst);
+    const float *pl = f32(el, n_dst * d.H);
+    f32(er, bounds[k] * d.H);
     const at::Tensor m = empty({n_dst, d.H}, at::kFloat, feat), dd = empty({n_dst, d.H}, at::kFloat, feat);
     const at::Tensor out = empty({n_dst, d.H, d.F}, feat.scalar_type(), feat);
     at::Tensor acc;
@@ -316,7 +351,7 @@ PyObject *gat_forward_parts(Args &a) {   // parts, bounds, n_dst, feat, el, er, 
     for (size_t q = 0; q < k; ++q) {
         unsigned flags = step_flags(q, k);
         if (q + 1 == k) flags |= (keep ? SAR_KEEP_NUMERATOR : 0u) | (relu ? SAR_RELU_OUT : 0u);
-        SAR(sar_gat_fwd, reinterpret_cast<const sar_part *>(parts[q]), rows(feat, bounds[q]), f32(el),
+        SAR(sar_gat_fwd, reinterpret_cast<const sar_part *>(parts[q]), rows(feat, bounds[q]), pl,
             reinterpret_cast<const float *>(rows(er, bounds[q])), d.H, d.F, d.t, (float)slope, flags, f32m(acc), f32m(m), f32m(dd), ptrm(out),
             ptrm(ws), ws.nbytes(), stream());
     }
@@ -332,14 +367,20 @@ PyObject *gat_backward_parts(Args &a) {   // parts, bounds, n_dst, feat, el, er,
     const bool numerator = a.flag();
     const Dims d(feat);
     const size_t k = parts.size();
+    const int64_t nh = n_dst * d.H;
+    require_pieces(parts, bounds, d.n, n_dst);
+    require_like(gout, feat, nh * d.F);
+    if (numerator) f32(oa, nh * d.F);
+    else require_like(oa, feat, nh * d.F);
+    const float *pl = f32(el, nh), *pm = f32(m, nh), *pd = f32(dd, nh);
+    f32(er, bounds[k] * d.H);
     const Backward r = backward_outputs(feat, d, n_dst);
     const at::Tensor ws = bytes(parts_workspace(parts, d), feat);
-    SAR(sar_gat_bwd_prepare, n_dst, d.H, d.F, code(gout), ptr(oa), numerator ? 1 : 0, ptr(gout), f32(el), f32(m), f32(dd), nullptr, ptrm(ws),
-        ws.nbytes(), stream());
+    SAR(sar_gat_bwd_prepare, n_dst, d.H, d.F, d.t, ptr(oa), numerator ? 1 : 0, ptr(gout), pl, pm, pd, nullptr, ptrm(ws), ws.nbytes(), stream());
     for (size_t q = 0; q < k; ++q) {
         const int64_t s = bounds[q];
-        SAR(sar_gat_bwd, reinterpret_cast<const sar_part *>(parts[q]), rows(feat, s), f32(el), reinterpret_cast<const float *>(rows(er, s)),
-            f32(m), f32(dd), ptr(gout), d.H, d.F, d.t, (float)slope, step_flags(q, k), rowsm(r.dfeat, s), f32m(r.del),
+        SAR(sar_gat_bwd, reinterpret_cast<const sar_part *>(parts[q]), rows(feat, s), pl, reinterpret_cast<const float *>(rows(er, s)),
+            pm, pd, ptr(gout), d.H, d.F, d.t, (float)slope, step_flags(q, k), rowsm(r.dfeat, s), f32m(r.del),
             reinterpret_cast<float *>(rowsm(r.der, s)), ptrm(ws), ws.nbytes(), stream());
     }
     return tuple(r.dfeat, r.del, r.der);
@@ -370,6 +411,8 @@ PyObject *spmm(Args &a) {   // part, feat, flags, deg_total
     const at::Tensor &x = a.tensor();
     const unsigned flags = (unsigned)a.integer();
     const at::Tensor deg = a.optional();
+    require_rows(x, g->n_src);
+    require(!deg.defined() || (deg.scalar_type() == at::kLong && deg.numel() >= g->n_dst), "expected an int64 degree per node");
     const at::Tensor out = empty({g->n_dst, x.size(1)}, x.scalar_type(), x);
     Scratch ws;
     void *w = ws.get(sum_workspace(g, x), x);
@@ -384,9 +427,11 @@ PyObject *spmm_scaled(Args &a) {   // part, feat, flags, src_scale, dst_scale, o
     const unsigned flags = (unsigned)a.integer();
     const at::Tensor src = a.optional(), dst = a.optional();
     at::Tensor out = a.optional();
-    if (!out.defined()) out = empty({g->n_dst, x.size(1)}, x.scalar_type(), x);
+    require_rows(x, g->n_src);
+    if (out.defined()) require_like(out, x, g->n_dst * x.size(1));
+    else out = empty({g->n_dst, x.size(1)}, x.scalar_type(), x);
     Scratch ws;
-    sum_scaled(g, ptr(x), x, flags, f32(src), f32(dst), ptrm(out), ws);
+    sum_scaled(g, ptr(x), x, flags, f32(src, g->n_src), f32(dst, g->n_dst), ptrm(out), ws);
     return wrap(out);
 }
 
@@ -399,25 +444,26 @@ PyObject *propagate(Args &a) {   // parts, bounds, x0, alpha, iters, src_scale, 
     if (iters <= 0) return wrap(x0.clone());
     std::vector<const sar_part *> ps;
     for (int64_t p : parts) ps.push_back(reinterpret_cast<const sar_part *>(p));
+    require_pieces(parts, bounds, x0.size(0), x0.size(0));
+    const float *ss = f32(src, ps[0]->n_dst), *ds = f32(dst, ps[0]->n_dst);
     const int32_t k = (int32_t)ps.size(), F = (int32_t)x0.size(1);
     const at::Tensor out = empty(x0.sizes(), x0.scalar_type(), x0);
     const at::Tensor ws = bytes(L.sar_propagate_workspace_bytes(k, ps.data(), F, code(x0)), x0);
-    SAR(sar_propagate, k, ps.data(), bounds.data(), ptr(x0), F, code(x0), (float)alpha, iters, f32(src), f32(dst), ptrm(out), ptrm(ws), ws.nbytes(),
-        stream());
+    SAR(sar_propagate, k, ps.data(), bounds.data(), ptr(x0), F, code(x0), (float)alpha, iters, ss, ds, ptrm(out), ptrm(ws), ws.nbytes(), stream());
     return wrap(out);
 }
 
 // sum over the pieces of one graph of inv * A x
 void aggregate(const std::vector<int64_t> &parts, const std::vector<int64_t> &bounds, const at::Tensor &h, const at::Tensor &inv, const at::Tensor &agg, Scratch &ws) {
     for (size_t q = 0; q < parts.size(); ++q)
-        sum_scaled(reinterpret_cast<const sar_part *>(parts[q]), rows(h, bounds[q]), h, step_flags(q, parts.size()), nullptr, f32(inv), ptrm(agg), ws);
+        sum_scaled(reinterpret_cast<const sar_part *>(parts[q]), rows(h, bounds[q]), h, step_flags(q, parts.size()), nullptr, f32(inv, reinterpret_cast<const sar_part *>(parts[q])->n_dst), ptrm(agg), ws);
 }
 // dh of every piece's sources (+)= what their out-edges hand back of dagg
 void scatter(const std::vector<int64_t> &parts, const std::vector<int64_t> &bounds, const at::Tensor &dagg, const at::Tensor &inv, const at::Tensor &dh, unsigned first, Scratch &ws) {
     for (size_t q = 0; q < parts.size(); ++q) {
         const sar_part *g = reinterpret_cast<const sar_part *>(parts[q]);
         const sar_part t{g->n_src, g->n_dst, g->nnz, g->t_indptr, g->t_indices, g->indptr, g->indices, g->t_split, g->split};
-        sum_scaled(&t, ptr(dagg), dagg, first | SAR_LAST, f32(inv), nullptr, rowsm(dh, bounds[q]), ws);
+        sum_scaled(&t, ptr(dagg), dagg, first | SAR_LAST, f32(inv, g->n_dst), nullptr, rowsm(dh, bounds[q]), ws);
     }
 }
 
@@ -431,15 +477,18 @@ PyObject *layer_forward(Args &a) {   // part, bounds, h, W, a_l, a_r, slope, rel
     const int64_t n = h.size(0);
     const int32_t d_in = (int32_t)h.size(1), H = (int32_t)al.size(0), F = (int32_t)al.size(1);
     const sar_dtype t = code(h);
+    require_matrix(W, h, d_in, (int64_t)H * F);
+    require_rows(h, g->n_src);
+    const float *pal = f32(al, (int64_t)H * F), *par = f32(ar, (int64_t)H * F);
     if (relu) SAR(sar_relu, h.numel(), t, ptrm(h), stream());
     const at::Tensor z = empty({n, H, F}, h.scalar_type(), h), el = empty({n, H}, at::kFloat, h), er = empty({n, H}, at::kFloat, h);
     {
         const at::Tensor ws = bytes(L.sar_linear_workspace_bytes(n, d_in, H * F), h);
         if (F % 8 == 0 && 128 % F == 0) {   // the scores leave the projection's epilogue
-            SAR(sar_linear_project, n, d_in, H, F, t, ptr(h), ptr(W), f32(al), f32(ar), ptrm(z), f32m(el), f32m(er), nullptr, ptrm(ws), ws.nbytes(), stream());
+            SAR(sar_linear_project, n, d_in, H, F, t, ptr(h), ptr(W), pal, par, ptrm(z), f32m(el), f32m(er), nullptr, ptrm(ws), ws.nbytes(), stream());
         } else {
             SAR(sar_linear, n, d_in, H * F, t, ptr(h), ptr(W), ptrm(z), ptrm(ws), ws.nbytes(), stream());
-            SAR(sar_gat_project, n, H, F, t, ptrm(z), f32(al), f32(ar), f32m(el), f32m(er), 0u, stream());
+            SAR(sar_gat_project, n, H, F, t, ptrm(z), pal, par, f32m(el), f32m(er), 0u, stream());
         }
     }
     const Forward r = forward_fused(g, bounds, z, el, er, slope, at::Tensor(), false);
@@ -456,11 +505,15 @@ PyObject *layer_backward(Args &a) {   // part, bounds, h, W, a_l, a_r, z, el, er
     const int64_t n = h.size(0);
     const int32_t d_in = (int32_t)h.size(1), H = (int32_t)al.size(0), F = (int32_t)al.size(1);
     const sar_dtype t = code(h);
+    require_matrix(W, h, d_in, (int64_t)H * F);
+    require(z.dim() == 3 && z.size(0) == n && z.size(1) == H && z.size(2) == F, "expected the z of the forward call");
+    require_like(z, h, 0);
+    const float *pal = f32(al, (int64_t)H * F), *par = f32(ar, (int64_t)H * F);
     const Backward b = backward_fused(g, bounds, z, el, er, m, d, gout, slope, at::Tensor());
     const at::Tensor dal = empty({H, F}, at::kFloat, h), dar = empty({H, F}, at::kFloat, h);
     {
         const at::Tensor ws = bytes(L.sar_gat_project_workspace_bytes(H, F), h);
-        SAR(sar_gat_project_bwd, n, H, F, t, ptr(z), f32(al), f32(ar), f32(b.del), f32(b.der), ptrm(b.dfeat), f32m(dal), f32m(dar), 0u, ptrm(ws), ws.nbytes(), stream());
+        SAR(sar_gat_project_bwd, n, H, F, t, ptr(z), pal, par, f32(b.del, n * H), f32(b.der, n * H), ptrm(b.dfeat), f32m(dal), f32m(dar), 0u, ptrm(ws), ws.nbytes(), stream());
     }
     const at::Tensor ws = bytes(L.sar_linear_workspace_bytes(n, d_in, H * F), h);
     const at::Tensor dW = empty({d_in, (int64_t)H * F}, at::kFloat, h), dh = empty(h.sizes(), h.scalar_type(), h);
@@ -478,6 +531,9 @@ PyObject *sage_forward(Args &a) {   // parts, bounds, h, W, W_res, inv
     const int64_t n = h.size(0);
     const int32_t d_in = (int32_t)h.size(1), d_out = (int32_t)W.size(1);
     const sar_dtype t = code(h);
+    require_pieces(parts, bounds, n, n);
+    require_matrix(W, h, d_in, d_out);
+    require_matrix(Wr, h, d_in, d_out);
     const at::Tensor agg = empty(h.sizes(), h.scalar_type(), h), pre = empty({n, d_out}, h.scalar_type(), h);
     Scratch sws;
     aggregate(parts, bounds, h, inv, agg, sws);
@@ -493,6 +549,11 @@ PyObject *sage_backward(Args &a) {   // parts, bounds, h, W, W_res, agg, inv, gp
     const int64_t n = h.size(0);
     const int32_t d_in = (int32_t)h.size(1), d_out = (int32_t)W.size(1);
     const sar_dtype t = code(h);
+    require_pieces(parts, bounds, n, n);
+    require_matrix(W, h, d_in, d_out);
+    require_matrix(Wr, h, d_in, d_out);
+    require_like(agg, h, n * d_in);
+    require_like(g, h, n * d_out);
     const at::Tensor ws = bytes(L.sar_linear_workspace_bytes(n, d_in, d_out), h);
     const at::Tensor dW = empty({d_in, d_out}, at::kFloat, h), dWr = empty({d_in, d_out}, at::kFloat, h);
     SAR(sar_linear_bwd_weight, n, d_in, d_out, t, ptr(agg), ptr(g), f32m(dW), ptrm(ws), ws.nbytes(), stream());
@@ -513,12 +574,13 @@ PyObject *bn_forward(Args &a) {   // x, eps, gamma, beta
     const int64_t n = x.size(0);
     const int32_t C = (int32_t)x.size(1);
     const sar_dtype t = code(x);
+    const float *pg = f32(gamma, C), *pb = f32(beta, C);
     const at::Tensor ws = bytes(L.sar_bn_workspace_bytes(C), x);
     const at::Tensor mean = empty({C}, at::kFloat, x), m2 = empty({C}, at::kFloat, x), rstd = empty({C}, at::kFloat, x);
     const at::Tensor y = empty(x.sizes(), x.scalar_type(), x);
     SAR(sar_bn_stats, n, C, t, ptr(x), f32m(mean), f32m(m2), ptrm(ws), ws.nbytes(), stream());
-    SAR(sar_bn_rstd, C, f32(m2), n > 1 ? n : 1, (float)eps, f32m(rstd), stream());
-    SAR(sar_bn_apply, n, C, t, ptr(x), f32(mean), f32(rstd), f32(gamma), f32(beta), ptrm(y), stream());
+    SAR(sar_bn_rstd, C, f32(m2, C), n > 1 ? n : 1, (float)eps, f32m(rstd), stream());
+    SAR(sar_bn_apply, n, C, t, ptr(x), f32(mean, C), f32(rstd, C), pg, pb, ptrm(y), stream());
     return tuple(y, mean, rstd);
 }
 
@@ -528,10 +590,12 @@ PyObject *bn_backward(Args &a) {   // x, gy, mean, rstd, gamma, count
     const int64_t count = a.integer(), n = x.size(0);
     const int32_t C = (int32_t)x.size(1);
     const sar_dtype t = code(x);
+    require_like(gy, x, n * C);
+    const float *pm = f32(mean, C), *pr = f32(rstd, C), *pg = f32(gamma, C);
     const at::Tensor ws = bytes(L.sar_bn_workspace_bytes(C), x);
     const at::Tensor s0 = empty({C}, at::kFloat, x), s1 = empty({C}, at::kFloat, x), gx = empty(x.sizes(), x.scalar_type(), x);
-    SAR(sar_bn_bwd_stats, n, C, t, ptr(x), f32(mean), f32(rstd), ptr(gy), f32m(s0), f32m(s1), ptrm(ws), ws.nbytes(), stream());
-    SAR(sar_bn_bwd_apply, n, C, t, ptr(x), f32(mean), f32(rstd), f32(gamma), ptr(gy), f32(s0), f32(s1), (float)(1.0 / (double)(count > 1 ? count : 1)), ptrm(gx), stream());
+    SAR(sar_bn_bwd_stats, n, C, t, ptr(x), pm, pr, ptr(gy), f32m(s0), f32m(s1), ptrm(ws), ws.nbytes(), stream());
+    SAR(sar_bn_bwd_apply, n, C, t, ptr(x), pm, pr, pg, ptr(gy), f32(s0, C), f32(s1, C), (float)(1.0 / (double)(count > 1 ? count : 1)), ptrm(gx), stream());
     return tuple(gx, s1, s0);
 }
 
