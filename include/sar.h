@@ -77,6 +77,7 @@ typedef enum { SAR_F32 = 0, SAR_BF16 = 1 } sar_dtype;
 #define SAR_MEAN 4u  /* sar_spmm_agg with SAR_LAST: divide by `deg_total`                    */
 #define SAR_KEEP_NUMERATOR 8u /* sar_gat_fwd with SAR_LAST: also leave the complete numerator in acc */
 #define SAR_RELU_OUT 16u      /* sar_gat_fwd with SAR_LAST: out = max(acc/d, 0), the f_node of Algorithm 1 as a ReLU */
+#define SAR_SAME_WORKSPACE 32u /* sar_gat_bwd after the first step: the workspace is as an earlier step left it */
 
 #define SAR_MAX_HEADS 16
 #define SAR_MAX_PARTS 64
@@ -318,7 +319,10 @@ SAR_API sar_status sar_gat_bwd_prepare(int64_t n_dst, int32_t H, int32_t F, sar_
  *   SAR_FIRST and accumulated otherwise.
  *   With SAR_FIRST|SAR_LAST (one partition holding all sources) D is rebuilt from the edges and
  *   sar_gat_bwd_prepare is not needed; otherwise `workspace` must hold what sar_gat_bwd_prepare
- *   wrote for these (gout, m, d).  Needs g->t_indptr / g->t_indices. */
+ *   wrote for these (gout, m, d).  SAR_SAME_WORKSPACE (not with SAR_FIRST) says that it also still holds what an earlier
+ *   step of the same pass left there - same workspace, gout, H, F, t and n_dst, and workspace_bytes at least the largest of
+ *   the partitions' sar_gat_workspace_bytes in all these steps: the step may then use that step's padded copy of gout.
+ *   Needs g->t_indptr / g->t_indices. */
 SAR_API sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, const float *er_q,
                        const float *m, const float *d, const void *gout, int32_t H, int32_t F, sar_dtype t,
                        float slope, uint32_t flags, void *dfeat_q, float *del, float *der_q, void *workspace,

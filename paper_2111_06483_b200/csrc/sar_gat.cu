@@ -85,13 +85,19 @@ static RowShape sum_shape(int F, sar_dtype t) {
     return r;
 }
 
-// [n,H,F] -> [n,H,vph*EPV], zeros behind the F elements of a head; one 16-byte vector per thread
+// [n,H,F] -> [n,H,vph*EPV], zeros behind the F elements of a head, of one array or of two (n2 > 0); one 16-byte vector per thread
 template <typename T>
-__global__ void __launch_bounds__(256) pad_rows_kernel(long long vecs, int F, int vph, const T *__restrict__ in, uint4 *__restrict__ out) {
+__global__ void __launch_bounds__(256) pad_rows_kernel(long long vecs, long long vecs2, int F, int vph, const T *__restrict__ in, uint4 *__restrict__ out,
+                                                       const T *__restrict__ in2, uint4 *__restrict__ out2) {
     after_predecessor();
     constexpr int EPV = Elem<T>::EPV;
-    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
-    if (i >= vecs) return;
+    long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (i >= vecs) {
+        i -= vecs;
+        if (i >= vecs2) return;
+        in = in2;
+        out = out2;
+    }
     const long long nh = i / vph;
     const int f0 = (int)(i - nh * vph) * EPV;
     const T *p = in + nh * F + f0;
@@ -101,14 +107,16 @@ __global__ void __launch_bounds__(256) pad_rows_kernel(long long vecs, int F, in
     out[i] = Elem<T>::pack(x);
 }
 
-static sar_status pad_rows(long long n, int H, int F, const RowShape &r, sar_dtype t, const void *in, void *out, cudaStream_t st) {
-    const long long vecs = n * H * r.vph;
-    if (vecs == 0) return SAR_OK;
-    const unsigned blocks = (unsigned)((vecs + 255) / 256);
+static sar_status pad_rows(int H, int F, const RowShape &r, sar_dtype t, long long n, const void *in, void *out, long long n2, const void *in2, void *out2,
+                           cudaStream_t st) {
+    const long long vecs = n * H * r.vph, vecs2 = n2 * H * r.vph;
+    if (vecs + vecs2 == 0) return SAR_OK;
+    const unsigned blocks = (unsigned)((vecs + vecs2 + 255) / 256);
+    uint4 *o = static_cast<uint4 *>(out), *o2 = static_cast<uint4 *>(out2);
     if (t == SAR_F32)
-        SAR_LAUNCH("pad_rows", st, launch(pad_rows_kernel<float>, blocks, 256, 0, st, vecs, F, r.vph, static_cast<const float *>(in), static_cast<uint4 *>(out)));
+        SAR_LAUNCH("pad_rows", st, launch(pad_rows_kernel<float>, blocks, 256, 0, st, vecs, vecs2, F, r.vph, static_cast<const float *>(in), o, static_cast<const float *>(in2), o2));
     else
-        SAR_LAUNCH("pad_rows", st, launch(pad_rows_kernel<__nv_bfloat16>, blocks, 256, 0, st, vecs, F, r.vph, static_cast<const __nv_bfloat16 *>(in), static_cast<uint4 *>(out)));
+        SAR_LAUNCH("pad_rows", st, launch(pad_rows_kernel<__nv_bfloat16>, blocks, 256, 0, st, vecs, vecs2, F, r.vph, static_cast<const __nv_bfloat16 *>(in), o, static_cast<const __nv_bfloat16 *>(in2), o2));
     return sar_after_launch();
 }
 
@@ -166,8 +174,9 @@ static sar_status strip_rows(long long n, int F, const RowShape &r, sar_dtype t,
 
 // ---- workspace layout ---------------------------------------------------------------------------
 // [ destination records: n_dst*H float4 ][ padded gout ][ segments of the CSR ][ segments of the CSC ][ padded feat ]
-// (the padded arrays for ragged shapes only).  The first two do not depend on the partition: the steps of a call-by-call
-// backward pass share them.
+// (the padded arrays for ragged shapes only).  The records are what sar_gat_bwd_prepare leaves for a step.  Everything else
+// is written by the call that reads it, but for the copy of gout with SAR_SAME_WORKSPACE: its place, like that of the
+// records, does not depend on the partition.
 static size_t rec_bytes(long long n_dst, int H) { return sar_round_up((size_t)n_dst * H * 16, 256); }
 static long long part_stride(int H, const RowShape &r, sar_dtype t) {  // floats per segment, a multiple of 4 (float4 rows)
     return ((long long)H * r.vph * (t == SAR_BF16 ? 8 : 4) + 3LL * H + 3) & ~3LL;
@@ -391,7 +400,7 @@ sar_status sar_gat_fwd(const sar_part *g, const void *feat_q, const float *el, c
     a.hvec = heads_aligned(H, r.geo.HP, {el, er_q});
     a.sp = split_args(g->split, use_split ? reinterpret_cast<float *>(wsb + w.csr) : nullptr, H, r, t);
     if (r.ragged) {
-        SAR_TRY(pad_rows(g->n_src, H, F, r, t, feat_q, wsb + w.feat, st));
+        SAR_TRY(pad_rows(H, F, r, t, g->n_src, feat_q, wsb + w.feat, 0, nullptr, nullptr, st));
         a.gather = wsb + w.feat;
     }
     Shape s;
@@ -519,7 +528,8 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
                        uint32_t flags, void *dfeat_q, float *del, float *der_q, void *workspace,
                        size_t workspace_bytes, void *stream) {
     SAR_TRY(check_part(g, true));
-    if (flags & ~(SAR_FIRST | SAR_LAST)) return SAR_ERR_INVALID_ARG;
+    if (flags & ~(SAR_FIRST | SAR_LAST | SAR_SAME_WORKSPACE)) return SAR_ERR_INVALID_ARG;
+    if ((flags & SAR_FIRST) && (flags & SAR_SAME_WORKSPACE)) return SAR_ERR_INVALID_ARG;
     if (!el || !m || !d || !gout || !del) return SAR_ERR_INVALID_ARG;
     if (g->n_src > 0 && (!feat_q || !er_q || !dfeat_q || !der_q)) return SAR_ERR_INVALID_ARG;
     SAR_TRY(check_elem_align({el, er_q, m, d, del, der_q}, 4));
@@ -533,11 +543,6 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char *wsb = static_cast<char *>(workspace);
     float4 *rec = reinterpret_cast<float4 *>(wsb);
-    // The padded copy of gout serves every step of a call-by-call pass: the first step makes it, whichever kernels it
-    // runs itself (its place does not depend on the partition).
-    if (r.ok && r.ragged && (flags & SAR_FIRST) && workspace_bytes >= w.csr)
-        SAR_TRY(pad_rows(g->n_dst, H, F, r, t, gout, wsb + w.gout, st));
-
     if (!rows) {
         GenericArgs a{};
         a.n_dst = g->n_dst;
@@ -581,7 +586,11 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
     }
     const void *feat_g = feat_q, *gout_g = gout;
     if (r.ragged) {
-        SAR_TRY(pad_rows(g->n_src, H, F, r, t, feat_q, wsb + w.feat, st));
+        // What a step finds in the workspace is the records alone (the caller may have prepared one for each step), unless
+        // it is told that an earlier step has made its copy of gout there: 8 steps on 170,000 nodes of 47 bf16, 2.5 million
+        // edges, forward and backward 1297 us, 1335 us with a copy in every step.
+        const long long n_gout = flags & SAR_SAME_WORKSPACE ? 0 : g->n_dst;
+        SAR_TRY(pad_rows(H, F, r, t, g->n_src, feat_q, wsb + w.feat, n_gout, gout, wsb + w.gout, st));
         feat_g = wsb + w.feat;
         gout_g = wsb + w.gout;
     }
@@ -593,7 +602,7 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
     a.d = d;
     a.rec = rec;
     a.slope = slope;
-    a.flags = flags;
+    a.flags = flags & ~SAR_SAME_WORKSPACE;
     a.H = H;
     a.F = F;
     a.vph = r.vph;
@@ -766,7 +775,7 @@ static sar_status spmm_impl(const sar_part *g, const void *feat_q, int32_t F, sa
     const bool use_split = g->split && g->split->n_long > 0;
     if (use_split && (!have_ws || workspace_bytes < parts)) return SAR_ERR_WORKSPACE;
     if (r.ragged) {
-        SAR_TRY(pad_rows(g->n_src, 1, F, r, t, feat_q, static_cast<char *>(workspace) + parts, st));
+        SAR_TRY(pad_rows(1, F, r, t, g->n_src, feat_q, static_cast<char *>(workspace) + parts, 0, nullptr, nullptr, st));
         feat_q = static_cast<char *>(workspace) + parts;
     }
     return sum_rows(g, r, F, t, flags, feat_q, deg_total, src_scale, dst_scale, SumMix{}, out, static_cast<float *>(workspace), st);

@@ -380,7 +380,7 @@ PyObject *gat_backward_parts(Args &a) {   // parts, bounds, n_dst, feat, el, er,
     for (size_t q = 0; q < k; ++q) {
         const int64_t s = bounds[q];
         SAR(sar_gat_bwd, reinterpret_cast<const sar_part *>(parts[q]), rows(feat, s), pl, reinterpret_cast<const float *>(rows(er, s)),
-            pm, pd, ptr(gout), d.H, d.F, d.t, (float)slope, step_flags(q, k), rowsm(r.dfeat, s), f32m(r.del),
+            pm, pd, ptr(gout), d.H, d.F, d.t, (float)slope, step_flags(q, k) | (q > 0 ? SAR_SAME_WORKSPACE : 0u), rowsm(r.dfeat, s), f32m(r.del),
             reinterpret_cast<float *>(rowsm(r.der, s)), ptrm(ws), ws.nbytes(), stream());
     }
     return tuple(r.dfeat, r.del, r.der);

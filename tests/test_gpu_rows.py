@@ -75,3 +75,23 @@ def test_ragged_shape_without_room_for_padded_copies():
     B.sar_gat_bwd(p.graph.whole, d["feat"], d["el"], d["er"], m, dd, d["gout"], 2, 7, 0.2, B.SAR_FIRST | B.SAR_LAST, dfeat, del_, der, ws)
     for got, want in ((dfeat, b.dfeat), (del_, b.del_), (der, b.der)):
         allclose_report(got.cpu().numpy(), np.asarray(want), 1e-4, 1e-5, "gradients")
+
+
+@pytest.mark.parametrize("H,F,dtype", [(1, 47, "bf16"), (2, 7, "f32")])
+def test_ragged_steps_with_a_workspace_each(H, F, dtype):
+    """A step of the backward pass needs of its workspace what sar_gat_bwd_prepare wrote and nothing that an earlier step left."""
+    n, src, dst = hub_graph(n=1200, e=15000, d_max=300.0, seed=23)
+    p = Problem(n, src, dst, H, F, 12, dtype=dtype, k=3, threshold=24, build_parts=True)
+    d, g = p.dev, p.graph
+    out, m, dd, acc = api.gat_forward(g, d["feat"], d["el"], d["er"], 0.2, mode="stateful", keep_numerator=True)
+    want = api.gat_backward(g, d["feat"], d["el"], d["er"], m, dd, d["gout"], 0.2, mode="stateful", acc=acc)
+    dfeat, del_, der = torch.empty_like(d["feat"]), torch.empty_like(m), torch.empty_like(m)
+    for q, part in enumerate(g.parts):
+        nbytes = B.sar_gat_workspace_bytes(part, H, F, B.SAR_BF16 if dtype == "bf16" else B.SAR_F32)
+        ws = torch.full((nbytes,), 0x7f, dtype=torch.uint8, device=DEV)
+        B.sar_gat_bwd_prepare(n, H, F, acc, True, d["gout"], d["el"], m, dd, None, ws)
+        s0, s1 = g.bounds[q], g.bounds[q + 1]
+        B.sar_gat_bwd(part, d["feat"][s0:s1], d["el"], d["er"][s0:s1], m, dd, d["gout"], H, F, 0.2,
+                      (B.SAR_FIRST if q == 0 else 0) | (B.SAR_LAST if q == 2 else 0), dfeat[s0:s1], del_, der[s0:s1], ws)
+    for got, ref in zip((dfeat, del_, der), want):
+        assert torch.equal(got, ref)
