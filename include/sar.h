@@ -386,8 +386,13 @@ SAR_API sar_status sar_spmm_agg_scaled(const sar_part *g, const void *feat_q, in
  * out = X_iters.  parts: HOST array of k partitions (k <= SAR_MAX_PARTS) that together hold the graph, part q the sources
  * bounds[q] .. bounds[q + 1] (HOST bounds, bounds[0] = 0, bounds[k] = n_dst of every part).  x0, out: [n, F] of type t,
  * x0 != out; rows are accumulated in float32 and stored in type t between the steps, multiplied by src_scale (a source is
- * scaled once, where its row is stored, not on every edge).  workspace: sar_propagate_workspace_bytes, 256-byte aligned. */
+ * scaled once, where its row is stored, not on every edge).  workspace: 256-byte aligned; sar_propagate_workspace_bytes is
+ * enough wherever x0 and out lie, sar_propagate_workspace_bytes_at for these two pointers: with rows of whole 16-byte
+ * vectors and 16-byte aligned x0 and out one array of [n, F] (the other one that the steps alternate between is out), up
+ * to three otherwise. */
 SAR_API size_t sar_propagate_workspace_bytes(int32_t k, const sar_part *const *parts, int32_t F, sar_dtype t);
+SAR_API size_t sar_propagate_workspace_bytes_at(int32_t k, const sar_part *const *parts, const void *x0, int32_t F,
+                                                sar_dtype t, const void *out);
 SAR_API sar_status sar_propagate(int32_t k, const sar_part *const *parts, const int64_t *bounds, const void *x0, int32_t F,
                                  sar_dtype t, float alpha, int64_t iters, const float *src_scale, const float *dst_scale,
                                  void *out, void *workspace, size_t workspace_bytes, void *stream);

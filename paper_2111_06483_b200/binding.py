@@ -37,7 +37,7 @@ EXPORTS = [
     "sar_gat_storing_workspace_bytes", "sar_gat_fwd_storing", "sar_gat_bwd_storing", "sar_bn_combine_moments",
     "sar_bn_combine_sums", "sar_degree_order_workspace_bytes", "sar_degree_order", "sar_relabel", "sar_permute_rows", "sar_linear_project", "sar_linear_bwd_input_relu",
     "sar_graph_from_coo", "sar_plan_many_workspace_bytes", "sar_plan_count_many", "sar_plan_fill_many", "sar_gather_i64",
-    "sar_propagate_workspace_bytes", "sar_propagate",
+    "sar_propagate_workspace_bytes", "sar_propagate_workspace_bytes_at", "sar_propagate",
 ]
 
 
@@ -81,7 +81,7 @@ def lib() -> ctypes.CDLL:
         for name in ("sar_graph_workspace_bytes", "sar_gat_workspace_bytes", "sar_spmm_workspace_bytes",
                      "sar_gat_stack_arena_bytes", "sar_gat_bwd_noalloc_limit", "sar_gat_project_workspace_bytes",
                      "sar_bn_workspace_bytes", "sar_linear_workspace_bytes", "sar_gat_storing_workspace_bytes",
-                     "sar_degree_order_workspace_bytes", "sar_plan_many_workspace_bytes", "sar_propagate_workspace_bytes"):
+                     "sar_degree_order_workspace_bytes", "sar_plan_many_workspace_bytes", "sar_propagate_workspace_bytes", "sar_propagate_workspace_bytes_at"):
             getattr(L, name).restype = c_size_t
         _lib = L
     return _lib
@@ -791,6 +791,11 @@ def _part_array(parts: Sequence[Part]):
 
 def sar_propagate_workspace_bytes(parts: Sequence[Part], F: int, dtype: int) -> int:
     return int(lib().sar_propagate_workspace_bytes(c_int32(len(parts)), _part_array(parts), c_int32(F), ctypes.c_int(dtype)))
+
+
+def sar_propagate_workspace_bytes_at(parts: Sequence[Part], x0: torch.Tensor, dtype: int, out: torch.Tensor) -> int:
+    return int(lib().sar_propagate_workspace_bytes_at(c_int32(len(parts)), _part_array(parts), _ptr(x0), c_int32(x0.shape[1]),
+                                                      ctypes.c_int(dtype), _ptr(out)))
 
 
 def sar_propagate(parts: Sequence[Part], bounds: Sequence[int], x0: torch.Tensor, alpha: float, iters: int,

@@ -794,7 +794,13 @@ sar_status sar_spmm_agg_scaled(const sar_part *g, const void *feat_q, int32_t F,
     return spmm_impl(g, feat_q, F, t, flags, nullptr, src_scale, dst_scale, out, workspace, workspace_bytes, stream);
 }
 
-// Workspace of a propagation: [ segments of the long rows ][ two arrays of padded rows ][ x0 with padded rows ]
+// Workspace of a propagation: [ segments of the long rows ][ the array a step reads while the next one is written ], and
+// where rows are ragged or arrays misaligned [ the latter, in place of out ][ x0 with padded rows ].
+static bool propagate_reads_x0(const RowShape &r, const void *x0) { return !r.ragged && all16({x0}); }
+static bool propagate_writes_out(const RowShape &r, const void *out) { return !r.ragged && all16({out}); }
+static int propagate_arrays(const RowShape &r, const void *x0, const void *out) {
+    return 1 + (propagate_writes_out(r, out) ? 0 : 1) + (propagate_reads_x0(r, x0) ? 0 : 1);
+}
 static size_t propagate_parts(int32_t k, const sar_part *const *parts, const RowShape &r, sar_dtype t) {
     size_t b = 0;
     for (int32_t q = 0; q < k; ++q) {
@@ -803,12 +809,18 @@ static size_t propagate_parts(int32_t k, const sar_part *const *parts, const Row
     }
     return b;
 }
-size_t sar_propagate_workspace_bytes(int32_t k, const sar_part *const *parts, int32_t F, sar_dtype t) {
+static size_t propagate_bytes(int32_t k, const sar_part *const *parts, int32_t F, sar_dtype t, bool any, const void *x0, const void *out) {
     if (k < 1 || !parts || F < 1) return 0;
     for (int32_t q = 0; q < k; ++q)
         if (!parts[q]) return 0;
     const RowShape r = sum_shape(F, t);
-    return propagate_parts(k, parts, r, t) + 3 * sar_round_up((size_t)parts[0]->n_dst * r.row_bytes, 256) + 256;
+    return propagate_parts(k, parts, r, t) + (any ? 3 : propagate_arrays(r, x0, out)) * sar_round_up((size_t)parts[0]->n_dst * r.row_bytes, 256) + 256;
+}
+size_t sar_propagate_workspace_bytes(int32_t k, const sar_part *const *parts, int32_t F, sar_dtype t) {
+    return propagate_bytes(k, parts, F, t, true, nullptr, nullptr);
+}
+size_t sar_propagate_workspace_bytes_at(int32_t k, const sar_part *const *parts, const void *x0, int32_t F, sar_dtype t, const void *out) {
+    return propagate_bytes(k, parts, F, t, false, x0, out);
 }
 
 sar_status sar_propagate(int32_t k, const sar_part *const *parts, const int64_t *bounds, const void *x0, int32_t F, sar_dtype t, float alpha,
@@ -831,19 +843,22 @@ sar_status sar_propagate(int32_t k, const sar_part *const *parts, const int64_t 
     const int32_t Fp = (int32_t)(ragged.row_bytes / sar_elem_size(t));
     const RowShape r = sum_shape(Fp, t);   // the same rows, every vector of them whole
     const size_t array = sar_round_up((size_t)n * r.row_bytes, 256), seg = propagate_parts(k, parts, r, t);
-    if (!workspace || !sar_aligned(workspace, 256) || workspace_bytes < seg + 3 * array) return SAR_ERR_WORKSPACE;
-    char *ws = static_cast<char *>(workspace), *y[2] = {ws + seg, ws + seg + array};
-    const bool in_place = !ragged.ragged && all16({x0});                  // x0 can be read as it lies
-    const bool out_direct = !ragged.ragged && all16({out});
-    const void *x0p = in_place ? x0 : ws + seg + 2 * array;
+    const int arrays = propagate_arrays(ragged, x0, out);
+    if (!workspace || !sar_aligned(workspace, 256) || workspace_bytes < seg + arrays * array) return SAR_ERR_WORKSPACE;
+    const bool in_place = propagate_reads_x0(ragged, x0), out_direct = propagate_writes_out(ragged, out);
+    char *ws = static_cast<char *>(workspace);
+    void *y[2] = {out_direct ? out : ws + seg + array, ws + seg};         // written in turn; the last step writes y[0]
+    char *padded = in_place ? nullptr : ws + seg + (arrays - 1) * array;
+    const void *x0p = in_place ? x0 : padded;
     const void *cur = x0p;
     if (!in_place || src_scale) {
-        if (src_scale) cur = y[0];
-        SAR_TRY(propagate_start(n, F, r, t, x0, src_scale, in_place ? nullptr : ws + seg + 2 * array, src_scale ? y[0] : nullptr, st));
+        void *scaled = src_scale ? y[iters & 1] : nullptr;
+        if (src_scale) cur = scaled;
+        SAR_TRY(propagate_start(n, F, r, t, x0, src_scale, padded, scaled, st));
     }
     for (int64_t i = 0; i < iters; ++i) {
         const bool end = i + 1 == iters;
-        void *nxt = end && out_direct ? out : y[(i + 1) & 1];
+        void *nxt = y[(iters - 1 - i) & 1];
         const SumMix mix{x0p, 1.f - alpha, alpha, end ? nullptr : src_scale};
         for (int32_t q = 0; q < k; ++q)
             SAR_TRY(sum_rows(parts[q], r, Fp, t, (q == 0 ? SAR_FIRST : 0u) | (q + 1 == k ? SAR_LAST : 0u),

@@ -21,7 +21,7 @@ namespace {
 #define SAR_TABLE(X)                                                                                                   \
     X(sar_status_string) X(sar_gat_workspace_bytes) X(sar_gat_fwd) X(sar_gat_fwd_fused) X(sar_gat_bwd_prepare)         \
     X(sar_gat_bwd) X(sar_gat_bwd_fused) X(sar_spmm_agg) X(sar_spmm_workspace_bytes) X(sar_spmm_agg_scaled)             \
-    X(sar_propagate) X(sar_propagate_workspace_bytes) X(sar_relu) X(sar_gat_project) X(sar_gat_project_bwd) X(sar_gat_project_workspace_bytes)              \
+    X(sar_propagate) X(sar_propagate_workspace_bytes_at) X(sar_relu) X(sar_gat_project) X(sar_gat_project_bwd) X(sar_gat_project_workspace_bytes)              \
     X(sar_linear_workspace_bytes) X(sar_linear) X(sar_linear_accumulate) X(sar_linear_project)                         \
     X(sar_linear_bwd_input) X(sar_linear_bwd_input_relu) X(sar_linear_bwd_weight) X(sar_bn_workspace_bytes)            \
     X(sar_bn_stats) X(sar_bn_rstd) X(sar_bn_apply) X(sar_bn_bwd_stats) X(sar_bn_bwd_apply)                             \
@@ -448,7 +448,7 @@ PyObject *propagate(Args &a) {   // parts, bounds, x0, alpha, iters, src_scale, 
     const float *ss = f32(src, ps[0]->n_dst), *ds = f32(dst, ps[0]->n_dst);
     const int32_t k = (int32_t)ps.size(), F = (int32_t)x0.size(1);
     const at::Tensor out = empty(x0.sizes(), x0.scalar_type(), x0);
-    const at::Tensor ws = bytes(L.sar_propagate_workspace_bytes(k, ps.data(), F, code(x0)), x0);
+    const at::Tensor ws = bytes(L.sar_propagate_workspace_bytes_at(k, ps.data(), ptr(x0), F, code(x0), ptr(out)), x0);
     SAR(sar_propagate, k, ps.data(), bounds.data(), ptr(x0), F, code(x0), (float)alpha, iters, ss, ds, ptrm(out), ptrm(ws), ws.nbytes(), stream());
     return wrap(out);
 }

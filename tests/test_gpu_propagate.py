@@ -14,7 +14,8 @@ DEV = "cuda"
 
 @pytest.mark.parametrize("n,F,dtype,k,iters,scaled,shift", [
     (1, 1, "f32", 1, 1, True, 0), (900, 3, "f32", 1, 3, True, 0), (900, 47, "f32", 4, 2, False, 0), (900, 300, "f32", 1, 1, True, 0),
-    (900, 16, "f32", 1, 2, True, 1), (900, 16, "f32", 3, 1, False, 0), (900, 9, "bf16", 2, 2, True, 0), (70_000, 47, "f32", 1, 3, True, 0),
+    (900, 16, "f32", 1, 2, True, 1), (900, 16, "f32", 3, 3, True, 1), (900, 16, "f32", 3, 1, False, 0), (900, 16, "f32", 1, 1, True, 0),
+    (900, 16, "f32", 2, 4, False, 0), (900, 16, "f32", 2, 3, True, 0), (900, 9, "bf16", 2, 2, True, 0), (70_000, 47, "f32", 1, 3, True, 0),
     (70_000, 48, "f32", 3, 2, True, 0), (70_000, 100, "bf16", 1, 2, False, 0)])
 def test_propagation_in_one_call(n, F, dtype, k, iters, scaled, shift):
     tdt = torch.float32 if dtype == "f32" else torch.bfloat16
@@ -38,3 +39,40 @@ def test_propagation_in_one_call(n, F, dtype, k, iters, scaled, shift):
     tol = dict(rtol=1e-5, atol=1e-5) if dtype == "f32" else dict(rtol=2e-2, atol=2e-2)
     allclose_report(got.double().cpu().numpy(), want.numpy(), what="propagation", **tol)
     assert np.isfinite(got.float().cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("F,shift_in,shift_out,arrays", [(16, 0, 0, 1), (16, 1, 0, 2), (16, 0, 1, 2), (16, 1, 1, 3), (15, 0, 0, 3)])
+@pytest.mark.parametrize("iters,scaled", [(1, True), (2, True), (3, False)])
+def test_workspace_for_the_pointers_given(F, shift_in, shift_out, arrays, iters, scaled):
+    """The workspace asked for holds no array that the call does not use, and the call stays within it."""
+    from paper_2111_06483_b200 import binding as B
+    n = 700
+    gen = torch.Generator().manual_seed(F)
+    src, dst = (torch.randint(0, n, (5 * n,), generator=gen, dtype=torch.int32).to(DEV) for _ in range(2))
+    g = api.Graph.from_coo(n, src, dst)
+    x, out = (torch.empty(n * F + s, device=DEV)[s:].view(n, F) for s in (shift_in, shift_out))
+    x.copy_(torch.randn((n, F), generator=gen))
+    s = torch.rand(n, device=DEV) if scaled else None
+    nbytes = B.sar_propagate_workspace_bytes_at([g.whole], x, B.SAR_F32, out)
+    assert nbytes == arrays * ((n * ((F + 3) // 4) * 16 + 255) // 256 * 256) + 256
+    assert B.sar_propagate_workspace_bytes([g.whole], F, B.SAR_F32) >= nbytes
+    ws = torch.full((nbytes + 4096,), 0xA5, dtype=torch.uint8, device=DEV)
+    B.sar_propagate([g.whole], g.bounds, x, 0.7, iters, s, None, out, ws[:nbytes])
+    assert torch.equal(out, api.propagate(g, x.clone(), 0.7, iters, s))
+    assert bool((ws[nbytes:] == 0xA5).all())
+    with pytest.raises(B.SarError):
+        B.sar_propagate([g.whole], g.bounds, x, 0.7, iters, s, None, out, ws[:nbytes - 512])
+
+
+def test_propagation_takes_one_array_beside_its_result():
+    n, F = 200_000, 64
+    src, dst = (torch.randint(0, n, (n,), device=DEV, dtype=torch.int32) for _ in range(2))
+    g = api.Graph.from_coo(n, src, dst)
+    x = torch.randn(n, F, device=DEV)
+    api.propagate(g, x, 0.5, 2)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    torch.cuda.reset_peak_memory_stats()
+    before = torch.cuda.memory_allocated()
+    api.propagate(g, x, 0.5, 3)
+    assert torch.cuda.max_memory_allocated() - before < 2.1 * x.nbytes
