@@ -641,17 +641,9 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
                 SAR_TRY(t == SAR_F32 ? lean_bwd_dst_f32(s, la, g->nnz, st) : lean_bwd_dst_bf16(s, la, g->nnz, st));
             else
                 SAR_TRY(t == SAR_F32 ? lean_bwd_dst_part_f32(s, la, g->nnz, st) : lean_bwd_dst_part_bf16(s, la, g->nnz, st));
-        } else if (use_span(s, g->n_src) || short_rows(s, g->n_dst, g->nnz, true, !whole)) {
-            a.n_rows = 0;   // the segments first, the rows beside them
-            if (a.sp.n_seg > 0) {
-                if (whole)
-                    SAR_TRY(t == SAR_F32 ? rows_dst_f32(a, r.geo, g->nnz, st) : rows_dst_bf16(a, r.geo, g->nnz, st));
-                else
-                    SAR_TRY(t == SAR_F32 ? rows_dst_part_f32(a, r.geo, g->nnz, st) : rows_dst_part_bf16(a, r.geo, g->nnz, st));
-            }
-            a.n_rows = g->n_dst;
+        } else if (use_span(s, g->n_src) || short_rows(s, g->n_dst, g->nnz, true, !whole))
             SAR_TRY(span_dst(s, a, g->nnz, !whole, st));
-        } else if (whole)
+        else if (whole)
             SAR_TRY(t == SAR_F32 ? rows_dst_f32(a, r.geo, g->nnz, st) : rows_dst_bf16(a, r.geo, g->nnz, st));
         else
             SAR_TRY(t == SAR_F32 ? rows_dst_part_f32(a, r.geo, g->nnz, st) : rows_dst_part_bf16(a, r.geo, g->nnz, st));
@@ -682,13 +674,10 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
             la.sp = a.sp;
             la.sp.threshold = g->t_split->threshold;
             SAR_TRY(t == SAR_F32 ? lean_bwd_src_f32(s, la, g->nnz, st) : lean_bwd_src_bf16(s, la, g->nnz, st));
-        } else {
-            const bool span = use_span(s, g->n_dst) || short_rows(s, g->n_src, g->nnz, true, !whole);
-            if (span) a.n_rows = 0;   // the segments first, the rows beside them
+        } else if (use_span(s, g->n_dst) || short_rows(s, g->n_src, g->nnz, true, !whole))
+            SAR_TRY(span_src(s, a, g->nnz, st));
+        else
             SAR_TRY(t == SAR_F32 ? rows_src_f32(a, r.geo, g->nnz, st) : rows_src_bf16(a, r.geo, g->nnz, st));
-            a.n_rows = g->n_src;
-            if (span) SAR_TRY(span_src(s, a, g->nnz, st));
-        }
         if (a.sp.n_long > 0) SAR_TRY(rows_src_merge(a, t, st));
     }
     return SAR_OK;

@@ -1,38 +1,22 @@
 // Launches that overlap the end of the launch before them (internal).
 //
 // A pass over a small graph is a chain of kernels of 3 to 5 us, and between two of them lies 1.5 us in which the second is
-// only being set up.  So every kernel of the aggregation and of the streaming steps around it is launched with programmatic stream serialisation and begins
-// with after_predecessor(): its blocks may be placed as soon as all blocks of the launch before run, wait there until that
-// launch has ended and its writes are visible, and then let the next launch be placed in turn.  Nothing is read or
-// written before the wait, so the order of the stream holds for every pair of launches, whoever issued them; a launch that
-// follows another kind of work, or carries the attribute without need, simply does not overlap.  2,000 nodes, 22,000 edges,
-// forward and backward (three launches): 18.6 -> 14.2 us.
-//
-// The segments of the long rows and the other rows are independent launches of one pass.  The segments go first (a segment
-// is the longest chain of work in the pass) and the rows launch, which follows with beside_segments(), does not wait
-// for their end: it is let in when all of their blocks run, that is, when they have passed their own wait, and fills
-// whatever they leave free.  Its last block waits for the segments' end, so that whatever follows the rows launch
-// follows both.  With the segments after the rows, a partition step over 100,000 rows and 250,000 edges spent 20 us of 80
-// on a handful of segments with the rest of the chip idle.
+// only being set up.  So every kernel of the aggregation and of the streaming steps around it is launched with programmatic
+// stream serialisation and begins with after_predecessor(): its blocks may be placed as soon as all blocks of the launch
+// before run, wait there until that launch has ended and its writes are visible, and then let the next launch be placed in
+// turn.  Every block waits, and nothing is read or written before: that is what makes the writes of a launch visible to
+// the next one and, since that one ends only after its own wait, to all that follow.  So the order of the stream holds
+// for every pair of launches, whoever issued them; a launch that follows another kind of work, or carries the attribute
+// without need, simply does not overlap.  2,000 nodes, 22,000 edges, forward and backward (three launches): 18.6 -> 14.2 us.
 #pragma once
 
 #include "sar_common.cuh"
 
 namespace sar {
 
-__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-__device__ __forceinline__ void let_successor_in() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void after_predecessor() {
-    wait_for_predecessor();
-    let_successor_in();
-}
-// the rows launch of a pass: begin, and end of every block
-__device__ __forceinline__ void beside_segments(bool segments) {
-    if (!segments) wait_for_predecessor();
-    let_successor_in();
-}
-__device__ __forceinline__ void rows_end(bool segments) {
-    if (segments && blockIdx.x == gridDim.x - 1) wait_for_predecessor();
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
 // One grid that strides over its array: its blocks have to be spread evenly, and placed into what the launch before leaves

@@ -99,4 +99,29 @@ static inline int lean_rows_per_span(long long n_rows, long long nnz, int cap, i
     return (int)R;
 }
 
+// What the blocks of a launch work on: a segment of a long row each, a span of the other rows each, or both, the segments
+// first.  A segment is the longest chain of work in a pass: where there are few, the spans fill what they leave free (a
+// partition step's pass over 100,000 rows and 250,000 edges: 60 us, and 80 with the segments in a launch of their own).
+// Where the segments alone fill every SM several times over, one launch after the other costs their tail and no more, and
+// the segments run with the shared memory that they need themselves, more of them at a time.  Forward + backward, one launch
+// against two: 4,666 segments (300,000 nodes, 8 heads of 32, bf16) 0.92 against 1.00 ms; 12,000 (500,000 nodes, 4 heads of
+// 32) 1.09 against 1.11; 23,000 (a million nodes) 1.984 against 1.976; 30,000 (2 million, 4 heads of 16, float32) 2.57
+// against 2.60; 47,000 (200,000 nodes, 20 million edges, 8 heads of 32) 3.82 against 3.78; 130,000 (a million nodes, 4 heads
+// of 64) 11.5 against 11.0; 575,000 (200 edges per node, 8 heads of 32) 42.7 against 41.6 ms.
+enum { kLeanBoth = 0, kLeanSegments = 1, kLeanRows = 2 };
+constexpr long long kLeanSegmentsAlone = 148 * 256;
+template <typename LR, typename LS, typename K, typename A>
+static sar_status launch_lean(const char *name, const char *seg_name, K both, K segments, K rows, const A &a, cudaStream_t st) {
+    const long long spans = (a.n_rows + a.R - 1) / a.R, n_seg = a.sp.n_seg;
+    auto go = [&](const char *what, K kern, size_t smem, long long blocks) -> sar_status {
+        if (blocks <= 0) return SAR_OK;
+        SAR_TRY(ensure_smem(kern, smem));
+        SAR_LAUNCH(what, st, launch(kern, (unsigned)blocks, 32, smem, st, a));
+        return sar_after_launch();
+    };
+    if (n_seg > 0 && n_seg < kLeanSegmentsAlone) return go(name, both, LR::total > LS::total ? LR::total : LS::total, n_seg + spans);
+    SAR_TRY(go(seg_name, segments, LS::total, n_seg));
+    return go(name, rows, LR::total, spans);
+}
+
 }  // namespace sar

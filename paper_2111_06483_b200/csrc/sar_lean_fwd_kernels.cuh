@@ -59,8 +59,8 @@ struct LeanFwdLayout {
     static constexpr int total = rowst + ((PART && !SEG) ? kLeanPartStagedFwd * SROWB : 0);
 };
 
-template <typename T, int G, int V, int H, bool SEG, int CAP, int P, int NS, int MINB, bool PART = false, bool FIRST = false>
-__global__ void __launch_bounds__(32, MINB) lean_fwd_kernel(const LeanArgs a) {
+template <typename T, int G, int V, int H, bool SEG, int CAP, int P, int NS, bool PART = false, bool FIRST = false>
+__device__ __forceinline__ void lean_fwd_warp(const LeanArgs &a, long long item) {
     static_assert(!(PART && SEG), "the segments of a partition step run the whole-graph segment kernel");
     static_assert(PART || !FIRST, "FIRST is the first partition step");
     using L = LeanFwdLayout<G, V, H, SEG, CAP, P, NS, PART, Elem<T>::EPV>;
@@ -75,8 +75,6 @@ __global__ void __launch_bounds__(32, MINB) lean_fwd_kernel(const LeanArgs a) {
     static_assert((1 << LGNVEC) == NVEC, "row geometry");
     static_assert(P <= 32 && 32 % P == 0 && (SPS == 4 || SPS == 8), "stage geometry: four or eight slots per stage");
     static_assert(ITEMS <= 64 && 32 % H == 0, "at most two (position, head) pairs per lane, both of one head");
-    if constexpr (SEG) after_predecessor();
-    else beside_segments(a.sp.n_seg > 0);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const unsigned sbase = (unsigned)__cvta_generic_to_shared(smem_raw);
     const unsigned ring_s = sbase + L::ring, rec_s = sbase + L::rec, w_s = sbase + L::w, offs_s = sbase + L::offs;
@@ -93,7 +91,6 @@ __global__ void __launch_bounds__(32, MINB) lean_fwd_kernel(const LeanArgs a) {
     auto perm = [](int q) { return (q / P) * P + ((q % P) % EPW) * SPS + (q % P) / EPW; };
 
     // ---- which rows ---------------------------------------------------------------------------
-    const long long item = blockIdx.x;
     long long row0, eb = 0, ee = 0;
     int nrows;
     bool excluded = false;
@@ -111,7 +108,6 @@ __global__ void __launch_bounds__(32, MINB) lean_fwd_kernel(const LeanArgs a) {
             excluded = ee - eb > a.sp.threshold;
         }
     } else {
-        if (item >= a.sp.n_seg) return;
         int lo = 0, hi = a.sp.n_long;
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
@@ -659,7 +655,14 @@ __global__ void __launch_bounds__(32, MINB) lean_fwd_kernel(const LeanArgs a) {
         }
         r = r2;
     }
-    if constexpr (!SEG) rows_end(a.sp.n_seg > 0);
+}
+
+template <typename T, int G, int V, int H, int CAP, int P, int NS, int MINB, int ITEMS, bool PART = false, bool FIRST = false>
+__global__ void __launch_bounds__(32, MINB) lean_fwd_kernel(const LeanArgs a) {
+    after_predecessor();
+    const long long item = blockIdx.x;
+    if (ITEMS == kLeanSegments || (ITEMS == kLeanBoth && item < a.sp.n_seg)) lean_fwd_warp<T, G, V, H, true, CAP, P, NS>(a, item);
+    else lean_fwd_warp<T, G, V, H, false, CAP, P, NS, PART, FIRST>(a, ITEMS == kLeanBoth ? item - a.sp.n_seg : item);
 }
 
 // ---- launcher ------------------------------------------------------------------------------------------------------
@@ -670,24 +673,13 @@ static sar_status launch_lean_fwd(LeanArgs a, long long nnz, cudaStream_t st) {
     using LR = LeanFwdLayout<G, V, H, false, kLeanCap, P, NS>;
     using LS = LeanFwdLayout<G, V, H, true, kLeanCap, P, NS>;
     a.R = lean_rows_per_span(a.n_rows, nnz, kLeanCap);
-    const long long spans = (a.n_rows + a.R - 1) / a.R;
-    if (a.sp.n_seg > 0) {
-        auto kern = lean_fwd_kernel<T, G, V, H, true, kLeanCap, P, NS, kLeanMinBlocks>;
-        SAR_TRY(ensure_smem(kern, LS::total));
-        SAR_LAUNCH("gat_fwd_seg", st, launch(kern, (unsigned)a.sp.n_seg, 32, LS::total, st, a));
-        SAR_TRY(sar_after_launch());
-    }
-    if (spans > 0) {
-        auto kern = lean_fwd_kernel<T, G, V, H, false, kLeanCap, P, NS, kLeanMinBlocks>;
-        SAR_TRY(ensure_smem(kern, LR::total));
-        SAR_LAUNCH("gat_fwd", st, launch(kern, (unsigned)spans, 32, LR::total, st, a));
-        SAR_TRY(sar_after_launch());
-    }
-    return SAR_OK;
+    return launch_lean<LR, LS>("gat_fwd", "gat_fwd_seg", lean_fwd_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocks, kLeanBoth>,
+                               lean_fwd_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocks, kLeanSegments>,
+                               lean_fwd_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocks, kLeanRows>, a, st);
 }
 
-// A partition step of a call-by-call forward pass: the rows launch is the PART variant, the segments of the long
-// rows run the whole-graph segment kernel (same partial records; the merge launch is the caller's and folds the state).
+// A partition step of a call-by-call forward pass: the rows are the PART variant, the segments of the long rows are the
+// whole graph's (same partial records; the merge launch is the caller's and folds the state).
 template <typename T, int G, int V, int H>
 static sar_status launch_lean_fwd_part(LeanArgs a, long long nnz, cudaStream_t st) {
     constexpr int NS = 2;
@@ -695,22 +687,12 @@ static sar_status launch_lean_fwd_part(LeanArgs a, long long nnz, cudaStream_t s
     using LR = LeanFwdLayout<G, V, H, false, kLeanCap, P, NS, true, Elem<T>::EPV>;
     using LS = LeanFwdLayout<G, V, H, true, kLeanCap, P, NS>;
     a.R = lean_rows_per_span(a.n_rows, nnz, kLeanCap, kLeanPartRows);
-    const long long spans = (a.n_rows + a.R - 1) / a.R;
-    if (a.sp.n_seg > 0) {
-        auto kern = lean_fwd_kernel<T, G, V, H, true, kLeanCap, P, NS, kLeanMinBlocks>;
-        SAR_TRY(ensure_smem(kern, LS::total));
-        SAR_LAUNCH("gat_fwd_seg", st, launch(kern, (unsigned)a.sp.n_seg, 32, LS::total, st, a));
-        SAR_TRY(sar_after_launch());
-    }
-    if (spans > 0) {
-        auto kern = a.first ? lean_fwd_kernel<T, G, V, H, false, kLeanCap, P, NS, kLeanMinBlocksPart, true, true>
-                            : lean_fwd_kernel<T, G, V, H, false, kLeanCap, P, NS, kLeanMinBlocksPart, true, false>;
-        SAR_TRY(ensure_smem(lean_fwd_kernel<T, G, V, H, false, kLeanCap, P, NS, kLeanMinBlocksPart, true, true>, LR::total));
-        SAR_TRY(ensure_smem(lean_fwd_kernel<T, G, V, H, false, kLeanCap, P, NS, kLeanMinBlocksPart, true, false>, LR::total));
-        SAR_LAUNCH("gat_fwd", st, launch(kern, (unsigned)spans, 32, LR::total, st, a));
-        SAR_TRY(sar_after_launch());
-    }
-    return SAR_OK;
+    auto segments = lean_fwd_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocks, kLeanSegments>;
+    if (a.first)
+        return launch_lean<LR, LS>("gat_fwd", "gat_fwd_seg", lean_fwd_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocksPart, kLeanBoth, true, true>, segments,
+                                   lean_fwd_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocksPart, kLeanRows, true, true>, a, st);
+    return launch_lean<LR, LS>("gat_fwd", "gat_fwd_seg", lean_fwd_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocksPart, kLeanBoth, true, false>, segments,
+                               lean_fwd_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocksPart, kLeanRows, true, false>, a, st);
 }
 
 template <typename T>

@@ -42,8 +42,8 @@ struct LeanSrcLayout {
     static constexpr int total = endm + ((MASKW * 4 + 15) / 16) * 16;
 };
 
-template <typename T, int G, int V, int H, bool SEG, int CAP, int P, int NS, int MINB>
-__global__ void __launch_bounds__(32, MINB) lean_src_kernel(const LeanSrcArgs a) {
+template <typename T, int G, int V, int H, bool SEG, int CAP, int P, int NS>
+__device__ __forceinline__ void lean_src_warp(const LeanSrcArgs a, long long item) {
     using L = LeanSrcLayout<G, V, H, SEG, CAP, P, NS>;
     constexpr int EPV = Elem<T>::EPV, NP = EPV / 2;
     constexpr int EPW = L::EPW, ROWB = L::ROWB, STAGE = L::STAGE;
@@ -55,8 +55,6 @@ __global__ void __launch_bounds__(32, MINB) lean_src_kernel(const LeanSrcArgs a)
     static_assert((1 << LGNVEC) == NVEC, "row geometry");
     static_assert(P <= 32 && 32 % P == 0 && (SPS == 4 || SPS == 8), "stage geometry: four or eight slots per stage");
     static_assert(ITEMS <= 64, "at most two (position, head) pairs per lane");
-    if constexpr (SEG) after_predecessor();
-    else beside_segments(a.sp.n_seg > 0);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const unsigned sbase = (unsigned)__cvta_generic_to_shared(smem_raw);
     const unsigned ring_s = sbase + L::ring, rec_s = sbase + L::rec, w_s = sbase + L::w, offs_s = sbase + L::offs;
@@ -69,7 +67,6 @@ __global__ void __launch_bounds__(32, MINB) lean_src_kernel(const LeanSrcArgs a)
     auto perm = [](int q) { return (q / P) * P + ((q % P) % EPW) * SPS + (q % P) / EPW; };
 
     // ---- which rows ---------------------------------------------------------------------------
-    const long long item = blockIdx.x;
     long long row0, eb = 0, ee = 0;
     int nrows;
     bool excluded = false;
@@ -87,7 +84,6 @@ __global__ void __launch_bounds__(32, MINB) lean_src_kernel(const LeanSrcArgs a)
             excluded = ee - eb > a.sp.threshold;
         }
     } else {
-        if (item >= a.sp.n_seg) return;
         int lo = 0, hi = a.sp.n_long;
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
@@ -438,7 +434,14 @@ __global__ void __launch_bounds__(32, MINB) lean_src_kernel(const LeanSrcArgs a)
         }
         r = r2;
     }
-    if constexpr (!SEG) rows_end(a.sp.n_seg > 0);
+}
+
+template <typename T, int G, int V, int H, int CAP, int P, int NS, int MINB, int ITEMS>
+__global__ void __launch_bounds__(32, MINB) lean_src_kernel(const LeanSrcArgs a) {
+    after_predecessor();
+    const long long item = blockIdx.x;
+    if (ITEMS == kLeanSegments || (ITEMS == kLeanBoth && item < a.sp.n_seg)) lean_src_warp<T, G, V, H, true, CAP, P, NS>(a, item);
+    else lean_src_warp<T, G, V, H, false, CAP, P, NS>(a, ITEMS == kLeanBoth ? item - a.sp.n_seg : item);
 }
 
 // ---- launcher ------------------------------------------------------------------------------------------------------
@@ -449,20 +452,9 @@ static sar_status launch_lean_src(LeanSrcArgs a, long long nnz, cudaStream_t st)
     using LR = LeanSrcLayout<G, V, H, false, kLeanCap, P, NS>;
     using LS = LeanSrcLayout<G, V, H, true, kLeanCap, P, NS>;
     a.R = lean_rows_per_span(a.n_rows, nnz, kLeanCap);
-    const long long spans = (a.n_rows + a.R - 1) / a.R;
-    if (a.sp.n_seg > 0) {
-        auto kern = lean_src_kernel<T, G, V, H, true, kLeanCap, P, NS, kLeanMinBlocks>;
-        SAR_TRY(ensure_smem(kern, LS::total));
-        SAR_LAUNCH("gat_bwd_src_seg", st, launch(kern, (unsigned)a.sp.n_seg, 32, LS::total, st, a));
-        SAR_TRY(sar_after_launch());
-    }
-    if (spans > 0) {
-        auto kern = lean_src_kernel<T, G, V, H, false, kLeanCap, P, NS, kLeanMinBlocksBwdRows>;
-        SAR_TRY(ensure_smem(kern, LR::total));
-        SAR_LAUNCH("gat_bwd_src", st, launch(kern, (unsigned)spans, 32, LR::total, st, a));
-        SAR_TRY(sar_after_launch());
-    }
-    return SAR_OK;
+    return launch_lean<LR, LS>("gat_bwd_src", "gat_bwd_src_seg", lean_src_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocksBwdRows, kLeanBoth>,
+                               lean_src_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocks, kLeanSegments>,
+                               lean_src_kernel<T, G, V, H, kLeanCap, P, NS, kLeanMinBlocksBwdRows, kLeanRows>, a, st);
 }
 
 template <typename T>

@@ -8,7 +8,6 @@ namespace sar {
 
 // ---- span kernels ---------------------------------------------------------------------------------
 constexpr int kCapFwd = 256, kCapDst = 256, kCapSrc = 192, kCapSum = 256;
-constexpr int kCapSeg = 128;  // capacity of the segment launches (segments hold at most the plan threshold)
 constexpr int kMinBlocksFwd = 24, kMinBlocksBwd = 20;  // resident blocks per SM the register budget is cut for
 constexpr size_t kStageBytes = 16 * 1024;              // shared memory a partition step may spend on the rows' own data
 
@@ -22,17 +21,9 @@ static int rows_per_span(long long n_rows, long long nnz, int cap) {
     return R;
 }
 
-// Launches span_kernel<MODE> over the rows (mode 0) and, with a long-row plan, over the segments (mode 1; the backward
-// passes' segments are the caller's).  The merge launch is the caller's.
+// Launches span_kernel<MODE> over the segments of the long rows and the spans of the others.  The merge launch is the caller's.
 template <typename T, int G, int V, int S, int MODE, int CAP, int MINB>
-static sar_status launch_span(SpanArgs a, long long nnz, const char *name, const char *seg_name, cudaStream_t st) {
-    // The segment launch never stages more than `threshold` edges at a time: when that fits the small
-    // capacity it runs the instantiation with the smaller shared-memory footprint (more resident warps).
-    constexpr int CAP_SEG = CAP < kCapSeg ? CAP : kCapSeg;
-    auto kern = span_kernel<T, G, V, S, MODE, CAP, MINB>;
-    const size_t smem = (size_t)kSpanWarps * span_layout<MODE>(a.g.Hp, V, CAP, S, 32 / G).total;
-    SAR_TRY(ensure_smem(kern, smem));
-    a.mode = 0;
+static sar_status launch_span(SpanArgs a, long long nnz, const char *name, cudaStream_t st) {
     constexpr bool kIsSum = MODE == kSum || MODE == kSumW;
     constexpr int kGeo = (kIsSum || G * V >= 4) ? 1 : 0;
     const bool geo = kGeo && a.g.n_vec == G * V && (kIsSum ? a.g.H == 1 : (a.g.H == 4 && a.g.Hp == 4 && a.hvec));
@@ -50,45 +41,16 @@ static sar_status launch_span(SpanArgs a, long long nnz, const char *name, const
             stage_bytes = (size_t)a.R * rsb;
         }
     }
-    if constexpr (MODE == kFwd || kIsSum) if (a.sp.threshold > 0 && a.sp.n_seg > 0) {
-        a.mode = 1;
-        const unsigned blocks = (unsigned)((a.sp.n_seg + kSpanWarps - 1) / kSpanWarps);
-        if (a.sp.threshold <= CAP_SEG) {
-            const size_t seg_smem = (size_t)kSpanWarps * span_layout<MODE>(a.g.Hp, V, CAP_SEG, S, 32 / G).total;
-            auto seg_kern = geo ? span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2, kGeo> : span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2>;
-            SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2, kGeo>, seg_smem));
-            SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP_SEG, MINB, 2>, seg_smem));
-            SAR_LAUNCH(seg_name, st, launch(seg_kern, blocks, kSpanThreads, seg_smem, st, a));
-        } else {
-            auto seg_kern = geo ? span_kernel<T, G, V, S, MODE, CAP, MINB, 2, kGeo> : span_kernel<T, G, V, S, MODE, CAP, MINB, 2>;
-            SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP, MINB, 2, kGeo>, smem));
-            SAR_TRY(ensure_smem(span_kernel<T, G, V, S, MODE, CAP, MINB, 2>, smem));
-            SAR_LAUNCH(seg_name, st, launch(seg_kern, blocks, kSpanThreads, smem, st, a));
-        }
-        SAR_TRY(sar_after_launch());
-    }
-    a.mode = 0;
-    const long long spans = (a.n_rows + a.R - 1) / a.R;
-    if (spans > 0) {
-        const unsigned blocks = (unsigned)((spans + kSpanWarps - 1) / kSpanWarps);
-        if (kIsSum || (whole && !(a.flags & (SAR_KEEP_NUMERATOR | SAR_RELU_OUT)))) {  // the epilogue's flag tests decided at compile time
-            if (geo) {
-                auto wk = span_kernel<T, G, V, S, MODE, CAP, MINB, 1, kGeo>;
-                SAR_TRY(ensure_smem(wk, smem));
-                SAR_LAUNCH(name, st, launch(wk, blocks, kSpanThreads, smem, st, a));
-            } else {
-                auto wk = span_kernel<T, G, V, S, MODE, CAP, MINB, 1>;
-                SAR_TRY(ensure_smem(wk, smem));
-                SAR_LAUNCH(name, st, launch(wk, blocks, kSpanThreads, smem, st, a));
-            }
-        } else {
-            const size_t smem_st = (size_t)kSpanWarps * span_layout<MODE>(a.g.Hp, V, CAP, S, 32 / G, stage_bytes).total;
-            SAR_TRY(ensure_smem(kern, smem_st));
-            SAR_LAUNCH(name, st, launch(kern, blocks, kSpanThreads, smem_st, st, a));
-        }
-        SAR_TRY(sar_after_launch());
-    }
-    return SAR_OK;
+    const long long blocks = a.sp.n_seg + (a.n_rows + a.R - 1) / a.R;
+    if (blocks <= 0) return SAR_OK;
+    // the epilogue's flag tests are decided at compile time where the call holds the whole graph (a sum reads its flags)
+    const bool fixed = kIsSum || (whole && !(a.flags & (SAR_KEEP_NUMERATOR | SAR_RELU_OUT)));
+    auto kern = span_kernel<T, G, V, S, MODE, CAP, MINB, kIsSum ? 1 : 0, 0>;
+    if (fixed) kern = geo ? span_kernel<T, G, V, S, MODE, CAP, MINB, 1, kGeo> : span_kernel<T, G, V, S, MODE, CAP, MINB, 1, 0>;
+    const size_t smem = span_layout<MODE>(a.g.Hp, V, CAP, S, 32 / G, stage_bytes).total;
+    SAR_TRY(ensure_smem(kern, smem));
+    SAR_LAUNCH(name, st, launch(kern, (unsigned)blocks, kSpanThreads, smem, st, a));
+    return sar_after_launch();
 }
 
 // stages of the gather ring: 8 x 512 bytes in flight per warp for one-vector rows
@@ -130,15 +92,15 @@ sar_status span_fwd(const Shape &s, const RowArgs &r, long long nnz, cudaStream_
     const SpanArgs a = span_args(s, r);
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
-        return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kFwd, kCapFwd, kMinBlocksFwd>(a, nnz, "gat_fwd", "gat_fwd_seg", st);
+        return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kFwd, kCapFwd, kMinBlocksFwd>(a, nnz, "gat_fwd", st);
     });
 }
 sar_status span_dst(const Shape &s, const RowArgs &r, long long nnz, bool part, cudaStream_t st) {
     const SpanArgs a = span_args(s, r);
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
-        if (part) return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDstGivenD, kCapDst, kMinBlocksBwd>(a, nnz, "gat_bwd_dst", "", st);
-        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDst, kCapDst, kMinBlocksBwd>(a, nnz, "gat_bwd_dst", "", st);
+        if (part) return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDstGivenD, kCapDst, kMinBlocksBwd>(a, nnz, "gat_bwd_dst", st);
+        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDst, kCapDst, kMinBlocksBwd>(a, nnz, "gat_bwd_dst", st);
     });
 }
 sar_status span_src(const Shape &s, const RowArgs &r, long long nnz, cudaStream_t st) {
@@ -146,15 +108,15 @@ sar_status span_src(const Shape &s, const RowArgs &r, long long nnz, cudaStream_
     a.hvec = s.geom.H % 4 == 0;
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
-        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdSrc, kCapSrc, kMinBlocksBwd>(a, nnz, "gat_bwd_src", "", st);
+        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdSrc, kCapSrc, kMinBlocksBwd>(a, nnz, "gat_bwd_src", st);
     });
 }
 sar_status span_sum(const Shape &s, const RowArgs &r, long long nnz, bool weighted, cudaStream_t st) {
     const SpanArgs a = span_args(s, r);
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
-        if (weighted) return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kSumW, kCapSum, kMinBlocksFwd>(a, nnz, "spmm", "spmm_seg", st);
-        return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kSum, kCapSum, kMinBlocksFwd>(a, nnz, "spmm", "spmm_seg", st);
+        if (weighted) return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kSumW, kCapSum, kMinBlocksFwd>(a, nnz, "spmm", st);
+        return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kSum, kCapSum, kMinBlocksFwd>(a, nnz, "spmm", st);
     });
 }
 

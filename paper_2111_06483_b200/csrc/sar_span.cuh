@@ -5,7 +5,7 @@
 
 namespace sar {
 
-// Rows launch, in the forward pass and the sums the segment launch too.
+// One launch over the segments of the long rows and the spans of the other rows.
 sar_status span_fwd(const Shape &s, const RowArgs &r, long long nnz, cudaStream_t st);
 sar_status span_dst(const Shape &s, const RowArgs &r, long long nnz, bool part, cudaStream_t st);
 sar_status span_src(const Shape &s, const RowArgs &r, long long nnz, cudaStream_t st);

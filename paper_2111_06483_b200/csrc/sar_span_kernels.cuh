@@ -19,12 +19,12 @@
 // Nothing per edge is written to global memory.  No floating-point atomics: every output element
 // has one writer (the per-(row, head) max of the forward pass is a shared-memory atomicMax on an
 // order-preserving integer key, whose result does not depend on the order).
-// Rows above the plan's threshold are skipped here and processed as independent segments by a second launch that writes
-// partial results - mode 1 of this kernel in the forward pass and the sums, the row kernels in the backward passes - which
-// the merge kernels of sar_rows_merge.cu fold.
+// Rows above the plan's threshold are skipped by the spans and processed as independent segments that leave partial
+// results, which the merge kernels of sar_rows_merge.cu fold.  Segments and spans are blocks of one grid, the segments
+// first: a segment is the longest chain of work in a pass, and the spans fill whatever the segments leave free.
 //
-// Where it runs: gathered arrays larger than the L2 (span_applies in sar_span.cuh).  What bounds a gather there is bytes
-// in flight, and the ring holds them without registers; out of the L2 the row kernels (sar_rows_kernel.cuh) are faster.
+// Where it runs: use_span and short_rows in sar_gat.cu.  What bounds a gather beyond the L2 is bytes in flight, and the
+// ring holds them without registers; out of the L2 the row kernels (sar_rows_kernel.cuh) are faster unless rows are short.
 #pragma once
 
 #include "sar_device.cuh"
@@ -44,8 +44,7 @@ struct WeightOf<kBwdSrc> {
     using type = float2;
 };
 
-constexpr int kSpanWarps = 1;             // warps per block
-constexpr int kSpanThreads = kSpanWarps * 32;
+constexpr int kSpanThreads = 32;          // a warp per block
 constexpr int kMaxSpanRows = 16;          // rows per span
 
 struct SpanArgs {
@@ -69,10 +68,9 @@ struct SpanArgs {
     unsigned flags;
     RowGeom g;
     SplitArgs sp;
-    int mode;                // 0: spans of R rows; 1: one long-row segment per warp
     int R;                   // rows per span (<= kMaxSpanRows)
     int hvec;                // heads are scored four at a time (H % 4 == 0 and er is 16-byte aligned)
-    int stage_rows;          // mode 0: rows whose own data is staged in shared memory per chunk (R, or 0: none)
+    int stage_rows;          // spans: rows whose own data is staged in shared memory per chunk (R, or 0: none)
 };
 
 // 16-byte asynchronous copy global -> shared that bypasses L1; src_bytes = 0 writes zeros.
@@ -123,17 +121,17 @@ __host__ __device__ inline SpanSmem span_layout(int Hp, int V, int cap, int stag
     return L;
 }
 
-// STATIC decides the launch mode at compile time, so that the flag tests of the row epilogue fold away:
-// 1 = rows (mode 0) of a partition that holds all sources (SAR_FIRST | SAR_LAST), in the sums of any partition;
-// 2 = long-row segments (mode 1); 0 = whatever SpanArgs says.
+// STATIC says what the warp works on, and decides the flag tests of the row epilogue at compile time where it can:
+// 0 = a span of rows; 1 = a span of rows of a partition that holds all sources (SAR_FIRST | SAR_LAST; the sums take this
+// variant with any flags); 2 = a segment of a long row.
 // GEO = 1 fixes the row geometry at compile time as well: rows of exactly G*V vectors and, for the attention modes,
 // 4 heads scored four at a time (SpanArgs::hvec set; the paper's GAT: 4 heads, hidden size 128), for the sums one
 // head, so that head arithmetic becomes shifts and the lane predicates vanish.
-template <typename T, int G, int V, int S, int MODE, int CAP, int MINB, int STATIC = 0, int GEO = 0>
-__global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs a) {
+template <typename T, int G, int V, int S, int MODE, int CAP, int STATIC, int GEO>
+__device__ __forceinline__ void span_warp(const SpanArgs &a, long long item) {
     constexpr int EPV = Elem<T>::EPV;
     constexpr int EPW = 32 / G;  // edges per slot
-    const int mode_ = STATIC == 1 ? 0 : (STATIC == 2 ? 1 : a.mode);
+    constexpr bool kSeg = STATIC == 2;
     const unsigned flags_ = STATIC == 1 && MODE != kSum && MODE != kSumW ? (unsigned)(SAR_FIRST | SAR_LAST) : a.flags;
     using W = typename WeightOf<MODE>::type;
     constexpr bool kFwdMode = MODE == kFwd;
@@ -141,12 +139,9 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
     constexpr bool kSrc = MODE == kBwdSrc;
     constexpr bool kAcc0 = MODE != kBwdDstGivenD;                  // accumulator 0 live
     constexpr bool kAcc1 = kDst || kSrc;                           // accumulator 1 live
-    const bool beside = a.sp.threshold > 0 && a.sp.n_seg > 0;   // the segments (of the backward passes: the row kernel's) go first
-    if (mode_ == 1) after_predecessor();
-    else beside_segments(beside);
     extern __shared__ __align__(16) unsigned char smem_raw[];
 
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     const int gl = lane & (G - 1), half = lane / G;
     constexpr int kGeoH = (MODE == kSum || MODE == kSumW) ? 1 : 4;  // heads of the compile-time geometry
     const int H = GEO ? kGeoH : a.g.H, Hp = GEO ? kGeoH : a.g.Hp, lgHp = GEO ? (kGeoH == 4 ? 2 : 0) : a.g.lgHp;
@@ -161,10 +156,10 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
     // (Measured on the large workload, 16 partitions: 129 -> 108 ms per layer.  The same for the forward pass's running
     // numerator, 512 bytes per row, costs more in resident warps than it saves: 98 -> 127 ms.)
     constexpr bool kStageMode = MODE == kBwdDst || MODE == kBwdDstGivenD;
-    const bool staged = kStageMode && STATIC == 0 && a.mode == 0 && a.stage_rows != 0;
+    const bool staged = kStageMode && STATIC == 0 && a.stage_rows != 0;
     const unsigned rsb = (unsigned)n_vec * 16u;   // bytes of a staged row
     const SpanSmem L = span_layout<MODE>(Hp, V, CAP, S, EPW, staged ? (size_t)a.stage_rows * rsb : 0);
-    unsigned char *wb = smem_raw + (size_t)warp * L.total;
+    unsigned char *wb = smem_raw;
     uint4 *stage = reinterpret_cast<uint4 *>(wb + L.stage);  // [S][V][32]
     int *sj = reinterpret_cast<int *>(wb + L.sj);
     W *sw = reinterpret_cast<W *>(wb + L.w);
@@ -183,12 +178,11 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
     unsigned *skey = reinterpret_cast<unsigned *>(sc1);
 
     // ---- which rows ---------------------------------------------------------------------------
-    const long long item = (long long)blockIdx.x * kSpanWarps + warp;
     long long row0, eb = 0, ee = 0;   // lane r: edge range of row row0 + r
     int nrows;
     bool excluded = false;            // long row left to the segment launch
     long long seg = -1;
-    if (mode_ == 0) {
+    if constexpr (!kSeg) {
         row0 = item * a.R;
         if (row0 >= a.n_rows) return;
         nrows = (int)((a.n_rows - row0) < a.R ? (a.n_rows - row0) : a.R);
@@ -201,7 +195,6 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
             excluded = a.sp.threshold > 0 && ee - eb > a.sp.threshold;
         }
     } else {
-        if (item >= a.sp.n_seg) return;
         int lo = 0, hi = a.sp.n_long;
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
@@ -217,8 +210,8 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
             ee = eb + a.sp.threshold < re_ ? eb + a.sp.threshold : re_;
         }
     }
-    const bool first_part = (flags_ & SAR_FIRST) || mode_ == 1;
-    const bool last_part = (flags_ & SAR_LAST) && mode_ == 0;
+    const bool first_part = (flags_ & SAR_FIRST) || kSeg;
+    const bool last_part = (flags_ & SAR_LAST) && !kSeg;
     const bool mean_now = (flags_ & SAR_MEAN) && (flags_ & SAR_LAST);
     // does a row without edges (in this partition) still have to be written?
     bool write_empty;
@@ -227,7 +220,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
     else if (MODE == kBwdDstGivenD) write_empty = flags_ & SAR_FIRST;
     else if (kSrc) write_empty = true;
     else write_empty = (flags_ & SAR_FIRST) || mean_now || (a.mix.x0 && (flags_ & SAR_LAST));
-    if (mode_ == 1) write_empty = false;
+    if (kSeg) write_empty = false;
 
     // ---- lane geometry ------------------------------------------------------------------------
     int hv[V];
@@ -428,7 +421,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
         __syncwarp();
 
         if constexpr (kDst || kSrc) {
-            if (mode_ == 0 && !staged_now) {  // the first row that starts in this chunk (a continued row brought its vector along)
+            if (!staged_now) {  // the first row that starts in this chunk (a continued row brought its vector along)
                 const int first = cont ? 1 : 0;
                 if (first < nr) request_rowvec(row0 + r + first, rvq_next);
             }
@@ -488,9 +481,9 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
             __syncwarp();
         } else if constexpr (MODE != kSum) {
             const bool vec4 = GEO ? true : a.hvec != 0;  // heads handled four at a time with 16-byte accesses
-            // A segment launch of the four-head geometry stages one row: every position would hit the same four
+            // A segment of the four-head geometry stages one row: every position would hit the same four
             // shared-memory words, so each lane keeps its own maxima and the warp reduces them once per chunk.
-            constexpr bool kLaneMax = kFwdMode && STATIC == 2 && GEO == 1;
+            constexpr bool kLaneMax = kFwdMode && kSeg && GEO == 1;
             unsigned kmax[4] = {kKeyNegInf, kKeyNegInf, kKeyNegInf, kKeyNegInf};
             int i = 0;
             for (int q0 = lane; q0 < npos; q0 += 64) {
@@ -698,7 +691,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
             const bool row_starts = !(cont && ri == 0);
             const bool row_ends = !(unfinished && ri == nr - 1);
             if constexpr (kDst || kSrc) {
-                if (mode_ == 0 && row_starts && !staged_now) {
+                if (row_starts && !staged_now) {
 #pragma unroll
                     for (int v = 0; v < V; ++v) rvq[v] = rvq_next[v];
                     if (ri + 1 < nr) request_rowvec(row + 1, rvq_next);
@@ -797,7 +790,7 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
             }
             const bool writer = half == 0;  // every edge lane now holds the full sums; one writes
             if constexpr (kFwdMode) {
-                if (mode_ == 1) {
+                if constexpr (kSeg) {
                     if (writer) {
                         float *rec = a.sp.part + seg * a.sp.pstride;
                         store_acc_row<G, V, EPV>(rec, gl, vok, acc0);
@@ -891,12 +884,19 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
                             DA += scratch[32 * V + lane * vph + k];
                         }
                         const float Sh = scratch[64 * V + lane];
+                        if constexpr (kSeg) {   // the segment's D (not where it is given), B and S, for the merge launch
+                            float *rec = a.sp.part + seg * a.sp.pstride;
+                            if constexpr (MODE == kBwdDst) rec[lane] = DA;
+                            rec[H + lane] = DB;
+                            rec[2 * H + lane] = Sh;
+                        } else {
                         const float D = MODE == kBwdDstGivenD ? (staged_now ? sc3[ri * Hp + lane] : a.rec_in[row * H + lane].w) : DA;
                         const float val = DB - D * Sh;
                         float *p = a.del + row * H + lane;
                         *p = (flags_ & SAR_FIRST) ? val : (staged_now ? sc4[ri * Hp + lane] : *p) + val;
                         if constexpr (MODE == kBwdDst)
                             a.rec_out[row * H + lane] = make_float4(sc0[ri * Hp + lane], sc1[ri * Hp + lane], sc2[ri * Hp + lane], D);
+                        }
                     }
                     __syncwarp();
                 }
@@ -911,7 +911,8 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
                         for (int e = 0; e < EPV; ++e) pC[v] = fmaf(rv[v][e], acc1[v][e], pC[v]);
                     }
                     if (writer) {
-                        store_row_vec<T, G, V>(a.out, row, n_vec, gl, vok, acc0);
+                        if constexpr (kSeg) store_acc_row<G, V, EPV>(a.sp.part + seg * a.sp.pstride, gl, vok, acc0);
+                        else store_row_vec<T, G, V>(a.out, row, n_vec, gl, vok, acc0);
 #pragma unroll
                         for (int v = 0; v < V; ++v)
                             if (vok[v]) {
@@ -923,12 +924,13 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
                     if (lane < H) {
                         float DC = 0.f;
                         for (int k = 0; k < vph; ++k) DC += scratch[lane * vph + k];
-                        a.der[row * H + lane] = DC - scratch[64 * V + lane];
+                        float *der = kSeg ? a.sp.part + seg * a.sp.pstride + rowf : a.der + row * H;
+                        der[lane] = DC - scratch[64 * V + lane];
                     }
                     __syncwarp();
                 }
             } else {  // sum aggregation
-                if (mode_ == 1) {
+                if constexpr (kSeg) {
                     if (writer) store_acc_row<G, V, EPV>(a.sp.part + seg * a.sp.pstride, gl, vok, acc0);
                 } else if (writer) {
                     if (a.dst_scale) {
@@ -991,7 +993,14 @@ __global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs
             r = r2;
         }
     }
-    if (mode_ == 0) rows_end(beside);
+}
+
+template <typename T, int G, int V, int S, int MODE, int CAP, int MINB, int STATIC, int GEO>
+__global__ void __launch_bounds__(kSpanThreads, MINB) span_kernel(const SpanArgs a) {
+    after_predecessor();
+    const long long item = (long long)blockIdx.x - a.sp.n_seg;
+    if (item < 0) span_warp<T, G, V, S, MODE, CAP, 2, GEO>(a, blockIdx.x);
+    else span_warp<T, G, V, S, MODE, CAP, STATIC, GEO>(a, item);
 }
 
 }  // namespace sar

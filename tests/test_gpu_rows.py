@@ -95,3 +95,28 @@ def test_ragged_steps_with_a_workspace_each(H, F, dtype):
                       (B.SAR_FIRST if q == 0 else 0) | (B.SAR_LAST if q == 2 else 0), dfeat[s0:s1], del_, der[s0:s1], ws)
     for got, ref in zip((dfeat, del_, der), want):
         assert torch.equal(got, ref)
+
+
+@pytest.mark.parametrize("H,F,dtype", [(4, 16, "f32"), (4, 32, "f32"), (8, 32, "bf16"), (4, 64, "f32")])
+@pytest.mark.parametrize("threshold,many", [(3, True), (100, False)])
+def test_segments_of_the_lean_kernels(H, F, dtype, threshold, many):
+    """Few segments run as the first blocks of the rows' grid, from 148 * 256 on in a launch of their own."""
+    n, src, dst = hub_graph(n=9000, e=300_000, d_max=1500.0, seed=H * F)
+    p = Problem(n, src, dst, H, F, 5, dtype=dtype, k=2, threshold=threshold, build_parts=True)
+    for part in [p.graph.whole] + p.graph.parts:
+        for split in (part.split, part.t_split):
+            assert split.n_seg >= 148 * 256 if many else 0 < split.n_seg < 148 * 256
+    _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
+
+
+@pytest.mark.parametrize("H,F,dtype", [(6, 48, "bf16"), (12, 16, "f32")])
+@pytest.mark.parametrize("threshold", [7, 150, 230, 600])
+def test_segments_of_the_span_kernels(H, F, dtype, threshold):
+    """Segments shorter and longer than the chunks a span kernel stages (192 and 256 edges), whole and step by step.
+    Heavier hubs than these leave the fixed tolerance: an element of dfeat sums D terms alpha * gout whose alpha carries about
+    2^-21 (an exponential of an argument of up to 16), that is an error of 2^-21 sqrt(D sum alpha^2 / D): 1e-5 for D = 1500 and
+    mean alpha^2 = 0.3, the tolerance's floor, and 2e-5 for D = 5000 (seen there: 5e-5, one element in four million)."""
+    n, src, dst = hub_graph(n=20_500, e=170_000, d_max=1500.0, seed=H + F)
+    p = Problem(n, src, dst, H, F, 9, dtype=dtype, k=2, threshold=threshold, build_parts=True)
+    assert p.graph.whole.split.n_seg > 0 and p.graph.whole.t_split.n_seg > 0
+    _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
