@@ -8,7 +8,13 @@ namespace sar {
 
 // ---- span kernels ---------------------------------------------------------------------------------
 constexpr int kCapFwd = 256, kCapDst = 256, kCapSrc = 192, kCapSum = 256;
-constexpr int kMinBlocksFwd = 24, kMinBlocksBwd = 20;  // resident blocks per SM the register budget is cut for
+// Resident blocks per SM the register budget is cut for.  The backward passes hold two accumulators of V vectors; over rows of
+// more than 1 KB (V > 2) they spilled a hundred bytes and more at 20 blocks, twice that with the bodies for spans and segments
+// in one kernel, where shared memory leaves room for 18 blocks (V = 4) or fewer.  Forward + backward, a kernel per body at 20
+// blocks / one kernel at 20 / one at 16: 250,000 nodes, 3 million edges, 8 heads of 64, float32 3.33 / 3.54 / 2.68 ms, 4 heads
+// of 128 2.19 / 2.32 / 2.07, 6 heads of 128, bf16 5.33 / 5.97 / 4.07; 600,000 nodes, 8 heads of 64 5.52 / 6.32 / 4.25.
+constexpr int kMinBlocksFwd = 24;
+template <int V> constexpr int kMinBlocksBwd = V <= 2 ? 20 : V == 4 ? 16 : 12;
 constexpr size_t kStageBytes = 16 * 1024;              // shared memory a partition step may spend on the rows' own data
 
 static int rows_per_span(long long n_rows, long long nnz, int cap) {
@@ -99,8 +105,8 @@ sar_status span_dst(const Shape &s, const RowArgs &r, long long nnz, bool part, 
     const SpanArgs a = span_args(s, r);
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
-        if (part) return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDstGivenD, kCapDst, kMinBlocksBwd>(a, nnz, "gat_bwd_dst", st);
-        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDst, kCapDst, kMinBlocksBwd>(a, nnz, "gat_bwd_dst", st);
+        if (part) return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDstGivenD, kCapDst, kMinBlocksBwd<C::v>>(a, nnz, "gat_bwd_dst", st);
+        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDst, kCapDst, kMinBlocksBwd<C::v>>(a, nnz, "gat_bwd_dst", st);
     });
 }
 sar_status span_src(const Shape &s, const RowArgs &r, long long nnz, cudaStream_t st) {
@@ -108,7 +114,7 @@ sar_status span_src(const Shape &s, const RowArgs &r, long long nnz, cudaStream_
     a.hvec = s.geom.H % 4 == 0;
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
-        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdSrc, kCapSrc, kMinBlocksBwd>(a, nnz, "gat_bwd_src", st);
+        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdSrc, kCapSrc, kMinBlocksBwd<C::v>>(a, nnz, "gat_bwd_src", st);
     });
 }
 sar_status span_sum(const Shape &s, const RowArgs &r, long long nnz, bool weighted, cudaStream_t st) {
