@@ -228,32 +228,41 @@ static sar_status check_part(const sar_part *g, bool need_csc) {
 }
 
 
-// The row kernels, or the span kernels?  Out of the L2 (126 MB) the row kernels are the faster ones, for arrays that do
-// not fit it the span kernels, whose ring keeps more bytes in flight.  Forward + backward, row against span kernels:
-// 100,000 nodes of 256 bytes 0.39 against 0.50 ms, 233,000 (forward alone) 0.41 against 0.57 ms, 400,000 1.43 against
-// 1.55 ms, 1 million of 576 bytes 12.0 against 10.3 ms.  A sum has nothing between its ids and its rows, and there the
-// ring is ahead much earlier: 100,000 nodes of 128 bytes 0.175 against 0.172 ms, 500,000 of 192 bytes 0.72 against
-// 0.67 ms, 2.45 million of 1 KB 15.0 against 12.5 ms; below that the row kernels' single launch counts.
+// The row kernels, or the span kernels (for the shapes that the lean kernels do not cover)?  Times of the span kernels over
+// those of the row kernels, on 8,000 to a million nodes with 2 to 32 edges per node, endpoints uniform and with hubs of
+// n^0.65 edges, plans of 256:
+//  * Arrays that do not fit the L2 (126 MB): the span kernels, whose ring keeps more bytes in flight.  Forward + backward
+//    400,000 nodes of 256 bytes 1.55 against 1.43 ms, 1 million of 576 bytes 10.3 against 12.0.
+//  * Heads: the row kernel holds the scalars of a tile's heads in registers (four or eight heads spill, see there).  One or
+//    two heads: backward 1.0 to 1.5.  Tiles of eight heads: backward 0.42 to 1.05, steps 0.55 to 1.15.  Tiles of four: backward
+//    0.6 to 0.95 with up to 16 edges per row from 20,000 rows on, 1.0 to 1.24 else.
+//  * Rows of 512 bytes to 1 KB in tiles of four or eight heads: backward 0.42 to 0.9, forward steps 0.5 to 1.0 (8,000
+//    uniform rows: up to 1.1), forward 0.55 to 0.98 with up to 12 edges per row.
+//  * Short rows: a row kernel's warp spends its time on the starts and ends of rows, a span kernel's gathers across them.
+//    Forward, from 60,000 rows on: 0.56 to 1.05 with up to 6 edges per row (in a step up to 4), 1.0 to 1.8 with more; with
+//    20,000 rows 0.9 to 1.5.  Rows below 128 bytes: 0.95 to 1.6 throughout.
+//  * Rows of more than 1 KB, backward, where they fit the L2: steps 0.85 to 1.45 (4 heads of 256, float32: 1.3 to 2.1); whole 0.52 to
+//    1.05 with four heads or more, from 20,000 rows on with up to 16 edges per row (6 heads of 128, bf16: 1.1 to 1.25), 0.86
+//    to 1.5 else.
+// With these lines the choice costs 1.1 % over the better kernel of each call in the mean, over shapes of up to 1 KB; with lines drawn
+// by the number of heads alone it was 2.8 %.
 constexpr unsigned long long kSpanBytes = 128ull << 20, kSpanSumBytes = 12ull << 20;
-static bool use_span(const Shape &s, long long n_gathered, unsigned long long bytes = kSpanBytes) {
-    return s.fast && (unsigned long long)n_gathered * s.row_bytes > bytes;
+static bool takes_span(const Shape &s, const RowGeo &geo, long long n_gathered, long long n_rows, long long nnz, bool backward, bool part) {
+    if (!s.fast) return false;
+    if ((unsigned long long)n_gathered * s.row_bytes > kSpanBytes) return true;
+    if (s.row_bytes < 128) return false;
+    const bool over_1k = s.row_bytes > 1024, wide = geo.HP >= 4 && geo.NV >= 64 && !over_1k;
+    const bool short_rows = n_rows >= 20000 && nnz <= 16 * n_rows;
+    if (backward && over_1k) return !part && s.geom.H >= 4 && short_rows;
+    if (backward) return wide || geo.HP == 8 || (geo.HP == 4 && short_rows);
+    if (wide) return part || nnz <= 12 * n_rows;
+    return n_rows >= 60000 && nnz <= (part ? 4 : 6) * n_rows;
 }
-// Short rows: a row kernel's warp spends its time on the starts and ends of rows, a span kernel's gathers across them, so
-// the latter take over below some edges per row, once there are rows enough to fill the chip with spans.  Where the lines
-// lie, from 2 to 32 edges per row and 4,000 to 1.2 million rows, time of the span kernels over that of the row kernels:
-//   forward, 2 / 4 / 8 / 16 edges, 300,000 rows: 4 heads of 8, float32 0.72 / 0.78 / 0.91 / 1.19; 2 of 64, float32 0.76 /
-//     0.83 / 0.95 / 1.17; 3 of 32, bf16 0.82 / 0.87 / 0.99 / 1.25; 6 of 48, bf16 0.59 / 0.66 / 0.81 / 0.95; 1 of 16, bf16
-//     0.98 / 1.00 / 1.09 / 1.33; with 20,000 rows 1.1 to 1.7 but for 6 of 48 (0.88 / 0.89 / 1.02 / 1.26).
-//   backward: 4 of 8 0.64 / 0.67 / 0.72 / 0.85 (32 edges 0.93); 2 of 64 0.89 / 0.90 / 0.99 / 1.04; 3 of 32 0.81 / 0.84 /
-//     0.90 / 1.02; 6 of 48 0.43 / 0.49 / 0.61 / 0.73 (tiles of eight heads spill), 0.5 to 0.9 in partition steps of any
-//     size; 1 of 16 1.13 to 1.32; partition steps of the other shapes 0.93 to 1.26.
-static bool short_rows(const Shape &s, long long n_rows, long long nnz, bool backward, bool part) {
-    const int H = s.geom.H;
-    if (!s.fast || s.row_bytes < 128) return false;
-    if (H > 4) return backward ? part || n_rows >= 10000 : n_rows >= 20000 && nnz <= 10 * n_rows;
-    if (!backward) return n_rows >= 60000 && nnz <= (part ? 4 : 6) * n_rows;
-    if (part) return H == 3 && n_rows >= 60000 && nnz <= 5 * n_rows;
-    return H == 4 ? n_rows >= 20000 && nnz <= 32 * n_rows : H == 3 ? n_rows >= 20000 && nnz <= 10 * n_rows : n_rows >= 60000 && nnz <= 5 * n_rows;
+// A sum has nothing between its ids and its rows, and there the ring is ahead much earlier: 100,000 nodes of 128 bytes 0.172
+// against 0.175 ms, 500,000 of 192 bytes 0.67 against 0.72 ms, 2.45 million of 1 KB 12.5 against 15.0 ms; below that the row
+// kernels' smaller start counts.
+static bool sum_takes_span(const Shape &s, long long n_gathered) {
+    return s.fast && (unsigned long long)n_gathered * s.row_bytes > kSpanSumBytes;
 }
 
 static sar_status check_shape(int32_t H, int32_t F, sar_dtype t) {
@@ -439,7 +448,7 @@ sar_status sar_gat_fwd(const sar_part *g, const void *feat_q, const float *el, c
         }
         return SAR_OK;
     }
-    if (use_span(s, g->n_src) || short_rows(s, g->n_dst, g->nnz, false, part))
+    if (takes_span(s, r.geo, g->n_src, g->n_dst, g->nnz, false, part))
         SAR_TRY(span_fwd(s, a, g->nnz, st));
     else if (part)
         SAR_TRY(t == SAR_F32 ? rows_fwd_part_f32(a, r.geo, g->nnz, st) : rows_fwd_part_bf16(a, r.geo, g->nnz, st));
@@ -641,7 +650,7 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
                 SAR_TRY(t == SAR_F32 ? lean_bwd_dst_f32(s, la, g->nnz, st) : lean_bwd_dst_bf16(s, la, g->nnz, st));
             else
                 SAR_TRY(t == SAR_F32 ? lean_bwd_dst_part_f32(s, la, g->nnz, st) : lean_bwd_dst_part_bf16(s, la, g->nnz, st));
-        } else if (use_span(s, g->n_src) || short_rows(s, g->n_dst, g->nnz, true, !whole))
+        } else if (takes_span(s, r.geo, g->n_src, g->n_dst, g->nnz, true, !whole))
             SAR_TRY(span_dst(s, a, g->nnz, !whole, st));
         else if (whole)
             SAR_TRY(t == SAR_F32 ? rows_dst_f32(a, r.geo, g->nnz, st) : rows_dst_bf16(a, r.geo, g->nnz, st));
@@ -674,7 +683,7 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
             la.sp = a.sp;
             la.sp.threshold = g->t_split->threshold;
             SAR_TRY(t == SAR_F32 ? lean_bwd_src_f32(s, la, g->nnz, st) : lean_bwd_src_bf16(s, la, g->nnz, st));
-        } else if (use_span(s, g->n_dst) || short_rows(s, g->n_src, g->nnz, true, !whole))
+        } else if (takes_span(s, r.geo, g->n_dst, g->n_src, g->nnz, true, !whole))
             SAR_TRY(span_src(s, a, g->nnz, st));
         else
             SAR_TRY(t == SAR_F32 ? rows_src_f32(a, r.geo, g->nnz, st) : rows_src_bf16(a, r.geo, g->nnz, st));
@@ -717,7 +726,7 @@ static sar_status sum_rows(const sar_part *g, const RowShape &r, int32_t F, sar_
     const bool weighted = src_scale != nullptr;
     Shape s;
     SAR_TRY(make_shape(1, F, t, !r.ragged, &s));
-    if (use_span(s, g->n_src, kSpanSumBytes))
+    if (sum_takes_span(s, g->n_src))
         SAR_TRY(span_sum(s, a, g->nnz, weighted, st));
     else
         SAR_TRY(t == SAR_F32 ? rows_sum_f32(a, r.geo, g->nnz, weighted, st) : rows_sum_bf16(a, r.geo, g->nnz, weighted, st));

@@ -23,7 +23,7 @@
 // results, which the merge kernels of sar_rows_merge.cu fold.  Segments and spans are blocks of one grid, the segments
 // first: a segment is the longest chain of work in a pass, and the spans fill whatever the segments leave free.
 //
-// Where it runs: use_span and short_rows in sar_gat.cu.  What bounds a gather beyond the L2 is bytes in flight, and the
+// Where it runs: takes_span in sar_gat.cu.  What bounds a gather beyond the L2 is bytes in flight, and the
 // ring holds them without registers; out of the L2 the row kernels (sar_rows_kernel.cuh) are faster unless rows are short.
 #pragma once
 
@@ -180,7 +180,7 @@ __device__ __forceinline__ void span_warp(const SpanArgs &a, long long item) {
     // ---- which rows ---------------------------------------------------------------------------
     long long row0, eb = 0, ee = 0;   // lane r: edge range of row row0 + r
     int nrows;
-    bool excluded = false;            // long row left to the segment launch
+    bool excluded = false;            // long row: its segments are blocks of their own
     long long seg = -1;
     if constexpr (!kSeg) {
         row0 = item * a.R;

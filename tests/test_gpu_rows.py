@@ -35,7 +35,10 @@ def test_attention_on_arrays_larger_than_the_l2(H, F, dtype, n):
 
 
 @pytest.mark.parametrize("H,F,dtype,n,deg,d_max", [(4, 8, "f32", 61_000, 3, 200.0), (2, 64, "bf16", 61_000, 2, 400.0), (3, 32, "bf16", 61_000, 4, 900.0),
-                                                   (6, 48, "bf16", 21_000, 9, 300.0), (12, 16, "f32", 10_100, 2, 500.0)])
+                                                   (6, 48, "bf16", 21_000, 9, 300.0), (12, 16, "f32", 10_100, 2, 500.0),
+                                                   (8, 24, "bf16", 700, 11, 200.0), (4, 48, "f32", 900, 20, 300.0), (3, 64, "f32", 900, 8, 300.0),
+                                                   (5, 24, "f32", 20_000, 16, 300.0), (4, 24, "bf16", 20_000, 15, 300.0), (6, 128, "bf16", 900, 6, 100.0),
+                                                   (3, 128, "f32", 1_500, 6, 100.0)])
 def test_attention_on_short_rows(H, F, dtype, n, deg, d_max):
     """Few edges per row: the span kernels on small arrays, whole and step by step, with long rows among them."""
     n, src, dst = hub_graph(n=n, e=deg * n, d_max=d_max, seed=H + F)
