@@ -1,6 +1,6 @@
 // Host-side interface of the lean span kernels (internal): arguments, applicability test and the launchers,
 // which are compiled in translation units of their own (sar_lean_*.cu), one per pass and storage type.
-// They cover the forward pass and both backward passes of a call that holds the whole graph.
+// They cover the forward pass and both backward passes, of a call that holds the whole graph and as partition steps.
 #pragma once
 
 #include "sar_rowkernels.cuh"
@@ -52,7 +52,7 @@ constexpr int kLeanCap = 256;   // edges a chunk stages; rows and segments must 
 
 // Do the lean kernels cover this shape?  Slope >= 0, heads in groups of four, rows of
 // exactly G*V vectors with V <= 2, the vectors of a head a power of two within one lane group, and a long-row
-// plan whose threshold fits a chunk (so that no row of the rows launch and no segment exceeds it), and a gathered
+// plan whose threshold fits a chunk (so that no span's row and no segment exceeds it), and a gathered
 // array of n_gathered rows whose 16-byte vectors can be counted in 32 bits (the staged row offsets are 32-bit).
 static inline bool lean_shape_applies(const Shape &s, float slope, const sar_split *sp, long long n_gathered) {
     if (!s.fast) return false;
@@ -65,14 +65,7 @@ static inline bool lean_shape_applies(const Shape &s, float slope, const sar_spl
     return (s.G == 16 && s.V == 1 && H == 4) || (s.G == 32 && s.V == 1 && (H == 4 || H == 8)) ||
            (s.G == 32 && s.V == 2 && H == 4);
 }
-// ... and is the call one that holds the whole graph (the forward pass and the destination-major pass of a partition
-// step have variants of their own; the source-major pass is the same for both, a source lies in one partition)?
-static inline bool lean_applies(const Shape &s, unsigned flags, float slope, const sar_split *sp, long long n_gathered) {
-    if ((flags & (SAR_FIRST | SAR_LAST | SAR_KEEP_NUMERATOR)) != (SAR_FIRST | SAR_LAST)) return false;
-    return lean_shape_applies(s, slope, sp, n_gathered);
-}
-
-// Rows launch + segment launch of one pass.
+// Segments of the long rows and spans of the other rows, of one pass.
 sar_status lean_fwd_f32(const Shape &s, const LeanArgs &a, long long nnz, cudaStream_t st);
 sar_status lean_fwd_bf16(const Shape &s, const LeanArgs &a, long long nnz, cudaStream_t st);
 sar_status lean_fwd_part_f32(const Shape &s, const LeanArgs &a, long long nnz, cudaStream_t st);

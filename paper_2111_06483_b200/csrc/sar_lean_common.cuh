@@ -21,8 +21,8 @@
 //     (slope >= 0) and runs online, stage by stage.
 //   * Dot products of the backward epilogues are taken on the un-folded accumulators and reduced with three shuffles
 //     per quantity; per-(row, head) scalars leave through shared memory, coalesced, once per chunk.
-// Preconditions (checked by the host, which otherwise launches the row kernels): SAR_FIRST|SAR_LAST, slope >= 0, every row of
-// the rows launch at most CAP edges (a long-row plan with threshold <= CAP), segments of at most CAP edges, fewer
+// Preconditions (checked by the host, which otherwise launches the row or span kernels): slope >= 0, every row that is no
+// long one at most CAP edges (a long-row plan with threshold <= CAP), segments of at most CAP edges, fewer
 // than 2^32 16-byte vectors in the gathered array.
 #pragma once
 
@@ -76,12 +76,12 @@ constexpr float kLog2e = 1.4426950408889634f;
 // One configuration: chunks of kLeanCap edges, ring of two stages of 2 KB (4 KB for rows of 512 bytes and more), measured
 // best on the large workload among stages of 2 / 4 KB, two to four stages, chunks of 128 / 192 / 256 edges.
 constexpr int kLeanMinBlocks = 8;
-// The rows launches of the two backward passes are compiled for 24 resident blocks per SM (72-78 registers instead of
-// 88, no spills): step of the large workload 153.1 -> 147.2 ms.  The same bound on the forward rows launch and on the
-// segment launches changes nothing (147.3 ms).
+// The rows of the two backward passes are compiled for 24 resident blocks per SM (64-80 registers instead of 88; no
+// spills but for bf16 rows of 1 KB source-major, 40 bytes): step of the large workload 153.1 -> 147.2 ms.  The same bound
+// on the forward rows and on launches over segments alone changes nothing (147.3 ms).
 constexpr int kLeanMinBlocksBwdRows = 24;
 
-// Resident blocks per SM the rows launch of a partition step is compiled for.
+// Resident blocks per SM the rows of a partition step are compiled for.
 constexpr int kLeanMinBlocksPart = 16;
 
 constexpr int kMaxSpanRows = 16;   // rows a span holds at most
