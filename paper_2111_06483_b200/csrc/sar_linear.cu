@@ -305,7 +305,12 @@ using GemmForward = LinearGemm<RowMajor, RowMajor, cutlass::bfloat16_t>;
 using GemmForwardProject = LinearGemm<RowMajor, RowMajor, cutlass::bfloat16_t, ProjectFusion>;
 // dh[n, d_in] = dz[n, d_out] W^T:           A = dz, B[k, n] = W[n, k]: K contiguous
 using GemmBwdInput = LinearGemm<RowMajor, ColMajor, cutlass::bfloat16_t>;
-// Outputs wider than 128 columns: tiles of 256, so that A, the large operand, is read once per 256 columns
+// Outputs wider than 128 columns: tiles of 256, so that A, the large operand, is read once per 256 columns, from some rows
+// on.  Time over that of tiles of 128, for widths of 136 to 512 and 32 to 256 columns of A: 2 million rows 0.63 to 1.06 (384
+// columns: a tile and a half), 200,000 0.71 to 1.0, 60,000 0.78 to 1.1; 20,000 rows 0.86 to 1.18, 8,000 and fewer 0.85 to
+// 1.24, for a wide tile is one CTA's work where two narrow ones are two CTAs'.
+constexpr int kWideRows = 2 * 148 * 128;   // two tiles of rows for every SM
+static bool wide_tiles(int64_t n, int columns) { return columns > 128 && n >= kWideRows; }
 using GemmForwardWide = LinearGemm<RowMajor, RowMajor, cutlass::bfloat16_t, void, false, Shape<_128, _256, _64>>;
 using GemmBwdInputWide = LinearGemm<RowMajor, ColMajor, cutlass::bfloat16_t, void, false, Shape<_128, _256, _64>>;
 // the same followed by the backward of the ReLU that produced the layer's input
@@ -388,7 +393,7 @@ sar_status sar_linear(int64_t n, int32_t d_in, int32_t d_out, sar_dtype t, const
                       void *workspace, size_t workspace_bytes, void *stream) {
     if (n == 0 && d_in > 0 && d_out > 0) return t == SAR_BF16 ? SAR_OK : SAR_ERR_UNSUPPORTED;
     SAR_TRY(linear_check(n, d_in, d_out, t, {h, w, z}));
-    return (d_out > 128 ? GemmForwardWide::run : GemmForward::run)((int)n, d_out, d_in, h, w, z, workspace, workspace_bytes,
+    return (wide_tiles(n, d_out) ? GemmForwardWide::run : GemmForward::run)((int)n, d_out, d_in, h, w, z, workspace, workspace_bytes,
                                                                    static_cast<cudaStream_t>(stream), "linear", 0.f, 1);
 }
 
@@ -416,7 +421,7 @@ sar_status sar_linear_accumulate(int64_t n, int32_t d_in, int32_t d_out, sar_dty
                                  void *workspace, size_t workspace_bytes, void *stream) {
     if (n == 0 && d_in > 0 && d_out > 0) return t == SAR_BF16 ? SAR_OK : SAR_ERR_UNSUPPORTED;
     SAR_TRY(linear_check(n, d_in, d_out, t, {h, w, z}));
-    return (d_out > 128 ? GemmForwardWide::run : GemmForward::run)((int)n, d_out, d_in, h, w, z, workspace, workspace_bytes,
+    return (wide_tiles(n, d_out) ? GemmForwardWide::run : GemmForward::run)((int)n, d_out, d_in, h, w, z, workspace, workspace_bytes,
                                                                    static_cast<cudaStream_t>(stream), "linear_accumulate", 1.f, 1);
 }
 
@@ -424,7 +429,7 @@ sar_status sar_linear_bwd_input(int64_t n, int32_t d_in, int32_t d_out, sar_dtyp
                                 void *dh, void *workspace, size_t workspace_bytes, void *stream) {
     if (n == 0 && d_in > 0 && d_out > 0) return t == SAR_BF16 ? SAR_OK : SAR_ERR_UNSUPPORTED;
     SAR_TRY(linear_check(n, d_in, d_out, t, {dz, w, dh}));
-    return (d_in > 128 ? GemmBwdInputWide::run : GemmBwdInput::run)((int)n, d_in, d_out, dz, w, dh, workspace, workspace_bytes,
+    return (wide_tiles(n, d_in) ? GemmBwdInputWide::run : GemmBwdInput::run)((int)n, d_in, d_out, dz, w, dh, workspace, workspace_bytes,
                                                                     static_cast<cudaStream_t>(stream), "linear_bwd_input", 0.f, 1);
 }
 

@@ -38,6 +38,13 @@ def test_projection_forward_and_backward(d_in, d_out, n):
     allclose_report(_np(dw), want_dw, 1e-4, 1e-5 * max(1.0, float(np.sqrt(n))), "dw")
 
 
+@pytest.mark.parametrize("d_in,d_out", [(136, 136), (264, 256), (72, 512)])
+@pytest.mark.parametrize("n", [2 * 148 * 128 - 1, 2 * 148 * 128])
+def test_projection_on_either_side_of_the_wide_tiles(d_in, d_out, n):
+    """Outputs wider than 128 columns take wider tiles from this many rows on."""
+    test_projection_forward_and_backward(d_in, d_out, n)
+
+
 @pytest.mark.parametrize("d_in,H,F", [(128, 4, 32), (64, 8, 32), (128, 2, 64), (40, 4, 16), (64, 1, 128), (128, 16, 8)])
 @pytest.mark.parametrize("n", [1, 100, 4097, 300001])
 def test_projection_with_scores_in_the_epilogue(d_in, H, F, n):
