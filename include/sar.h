@@ -597,9 +597,10 @@ SAR_API sar_status sar_bn_bwd_apply_act(int64_t n, int32_t C, sar_dtype t, const
  * cudaMalloc / cudaFree and no allocating library routine; inputs and outputs are the caller's, exactly
  * as for sar_gat_bwd.
  *
- *   - Limit: sar_gat_workspace_bytes(g, H, F, t) must not exceed SAR_NOALLOC_SCRATCH_BYTES (16 bytes per
- *     (destination, head) plus the long-row partials); larger problems return SAR_ERR_WORKSPACE and launch
- *     nothing.  Every GPU that loads the library carries the array until the process exits.
+ *   - Limit: the records and the long-row partials (16 bytes per (destination, head) plus the segments) must
+ *     fit SAR_NOALLOC_SCRATCH_BYTES; larger problems return SAR_ERR_WORKSPACE and launch nothing.  Where the
+ *     padded copies of a ragged F do not fit beside them, or arrays are misaligned, the scalar kernels run,
+ *     which need the records alone.  Every GPU that loads the library carries the array until the process exits.
  *   - The first call on each device looks up the array's device address (with that device current) and
  *     remembers it for the life of the process; make that first call before any stream capture begins.
  *     The remembered address belongs to the device's context at that time: after a cudaDeviceReset of

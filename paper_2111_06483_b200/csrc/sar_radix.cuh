@@ -12,7 +12,7 @@
 // No block waits for another one.
 //
 // What bounds a pass: 20 bytes of traffic an element would take 0.19 ms for 62 million pairs, the move takes 0.30 ms and
-// the counts 0.05.  The move issues 120 instructions per 32 elements, 76 of them on the half-rate integer pipe (78 % busy);
+// the counts 0.05.  The move issues 94 instructions per 32 elements, most of them on the half-rate integer pipe (67 to 77 % busy);
 // matching by shared-memory atomics or match_any instead of ballots, writing without the detour through shared memory,
 // and 11-bit digits (two passes of 0.7 ms: 2048 counters a tile, runs of 4) all measured the same or slower, and so did
 // 512 threads or 8 to 12 elements a thread.  Before, eight-bit passes over 8-byte keys of both endpoints took seven times

@@ -9,15 +9,19 @@
 //     registers before the first is accumulated.  What a lane holds per row is one vector of float32 sums (forward,
 //     source-major) or three numbers (destination-major).
 //
-// What bounds it: latency, then issue slots.  Out of the L2 a gather can move 20 TB/s on this GPU (random 512-byte rows
-// of a 64 MB array; 7.4 TB/s out of 2.5 GB), but a short row is a chain of dependent loads: row pointers, column ids,
-// rows.  So a warp keeps no stage and no ring, which leaves registers and shared memory for 32 of them per SM; the
+// What bounds it: latency, then issue slots.  The L2 is not what a gather out of it waits for (36 % of its throughput in the
+// two-head case below), but a short row is a chain of dependent loads: row pointers, column ids, rows.  So a warp keeps
+// no stage and no ring, and 32 of them fit an SM with 64 registers a thread (25 are there on average); the
 // row pointers of a warp's rows are one load, the column ids of the next 32 edges are asked for before the present ones
 // are used, and the score terms, the row's own data and the first U slots are all in flight together.  A row of up to
 // U slots costs one memory latency, which the other warps hide.  Measured, before (a warp staging 256 edges in shared
 // memory) and now: 233,000 nodes, 11.6 million edges, 2 heads of 64, bf16, forward 554 -> 408 us (7.3 TB/s of gathered
 // rows, 23 instructions per edge, issue slots 68 % busy); 20,000 nodes, 400,000 edges, 1 head of 64, float32, 4 partition
 // steps forward and backward 497 -> 274 us; 2,000 nodes, 22,000 edges, 4 heads of 16, one pass 15 -> 5 us.
+// 64 registers are not enough for every pass.  The sums and the forward pass of one head in float32 spill nothing; the other
+// passes of one or two heads 8 to 150 bytes a thread (0.3 to 6 % of the instructions they issue), tiles of four heads 60
+// to 200 (64 vectors of bf16: 116 to 372), of eight heads 90 to 560, and there the span kernels take over (takes_span in
+// sar_gat.cu).
 //
 // Forward: the softmax is taken against the exact maximum of the row's scores among 32 edges (one `redux` per head); a
 // row of more carries the running-max correction of Sec. 3.4.

@@ -18,7 +18,9 @@ static inline int rows_per_warp(long long n_rows) {
 
 template <typename T, int NV, int HP, int MODE>
 static sar_status launch_row_kernel(RowArgs a, RowGeo g, long long nnz, const char *name, cudaStream_t st) {
-    constexpr int MINB = NV >= 256 ? 2 : NV == 128 ? 4 : (NV == 64 || HP == 8) ? 7 : 8;   // 32 warps per SM at 64 registers (7 and 10 blocks: 2 and 10 % slower)
+    constexpr int MINB = NV >= 256 ? 2 : NV == 128 ? 4 : (NV == 64 || HP == 8) ? 7 : 8;
+    // 32 warps per SM at 64 registers (28 at 72 for 64 vectors or eight heads).  7 and 10 blocks were 2 and 10 % slower for two
+    // heads of 64, bf16, forward, where 8 spill 16 bytes; passes that spill more were not tried apart.
     a.nnz = nnz;
     a.R = rows_per_warp(a.n_rows);
     const long long items = a.sp.n_seg + (a.n_rows + a.R - 1) / a.R;
