@@ -258,6 +258,48 @@ static bool takes_span(const Shape &s, const RowGeo &geo, long long n_gathered, 
     if (wide) return part || nnz <= 12 * n_rows;
     return n_rows >= 60000 && nnz <= (part ? 4 : 6) * n_rows;
 }
+
+// The kernel for short rows (a row per group of lanes, sar_short_kernel.cuh) instead of either?  It wins where a row's start and
+// end cost the others more than its edges: few edges per row, narrow rows, many heads in a tile.  Times of the kernel that
+// takes the call otherwise over those of the kernel for short rows, 1,000 to 3 million nodes, 1 to 60 edges per node, endpoints
+// uniform / with hubs of n^0.65 edges, tiles of NV vectors and HP heads:
+//  * NV <= 8, HP <= 2.  From 16,000 rows on forward 1.2 to 5.2 / 1.1 to 3.2 with up to 12 edges per row, NV = 4 0.9 to 1.3 / 1.0 to
+//    1.4 and NV = 8 0.8 to 1.0 / 0.9 to 1.1 with 20, 0.7 to 0.9 / 0.8 to 1.3 with 30.  Backward 1.1 to 5 / 1.1 to 3.8, NV = 4 up to 28
+//    edges, NV = 8 0.85 to 1.1 with 20.
+//  * NV <= 8, HP = 4: forward 0.9 to 3.2 / 1.1 to 2.0 with up to 24; backward 1.1 to 4.4 / 1.2 to 2.7 with up to 60.
+//  * HP = 8: backward 1.3 to 5.7 / 1.1 to 4.0; forward 0.96 to 3.5 / 1.0 to 2.6 with up to 30 (NV = 32, where the array fits the
+//    L2: 0.96 to 1.5 / 0.9 to 1.2 with up to 14; else 0.73 to 1.2).
+//  * NV = 16, HP = 4: forward 1.0 to 1.75 / 0.95 to 1.07 with up to 10, backward 1.1 to 2.2 / 0.95 to 1.4 with up to 16.  HP = 2: forward
+//    1.0 to 1.67 / 0.85 to 1.05, backward 1.1 to 1.9 / 0.95 to 1.5 with up to 8.  HP = 1: 1.0 to 1.5 / 0.7 to 1.0 with up to 6.
+//  * NV = 32, HP = 4, backward: 1.0 to 1.5 / 0.9 to 1.1 with up to 10; forward, and HP <= 2, 0.5 to 1.2.
+//  * Few rows do not fill the chip with groups: 10,000 rows as above with up to 0.6 of these edges, 5,000 with 0.3, 2,000
+//    with 0.12 (with twice as many 0.5 to 0.9).
+static double short_edges(const RowGeo &geo, bool backward, bool hubs, bool fits_l2) {
+    const int NV = geo.NV, HP = geo.HP;
+    if (NV > 32) return 0;
+    if (HP == 8) return backward ? 100 : NV <= 16 ? 40 : fits_l2 ? 14 : 0;
+    if (NV == 32) return HP == 4 && backward ? 10 : 0;
+    if (NV == 16) return HP == 4 ? (backward ? 16 : 10) : HP == 2 ? (backward || !hubs ? 8 : 0) : hubs ? 0 : 6;
+    if (HP == 4) return backward ? 100 : 24;
+    return NV == 4 ? (backward ? 28 : 20) : backward ? 16 : 14;
+}
+static bool few_edges(double limit, long long n_rows, long long nnz) {
+    const double fill = n_rows < 16000 ? (double)n_rows / 16000 : 1.0;
+    return limit > 0 && nnz < (1LL << 30) && (double)nnz <= limit * fill * (double)n_rows;
+}
+static bool takes_short(const RowGeo &geo, long long n_gathered, unsigned row_bytes, long long n_rows, long long nnz, bool backward, bool hubs) {
+    const bool fits_l2 = (unsigned long long)n_gathered * row_bytes <= kSpanBytes;
+    return few_edges(short_edges(geo, backward, hubs, fits_l2), n_rows, nnz);
+}
+// Sums, likewise: rows of 64 bytes 1.0 to 4.1 / 1.0 to 2.4 with up to 20 edges per row; of 128 bytes, in arrays of up to 12 MB 1.1
+// to 2.4 / 1.0 to 1.4 with up to 14, up to 64 MB 1.1 to 1.9 / 1.0 to 1.3 with up to 8, beyond 1.1 to 1.6 / 1.0 to 1.2 with up to 3; of 256 bytes,
+// without hubs, in arrays of up to 12 MB 1.05 to 1.5 with up to 12; else 0.6 to 1.0.
+static bool sum_takes_short(const RowGeo &geo, long long n_gathered, unsigned row_bytes, long long n_rows, long long nnz, bool hubs) {
+    const unsigned long long bytes = (unsigned long long)n_gathered * row_bytes;
+    const double limit = geo.tiles > 1 || geo.NV > 16 ? 0 : geo.NV == 4 ? 20 : geo.NV == 8 ? (bytes <= kSpanSumBytes ? 14 : bytes <= (64ull << 20) ? 8 : 3)
+                                                     : !hubs && bytes <= kSpanSumBytes ? 12 : 0;
+    return few_edges(limit, n_rows, nnz);
+}
 // A sum has nothing between its ids and its rows, and there the ring is ahead much earlier: 100,000 nodes of 128 bytes 0.172
 // against 0.175 ms, 500,000 of 192 bytes 0.67 against 0.72 ms, 2.45 million of 1 KB 12.5 against 15.0 ms; below that the row
 // kernels' smaller start counts.
@@ -448,7 +490,8 @@ sar_status sar_gat_fwd(const sar_part *g, const void *feat_q, const float *el, c
         }
         return SAR_OK;
     }
-    if (takes_span(s, r.geo, g->n_src, g->n_dst, g->nnz, false, part))
+    a.lone = takes_short(r.geo, g->n_src, r.row_bytes, g->n_dst, g->nnz, false, use_split);
+    if (!a.lone && takes_span(s, r.geo, g->n_src, g->n_dst, g->nnz, false, part))
         SAR_TRY(span_fwd(s, a, g->nnz, st));
     else if (part)
         SAR_TRY(t == SAR_F32 ? rows_fwd_part_f32(a, r.geo, g->nnz, st) : rows_fwd_part_bf16(a, r.geo, g->nnz, st));
@@ -628,6 +671,7 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
         a.rowvec = gout_g;
         a.dscal = del;
         a.sp = split_args(g->split, reinterpret_cast<float *>(wsb + w.csr), H, r, t);
+        a.lone = takes_short(r.geo, g->n_src, r.row_bytes, g->n_dst, g->nnz, true, a.sp.n_long > 0);
         if (lean_shape_applies(s, slope, g->split, g->n_src) && sar_aligned(er_q, 16)) {
             LeanArgs la{};
             la.n_rows = g->n_dst;
@@ -650,7 +694,7 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
                 SAR_TRY(t == SAR_F32 ? lean_bwd_dst_f32(s, la, g->nnz, st) : lean_bwd_dst_bf16(s, la, g->nnz, st));
             else
                 SAR_TRY(t == SAR_F32 ? lean_bwd_dst_part_f32(s, la, g->nnz, st) : lean_bwd_dst_part_bf16(s, la, g->nnz, st));
-        } else if (takes_span(s, r.geo, g->n_src, g->n_dst, g->nnz, true, !whole))
+        } else if (!a.lone && takes_span(s, r.geo, g->n_src, g->n_dst, g->nnz, true, !whole))
             SAR_TRY(span_dst(s, a, g->nnz, !whole, st));
         else if (whole)
             SAR_TRY(t == SAR_F32 ? rows_dst_f32(a, r.geo, g->nnz, st) : rows_dst_bf16(a, r.geo, g->nnz, st));
@@ -668,6 +712,7 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
         a.out = dfeat_q;
         a.dscal = der_q;
         a.sp = split_args(g->t_split, reinterpret_cast<float *>(wsb + w.csc), H, r, t);
+        a.lone = takes_short(r.geo, g->n_dst, r.row_bytes, g->n_src, g->nnz, true, a.sp.n_long > 0);
         if (lean_shape_applies(s, slope, g->t_split, g->n_dst)) {
             LeanSrcArgs la{};
             la.n_rows = g->n_src;
@@ -683,7 +728,7 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
             la.sp = a.sp;
             la.sp.threshold = g->t_split->threshold;
             SAR_TRY(t == SAR_F32 ? lean_bwd_src_f32(s, la, g->nnz, st) : lean_bwd_src_bf16(s, la, g->nnz, st));
-        } else if (takes_span(s, r.geo, g->n_dst, g->n_src, g->nnz, true, !whole))
+        } else if (!a.lone && takes_span(s, r.geo, g->n_dst, g->n_src, g->nnz, true, !whole))
             SAR_TRY(span_src(s, a, g->nnz, st));
         else
             SAR_TRY(t == SAR_F32 ? rows_src_f32(a, r.geo, g->nnz, st) : rows_src_bf16(a, r.geo, g->nnz, st));
@@ -726,7 +771,8 @@ static sar_status sum_rows(const sar_part *g, const RowShape &r, int32_t F, sar_
     const bool weighted = src_scale != nullptr;
     Shape s;
     SAR_TRY(make_shape(1, F, t, !r.ragged, &s));
-    if (sum_takes_span(s, g->n_src))
+    a.lone = sum_takes_short(r.geo, g->n_src, r.row_bytes, g->n_dst, g->nnz, a.sp.n_long > 0);
+    if (!a.lone && sum_takes_span(s, g->n_src))
         SAR_TRY(span_sum(s, a, g->nnz, weighted, st));
     else
         SAR_TRY(t == SAR_F32 ? rows_sum_f32(a, r.geo, g->nnz, weighted, st) : rows_sum_bf16(a, r.geo, g->nnz, weighted, st));

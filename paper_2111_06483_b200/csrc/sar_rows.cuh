@@ -41,6 +41,7 @@ struct RowArgs {
     int ragged;              // out / acc rows are not made of aligned 16-byte vectors: element stores
     int hvec;                // the per-head scalars of a row can be loaded as float4 / float2
     int R;                   // rows per warp (<= 32)
+    int lone;                // a row per group of lanes (sar_short_kernel.cuh)
     SplitArgs sp;
 };
 

@@ -3,6 +3,7 @@
 
 #include "sar_dispatch.cuh"
 #include "sar_rows_kernel.cuh"
+#include "sar_short_kernel.cuh"
 
 namespace sar {
 
@@ -33,10 +34,27 @@ static sar_status launch_row_kernel(RowArgs a, RowGeo g, long long nnz, const ch
     return sar_after_launch();
 }
 
+template <typename T, int NV, int HP, int MODE>
+static sar_status launch_short_kernel(RowArgs a, RowGeo g, long long nnz, const char *name, cudaStream_t st) {
+    constexpr int NG = 32 / NV;
+    // 32 warps an SM at 64 registers; the backward passes over bf16 rows need 70 to 80 (24 warps, no spills)
+    constexpr int MINB = sizeof(T) == 2 && (MODE == kRowSrc || MODE == kRowDst || MODE == kRowDstPart) ? 6 : 8;
+    a.nnz = nnz;
+    const long long warps = a.sp.n_seg + (a.n_rows + NG - 1) / NG;
+    if (warps <= 0) return SAR_OK;
+    const dim3 grid((unsigned)((warps * 32 + kShortThreads - 1) / kShortThreads), (unsigned)g.tiles);
+    SAR_LAUNCH(name, st, launch(short_kernel<T, NV, HP, MODE, MINB>, grid, kShortThreads, 0, st, a));
+    return sar_after_launch();
+}
+
 template <typename T, int MODE>
 static sar_status dispatch_rows(const RowArgs &a, RowGeo g, long long nnz, const char *name, cudaStream_t st) {
 #define SAR_ROW_CASE(NV_, HP_) \
-    if (g.NV == NV_ && g.HP == HP_) return launch_row_kernel<T, NV_, HP_, MODE>(a, g, nnz, name, st);
+    if (g.NV == NV_ && g.HP == HP_) { \
+        if constexpr (NV_ <= 32) \
+            if (a.lone) return launch_short_kernel<T, NV_, HP_, MODE>(a, g, nnz, name, st); \
+        return launch_row_kernel<T, NV_, HP_, MODE>(a, g, nnz, name, st); \
+    }
     SAR_ROW_CASE(4, 1) SAR_ROW_CASE(8, 1) SAR_ROW_CASE(16, 1) SAR_ROW_CASE(32, 1) SAR_ROW_CASE(64, 1)
     SAR_ROW_CASE(128, 1) SAR_ROW_CASE(256, 1)
     if constexpr (MODE != kRowSum && MODE != kRowSumW) {

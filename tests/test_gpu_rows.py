@@ -46,6 +46,33 @@ def test_attention_on_short_rows(H, F, dtype, n, deg, d_max):
     _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
 
 
+@pytest.mark.parametrize("H,F,dtype", [(1, 5, "f32"), (1, 32, "bf16"), (2, 12, "bf16"), (4, 8, "f32"), (3, 16, "bf16"), (1, 47, "bf16"), (8, 8, "bf16"),
+                                       (2, 32, "f32"), (4, 24, "bf16"), (7, 8, "f32"), (8, 24, "bf16"), (3, 24, "f32")])
+@pytest.mark.parametrize("scale", [1.0, 60.0])
+def test_attention_of_a_row_per_lane_group(H, F, dtype, scale):
+    """Enough rows with few enough edges for the kernel for short rows: rows of 0, 1, 3 to 5, 23 to 25 and 95 to 97 edges (the ends of its
+    steps of four, and of what one group keeps to itself), segments of 100 and of 1, and scores that lead a row's first by more than 60."""
+    n, gen = 16_100, torch.Generator().manual_seed(H * F)
+    src, dst = [torch.randint(0, n, (3 * n,), generator=gen)], [torch.randint(500, n, (3 * n,), generator=gen)]
+    for row, deg in enumerate([1, 3, 4, 5, 23, 24, 25, 95, 96, 97, 100, 101, 350]):
+        src.append(torch.randint(0, n, (2 * deg,), generator=gen))
+        dst.append(torch.tensor([7 * row, 7 * row + 3]).repeat_interleave(deg))
+    src, dst = torch.cat(src).int(), torch.cat(dst).int()
+    both = torch.cat([src, dst]), torch.cat([dst, src])   # the same lengths among the columns, which the source-major pass walks
+    p = Problem(n, both[0], both[1], H, F, 3, dtype=dtype, k=2, threshold=100, build_parts=True, scale=scale)
+    if scale == 1.0:
+        return _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
+    # d = sum exp(e - m) with |e| up to 500: an ulp of e is 2^-15, and that is the relative error of its exponential
+    d, f = p.dev, p.oracle_fwd()
+    for mode in ("fused", "stateful"):
+        out, m, dd = api.gat_forward(p.graph, d["feat"], d["el"], d["er"], 0.2, mode=mode)[:3]
+        has = np.isfinite(f.m)
+        assert np.array_equal(np.isfinite(m.cpu().numpy()), has)
+        allclose_report(m.cpu().numpy()[has], f.m[has], 2.0 ** -23, 0.0, "m")
+        allclose_report(dd.cpu().numpy(), f.d, 2.0 ** -14, 0.0, "d")
+        allclose_report(out.float().cpu().numpy(), f.out, 2.0 ** -7, 2.0 ** -9, "out")
+
+
 @pytest.mark.parametrize("F", [1, 3, 47, 48, 127, 180, 260, 1030])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("n", [1500, 40_000])
