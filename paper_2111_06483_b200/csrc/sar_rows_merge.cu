@@ -1,7 +1,12 @@
-// Long rows, from their segments' records (see sar_rows_kernel.cuh): one block per long row.  The records of a hub row
-// (hundreds) are read by several streams of threads at once - a thread holds one float4 column of every kStreams-th
-// record - and the streams are added up in shared memory in a fixed order, so a result does not depend on the schedule.
-// Large workload, three merges of a layer (0.28-0.30 ms each with one lane group per long row walking all its records).
+// Long rows, from their segments' records (see sar_rows_kernel.cuh).  Most long rows have a handful of segments, and what their
+// merge costs is a chain of loads (which row, its records' statistics, its records), not the bytes: so a row of up to
+// kMergeFew segments is one warp's, four of them to a block, and its loads go out together.  With a block of 128 threads per
+// row, whatever its length, and a warp per row and head for the destination-major records, the three merges of 8 heads of 32
+// (1 million nodes, 200 edges per node, 575,000 segments) took 0.48, 0.50 and 0.29 ms, now 0.32, 0.08 and 0.19; the forward merge of 2 heads of
+// 64 (233,000 nodes, 11.6 million edges) 17 us, now 10.5.
+// The records of a hub row (hundreds) are read by all threads of the block, by several streams at once - a thread holds one
+// float4 column of every kStreams-th record - and the streams are added up in shared memory in a fixed order, so a result does
+// not depend on the schedule.
 #include "sar_dispatch.cuh"
 #include "sar_rows.cuh"
 
@@ -51,7 +56,130 @@ __device__ __forceinline__ float4 merge_columns(const RowArgs &a, long long s0, 
     return x;
 }
 
-// MODE: kRowFwd / kRowFwdPart, kRowSrc, kRowSum
+// One column (float4 x, its first float c of the padded row) of a finished row; what a forward row needs besides: its
+// denominator d and the factor `old` of the state's numerator.
+template <typename T, int MODE>
+__device__ __forceinline__ void merge_finish(const RowArgs &a, long long row, int c, const float4 &x, float d, float old) {
+    const bool first = a.flags & SAR_FIRST, last = a.flags & SAR_LAST;
+    T *out = reinterpret_cast<T *>(a.out);
+    if constexpr (MODE == kRowFwd) {
+        merge_store<T>(a, row, c, x, [&](long long o, int, float y) {
+            if (!first) y += a.acc[o] * old;
+            if (!last || (a.flags & SAR_KEEP_NUMERATOR)) a.acc[o] = y;
+            if (last) {
+                y *= d > 0.f ? 1.f / d : 0.f;
+                Elem<T>::store1(out + o, (a.flags & SAR_RELU_OUT) ? fmaxf(y, 0.f) : y);
+            }
+        });
+    } else if constexpr (MODE == kRowSrc) {
+        merge_store<T>(a, row, c, x, [&](long long o, int, float y) { Elem<T>::store1(out + o, y); });
+    } else {
+        const float ds = a.dst_scale ? a.dst_scale[row] : 1.f;
+        float inv = 1.f;
+        if ((a.flags & SAR_MEAN) && last) inv = a.deg[row] > 0 ? 1.f / (float)a.deg[row] : 0.f;
+        merge_store<T>(a, row, c, x, [&](long long o, int, float y) {
+            y *= ds;
+            if (!first) {
+                if constexpr (sizeof(T) == 4) y += out[o];
+                else y += __bfloat162float(out[o]);
+            }
+            y *= inv;
+            if (a.mix.x0 && last)
+                y = (a.mix.keep * Elem<T>::load1(reinterpret_cast<const T *>(a.mix.x0) + o) + a.mix.scale * y) * (a.mix.post ? a.mix.post[row] : 1.f);
+            Elem<T>::store1(out + o, y);
+        });
+    }
+}
+
+// A row of up to kMergeFew records and (forward, source-major) kMergeHeads heads, by one warp: a lane is a record for the
+// statistics and a float4 column, or several, for the sums.
+constexpr int kMergeFew = 16, kMergeHeads = 16;
+// long rows of a block; a sum has no statistics to wait for, and there a block per row is faster (2.45 million rows of 1 KB 55 us against 57 to 80)
+template <int MODE>
+struct MergeRows {
+    static constexpr int n = MODE == kRowSum ? 1 : kMergeThreads / 32;
+};
+template <typename T, int MODE>
+__device__ __forceinline__ void merge_few(const RowArgs &a, long long row, long long s0, int n, float (*fac)[kMergeHeads], float *sM, float *sD, float *sOld) {
+    constexpr int EPV = Elem<T>::EPV;
+    constexpr bool kF = MODE == kRowFwd;
+    const int lane = threadIdx.x & 31;
+    const int rowf = a.H * a.vph * EPV;
+    const bool first = a.flags & SAR_FIRST;
+    // two columns of four records at a time; the first ones are asked for before the statistics are there
+    float4 r[2][4];
+    auto ask = [&](int c, int s) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c + j * 128 < rowf && s + u < n) r[j][u] = *reinterpret_cast<const float4 *>(a.sp.part + (s0 + s + u) * a.sp.pstride + c + j * 128);
+    };
+    ask(lane * 4, 0);
+    const float *rec = a.sp.part + (s0 + (lane < n ? lane : n - 1)) * a.sp.pstride + rowf;
+    if constexpr (kF) {
+        for (int h0 = 0; h0 < a.H; h0 += 4) {
+            float m[4], d[4], mo[4], dold[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int h = h0 + k < a.H ? h0 + k : a.H - 1;
+                m[k] = rec[h];
+                d[k] = lane < n ? rec[a.H + h] : 0.f;
+                mo[k] = first ? SAR_NEG_INF : a.m_io[row * a.H + h];
+                dold[k] = first ? 0.f : a.d_io[row * a.H + h];
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float M = m[k];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+                const float mn = fmaxf(M, mo[k]), f = fast_exp(m[k] - mn);
+                float s = d[k] * f;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                const float fo = mo[k] == mn ? 1.f : fast_exp(mo[k] - mn);
+                if (h0 + k < a.H) {
+                    if (lane < n) fac[lane][h0 + k] = f;
+                    if (lane == 0) {
+                        sM[h0 + k] = mn;
+                        sD[h0 + k] = s + dold[k] * fo;
+                        sOld[h0 + k] = fo;
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        if (lane < a.H) {
+            a.m_io[row * a.H + lane] = sM[lane];
+            a.d_io[row * a.H + lane] = sD[lane];
+        }
+    }
+    if constexpr (MODE == kRowSrc) {
+        for (int h = 0; h < a.H; ++h) {
+            float d = lane < n ? rec[h] : 0.f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (lane == 0) a.dscal[row * a.H + h] = d;
+        }
+    }
+    for (int c = lane * 4; c < rowf; c += 256) {
+        const int head[2] = {c / (a.vph * EPV), (c + 128) / (a.vph * EPV)};
+        float4 x[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+        for (int s = 0; s < n; s += 4) {
+            if (c != lane * 4 || s > 0) ask(c, s);
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (c + j * 128 < rowf && s + u < n) add4(x[j], r[j][u], kF ? fac[s + u][head[j]] : 1.f);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (c + j * 128 < rowf) merge_finish<T, MODE>(a, row, c + j * 128, x[j], kF ? sD[head[j]] : 0.f, kF ? sOld[head[j]] : 0.f);
+    }
+}
+
+// MODE: kRowFwd, kRowSrc, kRowSum.  A block has MergeRows long rows, a warp each; then those of more records together.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs a) {
     constexpr int EPV = Elem<T>::EPV;
@@ -59,126 +187,130 @@ __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs
     after_predecessor();
     __shared__ float4 red[kMergeThreads];
     __shared__ float sM[SAR_MAX_HEADS], sD[SAR_MAX_HEADS], sOld[SAR_MAX_HEADS];
+    __shared__ float fac[MergeRows<MODE>::n][kF ? kMergeFew : 1][kMergeHeads], stat[MergeRows<MODE>::n][3][kMergeHeads];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long row = a.sp.long_row[blockIdx.x];
-    const long long s0 = a.sp.long_seg[blockIdx.x], s1 = a.sp.long_seg[blockIdx.x + 1];
     const int rowf = a.H * a.vph * EPV;
-    const bool first = a.flags & SAR_FIRST, last = a.flags & SAR_LAST;
-
-    if constexpr (kF) {   // statistics of the row: a warp per head
-        for (int h = warp; h < a.H; h += kMergeThreads / 32) {
-            float M = SAR_NEG_INF;
-            for (long long s = s0 + lane; s < s1; s += 32) M = fmaxf(M, a.sp.part[s * a.sp.pstride + rowf + h]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-            const float m_old = first ? SAR_NEG_INF : a.m_io[row * a.H + h], d_old = first ? 0.f : a.d_io[row * a.H + h];
-            const float mn = fmaxf(M, m_old);
-            float d = 0.f;
-            for (long long s = s0 + lane; s < s1; s += 32) {
-                const float *rec = a.sp.part + s * a.sp.pstride + rowf;
-                d += rec[a.H + h] * fast_exp(rec[h] - mn);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-            const float fo = m_old == mn ? 1.f : fast_exp(m_old - mn);
-            d += d_old * fo;
-            if (lane == 0) {
-                sM[h] = mn;
-                sD[h] = d;
-                sOld[h] = fo;
-            }
-        }
+    const bool first = a.flags & SAR_FIRST;
+    constexpr int kRows = MergeRows<MODE>::n;
+    const int lr0 = (int)blockIdx.x * kRows;
+    auto few = [&](int lr, long long &s0, long long &s1) {
+        s0 = a.sp.long_seg[lr];
+        s1 = a.sp.long_seg[lr + 1];
+        return MODE != kRowSum && s1 - s0 <= kMergeFew && a.H <= kMergeHeads;
+    };
+    if constexpr (MODE != kRowSum) {
+        const int lr = lr0 + warp;
+        long long s0, s1;
+        if (lr < a.sp.n_long && few(lr, s0, s1))
+            merge_few<T, MODE>(a, a.sp.long_row[lr], s0, (int)(s1 - s0), fac[warp], stat[warp][0], stat[warp][1], stat[warp][2]);
+    }
+    for (int lr = lr0; lr < lr0 + kRows && lr < a.sp.n_long; ++lr) {
+        long long s0, s1;
+        if (few(lr, s0, s1)) continue;
+        const long long row = a.sp.long_row[lr];
         __syncthreads();
-        if (tid < a.H) {
-            a.m_io[row * a.H + tid] = sM[tid];
-            a.d_io[row * a.H + tid] = sD[tid];
-        }
-    }
-    if constexpr (MODE == kRowSrc) {
-        for (int h = warp; h < a.H; h += kMergeThreads / 32) {
-            float d = 0.f;
-            for (long long s = s0 + lane; s < s1; s += 32) d += a.sp.part[s * a.sp.pstride + rowf + h];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-            if (lane == 0) a.dscal[row * a.H + h] = d;
-        }
-    }
 
-    const int cols = rowf / 4;
-    const int cols_pad = cols < kMergeThreads ? cols : kMergeThreads;
-    const int streams = (kMergeThreads / cols_pad) < (int)(s1 - s0) ? kMergeThreads / cols_pad : (int)(s1 - s0);
-    const int col = tid % cols_pad, stream = tid / cols_pad;
-    for (int c0 = 0; c0 < cols; c0 += cols_pad) {
-        const bool in = c0 + col < cols && stream < streams;
-        const int c = in ? (c0 + col) * 4 : 0;
-        const int head = c / (a.vph * EPV);
-        const float4 x = merge_columns(a, in ? s0 : s1, s1, c, stream, streams, red, cols_pad, col, [&](long long s) {
-            if constexpr (kF) return fast_exp(a.sp.part[s * a.sp.pstride + rowf + head] - sM[head]);
-            else return 1.f;
-        });
-        if (!in || stream != 0) continue;
-        T *out = reinterpret_cast<T *>(a.out);
-        if constexpr (kF) {
-            merge_store<T>(a, row, c, x, [&](long long o, int h, float y) {
-                if (!first) y += a.acc[o] * sOld[h];
-                if (!last || (a.flags & SAR_KEEP_NUMERATOR)) a.acc[o] = y;
-                if (last) {
-                    y *= sD[h] > 0.f ? 1.f / sD[h] : 0.f;
-                    Elem<T>::store1(out + o, (a.flags & SAR_RELU_OUT) ? fmaxf(y, 0.f) : y);
+        if constexpr (kF) {   // statistics of the row: a warp per head
+            for (int h = warp; h < a.H; h += kMergeThreads / 32) {
+                float M = SAR_NEG_INF;
+                for (long long s = s0 + lane; s < s1; s += 32) M = fmaxf(M, a.sp.part[s * a.sp.pstride + rowf + h]);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+                const float m_old = first ? SAR_NEG_INF : a.m_io[row * a.H + h], d_old = first ? 0.f : a.d_io[row * a.H + h];
+                const float mn = fmaxf(M, m_old);
+                float d = 0.f;
+                for (long long s = s0 + lane; s < s1; s += 32) {
+                    const float *rec = a.sp.part + s * a.sp.pstride + rowf;
+                    d += rec[a.H + h] * fast_exp(rec[h] - mn);
                 }
-            });
-        } else if constexpr (MODE == kRowSrc) {
-            merge_store<T>(a, row, c, x, [&](long long o, int, float y) { Elem<T>::store1(out + o, y); });
-        } else {
-            const float ds = a.dst_scale ? a.dst_scale[row] : 1.f;
-            float inv = 1.f;
-            if ((a.flags & SAR_MEAN) && last) inv = a.deg[row] > 0 ? 1.f / (float)a.deg[row] : 0.f;
-            merge_store<T>(a, row, c, x, [&](long long o, int, float y) {
-                y *= ds;
-                if (!first) {
-                    if constexpr (sizeof(T) == 4) y += out[o];
-                    else y += __bfloat162float(out[o]);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+                const float fo = m_old == mn ? 1.f : fast_exp(m_old - mn);
+                d += d_old * fo;
+                if (lane == 0) {
+                    sM[h] = mn;
+                    sD[h] = d;
+                    sOld[h] = fo;
                 }
-                y *= inv;
-                if (a.mix.x0 && last)
-                    y = (a.mix.keep * Elem<T>::load1(reinterpret_cast<const T *>(a.mix.x0) + o) + a.mix.scale * y) * (a.mix.post ? a.mix.post[row] : 1.f);
-                Elem<T>::store1(out + o, y);
+            }
+            __syncthreads();
+            if (tid < a.H) {
+                a.m_io[row * a.H + tid] = sM[tid];
+                a.d_io[row * a.H + tid] = sD[tid];
+            }
+        }
+        if constexpr (MODE == kRowSrc) {
+            for (int h = warp; h < a.H; h += kMergeThreads / 32) {
+                float d = 0.f;
+                for (long long s = s0 + lane; s < s1; s += 32) d += a.sp.part[s * a.sp.pstride + rowf + h];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+                if (lane == 0) a.dscal[row * a.H + h] = d;
+            }
+        }
+
+        const int cols = rowf / 4;
+        const int cols_pad = cols < kMergeThreads ? cols : kMergeThreads;
+        const int streams = (kMergeThreads / cols_pad) < (int)(s1 - s0) ? kMergeThreads / cols_pad : (int)(s1 - s0);
+        const int col = tid % cols_pad, stream = tid / cols_pad;
+        for (int c0 = 0; c0 < cols; c0 += cols_pad) {
+            const bool in = c0 + col < cols && stream < streams;
+            const int c = in ? (c0 + col) * 4 : 0;
+            const int head = c / (a.vph * EPV);
+            const float4 x = merge_columns(a, in ? s0 : s1, s1, c, stream, streams, red, cols_pad, col, [&](long long s) {
+                if constexpr (kF) return fast_exp(a.sp.part[s * a.sp.pstride + rowf + head] - sM[head]);
+                else return 1.f;
             });
+            if (!in || stream != 0) continue;
+            merge_finish<T, MODE>(a, row, c, x, kF ? sD[head] : 0.f, kF ? sOld[head] : 0.f);
         }
     }
 }
 
-// Destination-major: D, B and S of the segments are numbers; a warp per long row and head.
+// Destination-major: D, B and S of the segments are numbers, 3 H of them one after the other in a record; a warp per long row, a
+// lane per number (of the heads h0 .. h0 + 9, so that they fit a warp), half a warp per record where 15 lanes do.
 template <bool PART>
 __global__ void __launch_bounds__(kMergeThreads) rows_dst_merge_kernel(const RowArgs a) {
     after_predecessor();
     const int lane = threadIdx.x & 31;
-    const long long item = (long long)blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5);
-    const int lr = (int)(item / a.H), h = (int)(item % a.H);
+    const long long lr = (long long)blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5);
     if (lr >= a.sp.n_long) return;
-    const long long row = a.sp.long_row[lr], s1 = a.sp.long_seg[lr + 1];
-    float D = 0.f, Bs = 0.f, S = 0.f;
-    for (long long s = a.sp.long_seg[lr] + lane; s < s1; s += 32) {
-        const float *rec = a.sp.part + s * a.sp.pstride;
-        if (!PART) D += rec[h];
-        Bs += rec[a.H + h];
-        S += rec[2 * a.H + h];
-    }
+    const long long row = a.sp.long_row[lr], s0 = a.sp.long_seg[lr], s1 = a.sp.long_seg[lr + 1];
+    for (int h0 = 0; h0 < a.H; h0 += 10) {
+        const int H = min(a.H - h0, 10), lanes = H <= 5 ? 16 : 32, at = lane & (lanes - 1);
+        const int q = at / H, h = at - q * H;   // number q (D, B, S) of head h0 + h
+        float x = 0.f;
+        if (q < 3 && !(PART && q == 0)) {
+            float part[8];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        if (!PART) D += __shfl_xor_sync(0xffffffffu, D, o);
-        Bs += __shfl_xor_sync(0xffffffffu, Bs, o);
-        S += __shfl_xor_sync(0xffffffffu, S, o);
-    }
-    if (lane == 0) {
-        const long long o = row * a.H + h;
-        if (PART) {
-            const float x = Bs - a.rec[o].w * S;
-            a.dscal[o] = (a.flags & SAR_FIRST) ? x : a.dscal[o] + x;
-        } else {
-            const float dd = a.d[o];
-            a.dscal[o] = Bs - D * S;
-            a.rec[o] = make_float4(a.el[o], a.m[o], dd > 0.f ? __fdividef(1.f, dd) : 0.f, D);
+            for (int u = 0; u < 8; ++u) part[u] = 0.f;
+            const int step = 32 / lanes;
+            const float *p = a.sp.part + q * a.H + h0 + h;
+            long long s = s0 + lane / lanes;
+            for (; s + 7LL * step < s1; s += 8LL * step) {
+                float r[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) r[u] = p[(s + u * step) * a.sp.pstride];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) part[u] += r[u];
+            }
+#pragma unroll
+            for (int u = 0; u < 7; ++u)
+                if (s + u * step < s1) part[u] += p[(s + u * step) * a.sp.pstride];
+            x = ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
+        }
+        if (lanes == 16) x += __shfl_xor_sync(0xffffffffu, x, 16);
+        const float D = x, Bs = __shfl_sync(0xffffffffu, x, (lane + H) & 31), S = __shfl_sync(0xffffffffu, x, (lane + 2 * H) & 31);
+        if (lane < H) {
+            const long long o = row * a.H + h0 + lane;
+            if (PART) {
+                const float y = Bs - a.rec[o].w * S;
+                a.dscal[o] = (a.flags & SAR_FIRST) ? y : a.dscal[o] + y;
+            } else {
+                const float dd = a.d[o];
+                a.dscal[o] = Bs - D * S;
+                a.rec[o] = make_float4(a.el[o], a.m[o], dd > 0.f ? __fdividef(1.f, dd) : 0.f, D);
+            }
         }
     }
 }
@@ -214,10 +346,11 @@ __global__ void __launch_bounds__(256) rows_finalize_kernel(const RowArgs a) {
 
 template <int MODE>
 static sar_status launch_merge(const RowArgs &a, sar_dtype t, const char *name, cudaStream_t st) {
+    const unsigned blocks = (unsigned)((a.sp.n_long + MergeRows<MODE>::n - 1) / MergeRows<MODE>::n);
     if (t == SAR_F32)
-        SAR_LAUNCH(name, st, launch(rows_merge_kernel<float, MODE>, (unsigned)a.sp.n_long, kMergeThreads, 0, st, a));
+        SAR_LAUNCH(name, st, launch(rows_merge_kernel<float, MODE>, blocks, kMergeThreads, 0, st, a));
     else
-        SAR_LAUNCH(name, st, launch(rows_merge_kernel<__nv_bfloat16, MODE>, (unsigned)a.sp.n_long, kMergeThreads, 0, st, a));
+        SAR_LAUNCH(name, st, launch(rows_merge_kernel<__nv_bfloat16, MODE>, blocks, kMergeThreads, 0, st, a));
     return sar_after_launch();
 }
 
@@ -235,8 +368,7 @@ sar_status rows_fwd_finalize(const RowArgs &a, sar_dtype t, cudaStream_t st) {
 }
 
 sar_status rows_dst_merge(const RowArgs &a, bool part, cudaStream_t st) {
-    const long long warps = (long long)a.sp.n_long * a.H;
-    const unsigned blocks = (unsigned)((warps + kMergeThreads / 32 - 1) / (kMergeThreads / 32));
+    const unsigned blocks = (unsigned)((a.sp.n_long + kMergeThreads / 32 - 1) / (kMergeThreads / 32));
     if (part)
         SAR_LAUNCH("gat_bwd_dst_merge", st, launch(rows_dst_merge_kernel<true>, blocks, kMergeThreads, 0, st, a));
     else

@@ -73,6 +73,23 @@ def test_attention_of_a_row_per_lane_group(H, F, dtype, scale):
         allclose_report(out.float().cpu().numpy(), f.out, 2.0 ** -7, 2.0 ** -9, "out")
 
 
+@pytest.mark.parametrize("H,F,dtype", [(1, 64, "bf16"), (5, 8, "f32"), (6, 24, "bf16"), (10, 16, "f32"), (11, 8, "bf16"), (16, 32, "f32"),
+                                       (17, 8, "f32"), (1, 1030, "bf16")])
+def test_merges_on_either_side_of_what_a_warp_takes(H, F, dtype):
+    """Rows of 2 to 18, 33 and 40 segments next to each other (a warp merges up to 16, a block more), of a number that does not fill the
+    last block, with heads on either side of what one step of the destination-major merge (5 and 10) and a warp (16) take."""
+    n, size, gen = 900, 20, torch.Generator().manual_seed(H)
+    src, dst = [torch.randint(0, n, (3 * n,), generator=gen)], [torch.randint(100, n, (3 * n,), generator=gen)]
+    for i, segs in enumerate([2, 16, 17, 3, 15, 16, 18, 33, 16, 1, 4, 40, 8, 9]):
+        for row, deg in ((3 * i, segs * size), (3 * i + 1, segs * size - 1)):
+            src.append(torch.randint(100, n, (deg,), generator=gen))
+            dst.append(torch.full((deg,), row))
+    src, dst = torch.cat(src).int(), torch.cat(dst).int()
+    both = torch.cat([src, dst]), torch.cat([dst, src])   # long rows among the columns, which the source-major pass walks
+    p = Problem(n, both[0], both[1], H, F, 5, dtype=dtype, k=2, threshold=size, build_parts=True)
+    _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=max(10.0, F / 64))
+
+
 @pytest.mark.parametrize("F", [1, 3, 47, 48, 127, 180, 260, 1030])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("n", [1500, 40_000])
