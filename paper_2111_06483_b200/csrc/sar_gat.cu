@@ -153,23 +153,50 @@ static sar_status propagate_start(long long n, int F, const RowShape &r, sar_dty
         SAR_LAUNCH("propagate_start", st, launch(propagate_start_kernel<__nv_bfloat16>, blocks, 256, 0, st, vecs, F, r.vph, static_cast<const __nv_bfloat16 *>(in), scale, p, s));
     return sar_after_launch();
 }
-// padded rows -> rows of F elements; one element per thread
-template <typename T>
+// padded rows -> rows of F elements.  Sixteen bytes of the result per thread where it is aligned, else an element; the index of
+// the row by a 32-bit division where there are no more than 2^32 elements.  Bound by that index arithmetic, not by the bytes, with
+// an element per thread and 64 bits: 500,000 rows of 47 float32 100 us, now 34 (each with some 6 us of its launch; the bytes 29).
+template <typename T, typename I, int N>
 __global__ void __launch_bounds__(256) strip_rows_kernel(long long elems, int F, int pitch, const T *__restrict__ in, T *__restrict__ out) {
     after_predecessor();
-    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    const long long i = ((long long)blockIdx.x * 256 + threadIdx.x) * N;
     if (i >= elems) return;
-    const long long row = i / F;
-    out[i] = in[row * pitch + (i - row * F)];
+    long long row = (I)i / (I)F;
+    int at = (int)((I)i - (I)row * (I)F);
+    alignas(16) T x[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        if (i + k < elems) x[k] = in[row * pitch + at];
+        if (++at == F) {
+            at = 0;
+            ++row;
+        }
+    }
+    if (N > 1 && i + N <= elems) {
+        *reinterpret_cast<uint4 *>(out + i) = *reinterpret_cast<const uint4 *>(x);
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (i + k < elems) out[i + k] = x[k];
+    }
+}
+template <typename T>
+static sar_status strip_rows_as(long long elems, int F, int pitch, const void *in, void *out, cudaStream_t st) {
+    constexpr int N = 16 / sizeof(T);
+    const T *p = static_cast<const T *>(in);
+    T *o = static_cast<T *>(out);
+    const unsigned blocks = (unsigned)((elems + 255) / 256), blocks_n = (unsigned)((elems + 256 * N - 1) / (256 * N));
+    if (elems + N > 0xffffffffLL)
+        SAR_LAUNCH("strip_rows", st, launch(strip_rows_kernel<T, unsigned long long, 1>, blocks, 256, 0, st, elems, F, pitch, p, o));
+    else if (sar_aligned(out, 16))
+        SAR_LAUNCH("strip_rows", st, launch(strip_rows_kernel<T, unsigned, N>, blocks_n, 256, 0, st, elems, F, pitch, p, o));
+    else
+        SAR_LAUNCH("strip_rows", st, launch(strip_rows_kernel<T, unsigned, 1>, blocks, 256, 0, st, elems, F, pitch, p, o));
+    return sar_after_launch();
 }
 static sar_status strip_rows(long long n, int F, const RowShape &r, sar_dtype t, const void *in, void *out, cudaStream_t st) {
-    const unsigned blocks = (unsigned)((n * F + 255) / 256);
     const int pitch = (int)(r.row_bytes / sar_elem_size(t));
-    if (t == SAR_F32)
-        SAR_LAUNCH("strip_rows", st, launch(strip_rows_kernel<float>, blocks, 256, 0, st, n * F, F, pitch, static_cast<const float *>(in), static_cast<float *>(out)));
-    else
-        SAR_LAUNCH("strip_rows", st, launch(strip_rows_kernel<__nv_bfloat16>, blocks, 256, 0, st, n * F, F, pitch, static_cast<const __nv_bfloat16 *>(in), static_cast<__nv_bfloat16 *>(out)));
-    return sar_after_launch();
+    return t == SAR_F32 ? strip_rows_as<float>(n * F, F, pitch, in, out, st) : strip_rows_as<__nv_bfloat16>(n * F, F, pitch, in, out, st);
 }
 
 // ---- workspace layout ---------------------------------------------------------------------------

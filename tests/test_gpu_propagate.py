@@ -76,3 +76,22 @@ def test_propagation_takes_one_array_beside_its_result():
     before = torch.cuda.memory_allocated()
     api.propagate(g, x, 0.5, 3)
     assert torch.cuda.max_memory_allocated() - before < 2.1 * x.nbytes
+
+
+@pytest.mark.parametrize("n,F", [(1, 1), (37, 3), (1001, 1), (513, 2), (129, 5), (77, 7), (640, 8), (255, 47), (33, 301)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_rows_of_a_ragged_or_misaligned_result(n, F, dtype, shift):
+    """(1 - 0) x0 + 0 sum is x0 to the bit: every element of the result is written, at its place, and none beside it."""
+    from paper_2111_06483_b200 import binding as B
+    gen = torch.Generator().manual_seed(n)
+    src, dst = (torch.randint(0, n, (3 * n,), generator=gen, dtype=torch.int32).to(DEV) for _ in range(2))
+    g = api.Graph.from_coo(n, src, dst)
+    x = torch.randn((n, F), generator=gen).to(dtype).to(DEV)
+    buf = torch.full((shift + n * F + 16,), 7.0, dtype=dtype, device=DEV)
+    out = buf[shift:shift + n * F].view(n, F)
+    t = B.SAR_F32 if dtype == torch.float32 else B.SAR_BF16
+    ws = torch.empty(B.sar_propagate_workspace_bytes([g.whole], F, t), dtype=torch.uint8, device=DEV)
+    B.sar_propagate([g.whole], g.bounds, x, 0.0, 2, None, None, out, ws)
+    assert torch.equal(out, x)
+    assert bool((buf[:shift] == 7.0).all()) and bool((buf[shift + n * F:] == 7.0).all())
