@@ -327,11 +327,31 @@ static bool sum_takes_short(const RowGeo &geo, long long n_gathered, unsigned ro
                                                      : !hubs && bytes <= kSpanSumBytes ? 12 : 0;
     return few_edges(limit, n_rows, nnz);
 }
-// A sum has nothing between its ids and its rows, and there the ring is ahead much earlier: 100,000 nodes of 128 bytes 0.172
-// against 0.175 ms, 500,000 of 192 bytes 0.67 against 0.72 ms, 2.45 million of 1 KB 12.5 against 15.0 ms; below that the row
-// kernels' smaller start counts.
-static bool sum_takes_span(const Shape &s, long long n_gathered) {
-    return s.fast && (unsigned long long)n_gathered * s.row_bytes > kSpanSumBytes;
+// A sum has nothing between its ids and its rows.  Where the L2 doesn't hold the array the span kernels' ring keeps more loads in
+// flight (2.45 million rows of 1 KB 12.5 against 15.0 ms, 500,000 of 192 bytes with 20 edges each and hubs 0.67 against 0.72); where it does,
+// and a row has a dozen edges or more to spread the start of a row over, the row kernels issue less per edge.  They lose by
+// less than that the more edges a row has, so the line is a number of MB per edge of the mean row (up to 32 edges, 100 MB in all).  Over
+// 782 sizes of array, rows and graph, span / row on the row kernels' side of the line:
+//  * float32, rows of 144 to 512 bytes other than 256 (the span kernels leave lanes idle): plain 0.98 to 1.90, 1.35 in the median,
+//    weighted 1.05 to 1.83 / 1.46, with the propagation's mix 1.04 to 1.70 / 1.31; with long rows, whose hubs make the row kernels
+//    wait, 1.00 to 1.59 / 1.2 to 1.3; bf16 0.97 to 1.54 / 1.1 to 1.23.
+//  * rows of 528 to 768 bytes, no long rows, in up to 40 MB: float32 1.12 to 1.70 / 1.4, bf16 weighted 1.08 to 1.30.
+//  * rows of 128 and 256 bytes, full lanes in either: half the MB, 0.97 to 1.41 / 1.1 to 1.25, no mix.
+// Beyond the line 0.55 to 1.1.
+static bool sum_takes_rows(const RowArgs &a, sar_dtype t, long long n_gathered, long long nnz, bool weighted) {
+    const int vecs = (int)(a.row_bytes / 16);
+    const bool hubs = a.sp.n_long > 0, mix = a.mix.x0 != nullptr, f32 = t == SAR_F32;
+    if (vecs < 8 || vecs > 48 || nnz < (hubs ? 20 : 12) * a.n_rows) return false;
+    double mb = f32 ? (mix ? (hubs ? 1.25 : 1.8) : weighted ? (hubs ? 3.2 : 5.0) : hubs ? 2.5 : 3.2)
+                    : (mix ? (hubs ? 0.0 : 0.9) : weighted ? (hubs ? 1.5 : 2.4) : hubs ? 1.0 : 1.9);
+    if (vecs == 8 || vecs == 16) mb = mix || (!f32 && (!weighted || hubs)) ? 0.0 : 0.5 * mb;
+    else if (vecs > 32 && (hubs || (!f32 && (!weighted || mix)))) mb = 0.0;
+    else if (vecs < 16 && hubs && !f32 && !weighted) mb = 0.0;
+    const double mean = (double)nnz / (double)a.n_rows, most = vecs > 32 ? 40.0 : 100.0, line = mb * (mean < 32.0 ? mean : 32.0);
+    return (double)n_gathered * a.row_bytes <= (line < most ? line : most) * 1e6;
+}
+static bool sum_takes_span(const Shape &s, const RowArgs &a, sar_dtype t, long long n_gathered, long long nnz, bool weighted) {
+    return s.fast && (unsigned long long)n_gathered * s.row_bytes > kSpanSumBytes && !sum_takes_rows(a, t, n_gathered, nnz, weighted);
 }
 
 static sar_status check_shape(int32_t H, int32_t F, sar_dtype t) {
@@ -799,7 +819,7 @@ static sar_status sum_rows(const sar_part *g, const RowShape &r, int32_t F, sar_
     Shape s;
     SAR_TRY(make_shape(1, F, t, !r.ragged, &s));
     a.lone = sum_takes_short(r.geo, g->n_src, r.row_bytes, g->n_dst, g->nnz, a.sp.n_long > 0);
-    if (!a.lone && sum_takes_span(s, g->n_src))
+    if (!a.lone && sum_takes_span(s, a, t, g->n_src, g->nnz, weighted))
         SAR_TRY(span_sum(s, a, g->nnz, weighted, st));
     else
         SAR_TRY(t == SAR_F32 ? rows_sum_f32(a, r.geo, g->nnz, weighted, st) : rows_sum_bf16(a, r.geo, g->nnz, weighted, st));

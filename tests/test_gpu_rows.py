@@ -108,6 +108,28 @@ def test_sums_of_ragged_rows(F, dtype, n):
     assert torch.equal(out, (x.float() + 4.0 * want).to(x.dtype))
 
 
+@pytest.mark.parametrize("F,dtype", [(32, "f32"), (36, "f32"), (47, "f32"), (64, "f32"), (101, "f32"), (128, "f32"), (160, "f32"), (193, "f32"),
+                                     (72, "bf16"), (100, "bf16"), (256, "bf16"), (333, "bf16")])
+@pytest.mark.parametrize("mb,deg,long", [(13, 11, False), (13, 13, False), (13, 21, True), (39, 21, False), (42, 21, False)])
+def test_sums_on_either_side_of_the_span_kernels_line(F, dtype, mb, deg, long):
+    """Arrays of 13 to 42 MB and rows of 11 to 21 edges: where the number of edges, the size of the array, weights, long rows and the mix of
+    a propagation choose between the row and the span kernels.  Whole numbers, exact in float32: one rounding where the result is bf16."""
+    tdt, size = (torch.bfloat16, 2) if dtype == "bf16" else (torch.float32, 4)
+    n = mb * 1_000_000 // ((F * size + 15) // 16 * 16)
+    gen = torch.Generator(device=DEV).manual_seed(F + deg)
+    src, dst = (torch.randint(0, n, (deg * n,), generator=gen, device=DEV, dtype=torch.int32) for _ in range(2))
+    if long:
+        dst[:300], dst[300:1200] = 5, n - 1
+    g = api.Graph.from_coo(n, src, dst, threshold=200)
+    x = (torch.arange(n * F, device=DEV).view(n, F) % 3 == 0).to(tdt)
+    scale = 2.0 ** (torch.arange(n, device=DEV) % 3 - 1).float()
+    take = lambda y: torch.zeros(n, F, device=DEV).index_add_(0, dst.long(), y[src.long()])
+    want = take(x.float() * scale[:, None]) * scale[:, None]
+    assert torch.equal(api.spmm_sum(g.whole, x), take(x.float()).to(tdt))
+    assert torch.equal(api.spmm_scaled(g.whole, x, src_scale=scale, dst_scale=scale), want.to(tdt))
+    assert torch.equal(api.propagate(g, x, 0.5, 1, scale, scale), (0.5 * x.float() + 0.5 * want).to(tdt))
+
+
 def test_ragged_shape_without_room_for_padded_copies():
     """No workspace in the forward call, one that holds the records alone in the backward call: the scalar kernels."""
     n, src, dst = hub_graph(n=500, e=6000, d_max=100.0, seed=3)
