@@ -1,8 +1,9 @@
 // Long rows, from their segments' records (see sar_rows_kernel.cuh).  Most long rows have a handful of segments, and what their
-// merge costs is a chain of loads (which row, its records' statistics, its records), not the bytes: so a row of up to
-// kMergeFew segments is one warp's, four of them to a block, and its loads go out together.  With a block of 128 threads per
+// merge costs is a chain of loads (which row, its records' statistics, its records), not the bytes: so where there are more long
+// rows than a couple of blocks per SM, a row of up to kMergeFew segments is one warp's, four of them to a block, and its loads go out
+// together.  With a block of 128 threads per
 // row, whatever its length, and a warp per row and head for the destination-major records, the three merges of 8 heads of 32
-// (1 million nodes, 200 edges per node, 575,000 segments) took 0.48, 0.50 and 0.29 ms, now 0.32, 0.08 and 0.19; the forward merge of 2 heads of
+// (1 million nodes, 200 edges per node, 575,000 segments) took 0.48, 0.50 and 0.29 ms, now 0.30, 0.08 and 0.19; the forward merge of 2 heads of
 // 64 (233,000 nodes, 11.6 million edges) 17 us, now 10.5.
 // The records of a hub row (hundreds) are read by all threads of the block, by several streams at once - a thread holds one
 // float4 column of every kStreams-th record - and the streams are added up in shared memory in a fixed order, so a result does
@@ -93,8 +94,11 @@ __device__ __forceinline__ void merge_finish(const RowArgs &a, long long row, in
 
 // A row of up to kMergeFew records and (forward, source-major) kMergeHeads heads, by one warp: a lane is a record for the
 // statistics and a float4 column, or several, for the sums.
-constexpr int kMergeFew = 16, kMergeHeads = 16;
-// long rows of a block; a sum has no statistics to wait for, and there a block per row is faster (2.45 million rows of 1 KB 55 us against 57 to 80)
+constexpr int kMergeFew = 32, kMergeHeads = 16;
+// With up to two blocks per SM a block per row is as fast or faster: 128 rows of 6 segments, 8 heads of 48 bf16, source-major 8.6
+// against 10.6 us; 592 rows 12.6 against 10.7, 9600 rows 56 against 50 and forward 85 against 55.
+constexpr int kMergeMany = 296;
+// the most long rows of a block; a sum has no statistics to wait for, and there a block per row is faster (2.45 million rows of 1 KB 55 us against 57 to 80)
 template <int MODE>
 struct MergeRows {
     static constexpr int n = MODE == kRowSum ? 1 : kMergeThreads / 32;
@@ -179,7 +183,10 @@ __device__ __forceinline__ void merge_few(const RowArgs &a, long long row, long 
     }
 }
 
-// MODE: kRowFwd, kRowSrc, kRowSum.  A block has MergeRows long rows, a warp each; then those of more records together.
+// long rows of a block
+static __host__ __device__ int merge_rows(int n_long, int rows) { return n_long > kMergeMany ? rows : 1; }
+
+// MODE: kRowFwd, kRowSrc, kRowSum.  A block has merge_rows long rows, a warp each; then those of more records together.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs a) {
     constexpr int EPV = Elem<T>::EPV;
@@ -191,20 +198,20 @@ __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rowf = a.H * a.vph * EPV;
     const bool first = a.flags & SAR_FIRST;
-    constexpr int kRows = MergeRows<MODE>::n;
-    const int lr0 = (int)blockIdx.x * kRows;
+    const int rows = merge_rows(a.sp.n_long, MergeRows<MODE>::n);
+    const int lr0 = (int)blockIdx.x * rows;
     auto few = [&](int lr, long long &s0, long long &s1) {
         s0 = a.sp.long_seg[lr];
         s1 = a.sp.long_seg[lr + 1];
-        return MODE != kRowSum && s1 - s0 <= kMergeFew && a.H <= kMergeHeads;
+        return rows > 1 && s1 - s0 <= kMergeFew && a.H <= kMergeHeads;
     };
     if constexpr (MODE != kRowSum) {
         const int lr = lr0 + warp;
         long long s0, s1;
-        if (lr < a.sp.n_long && few(lr, s0, s1))
+        if (warp < rows && lr < a.sp.n_long && few(lr, s0, s1))
             merge_few<T, MODE>(a, a.sp.long_row[lr], s0, (int)(s1 - s0), fac[warp], stat[warp][0], stat[warp][1], stat[warp][2]);
     }
-    for (int lr = lr0; lr < lr0 + kRows && lr < a.sp.n_long; ++lr) {
+    for (int lr = lr0; lr < lr0 + rows && lr < a.sp.n_long; ++lr) {
         long long s0, s1;
         if (few(lr, s0, s1)) continue;
         const long long row = a.sp.long_row[lr];
@@ -346,7 +353,8 @@ __global__ void __launch_bounds__(256) rows_finalize_kernel(const RowArgs a) {
 
 template <int MODE>
 static sar_status launch_merge(const RowArgs &a, sar_dtype t, const char *name, cudaStream_t st) {
-    const unsigned blocks = (unsigned)((a.sp.n_long + MergeRows<MODE>::n - 1) / MergeRows<MODE>::n);
+    const int rows = merge_rows(a.sp.n_long, MergeRows<MODE>::n);
+    const unsigned blocks = (unsigned)((a.sp.n_long + rows - 1) / rows);
     if (t == SAR_F32)
         SAR_LAUNCH(name, st, launch(rows_merge_kernel<float, MODE>, blocks, kMergeThreads, 0, st, a));
     else

@@ -75,15 +75,19 @@ def test_attention_of_a_row_per_lane_group(H, F, dtype, scale):
 
 @pytest.mark.parametrize("H,F,dtype", [(1, 64, "bf16"), (5, 8, "f32"), (6, 24, "bf16"), (10, 16, "f32"), (11, 8, "bf16"), (16, 32, "f32"),
                                        (17, 8, "f32"), (1, 1030, "bf16")])
-def test_merges_on_either_side_of_what_a_warp_takes(H, F, dtype):
-    """Rows of 2 to 18, 33 and 40 segments next to each other (a warp merges up to 16, a block more), of a number that does not fill the
-    last block, with heads on either side of what one step of the destination-major merge (5 and 10) and a warp (16) take."""
+@pytest.mark.parametrize("many", [False, True])
+def test_merges_on_either_side_of_what_a_warp_takes(H, F, dtype, many):
+    """Rows of 2 to 40 segments next to each other (where there are many long rows a warp merges up to 32, a block more), of a number that does
+    not fill the last block, with heads on either side of what one step of the destination-major merge (5 and 10) and a warp (16) take."""
     n, size, gen = 900, 20, torch.Generator().manual_seed(H)
     src, dst = [torch.randint(0, n, (3 * n,), generator=gen)], [torch.randint(100, n, (3 * n,), generator=gen)]
-    for i, segs in enumerate([2, 16, 17, 3, 15, 16, 18, 33, 16, 1, 4, 40, 8, 9]):
+    for i, segs in enumerate([2, 32, 33, 3, 31, 32, 34, 65, 32, 1, 4, 40, 8, 9]):
         for row, deg in ((3 * i, segs * size), (3 * i + 1, segs * size - 1)):
             src.append(torch.randint(100, n, (deg,), generator=gen))
             dst.append(torch.full((deg,), row))
+    if many:
+        src.append(torch.randint(100, n, (300 * 2 * size,), generator=gen))
+        dst.append(torch.arange(500, 800).repeat_interleave(2 * size))
     src, dst = torch.cat(src).int(), torch.cat(dst).int()
     both = torch.cat([src, dst]), torch.cat([dst, src])   # long rows among the columns, which the source-major pass walks
     p = Problem(n, both[0], both[1], H, F, 5, dtype=dtype, k=2, threshold=size, build_parts=True)
