@@ -294,38 +294,42 @@ static bool takes_span(const Shape &s, const RowGeo &geo, long long n_gathered, 
 //    1.4 and NV = 8 0.8 to 1.0 / 0.9 to 1.1 with 20, 0.7 to 0.9 / 0.8 to 1.3 with 30.  Backward 1.1 to 5 / 1.1 to 3.8, NV = 4 up to 28
 //    edges, NV = 8 0.85 to 1.1 with 20.
 //  * NV <= 8, HP = 4: forward 0.9 to 3.2 / 1.1 to 2.0 with up to 24; backward 1.1 to 4.4 / 1.2 to 2.7 with up to 60.
-//  * HP = 8: backward 1.3 to 5.7 / 1.1 to 4.0; forward 0.96 to 3.5 / 1.0 to 2.6 with up to 30 (NV = 32, where the array fits the
-//    L2: 0.96 to 1.5 / 0.9 to 1.2 with up to 14; else 0.73 to 1.2).
-//  * NV = 16, HP = 4: forward 1.0 to 1.75 / 0.95 to 1.07 with up to 10, backward 1.1 to 2.2 / 0.95 to 1.4 with up to 16.  HP = 2: forward
-//    1.0 to 1.67 / 0.85 to 1.05, backward 1.1 to 1.9 / 0.95 to 1.5 with up to 8.  HP = 1: 1.0 to 1.5 / 0.7 to 1.0 with up to 6.
-//  * NV = 32, HP = 4, backward: 1.0 to 1.5 / 0.9 to 1.1 with up to 10; forward, and HP <= 2, 0.5 to 1.2.
-//  * Few rows do not fill the chip with groups: 10,000 rows as above with up to 0.6 of these edges, 5,000 with 0.3, 2,000
-//    with 0.12 (with twice as many 0.5 to 0.9).
-static double short_edges(const RowGeo &geo, bool backward, bool hubs, bool fits_l2) {
+//  * HP = 8: backward 1.3 to 5.7 / 1.1 to 4.0; forward 0.96 to 3.5 / 1.0 to 2.6 with up to 30 (NV = 32, in arrays of up to 32 MB:
+//    0.96 to 1.5 / 0.9 to 1.2 with up to 14; else 0.73 to 1.2).
+//  * NV = 16, HP = 4: forward 1.0 to 1.75 / 0.95 to 1.07 with up to 10, backward 1.1 to 2.2 / 0.95 to 1.4 with up to 16.
+// The rest is decided by rows of up to 100 or 240 edges, too short for segments, among ones of 2 to 20: a group waits for the longest
+// row of its warp, and the plan doesn't tell such graphs from uniform ones.
+//  * NV = 16, HP = 2: backward 1.0 to 1.24 with up to 6 (uniform up to 1.9); forward 0.84 to 1.13 and HP = 1 0.82 to 1.13 (uniform 1.0
+//    to 1.67): not taken.
+//  * NV = 32, HP = 4, backward: in arrays of up to 8 MB 1.0 to 1.23 with up to 10; of 12 MB 0.87 to 0.99, of 50 to 77 MB 0.74 to 0.89.
+//  * Few rows do not fill the chip with groups.  HP >= 4, backward: 8,000 rows as above with half of these edges (1.05 to 1.9).  Else
+//    16,000 rows with half (1.0 to 1.9; with as many 0.8 to 1.1), 8,000 with a quarter (1.0 to 1.24), with NV >= 8, HP = 1 or
+//    NV = 16, HP = 2 not (0.89 to 1.07).
+static double short_edges(const RowGeo &geo, bool backward, unsigned long long bytes) {
     const int NV = geo.NV, HP = geo.HP;
     if (NV > 32) return 0;
-    if (HP == 8) return backward ? 100 : NV <= 16 ? 40 : fits_l2 ? 14 : 0;
-    if (NV == 32) return HP == 4 && backward ? 10 : 0;
-    if (NV == 16) return HP == 4 ? (backward ? 16 : 10) : HP == 2 ? (backward || !hubs ? 8 : 0) : hubs ? 0 : 6;
+    if (HP == 8) return backward ? 100 : NV <= 16 ? 40 : bytes <= (32ull << 20) ? 14 : 0;
+    if (NV == 32) return HP == 4 && backward && bytes <= (8ull << 20) ? 10 : 0;
+    if (NV == 16) return HP == 4 ? (backward ? 16 : 10) : HP == 2 && backward ? 6 : 0;
     if (HP == 4) return backward ? 100 : 24;
     return NV == 4 ? (backward ? 28 : 20) : backward ? 16 : 14;
 }
-static bool few_edges(double limit, long long n_rows, long long nnz) {
-    const double fill = n_rows < 16000 ? (double)n_rows / 16000 : 1.0;
+// `filled`: rows with which the limit holds in full
+static bool few_edges(double limit, long long filled, long long n_rows, long long nnz) {
+    const double fill = n_rows < filled ? (double)n_rows / (double)filled : 1.0;
     return limit > 0 && nnz < (1LL << 30) && (double)nnz <= limit * fill * (double)n_rows;
 }
-static bool takes_short(const RowGeo &geo, long long n_gathered, unsigned row_bytes, long long n_rows, long long nnz, bool backward, bool hubs) {
-    const bool fits_l2 = (unsigned long long)n_gathered * row_bytes <= kSpanBytes;
-    return few_edges(short_edges(geo, backward, hubs, fits_l2), n_rows, nnz);
+static bool takes_short(const RowGeo &geo, long long n_gathered, unsigned row_bytes, long long n_rows, long long nnz, bool backward) {
+    if (n_rows < 12000 && ((geo.HP == 1 && geo.NV >= 8) || (geo.HP == 2 && geo.NV >= 16))) return false;
+    return few_edges(short_edges(geo, backward, (unsigned long long)n_gathered * row_bytes), geo.HP >= 4 && backward ? 16000 : 32000, n_rows, nnz);
 }
-// Sums, likewise: rows of 64 bytes 1.0 to 4.1 / 1.0 to 2.4 with up to 20 edges per row; of 128 bytes, in arrays of up to 12 MB 1.1
-// to 2.4 / 1.0 to 1.4 with up to 14, up to 64 MB 1.1 to 1.9 / 1.0 to 1.3 with up to 8, beyond 1.1 to 1.6 / 1.0 to 1.2 with up to 3; of 256 bytes,
-// without hubs, in arrays of up to 12 MB 1.05 to 1.5 with up to 12; else 0.6 to 1.0.
-static bool sum_takes_short(const RowGeo &geo, long long n_gathered, unsigned row_bytes, long long n_rows, long long nnz, bool hubs) {
+// Sums, likewise, from 12,000 rows on (8,000: 0.83 to 1.06): rows of 64 bytes 1.0 to 4.1 / 1.0 to 2.4 with up to 20 edges per row; of 128
+// bytes, in arrays of up to 12 MB 1.1 to 2.4 / 1.0 to 1.4 with up to 14, up to 64 MB 1.1 to 1.9 / 1.0 to 1.3 with up to 8, beyond 1.1 to
+// 1.6 / 1.0 to 1.2 with up to 3; of 256 bytes 0.91 to 1.2 (uniform up to 1.5): not taken.
+static bool sum_takes_short(const RowGeo &geo, long long n_gathered, unsigned row_bytes, long long n_rows, long long nnz) {
     const unsigned long long bytes = (unsigned long long)n_gathered * row_bytes;
-    const double limit = geo.tiles > 1 || geo.NV > 16 ? 0 : geo.NV == 4 ? 20 : geo.NV == 8 ? (bytes <= kSpanSumBytes ? 14 : bytes <= (64ull << 20) ? 8 : 3)
-                                                     : !hubs && bytes <= kSpanSumBytes ? 12 : 0;
-    return few_edges(limit, n_rows, nnz);
+    const double limit = geo.tiles > 1 || n_rows < 12000 ? 0 : geo.NV == 4 ? 20 : geo.NV == 8 ? (bytes <= kSpanSumBytes ? 14 : bytes <= (64ull << 20) ? 8 : 3) : 0;
+    return few_edges(limit, 32000, n_rows, nnz);
 }
 // A sum has nothing between its ids and its rows.  Where the L2 doesn't hold the array the span kernels' ring keeps more loads in
 // flight (2.45 million rows of 1 KB 12.5 against 15.0 ms, 500,000 of 192 bytes with 20 edges each and hubs 0.67 against 0.72); where it does,
@@ -336,12 +340,12 @@ static bool sum_takes_short(const RowGeo &geo, long long n_gathered, unsigned ro
 //    weighted 1.05 to 1.83 / 1.46, with the propagation's mix 1.04 to 1.70 / 1.31; with long rows, whose hubs make the row kernels
 //    wait, 1.00 to 1.59 / 1.2 to 1.3; bf16 0.97 to 1.54 / 1.1 to 1.23.
 //  * rows of 528 to 768 bytes, no long rows, in up to 40 MB: float32 1.12 to 1.70 / 1.4, bf16 weighted 1.08 to 1.30.
-//  * rows of 128 and 256 bytes, full lanes in either: half the MB, 0.97 to 1.41 / 1.1 to 1.25, no mix.
+//  * rows of 128 and 256 bytes, full lanes in either: half the MB, from 20 edges on, 0.97 to 1.41 / 1.1 to 1.25, no mix (12 edges 0.87 to 1.0).
 // Beyond the line 0.55 to 1.1.
 static bool sum_takes_rows(const RowArgs &a, sar_dtype t, long long n_gathered, long long nnz, bool weighted) {
     const int vecs = (int)(a.row_bytes / 16);
     const bool hubs = a.sp.n_long > 0, mix = a.mix.x0 != nullptr, f32 = t == SAR_F32;
-    if (vecs < 8 || vecs > 48 || nnz < (hubs ? 20 : 12) * a.n_rows) return false;
+    if (vecs < 8 || vecs > 48 || nnz < (hubs || vecs == 8 || vecs == 16 ? 20 : 12) * a.n_rows) return false;
     double mb = f32 ? (mix ? (hubs ? 1.25 : 1.8) : weighted ? (hubs ? 3.2 : 5.0) : hubs ? 2.5 : 3.2)
                     : (mix ? (hubs ? 0.0 : 0.9) : weighted ? (hubs ? 1.5 : 2.4) : hubs ? 1.0 : 1.9);
     if (vecs == 8 || vecs == 16) mb = mix || (!f32 && (!weighted || hubs)) ? 0.0 : 0.5 * mb;
@@ -537,7 +541,7 @@ sar_status sar_gat_fwd(const sar_part *g, const void *feat_q, const float *el, c
         }
         return SAR_OK;
     }
-    a.lone = takes_short(r.geo, g->n_src, r.row_bytes, g->n_dst, g->nnz, false, use_split);
+    a.lone = takes_short(r.geo, g->n_src, r.row_bytes, g->n_dst, g->nnz, false);
     if (!a.lone && takes_span(s, r.geo, g->n_src, g->n_dst, g->nnz, false, part))
         SAR_TRY(span_fwd(s, a, g->nnz, st));
     else if (part)
@@ -718,7 +722,7 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
         a.rowvec = gout_g;
         a.dscal = del;
         a.sp = split_args(g->split, reinterpret_cast<float *>(wsb + w.csr), H, r, t);
-        a.lone = takes_short(r.geo, g->n_src, r.row_bytes, g->n_dst, g->nnz, true, a.sp.n_long > 0);
+        a.lone = takes_short(r.geo, g->n_src, r.row_bytes, g->n_dst, g->nnz, true);
         if (lean_shape_applies(s, slope, g->split, g->n_src) && sar_aligned(er_q, 16)) {
             LeanArgs la{};
             la.n_rows = g->n_dst;
@@ -759,7 +763,7 @@ sar_status sar_gat_bwd(const sar_part *g, const void *feat_q, const float *el, c
         a.out = dfeat_q;
         a.dscal = der_q;
         a.sp = split_args(g->t_split, reinterpret_cast<float *>(wsb + w.csc), H, r, t);
-        a.lone = takes_short(r.geo, g->n_dst, r.row_bytes, g->n_src, g->nnz, true, a.sp.n_long > 0);
+        a.lone = takes_short(r.geo, g->n_dst, r.row_bytes, g->n_src, g->nnz, true);
         if (lean_shape_applies(s, slope, g->t_split, g->n_dst)) {
             LeanSrcArgs la{};
             la.n_rows = g->n_src;
@@ -818,7 +822,7 @@ static sar_status sum_rows(const sar_part *g, const RowShape &r, int32_t F, sar_
     const bool weighted = src_scale != nullptr;
     Shape s;
     SAR_TRY(make_shape(1, F, t, !r.ragged, &s));
-    a.lone = sum_takes_short(r.geo, g->n_src, r.row_bytes, g->n_dst, g->nnz, a.sp.n_long > 0);
+    a.lone = sum_takes_short(r.geo, g->n_src, r.row_bytes, g->n_dst, g->nnz);
     if (!a.lone && sum_takes_span(s, a, t, g->n_src, g->nnz, weighted))
         SAR_TRY(span_sum(s, a, g->nnz, weighted, st));
     else
