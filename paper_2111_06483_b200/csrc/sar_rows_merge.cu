@@ -183,35 +183,31 @@ __device__ __forceinline__ void merge_few(const RowArgs &a, long long row, long 
     }
 }
 
-// long rows of a block
-static __host__ __device__ int merge_rows(int n_long, int rows) { return n_long > kMergeMany ? rows : 1; }
-
-// MODE: kRowFwd, kRowSrc, kRowSum.  A block has merge_rows long rows, a warp each; then those of more records together.
-template <typename T, int MODE>
+// MODE: kRowFwd, kRowSrc, kRowSum.  A block has ROWS long rows, a warp each; then those of more records together.
+template <typename T, int MODE, int ROWS>
 __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs a) {
     constexpr int EPV = Elem<T>::EPV;
     constexpr bool kF = MODE == kRowFwd;
     after_predecessor();
     __shared__ float4 red[kMergeThreads];
     __shared__ float sM[SAR_MAX_HEADS], sD[SAR_MAX_HEADS], sOld[SAR_MAX_HEADS];
-    __shared__ float fac[MergeRows<MODE>::n][kF ? kMergeFew : 1][kMergeHeads], stat[MergeRows<MODE>::n][3][kMergeHeads];
+    __shared__ float fac[ROWS][kF && ROWS > 1 ? kMergeFew : 1][kMergeHeads], stat[ROWS][3][kMergeHeads];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rowf = a.H * a.vph * EPV;
     const bool first = a.flags & SAR_FIRST;
-    const int rows = merge_rows(a.sp.n_long, MergeRows<MODE>::n);
-    const int lr0 = (int)blockIdx.x * rows;
+    const int lr0 = (int)blockIdx.x * ROWS;
     auto few = [&](int lr, long long &s0, long long &s1) {
         s0 = a.sp.long_seg[lr];
         s1 = a.sp.long_seg[lr + 1];
-        return rows > 1 && s1 - s0 <= kMergeFew && a.H <= kMergeHeads;
+        return ROWS > 1 && s1 - s0 <= kMergeFew && a.H <= kMergeHeads;
     };
-    if constexpr (MODE != kRowSum) {
+    if constexpr (ROWS > 1) {
         const int lr = lr0 + warp;
         long long s0, s1;
-        if (warp < rows && lr < a.sp.n_long && few(lr, s0, s1))
+        if (lr < a.sp.n_long && few(lr, s0, s1))
             merge_few<T, MODE>(a, a.sp.long_row[lr], s0, (int)(s1 - s0), fac[warp], stat[warp][0], stat[warp][1], stat[warp][2]);
     }
-    for (int lr = lr0; lr < lr0 + rows && lr < a.sp.n_long; ++lr) {
+    for (int lr = lr0; lr < lr0 + ROWS && lr < a.sp.n_long; ++lr) {
         long long s0, s1;
         if (few(lr, s0, s1)) continue;
         const long long row = a.sp.long_row[lr];
@@ -351,15 +347,17 @@ __global__ void __launch_bounds__(256) rows_finalize_kernel(const RowArgs a) {
     reinterpret_cast<uint4 *>(a.out)[vi] = Elem<T>::pack(x);
 }
 
+template <typename T, int MODE, int ROWS>
+static sar_status launch_merge_rows(const RowArgs &a, const char *name, cudaStream_t st) {
+    SAR_LAUNCH(name, st, launch(rows_merge_kernel<T, MODE, ROWS>, (unsigned)((a.sp.n_long + ROWS - 1) / ROWS), kMergeThreads, 0, st, a));
+    return sar_after_launch();
+}
 template <int MODE>
 static sar_status launch_merge(const RowArgs &a, sar_dtype t, const char *name, cudaStream_t st) {
-    const int rows = merge_rows(a.sp.n_long, MergeRows<MODE>::n);
-    const unsigned blocks = (unsigned)((a.sp.n_long + rows - 1) / rows);
-    if (t == SAR_F32)
-        SAR_LAUNCH(name, st, launch(rows_merge_kernel<float, MODE>, blocks, kMergeThreads, 0, st, a));
-    else
-        SAR_LAUNCH(name, st, launch(rows_merge_kernel<__nv_bfloat16, MODE>, blocks, kMergeThreads, 0, st, a));
-    return sar_after_launch();
+    constexpr int R = MergeRows<MODE>::n;
+    if (R > 1 && a.sp.n_long > kMergeMany)
+        return t == SAR_F32 ? launch_merge_rows<float, MODE, R>(a, name, st) : launch_merge_rows<__nv_bfloat16, MODE, R>(a, name, st);
+    return t == SAR_F32 ? launch_merge_rows<float, MODE, 1>(a, name, st) : launch_merge_rows<__nv_bfloat16, MODE, 1>(a, name, st);
 }
 
 sar_status rows_fwd_merge(const RowArgs &a, sar_dtype t, cudaStream_t st) { return launch_merge<kRowFwd>(a, t, "gat_fwd_merge", st); }
