@@ -35,7 +35,7 @@ static sar_status launch_row_kernel(RowArgs a, RowGeo g, long long nnz, const ch
 }
 
 template <typename T, int NV, int HP, int MODE>
-static sar_status launch_short_kernel(RowArgs a, RowGeo g, long long nnz, const char *name, cudaStream_t st) {
+static sar_status launch_short_kernel(RowArgs a, RowGeo g, long long nnz, cudaStream_t st) {
     constexpr int NG = 32 / NV;
     // 32 warps an SM at 64 registers; the backward passes over bf16 rows need 70 to 80 (24 warps, no spills)
     constexpr int MINB = sizeof(T) == 2 && (MODE == kRowSrc || MODE == kRowDst || MODE == kRowDstPart) ? 6 : 8;
@@ -43,6 +43,8 @@ static sar_status launch_short_kernel(RowArgs a, RowGeo g, long long nnz, const 
     const long long warps = a.sp.n_seg + (a.n_rows + NG - 1) / NG;
     if (warps <= 0) return SAR_OK;
     const dim3 grid((unsigned)((warps * 32 + kShortThreads - 1) / kShortThreads), (unsigned)g.tiles);
+    constexpr const char *name = MODE == kRowFwd || MODE == kRowFwdPart ? "gat_fwd_short" : MODE == kRowDst || MODE == kRowDstPart ? "gat_bwd_dst_short"
+                                 : MODE == kRowSrc ? "gat_bwd_src_short" : "spmm_short";
     SAR_LAUNCH(name, st, launch(short_kernel<T, NV, HP, MODE, MINB>, grid, kShortThreads, 0, st, a));
     return sar_after_launch();
 }
@@ -52,7 +54,7 @@ static sar_status dispatch_rows(const RowArgs &a, RowGeo g, long long nnz, const
 #define SAR_ROW_CASE(NV_, HP_) \
     if (g.NV == NV_ && g.HP == HP_) { \
         if constexpr (NV_ <= 32) \
-            if (a.lone) return launch_short_kernel<T, NV_, HP_, MODE>(a, g, nnz, name, st); \
+            if (a.lone) return launch_short_kernel<T, NV_, HP_, MODE>(a, g, nnz, st); \
         return launch_row_kernel<T, NV_, HP_, MODE>(a, g, nnz, name, st); \
     }
     SAR_ROW_CASE(4, 1) SAR_ROW_CASE(8, 1) SAR_ROW_CASE(16, 1) SAR_ROW_CASE(32, 1) SAR_ROW_CASE(64, 1)

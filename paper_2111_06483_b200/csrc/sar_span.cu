@@ -98,15 +98,15 @@ sar_status span_fwd(const Shape &s, const RowArgs &r, long long nnz, cudaStream_
     const SpanArgs a = span_args(s, r);
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
-        return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kFwd, kCapFwd, kMinBlocksFwd>(a, nnz, "gat_fwd", st);
+        return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kFwd, kCapFwd, kMinBlocksFwd>(a, nnz, "gat_fwd_span", st);
     });
 }
 sar_status span_dst(const Shape &s, const RowArgs &r, long long nnz, bool part, cudaStream_t st) {
     const SpanArgs a = span_args(s, r);
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
-        if (part) return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDstGivenD, kCapDst, kMinBlocksBwd<C::v>>(a, nnz, "gat_bwd_dst", st);
-        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDst, kCapDst, kMinBlocksBwd<C::v>>(a, nnz, "gat_bwd_dst", st);
+        if (part) return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDstGivenD, kCapDst, kMinBlocksBwd<C::v>>(a, nnz, "gat_bwd_dst_span", st);
+        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdDst, kCapDst, kMinBlocksBwd<C::v>>(a, nnz, "gat_bwd_dst_span", st);
     });
 }
 sar_status span_src(const Shape &s, const RowArgs &r, long long nnz, cudaStream_t st) {
@@ -114,15 +114,15 @@ sar_status span_src(const Shape &s, const RowArgs &r, long long nnz, cudaStream_
     a.hvec = s.geom.H % 4 == 0;
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
-        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdSrc, kCapSrc, kMinBlocksBwd<C::v>>(a, nnz, "gat_bwd_src", st);
+        return launch_span<typename C::type, C::g, C::v, UBwd<C::v>::u, kBwdSrc, kCapSrc, kMinBlocksBwd<C::v>>(a, nnz, "gat_bwd_src_span", st);
     });
 }
 sar_status span_sum(const Shape &s, const RowArgs &r, long long nnz, bool weighted, cudaStream_t st) {
     const SpanArgs a = span_args(s, r);
     return dispatch(s, [&](auto cfg) -> sar_status {
         using C = decltype(cfg);
-        if (weighted) return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kSumW, kCapSum, kMinBlocksFwd>(a, nnz, "spmm", st);
-        return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kSum, kCapSum, kMinBlocksFwd>(a, nnz, "spmm", st);
+        if (weighted) return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kSumW, kCapSum, kMinBlocksFwd>(a, nnz, "spmm_span", st);
+        return launch_span<typename C::type, C::g, C::v, UFwd<C::v>::u, kSum, kCapSum, kMinBlocksFwd>(a, nnz, "spmm_span", st);
     });
 }
 

@@ -28,6 +28,7 @@ def test_pass_grouping_and_clock_parsing():
     p = bench.group_passes(k)
     assert p["gat_fwd"]["ms"] == 3.5 and sorted(p["gat_fwd"]["launches"]) == ["gat_fwd", "gat_fwd_merge", "gat_fwd_seg"]
     assert p["gat_bwd_src"]["ms"] == 3.0
+    assert list(bench.group_passes({"gat_bwd_dst_short": {"avg_ms": 1.0}, "gat_bwd_dst_span": {"avg_ms": 2.0}})) == ["gat_bwd_dst"]
     lines = ["1965, 1965, 410.2, Not Active, Not Active, Not Active, Not Active",
              "1500, 1965, 990.0, Not Active, Not Active, Not Active, Active",
              "1800, 1965, 700.0, Not Active, Not Active, Not Active, Not Active", "garbage"]
