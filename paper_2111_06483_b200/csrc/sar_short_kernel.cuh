@@ -16,8 +16,10 @@
 // edges 58 -> 36; the same head over 445,858 nodes in 16 steps, forward and backward, 2.74 -> 1.74 ms.
 //
 // Sums of four edges are formed first and added to the row's: chains of 4 + deg/4 additions, fewer with the groups' shares.
-// The softmax is taken against the score of the first edge, as in the lean kernels; where a score leads it by more than 60 the
-// shift moves up and the sums so far follow.  A row's arithmetic does not depend on the rows around it.
+// The softmax is taken against the running maximum of the row's scores: the sums so far times exp(m_before - m) in the
+// multiply-add that adds the next four edges, so that it costs one exponential per lane and step, and no weight exceeds 1 whatever the
+// scores and features.  The maximum starts at the lowest finite number: a score of -inf (a masked source) weighs nothing against it, and
+// a row without any other has m = -inf and d = 0, like one without edges.  A row's arithmetic does not depend on the rows around it.
 #pragma once
 
 #include "sar_rows_kernel.cuh"
@@ -35,8 +37,8 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
     constexpr bool kF = MODE == kRowFwd || MODE == kRowFwdPart, kD = MODE == kRowDst || MODE == kRowDstPart;
     constexpr bool kS = MODE == kRowSrc, kAgg = MODE == kRowSum || MODE == kRowSumW;
     constexpr bool kAcc = kF || kS || kAgg, kDot = kD || kS;
-    constexpr float kMaxLead = 60.f;
     constexpr unsigned kAll = 0xffffffffu;
+    constexpr float kLowest = -3.402823466e38f;
     static_assert(NV <= 32, "one vector per lane");
     const int lane = threadIdx.x & 31, gl = lane & (G - 1), grp = lane / G;
     const long long warp = (long long)blockIdx.x * (kShortThreads / 32) + (threadIdx.x >> 5);
@@ -115,7 +117,7 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
         }
         if constexpr (MODE == kRowFwdPart || MODE == kRowDstPart) __syncwarp();   // every lane of a head has read the state before one writes it
         f32x2 acc[NP], go[NP];
-        float l = 0.f, m = SAR_NEG_INF, c = 0.f, dD = 0.f, dB = 0.f;
+        float l = 0.f, m = kLowest, dD = 0.f, dB = 0.f;
 #pragma unroll
         for (int k = 0; k < NP; ++k) acc[k] = zero2();
         if constexpr (kDot) Pairs<T>::get(rv, go);
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
 
         // four edges at a time (positions past the end repeat the last edge with weight zero)
         for (int e = e0; e < n; e += step) {
-            float t[U], g4[U], ag[U];
+            float t[U], g4[U], ag[U], keep = 1.f;
             float4 rc[kS ? U : 1];
             uint4 x[U];
 #pragma unroll
@@ -140,24 +142,16 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
                 for (int u = 0; u < U; ++u) col[u] = column(e + step + u);
             }
             if constexpr (kF) {
-                float top = SAR_NEG_INF;
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     float gr;
                     t[u] = leaky(rs + t[u], a.slope, gr);
-                    top = fmaxf(top, t[u]);
                 }
-                if (e == e0) c = t[0];
-                if (top - c > kMaxLead) {   // the shift moves up, and the sums so far with it (Sec. 3.4)
-                    const float f = e == e0 ? 1.f : row_ex2((c - top) * kRowLog2e);
-                    c = top;
-                    l *= f;
+                const float top = fmaxf(fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3])), m);
+                keep = row_ex2((m - top) * kRowLog2e);   // the sums so far follow the maximum (Sec. 3.4)
+                m = top;
 #pragma unroll
-                    for (int k = 0; k < NP; ++k) acc[k] = fma2(acc[k], pack2(f, f), zero2());
-                }
-                m = fmaxf(m, top);
-#pragma unroll
-                for (int u = 0; u < U; ++u) t[u] = row_ex2((t[u] - c) * kRowLog2e);
+                for (int u = 0; u < U; ++u) t[u] = row_ex2((t[u] - top) * kRowLog2e);
             } else if constexpr (kD) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
@@ -176,7 +170,7 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
                 if (u > 0 && e + u >= n) t[u] = 0.f;
                 if constexpr (kDot) ag[u] = t[u] * g4[u];
             }
-            if constexpr (kF) l += (t[0] + t[1]) + (t[2] + t[3]);
+            if constexpr (kF) l = fmaf(l, keep, (t[0] + t[1]) + (t[2] + t[3]));
             if constexpr (kD) l += (ag[0] + ag[1]) + (ag[2] + ag[3]);
             if constexpr (kS) l += (ag[0] * rc[0].w + ag[1] * rc[1].w) + (ag[2] * rc[2].w + ag[3] * rc[3].w);
             f32x2 part[NP];
@@ -200,7 +194,7 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
             }
             if constexpr (kAcc) {
 #pragma unroll
-                for (int k = 0; k < NP; ++k) acc[k] = fma2(part[k], pack2(1.f, 1.f), acc[k]);
+                for (int k = 0; k < NP; ++k) acc[k] = fma2(acc[k], pack2(keep, keep), part[k]);
             }
             dB += b;
             dD += d;
@@ -214,15 +208,15 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
             y[2 * k + 1] = acc[k].y;
         }
         if (fold) {
-            if constexpr (kF) {   // the groups' sums against one shift, the maximum (-inf: a group without edges)
+            if constexpr (kF) {   // the groups' sums against one shift, the maximum
                 float mm = m;
 #pragma unroll
                 for (int off = G; off < 32; off <<= 1) mm = fmaxf(mm, __shfl_xor_sync(kAll, mm, off));
-                const float f = m == SAR_NEG_INF ? 0.f : c == mm ? 1.f : row_ex2((c - mm) * kRowLog2e);
+                const float f = row_ex2((m - mm) * kRowLog2e);
                 l *= f;
 #pragma unroll
                 for (int k = 0; k < EPV; ++k) y[k] *= f;
-                c = m = mm;
+                m = mm;
             }
 #pragma unroll
             for (int off = G; off < 32; off <<= 1) {
@@ -242,6 +236,7 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
                 }
             }
         }
+        if constexpr (kF) m = l == 0.f ? SAR_NEG_INF : m;
         if (!live || (fold && grp != 0)) return;
         if (seg) {
             float *part = a.sp.part + warp * a.sp.pstride;
@@ -265,7 +260,7 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
         }
         T *outp = reinterpret_cast<T *>(a.out) + row * (long long)HF + oel;
         if constexpr (MODE == kRowFwd) {
-            const float f = c == m ? 1.f : row_ex2((c - m) * kRowLog2e), inv = l > 0.f ? __fdividef(1.f, l) : 0.f;
+            const float inv = l > 0.f ? __fdividef(1.f, l) : 0.f;
 #pragma unroll
             for (int k = 0; k < EPV; ++k) {
                 y[k] *= inv;
@@ -274,7 +269,7 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
             if (left > 0) store_elems<T, EPV>(outp, y, left, a.ragged);
             if (head_lane) {
                 a.m_io[so] = m;
-                a.d_io[so] = n > 0 ? l * f : 0.f;
+                a.d_io[so] = l;
             }
         } else if constexpr (MODE == kRowFwdPart) {
             if (n == 0 && !first && !last) return;   // nothing to add, nothing to write
@@ -284,7 +279,7 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
 #pragma unroll
             for (int k = 0; k < EPV; ++k) pa[k] = 0.f;
             if (!first && left > 0) load_elems<float, EPV>(ap, pa, left, a.ragged);
-            const float fo = pm == mn ? 1.f : row_ex2((pm - mn) * kRowLog2e), fn = n == 0 || c == mn ? 1.f : row_ex2((c - mn) * kRowLog2e);
+            const float fo = pm == mn ? 1.f : row_ex2((pm - mn) * kRowLog2e), fn = m == mn ? 1.f : row_ex2((m - mn) * kRowLog2e);
             const float dn = pd * fo + l * fn;
 #pragma unroll
             for (int k = 0; k < EPV; ++k) y[k] = pa[k] * fo + y[k] * fn;

@@ -7,12 +7,30 @@ import torch
 
 import workloads
 from helpers import allclose_report
-from test_gpu_parity import DEV, Problem, _full_check, check_out, hub_graph
+from test_gpu_parity import DEV, Problem, _full_check, check_grad, check_out, hub_graph
 
 pytestmark = pytest.mark.gpu
 
 if torch.cuda.is_available():
     from paper_2111_06483_b200 import api, binding as B
+
+
+class Launches:
+    """The names of the gather kernels' launches inside the block."""
+
+    def __enter__(self):
+        self.names = []
+        B.sar_set_launch_hook(lambda name, phase: self.names.append(name) if phase == 0 else None)
+        return self
+
+    def __exit__(self, *exc):
+        B.sar_set_launch_hook(None)
+        return False
+
+    def only(self, suffix, passes=("gat_fwd", "gat_bwd_dst", "gat_bwd_src")):
+        """Every pass over edges was the kernel of that suffix (its merges aside)."""
+        seen = [x for x in self.names if x.startswith(tuple(passes)) and not x.endswith(("_merge", "_finalize"))]
+        return bool(seen) and all(x.endswith(suffix) for x in seen)
 
 
 @pytest.mark.parametrize("H,F,dtype", [(1, 47, "bf16"), (3, 33, "f32"), (6, 24, "bf16"), (2, 64, "bf16"), (7, 9, "f32"), (1, 300, "f32"),
@@ -71,6 +89,66 @@ def test_attention_of_a_row_per_lane_group(H, F, dtype, scale):
         allclose_report(m.cpu().numpy()[has], f.m[has], 2.0 ** -23, 0.0, "m")
         allclose_report(dd.cpu().numpy(), f.d, 2.0 ** -14, 0.0, "d")
         allclose_report(out.float().cpu().numpy(), f.out, 2.0 ** -7, 2.0 ** -9, "out")
+
+
+def _masked_problem(H, F, dtype, which, threshold, long_rows=()):
+    """Rows whose sources' score terms are partly -inf, three random edges per row besides rows of 6 to 96 edges with sources of
+    their own.  Every row keeps an edge from the last hundred sources, which are not masked."""
+    n, gen = 16_100, torch.Generator().manual_seed(H * F)
+    src, dst = [torch.randint(0, n, (2 * n,), generator=gen), n - 1 - torch.arange(n) % 100], [torch.randint(500, n, (2 * n,), generator=gen), torch.arange(n)]
+    masked, at = torch.zeros(n, dtype=torch.bool), 1000
+    groups = max(1, 32 // (4 if F * (2 if dtype == "bf16" else 4) * H <= 64 else 8))
+    for i, deg in enumerate([6, 8, 9, 23, 24, 25, 32, 48, 95, 96, *long_rows]):
+        src.append(torch.arange(at, at + deg))     # sources ascend within a row: position p of the row is source at + p
+        dst.append(torch.full((deg,), 7 * i))
+        pos = torch.arange(deg)
+        masked[at:at + deg] = pos < 4 if which == "first" else (pos // 4) % groups == i % groups
+        at += deg
+    if which == "step":
+        masked[:] = torch.arange(n) < n // 2
+    elif which == "half":
+        masked[:] = torch.rand(n, generator=gen) < 0.5
+    masked[n - 100:] = False
+    p = Problem(n, torch.cat(src).int(), torch.cat(dst).int(), H, F, 3, dtype=dtype, k=2, threshold=threshold, build_parts=True)
+    p.host["er"][masked.numpy()] = -np.inf
+    p.dev["er"][masked.to(DEV)] = -float("inf")
+    return p
+
+
+@pytest.mark.parametrize("H,F,dtype", [(1, 32, "bf16"), (1, 47, "bf16"), (1, 16, "f32"), (8, 8, "bf16"), (4, 8, "f32"), (8, 24, "bf16")])
+@pytest.mark.parametrize("which", ["first", "group", "step", "half"])
+def test_masked_sources_of_short_rows(H, F, dtype, which):
+    """er = -inf for a row's first four edges, for all that one group of lanes has of a row the warp shares, for every edge of a
+    partition step and for half of all sources: such an edge weighs nothing, and what came before the first other one is 0."""
+    p = _masked_problem(H, F, dtype, which, 0)
+    with Launches() as ran:
+        _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
+    assert ran.only("_short", ("gat_fwd",) if (H, F) == (8, 24) else ("gat_fwd", "gat_bwd_dst")), set(ran.names)
+
+
+@pytest.mark.parametrize("H,F,dtype", [(1, 32, "bf16"), (1, 16, "f32"), (8, 8, "bf16"), (4, 8, "f32")])
+@pytest.mark.parametrize("lead,power", [(50.0, 60), (20.0, 100)])
+def test_large_features_of_short_rows(H, F, dtype, lead, power):
+    """Features of 2^60 (1e18) and 2^100 (1e30) whose scores lead the row's others by 50 and 20: no weight exceeds 1, so that no sum exceeds
+    the features' by more than the number of edges.  Features and output gradients are scaled by powers of two, which is exact."""
+    p = _masked_problem(H, F, dtype, "none", 0)
+    pick = np.random.default_rng(5).random(p.host["er"].shape) < 0.5
+    p.host["el"][:] = 0.0
+    p.host["er"][:] = np.where(pick, 1.0, 1.0 + lead)
+    f = p.oracle_fwd()
+    b = p.oracle_bwd(f)
+    d = {k: torch.as_tensor(v, device=DEV) for k, v in p.host.items()}
+    feat, gout = p.dev["feat"] * 2.0 ** power, p.dev["gout"] * 2.0 ** -power
+    for mode in ("fused", "stateful"):
+        with Launches() as ran:
+            out, m, dd, *acc = api.gat_forward(p.graph, feat, d["el"], d["er"], 0.2, mode=mode, keep_numerator=mode == "stateful")
+        assert ran.only("_short"), set(ran.names)
+        check_out(out.float() * 2.0 ** -power, f.out, dtype, "out")
+        allclose_report(dd.cpu().numpy(), f.d, 1e-5, 1e-6, "d")
+        dfeat, del_, der = api.gat_backward(p.graph, feat, d["el"], d["er"], m, dd, gout, 0.2, out=out, mode=mode, acc=acc[0] if acc else None)
+        check_grad(dfeat.float() * 2.0 ** power, b.dfeat, dtype, "dfeat", stored=True)
+        check_grad(del_, b.del_, dtype, "del", 10.0)
+        check_grad(der, b.der, dtype, "der", 10.0)
 
 
 @pytest.mark.parametrize("H,F,dtype", [(1, 64, "bf16"), (5, 8, "f32"), (6, 24, "bf16"), (10, 16, "f32"), (11, 8, "bf16"), (16, 32, "f32"),
