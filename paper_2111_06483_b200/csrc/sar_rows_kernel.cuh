@@ -428,8 +428,6 @@ __global__ void __launch_bounds__(kRowWarps * 32, MINB) row_kernel(const RowArgs
                     const float al = lane < nb ? row_ex2((s - rc[h].y) * kRowLog2e) * rc[h].z : 0.f;
                     *reinterpret_cast<float4 *>(sw + (lane * HP + h) * 4) = make_float4(al, al * gr, al * gr * rc[h].w, 0.f);
                 }
-            } else {
-                if (lane >= nb) wcol = 0.f;
             }
             if constexpr (!kAgg) __syncwarp();
             if constexpr (kDot) {
@@ -446,7 +444,10 @@ __global__ void __launch_bounds__(kRowWarps * 32, MINB) row_kernel(const RowArgs
                 for (int u = 0; u < U; ++u) {
                     if (all || s + u < slots) {
                         float wsum = 1.f;
-                        if (kAgg && (MODE == kRowSumW || E > 1)) wsum = __shfl_sync(0xffffffffu, wcol, (s + u) * E + half);
+                        if (MODE == kRowSumW) wsum = __shfl_sync(0xffffffffu, wcol, (s + u) * E + half);
+                        // a sum's last slot may be short of edges: nothing is added for them (zero times the last edge's row is no zero if
+                        // that holds an infinity)
+                        const bool there = !kAgg || E == 1 || (s + u) * E + half < nb;
 #pragma unroll
                         for (int v = 0; v < V; ++v) {
                             f32x2 y[NP];
@@ -462,7 +463,8 @@ __global__ void __launch_bounds__(kRowWarps * 32, MINB) row_kernel(const RowArgs
                                     for (int k = 0; k < NP; ++k) acc[v][k] = fma2(y[k], w2, acc[v][k]);
                                 } else {
 #pragma unroll
-                                    for (int k = 0; k < NP; ++k) pin[v][k] = fma2(y[k], w2, pin[v][k]);
+                                    for (int k = 0; k < NP; ++k)
+                                        if (there) pin[v][k] = fma2(y[k], w2, pin[v][k]);
                                 }
                             } else {
                                 float al, ag, agd = 0.f;

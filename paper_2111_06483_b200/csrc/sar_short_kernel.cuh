@@ -123,7 +123,8 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
         if constexpr (kDot) Pairs<T>::get(rv, go);
         if constexpr (kD) ri = ri > 0.f ? __fdividef(1.f, ri) : 0.f;
 
-        // four edges at a time (positions past the end repeat the last edge with weight zero)
+        // four edges at a time; positions past the end repeat the last edge's loads and add nothing: not zero times its row, which may hold
+        // an infinity, but in a sum no product, in the other passes zero times zeros (the cheaper of the two for each)
         for (int e = e0; e < n; e += step) {
             float t[U], g4[U], ag[U], keep = 1.f;
             float4 rc[kS ? U : 1];
@@ -167,18 +168,24 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                if (u > 0 && e + u >= n) t[u] = 0.f;
+                if (!kAgg && u > 0 && e + u >= n) t[u] = 0.f;
                 if constexpr (kDot) ag[u] = t[u] * g4[u];
             }
             if constexpr (kF) l = fmaf(l, keep, (t[0] + t[1]) + (t[2] + t[3]));
             if constexpr (kD) l += (ag[0] + ag[1]) + (ag[2] + ag[3]);
             if constexpr (kS) l += (ag[0] * rc[0].w + ag[1] * rc[1].w) + (ag[2] * rc[2].w + ag[3] * rc[3].w);
+            if (!kAgg && e + U > n) {
+#pragma unroll
+                for (int u = 1; u < U; ++u)
+                    if (e + u >= n) x[u] = make_uint4(0u, 0u, 0u, 0u);
+            }
             f32x2 part[NP];
             float b = 0.f, d = 0.f;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 f32x2 y[NP];
                 Pairs<T>::get(x[u], y);
+                if (kAgg && u > 0 && e + u >= n) continue;
                 if constexpr (kAcc) {
 #pragma unroll
                     for (int k = 0; k < NP; ++k) part[k] = fma2(y[k], pack2(t[u], t[u]), u == 0 ? zero2() : part[k]);

@@ -151,6 +151,65 @@ def test_large_features_of_short_rows(H, F, dtype, lead, power):
         check_grad(der, b.der, dtype, "der", 10.0)
 
 
+def _infinite_last_sources(n):
+    """Rows of 1 to 50 edges whose last edge (the highest source) is one of 20 nodes with an infinite feature, and the same transposed.
+    Returns src, dst and the nodes; the other rows have three edges each."""
+    gen = torch.Generator(device=DEV).manual_seed(n)
+    src, dst = [torch.randint(0, n - 20, (3 * n,), generator=gen, device=DEV)], [torch.randint(0, n - 20, (3 * n,), generator=gen, device=DEV)]
+    for deg in range(1, 51):
+        src += [torch.randint(0, n - 20, (deg,), generator=gen, device=DEV), torch.tensor([n - 1 - deg % 20], device=DEV)]
+        dst += [torch.full((deg + 1,), 3 * deg, device=DEV)]
+    src, dst = torch.cat(src).int(), torch.cat(dst).int()
+    return torch.cat([src, dst]), torch.cat([dst, src]), torch.arange(n - 20, n, device=DEV)
+
+
+@pytest.mark.parametrize("n,F,dtype", [(1500, 12, "f32"), (1500, 32, "f32"), (1500, 47, "bf16"), (1500, 60, "f32"), (1500, 100, "f32"), (33_000, 16, "f32"),
+                                       (33_000, 27, "f32"), (33_000, 32, "bf16"), (33_000, 64, "bf16"), (70_000, 47, "f32"), (90_000, 72, "bf16")])
+def test_an_infinity_on_the_last_edge_of_a_sum(n, F, dtype):
+    """Whatever a kernel takes for the edges that a row's last step is short of, it is not zero times the last edge's row: a sum with an
+    infinite term is infinite in that column and finite in the others."""
+    src, dst, nodes = _infinite_last_sources(n)
+    if n > 33_000:   # rows of a dozen edges and more in an array that the L2 holds
+        gen = torch.Generator(device=DEV).manual_seed(1)
+        more = [torch.randint(0, n - 20, (20 * n,), generator=gen, device=DEV, dtype=torch.int32) for _ in range(2)]
+        src, dst = torch.cat([src, more[0]]), torch.cat([dst, more[1]])
+    g = api.Graph.from_coo(n, src, dst)
+    x = (torch.arange(n * F, device=DEV).view(n, F) % 3 == 0).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    x[nodes, torch.arange(20, device=DEV) % F] = torch.tensor([float("inf"), -float("inf")], device=DEV, dtype=x.dtype).repeat(10)
+    scale = 2.0 ** (torch.arange(n, device=DEV) % 3 - 1).float()
+    take = lambda y: torch.zeros(n, F, device=DEV).index_add_(0, dst.long(), y[src.long()])
+    want = take(x.float())
+    assert bool(want.isinf().any()) and not bool(want.isnan().any())
+    assert torch.equal(api.spmm_sum(g.whole, x), want.to(x.dtype))
+    assert torch.equal(api.spmm_scaled(g.whole, x, src_scale=scale, dst_scale=scale), (take(x.float() * scale[:, None]) * scale[:, None]).to(x.dtype))
+
+
+@pytest.mark.parametrize("H,F,dtype", [(1, 16, "f32"), (1, 32, "f32"), (2, 8, "bf16"), (4, 8, "bf16"), (4, 24, "bf16"), (8, 24, "bf16")])
+def test_an_infinity_on_the_last_edge_of_a_short_row(H, F, dtype):
+    n = 33_000
+    src, dst, nodes = _infinite_last_sources(n)
+    g = api.Graph.from_coo(n, src, dst)
+    gen = torch.Generator(device=DEV).manual_seed(H * F)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    feat, gout = (torch.randn(n, H, F, generator=gen, device=DEV).to(dt) for _ in range(2))
+    el, er = (torch.randn(n, H, generator=gen, device=DEV) for _ in range(2))
+    feat_inf, gout_inf = feat.clone(), gout.clone()
+    for x in (feat_inf, gout_inf):
+        x[nodes, :, torch.arange(20, device=DEV) % F] = float("inf")
+    with Launches() as ran:
+        out, m, d = api.gat_forward(g, feat_inf, el, er, 0.2)[:3]
+        # (with finite features, whose dot products with an infinite gradient do not enter dfeat)
+        dfeat = api.gat_backward(g, feat, el, er, m, d, gout_inf, 0.2)[0]
+    assert ran.only("_short"), set(ran.names)
+    s, t = src.long(), dst.long()
+    alpha = torch.exp(torch.nn.functional.leaky_relu(el[t].double() + er[s].double(), 0.2) - m[t].double()) / d[t].double()
+    for got, to, x in ((out, t, feat_inf[s]), (dfeat, s, gout_inf[t])):
+        want = torch.zeros(n, H, F, device=DEV, dtype=torch.float64).index_add_(0, to, alpha[..., None] * x.double())
+        assert bool(want.isinf().any()) and torch.equal(got.double().isinf(), want.isinf()) and not bool(got.isnan().any())
+        ok = want.isfinite().cpu().numpy()
+        check_grad(got[want.isfinite()], want.cpu().numpy()[ok], dtype, "finite columns", stored=True)
+
+
 @pytest.mark.parametrize("H,F,dtype", [(1, 64, "bf16"), (5, 8, "f32"), (6, 24, "bf16"), (10, 16, "f32"), (11, 8, "bf16"), (16, 32, "f32"),
                                        (17, 8, "f32"), (1, 1030, "bf16")])
 @pytest.mark.parametrize("many", [False, True])
