@@ -57,6 +57,10 @@ __device__ __forceinline__ float4 merge_columns(const RowArgs &a, long long s0, 
     return x;
 }
 
+// A record's factor: exp(its maximum - the row's).  A record of masked scores alone (maximum -inf) weighs nothing, also where the
+// row has had no other so far.
+__device__ __forceinline__ float merge_factor(float m, float mn) { return m == SAR_NEG_INF ? 0.f : fast_exp(m - mn); }
+
 // One column (float4 x, its first float c of the padded row) of a finished row; what a forward row needs besides: its
 // denominator d and the factor `old` of the state's numerator.
 template <typename T, int MODE>
@@ -137,7 +141,7 @@ __device__ __forceinline__ void merge_few(const RowArgs &a, long long row, long 
                 float M = m[k];
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-                const float mn = fmaxf(M, mo[k]), f = fast_exp(m[k] - mn);
+                const float mn = fmaxf(M, mo[k]), f = merge_factor(m[k], mn);
                 float s = d[k] * f;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -224,7 +228,7 @@ __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs
                 float d = 0.f;
                 for (long long s = s0 + lane; s < s1; s += 32) {
                     const float *rec = a.sp.part + s * a.sp.pstride + rowf;
-                    d += rec[a.H + h] * fast_exp(rec[h] - mn);
+                    d += rec[a.H + h] * merge_factor(rec[h], mn);
                 }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
@@ -261,7 +265,7 @@ __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs
             const int c = in ? (c0 + col) * 4 : 0;
             const int head = c / (a.vph * EPV);
             const float4 x = merge_columns(a, in ? s0 : s1, s1, c, stream, streams, red, cols_pad, col, [&](long long s) {
-                if constexpr (kF) return fast_exp(a.sp.part[s * a.sp.pstride + rowf + head] - sM[head]);
+                if constexpr (kF) return merge_factor(a.sp.part[s * a.sp.pstride + rowf + head], sM[head]);
                 else return 1.f;
             });
             if (!in || stream != 0) continue;

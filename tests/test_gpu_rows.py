@@ -127,6 +127,19 @@ def test_masked_sources_of_short_rows(H, F, dtype, which):
 
 
 @pytest.mark.parametrize("H,F,dtype", [(1, 32, "bf16"), (1, 16, "f32"), (8, 8, "bf16"), (4, 8, "f32")])
+@pytest.mark.parametrize("threshold,long_rows", [(100, (101, 350, 800)), (20, (21,) * 300)])
+def test_masked_sources_of_long_rows(H, F, dtype, threshold, long_rows):
+    """Rows in segments, all of whose edges in the first partition step are masked: their merge (of a block, and of a warp where there
+    are many such rows) leaves a state that the second step can go on from."""
+    p = _masked_problem(H, F, dtype, "step", threshold, long_rows)
+    with Launches() as ran:
+        _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
+    assert ran.only("_short", ("gat_fwd",)) and "gat_fwd_merge" in ran.names, set(ran.names)
+    part = p.graph.parts[0]
+    assert part.split.n_long > (296 if threshold == 20 else 0)
+
+
+@pytest.mark.parametrize("H,F,dtype", [(1, 32, "bf16"), (1, 16, "f32"), (8, 8, "bf16"), (4, 8, "f32")])
 @pytest.mark.parametrize("lead,power", [(50.0, 60), (20.0, 100)])
 def test_large_features_of_short_rows(H, F, dtype, lead, power):
     """Features of 2^60 (1e18) and 2^100 (1e30) whose scores lead the row's others by 50 and 20: no weight exceeds 1, so that no sum exceeds
