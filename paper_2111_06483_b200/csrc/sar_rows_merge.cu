@@ -4,7 +4,9 @@
 // together.  With a block of 128 threads per
 // row, whatever its length, and a warp per row and head for the destination-major records, the three merges of 8 heads of 32
 // (1 million nodes, 200 edges per node, 575,000 segments) took 0.48, 0.50 and 0.29 ms, now 0.30, 0.08 and 0.19; the forward merge of 2 heads of
-// 64 (233,000 nodes, 11.6 million edges) 17 us, now 10.5.
+// 64 (233,000 nodes, 11.6 million edges) 17 us, now 10.5.  Hubs (8 heads of 32, bf16, us each, by the block per row and head / by
+// four neighbouring rows and one warp / now): four of 100,000 edges beside 400 of 600, forward 45 / 167 / 48, destination-major 19 / 52 / 13;
+// one of a million, destination-major 212 / 487 / 79.
 // The records of a hub row (hundreds) are read by all threads of the block, by several streams at once - a thread holds one
 // float4 column of every kStreams-th record - and the streams are added up in shared memory in a fixed order, so a result does
 // not depend on the schedule.
@@ -57,9 +59,9 @@ __device__ __forceinline__ float4 merge_columns(const RowArgs &a, long long s0, 
     return x;
 }
 
-// A record's factor: exp(its maximum - the row's).  A record of masked scores alone (maximum -inf) weighs nothing, also where the
-// row has had no other so far.
-__device__ __forceinline__ float merge_factor(float m, float mn) { return m == SAR_NEG_INF ? 0.f : fast_exp(m - mn); }
+// What a row's records are scaled against: its maximum, or the lowest finite number where that is -inf, so that a record of masked
+// scores alone (maximum -inf) weighs nothing.
+__device__ __forceinline__ float merge_shift(float m) { return fmaxf(m, -3.402823466e38f); }
 
 // One column (float4 x, its first float c of the padded row) of a finished row; what a forward row needs besides: its
 // denominator d and the factor `old` of the state's numerator.
@@ -141,7 +143,7 @@ __device__ __forceinline__ void merge_few(const RowArgs &a, long long row, long 
                 float M = m[k];
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-                const float mn = fmaxf(M, mo[k]), f = merge_factor(m[k], mn);
+                const float mn = fmaxf(M, mo[k]), f = fast_exp(m[k] - merge_shift(mn));
                 float s = d[k] * f;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -187,6 +189,10 @@ __device__ __forceinline__ void merge_few(const RowArgs &a, long long row, long 
     }
 }
 
+// The w-th long row of a block: the rows of a block are far apart, for the heaviest often follow one another (nodes in the order of
+// their degrees), and a block takes its heavy rows one after the other.
+__device__ __forceinline__ int merge_row_of(unsigned block, int w) { return (int)(block + (unsigned)w * gridDim.x); }
+
 // MODE: kRowFwd, kRowSrc, kRowSum.  A block has ROWS long rows, a warp each; then those of more records together.
 template <typename T, int MODE, int ROWS>
 __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs a) {
@@ -199,21 +205,21 @@ __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rowf = a.H * a.vph * EPV;
     const bool first = a.flags & SAR_FIRST;
-    const int lr0 = (int)blockIdx.x * ROWS;
     auto few = [&](int lr, long long &s0, long long &s1) {
         s0 = a.sp.long_seg[lr];
         s1 = a.sp.long_seg[lr + 1];
         return ROWS > 1 && s1 - s0 <= kMergeFew && a.H <= kMergeHeads;
     };
     if constexpr (ROWS > 1) {
-        const int lr = lr0 + warp;
+        const int lr = merge_row_of(blockIdx.x, warp);
         long long s0, s1;
         if (lr < a.sp.n_long && few(lr, s0, s1))
             merge_few<T, MODE>(a, a.sp.long_row[lr], s0, (int)(s1 - s0), fac[warp], stat[warp][0], stat[warp][1], stat[warp][2]);
     }
-    for (int lr = lr0; lr < lr0 + ROWS && lr < a.sp.n_long; ++lr) {
+    for (int w = 0; w < ROWS; ++w) {
+        const int lr = merge_row_of(blockIdx.x, w);
         long long s0, s1;
-        if (few(lr, s0, s1)) continue;
+        if (lr >= a.sp.n_long || few(lr, s0, s1)) continue;
         const long long row = a.sp.long_row[lr];
         __syncthreads();
 
@@ -228,7 +234,7 @@ __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs
                 float d = 0.f;
                 for (long long s = s0 + lane; s < s1; s += 32) {
                     const float *rec = a.sp.part + s * a.sp.pstride + rowf;
-                    d += rec[a.H + h] * merge_factor(rec[h], mn);
+                    d += rec[a.H + h] * fast_exp(rec[h] - merge_shift(mn));
                 }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
@@ -264,8 +270,9 @@ __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs
             const bool in = c0 + col < cols && stream < streams;
             const int c = in ? (c0 + col) * 4 : 0;
             const int head = c / (a.vph * EPV);
+            const float shift = kF ? merge_shift(sM[head]) : 0.f;
             const float4 x = merge_columns(a, in ? s0 : s1, s1, c, stream, streams, red, cols_pad, col, [&](long long s) {
-                if constexpr (kF) return merge_factor(a.sp.part[s * a.sp.pstride + rowf + head], sM[head]);
+                if constexpr (kF) return fast_exp(a.sp.part[s * a.sp.pstride + rowf + head] - shift);
                 else return 1.f;
             });
             if (!in || stream != 0) continue;
@@ -274,51 +281,78 @@ __global__ void __launch_bounds__(kMergeThreads) rows_merge_kernel(const RowArgs
     }
 }
 
-// Destination-major: D, B and S of the segments are numbers, 3 H of them one after the other in a record; a warp per long row, a
-// lane per number (of the heads h0 .. h0 + 9, so that they fit a warp), half a warp per record where 15 lanes do.
+// Destination-major: D, B and S of the segments are numbers, 3 H of them one after the other in a record; a lane per number (of the
+// heads h0 .. h0 + 9, so that they fit a warp), half a warp per record where 15 lanes do.  A row of up to kMergeAlone records is one
+// warp's; one of more is summed by the warps of the block together, every fourth step's records a warp's, and added up in shared
+// memory in a fixed order.
+constexpr int kMergeAlone = 64;
+// the sum of number p over the records s, s + step, .., eight loads in flight
+__device__ __forceinline__ float merge_numbers(const float *p, long long pstride, long long s, long long s1, int step) {
+    constexpr int U = 8;
+    float part[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) part[u] = 0.f;
+    p += s * pstride;
+    pstride *= step;
+    int n = s < s1 ? (int)((s1 - s + step - 1) / step) : 0;
+    for (; n >= U; n -= U, p += U * pstride) {
+        float r[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) r[u] = __ldg(p + u * pstride);
+#pragma unroll
+        for (int u = 0; u < U; ++u) part[u] += r[u];
+    }
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+        if (u < n) part[u] += __ldg(p + u * pstride);
+    return ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
+}
 template <bool PART>
 __global__ void __launch_bounds__(kMergeThreads) rows_dst_merge_kernel(const RowArgs a) {
     after_predecessor();
-    const int lane = threadIdx.x & 31;
-    const long long lr = (long long)blockIdx.x * (kMergeThreads / 32) + (threadIdx.x >> 5);
-    if (lr >= a.sp.n_long) return;
-    const long long row = a.sp.long_row[lr], s0 = a.sp.long_seg[lr], s1 = a.sp.long_seg[lr + 1];
-    for (int h0 = 0; h0 < a.H; h0 += 10) {
-        const int H = min(a.H - h0, 10), lanes = H <= 5 ? 16 : 32, at = lane & (lanes - 1);
-        const int q = at / H, h = at - q * H;   // number q (D, B, S) of head h0 + h
-        float x = 0.f;
-        if (q < 3 && !(PART && q == 0)) {
-            float part[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) part[u] = 0.f;
-            const int step = 32 / lanes;
-            const float *p = a.sp.part + q * a.H + h0 + h;
-            long long s = s0 + lane / lanes;
-            for (; s + 7LL * step < s1; s += 8LL * step) {
-                float r[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) r[u] = p[(s + u * step) * a.sp.pstride];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) part[u] += r[u];
+    constexpr int W = kMergeThreads / 32;
+    __shared__ float red[W][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto merge_row = [&](int lr, bool alone) {   // by this warp, or by all of the block
+        const long long row = a.sp.long_row[lr], s0 = a.sp.long_seg[lr], s1 = a.sp.long_seg[lr + 1];
+        for (int h0 = 0; h0 < a.H; h0 += 10) {
+            const int H = min(a.H - h0, 10), lanes = H <= 5 ? 16 : 32, at = lane & (lanes - 1), step = 32 / lanes;
+            const int q = at / H, h = at - q * H;   // number q (D, B, S) of head h0 + h
+            float x = 0.f;
+            if (q < 3 && !(PART && q == 0)) {
+                const float *p = a.sp.part + q * a.H + h0 + h;
+                x = merge_numbers(p, a.sp.pstride, s0 + (alone ? 0 : warp * step) + lane / lanes, s1, alone ? step : W * step);
             }
-#pragma unroll
-            for (int u = 0; u < 7; ++u)
-                if (s + u * step < s1) part[u] += p[(s + u * step) * a.sp.pstride];
-            x = ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
-        }
-        if (lanes == 16) x += __shfl_xor_sync(0xffffffffu, x, 16);
-        const float D = x, Bs = __shfl_sync(0xffffffffu, x, (lane + H) & 31), S = __shfl_sync(0xffffffffu, x, (lane + 2 * H) & 31);
-        if (lane < H) {
-            const long long o = row * a.H + h0 + lane;
-            if (PART) {
-                const float y = Bs - a.rec[o].w * S;
-                a.dscal[o] = (a.flags & SAR_FIRST) ? y : a.dscal[o] + y;
-            } else {
-                const float dd = a.d[o];
-                a.dscal[o] = Bs - D * S;
-                a.rec[o] = make_float4(a.el[o], a.m[o], dd > 0.f ? __fdividef(1.f, dd) : 0.f, D);
+            if (!alone) {
+                red[warp][lane] = x;
+                __syncthreads();
+                x = (red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane]);
+                __syncthreads();
+            }
+            if (lanes == 16) x += __shfl_xor_sync(0xffffffffu, x, 16);
+            const float D = x, Bs = __shfl_sync(0xffffffffu, x, (lane + H) & 31), S = __shfl_sync(0xffffffffu, x, (lane + 2 * H) & 31);
+            if (lane < H && (alone || warp == 0)) {
+                const long long o = row * a.H + h0 + lane;
+                if (PART) {
+                    const float y = Bs - a.rec[o].w * S;
+                    a.dscal[o] = (a.flags & SAR_FIRST) ? y : a.dscal[o] + y;
+                } else {
+                    const float dd = a.d[o];
+                    a.dscal[o] = Bs - D * S;
+                    a.rec[o] = make_float4(a.el[o], a.m[o], dd > 0.f ? __fdividef(1.f, dd) : 0.f, D);
+                }
             }
         }
+    };
+    static_assert(W == 4, "four shares");
+    auto is_few = [&](int lr) { return a.sp.long_seg[lr + 1] - a.sp.long_seg[lr] <= kMergeAlone; };
+    const int mine = merge_row_of(blockIdx.x, warp);
+    const bool there = mine < a.sp.n_long, few = there && is_few(mine);
+    if (few) merge_row(mine, true);
+    if (!__syncthreads_or(there && !few)) return;
+    for (int w = 0; w < W; ++w) {
+        const int lr = merge_row_of(blockIdx.x, w);
+        if (lr < a.sp.n_long && !is_few(lr)) merge_row(lr, false);
     }
 }
 
@@ -378,7 +412,8 @@ sar_status rows_fwd_finalize(const RowArgs &a, sar_dtype t, cudaStream_t st) {
 }
 
 sar_status rows_dst_merge(const RowArgs &a, bool part, cudaStream_t st) {
-    const unsigned blocks = (unsigned)((a.sp.n_long + kMergeThreads / 32 - 1) / (kMergeThreads / 32));
+    constexpr int W = kMergeThreads / 32;
+    const unsigned blocks = (unsigned)(a.sp.n_long > kMergeMany ? (a.sp.n_long + W - 1) / W : a.sp.n_long);
     if (part)
         SAR_LAUNCH("gat_bwd_dst_merge", st, launch(rows_dst_merge_kernel<true>, blocks, kMergeThreads, 0, st, a));
     else

@@ -244,6 +244,26 @@ def test_merges_on_either_side_of_what_a_warp_takes(H, F, dtype, many):
     _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=max(10.0, F / 64))
 
 
+@pytest.mark.parametrize("H,F,dtype", [(1, 64, "bf16"), (5, 8, "f32"), (8, 24, "bf16"), (10, 16, "f32"), (16, 8, "f32")])
+@pytest.mark.parametrize("many", [False, True])
+def test_merges_of_hubs(H, F, dtype, many):
+    """Rows of 520 segments among short ones, four of them in a block or one after the other, and rows on either side of the 64 that one
+    warp sums for the destination-major pass and of the steps in which four warps do."""
+    n, size, gen = 1200, 3, torch.Generator().manual_seed(H)
+    segs = [520, 2, 519, 64, 65, 521, 63, 66, 520, 127, 128, 129, 130, 512, 3]
+    if many:   # of 300 to 303 long rows a block has every 75th or 76th
+        segs += [2] * 288
+        for at in (75, 76, 150, 152, 225, 228):
+            segs[at] = 520
+    deg = torch.tensor([s * size - i % 2 for i, s in enumerate(segs)])
+    src = [torch.randint(600, n, (n,), generator=gen), torch.randint(600, n, (int(deg.sum()),), generator=gen)]
+    dst = [torch.randint(600, n, (n,), generator=gen), torch.arange(len(segs)).repeat_interleave(deg)]
+    src, dst = torch.cat(src).int(), torch.cat(dst).int()
+    both = torch.cat([src, dst]), torch.cat([dst, src])
+    p = Problem(n, both[0], both[1], H, F, 5, dtype=dtype, k=2, threshold=size, build_parts=True)
+    _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
+
+
 @pytest.mark.parametrize("F", [1, 3, 47, 48, 127, 180, 260, 1030])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("n", [1500, 40_000])
