@@ -40,8 +40,9 @@ struct RowArgs {
     int vph;                 // 16-byte vectors per head in gather and rowvec
     int ragged;              // out / acc rows are not made of aligned 16-byte vectors: element stores
     int hvec;                // the per-head scalars of a row can be loaded as float4 / float2
-    int R;                   // rows per warp (<= 32)
+    int R;                   // rows per warp (<= 32); sar_short_kernel.cuh: the most edges of a row that is one warp's
     int lone;                // a row per group of lanes (sar_short_kernel.cuh)
+    int wide;                // ... and a segment per block
     SplitArgs sp;
 };
 

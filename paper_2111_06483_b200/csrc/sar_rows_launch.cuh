@@ -34,19 +34,34 @@ static sar_status launch_row_kernel(RowArgs a, RowGeo g, long long nnz, const ch
     return sar_after_launch();
 }
 
+constexpr long long kShortBlock = 96, kShortFew = 4 * 32 * kRowSMs;   // edges (64: 0.79 to 1.0 of the speed with rows of 60); rows: four waves
 template <typename T, int NV, int HP, int MODE>
 static sar_status launch_short_kernel(RowArgs a, RowGeo g, long long nnz, cudaStream_t st) {
     constexpr int NG = 32 / NV;
-    // 32 warps an SM at 64 registers; the backward passes over bf16 rows need 70 to 80 (24 warps, no spills)
+    // 32 warps an SM at 64 registers; the backward passes over bf16 rows need 70 and more (24 warps at 80)
     constexpr int MINB = sizeof(T) == 2 && (MODE == kRowSrc || MODE == kRowDst || MODE == kRowDstPart) ? 6 : 8;
     a.nnz = nnz;
-    const long long warps = a.sp.n_seg + (a.n_rows + NG - 1) / NG;
-    if (warps <= 0) return SAR_OK;
-    const dim3 grid((unsigned)((warps * 32 + kShortThreads - 1) / kShortThreads), (unsigned)g.tiles);
     constexpr const char *name = MODE == kRowFwd || MODE == kRowFwdPart ? "gat_fwd_short" : MODE == kRowDst || MODE == kRowDstPart ? "gat_bwd_dst_short"
                                  : MODE == kRowSrc ? "gat_bwd_src_short" : "spmm_short";
-    SAR_LAUNCH(name, st, launch(short_kernel<T, NV, HP, MODE, MINB>, grid, kShortThreads, 0, st, a));
-    return sar_after_launch();
+    auto go = [&](auto kernel) {
+        const long long warps = (a.wide ? a.sp.n_seg * kShortWarps : a.sp.n_seg) + (a.n_rows + NG - 1) / NG;
+        if (warps <= 0) return SAR_OK;
+        SAR_LAUNCH(name, st, launch(kernel, dim3((unsigned)((warps + kShortWarps - 1) / kShortWarps), (unsigned)g.tiles), kShortThreads, 0, st, a));
+        return sar_after_launch();
+    };
+    if constexpr (NG == 1) {
+        // A long row is a chain of steps, and where a row fills the warp that chain decides how long a launch of few rows takes: there
+        // rows much longer than the others are shared by the warps of a block, and so are segments where a block for each fits the chip
+        // at once.  Times without over with it, backward, rows of 240 to 256 edges among ones of 2 to 20: 1.1 to 1.8; without such rows
+        // 0.91 to 1.0, and with ones of 40 to 100 0.88 to 1.05, so that launches of more rows, which hide the chain, go without.
+        a.wide = a.sp.n_seg > 0 && a.sp.n_seg * g.tiles <= kRowSMs * MINB;
+        if (a.n_rows * g.tiles <= (a.wide ? 2 : 1) * kShortFew) {
+            a.R = (int)(3 * nnz < kShortBlock * a.n_rows ? kShortBlock : 3 * nnz / a.n_rows);
+            return go(short_kernel<T, NV, HP, MODE, MINB, true>);
+        }
+    }
+    a.wide = 0;
+    return go(short_kernel<T, NV, HP, MODE, MINB, false>);
 }
 
 template <typename T, int MODE>

@@ -8,6 +8,9 @@
 // kernel spends 500 and more instructions of a whole warp on the start and the end of each.  So rows of more than kShortEdges
 // edges are left for last and shared by all groups of the warp (four edges to each at a time), and a segment of a long row has a
 // warp to itself from the start: without that a segment of 256 edges was a chain of 64 loads, 50 us, whatever the rest did.
+// Where a row fills the warp there are no groups to share it, and in a launch of few rows a segment or a row of a hundred edges and more is
+// taken by the four warps of a block (rest_of_block): 8 heads of 24, bf16, 3,200 nodes with 2 edges and hubs of 400, backward 70 -> 32 us
+// (span kernels 57), 5 heads of 24, 8,600 nodes, likewise 73 -> 35 (51).
 //
 // What bounds it: the chain row pointers -> column ids -> rows of a warp, which 32 warps an SM hide, then the issue slots of groups that
 // wait for longer ones.  Measured against the kernels that took these rows before (kShortEdges 12 and 48 within 5 %, but for
@@ -19,69 +22,86 @@
 // The softmax is taken against the running maximum of the row's scores: the sums so far times exp(m_before - m) in the
 // multiply-add that adds the next four edges, so that it costs one exponential per lane and step, and no weight exceeds 1 whatever the
 // scores and features.  The maximum starts at the lowest finite number: a score of -inf (a masked source) weighs nothing against it, and
-// a row without any other has m = -inf and d = 0, like one without edges.  A row's arithmetic does not depend on the rows around it.
+// a row without any other has m = -inf and d = 0, like one without edges.  A row's arithmetic does not depend on the rows around it, but for
+// those that a block may share.
 #pragma once
 
 #include "sar_rows_kernel.cuh"
 
 namespace sar {
 
-constexpr int kShortThreads = 128;
+constexpr int kShortThreads = 128, kShortWarps = kShortThreads / 32;
 constexpr int kShortEdges = 24;   // rows of more are shared by the groups of the warp
 
-template <typename T, int NV, int HP, int MODE, int MINB>
-__global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArgs a) {
-    after_predecessor();
-    constexpr int EPV = Elem<T>::EPV, NP = EPV / 2, U = 4;
-    constexpr int G = NV, NG = 32 / G, VPHP = NV / HP;
-    constexpr bool kF = MODE == kRowFwd || MODE == kRowFwdPart, kD = MODE == kRowDst || MODE == kRowDstPart;
-    constexpr bool kS = MODE == kRowSrc, kAgg = MODE == kRowSum || MODE == kRowSumW;
-    constexpr bool kAcc = kF || kS || kAgg, kDot = kD || kS;
+// A row, or a segment of one
+struct ShortItem {
+    long long row, p;   // row, first edge
+    int n, seg;         // edges (< 0: nothing to do); segment (< 0: a row)
+};
+// The rows of a block (or the segment, where it has one): one row per group of NG to a warp, or a segment per warp.
+template <int NG, bool SHARE>
+__device__ __forceinline__ ShortItem short_item(const RowArgs &a, unsigned block) {
     constexpr unsigned kAll = 0xffffffffu;
-    constexpr float kLowest = -3.402823466e38f;
-    static_assert(NV <= 32, "one vector per lane");
-    const int lane = threadIdx.x & 31, gl = lane & (G - 1), grp = lane / G;
-    const long long warp = (long long)blockIdx.x * (kShortThreads / 32) + (threadIdx.x >> 5);
-    const int h0 = kAgg ? 0 : (int)blockIdx.y * HP, have = a.H - h0;
-    const int hv = gl / VPHP, vec = gl % VPHP + (kAgg ? (int)blockIdx.y * NV : 0);
-    const bool okv = hv < have && vec < a.vph;
-    const int hc = h0 + (hv < have ? hv : have - 1), vc = vec < a.vph ? vec : a.vph - 1;   // a lane without a vector repeats the last one
-    const bool first = a.flags & SAR_FIRST, last = a.flags & SAR_LAST;
-    const unsigned HF = (unsigned)(a.H * a.F);
-    const int oel = hc * a.F + vec * EPV, left = okv ? a.F - vec * EPV : 0;
-    const bool head_lane = okv && gl % VPHP == 0;
-    const unsigned gofs = (unsigned)(hc * a.vph + vc) * 16u;
-    const char *gsrc = reinterpret_cast<const char *>(a.gather) + gofs;
-
-    // ---- which rows: one segment of a long row per warp, or one row per group ---------------------------------------------
-    const bool seg = warp < a.sp.n_seg;
-    long long row, p = 0;
-    int n = -1;                         // edges; < 0: nothing to do
-    if (seg) {
-        int lo = 0, hi = a.sp.n_long;   // last lo with long_seg[lo] <= warp, 32 probes at a time
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long item = SHARE && a.wide ? (block < a.sp.n_seg ? block : a.sp.n_seg + (block - a.sp.n_seg) * kShortWarps + wid) : (long long)block * kShortWarps + wid;
+    ShortItem x{0, 0, -1, -1};
+    if (item < a.sp.n_seg) {
+        x.seg = (int)item;
+        int lo = 0, hi = a.sp.n_long;   // last lo with long_seg[lo] <= item, 32 probes at a time
         while (hi - lo > 1) {
             const int step = (hi - lo + 31) >> 5;
             const int at = lo + lane * step;
-            const bool ok = at < hi && __ldg(a.sp.long_seg + at) <= warp;
+            const bool ok = at < hi && __ldg(a.sp.long_seg + at) <= item;
             lo += (__popc(__ballot_sync(kAll, ok)) - 1) * step;
             hi = min(hi, lo + step);
         }
-        row = __ldg(a.sp.long_row + lo);
-        p = __ldg(a.indptr + row) + (warp - __ldg(a.sp.long_seg + lo)) * a.sp.threshold;
-        const long long rest = __ldg(a.indptr + row + 1) - p;
-        n = (int)(rest < a.sp.threshold ? rest : a.sp.threshold);
+        x.row = __ldg(a.sp.long_row + lo);
+        x.p = __ldg(a.indptr + x.row) + (item - __ldg(a.sp.long_seg + lo)) * a.sp.threshold;
+        const long long rest = __ldg(a.indptr + x.row + 1) - x.p;
+        x.n = (int)(rest < a.sp.threshold ? rest : a.sp.threshold);
     } else {
-        row = (warp - a.sp.n_seg) * NG + grp;
-        if (row < a.n_rows) {
-            p = __ldg(a.indptr + row);
-            const long long len = __ldg(a.indptr + row + 1) - p;
-            if (a.sp.threshold <= 0 || len <= a.sp.threshold) n = (int)min(len, 0x7fffffffLL);   // else its segments are items of their own
+        x.row = (item - a.sp.n_seg) * NG + lane / (32 / NG);
+        if (x.row < a.n_rows) {
+            x.p = __ldg(a.indptr + x.row);
+            const long long len = __ldg(a.indptr + x.row + 1) - x.p;
+            if (a.sp.threshold <= 0 || len <= a.sp.threshold) x.n = (int)min(len, 0x7fffffffLL);   // else its segments are items of their own
         }
     }
+    return x;
+}
 
-    // One row (or segment) of n edges from position p on, every `step`-th four of them from the e0-th on.  fold: the groups of the warp share
-    // it, group 0 writes.
-    auto process = [&](long long row, long long p, int n, int e0, int step, bool fold, bool live) {
+// One row (or segment) of n edges from position p on, every `step`-th four of them from the e0-th on.  FOLD: the groups of the warp share
+// it, group 0 writes; with `share` the warps of the block too, warp 0 writes.
+template <typename T, int NV, int HP, int MODE>
+struct ShortRow {
+    static constexpr int EPV = Elem<T>::EPV, NP = EPV / 2, U = 4;
+    static constexpr int G = NV, NG = 32 / G, VPHP = NV / HP;
+    static constexpr bool kF = MODE == kRowFwd || MODE == kRowFwdPart, kD = MODE == kRowDst || MODE == kRowDstPart;
+    static constexpr bool kS = MODE == kRowSrc, kAgg = MODE == kRowSum || MODE == kRowSumW;
+    static constexpr bool kAcc = kF || kS || kAgg, kDot = kD || kS;
+    // Floats per lane that warps hand over: up to EPV + 2.  The same for every pass, for between two launches that need different shares of the
+    // L1 as shared memory an SM has to run empty (backward passes of 1,500 rows 13.6 -> 15.8 us).
+    static constexpr int kShare = 10;
+    static_assert(NV <= 32, "one vector per lane");
+
+    template <bool FOLD>
+    static __device__ __forceinline__ void process(const RowArgs &a, const ShortItem &item, int e0, int step, bool live, float (*share)[G][kShare]) {
+        constexpr unsigned kAll = 0xffffffffu;
+        constexpr float kLowest = -3.402823466e38f;
+        const int lane = threadIdx.x & 31, gl = lane & (G - 1), grp = lane / G;
+        const int h0 = kAgg ? 0 : (int)blockIdx.y * HP, have = a.H - h0;
+        const int hv = gl / VPHP, vec = gl % VPHP + (kAgg ? (int)blockIdx.y * NV : 0);
+        const bool okv = hv < have && vec < a.vph;
+        const int hc = h0 + (hv < have ? hv : have - 1), vc = vec < a.vph ? vec : a.vph - 1;   // a lane without a vector repeats the last one
+        const bool first = a.flags & SAR_FIRST, last = a.flags & SAR_LAST;
+        const unsigned HF = (unsigned)(a.H * a.F);
+        const int oel = hc * a.F + vec * EPV, left = okv ? a.F - vec * EPV : 0;
+        const bool head_lane = okv && gl % VPHP == 0;
+        const unsigned gofs = (unsigned)(hc * a.vph + vc) * 16u;
+        const char *gsrc = reinterpret_cast<const char *>(a.gather) + gofs;
+        const long long row = item.row, p = item.p;
+        const int n = item.n;
+        const bool seg = FOLD && item.seg >= 0;
         const long long so = row * a.H + hc;
         // an inconsistent graph gives wrong sums, not a wrong address
         auto column = [&](int e) {
@@ -214,7 +234,7 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
             y[2 * k] = acc[k].x;
             y[2 * k + 1] = acc[k].y;
         }
-        if (fold) {
+        if constexpr (FOLD) {
             if constexpr (kF) {   // the groups' sums against one shift, the maximum
                 float mm = m;
 #pragma unroll
@@ -237,16 +257,57 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
         if constexpr (kDot) {
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
-                if (off < VPHP || (fold && off >= G)) {
+                if (off < VPHP || (FOLD && off >= G)) {
                     if constexpr (MODE == kRowDst) dD += __shfl_xor_sync(kAll, dD, off);
                     dB += __shfl_xor_sync(kAll, dB, off);
                 }
             }
         }
+        if (FOLD && share) {
+            const int wid = threadIdx.x >> 5;
+            if (grp == 0) {
+                float *mine = share[wid][gl];
+                if constexpr (kAcc) {
+#pragma unroll
+                    for (int k = 0; k < EPV; ++k) mine[k] = y[k];
+                }
+                if constexpr (!kAgg) mine[kAcc ? EPV : 0] = l;
+                if constexpr (kF) mine[EPV + 1] = m;
+                if constexpr (kDot) mine[kAcc ? EPV + 1 : 1] = dB;
+                if constexpr (kD) mine[2] = dD;
+            }
+            __syncthreads();
+            if (wid == 0) {
+                float mm = m;
+                if constexpr (kF) {
+#pragma unroll
+                    for (int w = 1; w < kShortWarps; ++w) mm = fmaxf(mm, share[w][gl][EPV + 1]);
+                    const float f = row_ex2((m - mm) * kRowLog2e);
+                    l *= f;
+#pragma unroll
+                    for (int k = 0; k < EPV; ++k) y[k] *= f;
+                }
+#pragma unroll
+                for (int w = 1; w < kShortWarps; ++w) {
+                    const float *x = share[w][gl];
+                    const float f = kF ? row_ex2((x[kF ? EPV + 1 : 0] - mm) * kRowLog2e) : 1.f;
+                    if constexpr (kAcc) {
+#pragma unroll
+                        for (int k = 0; k < EPV; ++k) y[k] = fmaf(x[k], f, y[k]);
+                    }
+                    if constexpr (!kAgg) l = fmaf(x[kAcc ? EPV : 0], f, l);
+                    if constexpr (kDot) dB += x[kAcc ? EPV + 1 : 1];
+                    if constexpr (kD) dD += x[2];
+                }
+                m = mm;
+            }
+            __syncthreads();
+            live = wid == 0;
+        }
         if constexpr (kF) m = l == 0.f ? SAR_NEG_INF : m;
-        if (!live || (fold && grp != 0)) return;
+        if (!live || (FOLD && grp != 0)) return;
         if (seg) {
-            float *part = a.sp.part + warp * a.sp.pstride;
+            float *part = a.sp.part + item.seg * a.sp.pstride;
             const long long rowf = (long long)a.H * a.vph * EPV;
             if constexpr (kAcc) {
                 if (okv) store_elems<float, EPV>(part + (hc * a.vph + vc) * EPV, y, EPV, false);
@@ -337,20 +398,65 @@ __global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const RowArg
             }
             store_elems<T, EPV>(outp, y, left, a.ragged);
         }
-    };
+    }
 
-    // short rows, one per group; then the others and segments, one after the other, the groups of the warp together
-    const bool mine = !seg && n >= 0 && (NG == 1 || n <= kShortEdges);
-    if (!seg) process(row, p, mine ? n : 0, 0, U, false, mine);
-    if constexpr (NG > 1) {
-        unsigned rest = seg ? 1u : __ballot_sync(kAll, n > kShortEdges && gl == 0);
+    // Where a row fills the warp: rows of more than a.R edges are taken by the warps of the block together, one after the other, unless that
+    // takes longer than each warp with its own (a step per four edges, two to end a shared row); or the block's segment (a.wide).  A
+    // function of its own that looks its rows up again: compiled into the kernel it took registers from the short rows and cost them up to 25 %.
+    static __device__ __noinline__ void rest_of_block(const RowArgs &a) {
+        __shared__ float share[kShortWarps][G][kShare];
+        __shared__ ShortItem items[kShortWarps];
+        const int wid = threadIdx.x >> 5;
+        const ShortItem x = short_item<1, true>(a, blockIdx.x);
+        if ((threadIdx.x & 31) == 0) items[wid] = x;
+        __syncthreads();
+        auto shared = [&](const ShortItem &y) { return y.seg < 0 && y.n > a.R; };
+        bool own = false;
+        int entries = a.wide && x.seg >= 0 ? 1 : kShortWarps;
+        if (entries > 1) {
+            int block_steps = 0, warp_steps = 0;
+            for (int w = 0; w < kShortWarps; ++w) {
+                const int steps = shared(items[w]) ? (items[w].n + U - 1) / U : 0;
+                if (steps > 0) block_steps += (steps + kShortWarps - 1) / kShortWarps + 2;
+                warp_steps = max(warp_steps, steps);
+            }
+            if (block_steps >= warp_steps) {
+                own = shared(x);
+                entries = 0;
+            }
+        }
+        for (int at = own ? -1 : 0; at < entries; ++at) {
+            const bool block = at >= 0;
+            const ShortItem y = block ? items[at] : x;
+            if (entries > 1 && !shared(y)) continue;
+            process<true>(a, y, block ? wid * U : 0, (block ? kShortWarps : 1) * U, true, block ? share : nullptr);
+        }
+    }
+};
+
+// SHARE (where a row fills the warp): what the warps of a block share is left to rest_of_block.
+template <typename T, int NV, int HP, int MODE, int MINB, bool SHARE>
+__global__ void __launch_bounds__(kShortThreads, MINB) short_kernel(const __grid_constant__ RowArgs a) {
+    after_predecessor();
+    using Row = ShortRow<T, NV, HP, MODE>;
+    const ShortItem x = short_item<Row::NG, SHARE>(a, blockIdx.x);
+    const int most = SHARE ? a.R : Row::NG > 1 ? kShortEdges : 0x7fffffff;   // edges of a row that is one group's
+    const bool alone = x.n >= 0 && x.n <= most;
+    if (x.seg < 0) Row::template process<false>(a, alone ? x : ShortItem{x.row, x.p, 0, -1}, 0, Row::U, alone, nullptr);
+    if constexpr (SHARE) {
+        const bool wide = a.wide && x.seg >= 0;
+        if (x.seg >= 0 && !wide) Row::template process<true>(a, x, 0, Row::U, true, nullptr);
+        if (__syncthreads_or(wide || (x.seg < 0 && x.n > most))) Row::rest_of_block(a);
+    } else {
+        // segments, and rows of more edges, one after the other, the groups of the warp together
+        const int lane = threadIdx.x & 31;
+        unsigned rest = x.seg >= 0 ? 1u : Row::NG > 1 ? __ballot_sync(0xffffffffu, x.n > most && (lane & (Row::G - 1)) == 0) : 0u;
         while (rest) {
             const int from = __ffs(rest) - 1;
             rest &= rest - 1;
-            process(__shfl_sync(kAll, row, from), __shfl_sync(kAll, p, from), __shfl_sync(kAll, n, from), grp * U, NG * U, true, true);
+            const ShortItem y{__shfl_sync(0xffffffffu, x.row, from), __shfl_sync(0xffffffffu, x.p, from), __shfl_sync(0xffffffffu, x.n, from), x.seg};
+            Row::template process<true>(a, y, lane / Row::G * Row::U, Row::NG * Row::U, true, nullptr);
         }
-    } else if (seg) {
-        process(row, p, n, 0, U, true, true);
     }
 }
 

@@ -197,6 +197,30 @@ def test_an_infinity_on_the_last_edge_of_a_sum(n, F, dtype):
     assert torch.equal(api.spmm_scaled(g.whole, x, src_scale=scale, dst_scale=scale), (take(x.float() * scale[:, None]) * scale[:, None]).to(x.dtype))
 
 
+@pytest.mark.parametrize("H,F,dtype", [(5, 24, "bf16"), (8, 24, "bf16"), (6, 12, "f32"), (5, 16, "f32")])
+@pytest.mark.parametrize("threshold", [0, 100, 256])
+@pytest.mark.parametrize("masked", [False, True])
+def test_long_rows_that_the_warps_of_a_block_share(H, F, dtype, threshold, masked):
+    """Rows that fill a warp, with ones on either side of 96 edges among them: one to four in a block, of lengths that are and are not worth sharing;
+    segments of 100, of 256 and of less, a block each; unsplit rows of 1,000.  With half of the sources masked whole warps have nothing to add."""
+    n, gen = 16_100, torch.Generator().manual_seed(H * F)
+    degs = [(96, 2, 1, 0), (97, 1, 2, 3), (0, 98, 0, 0), (1, 2, 129, 97), (200, 200, 200, 200), (255, 97, 100, 1), (97, 97, 97, 97), (240, 0, 200, 5),
+            (300, 0, 0, 1), (1000, 1, 0, 2), (101, 350, 1, 99), (256, 257, 3, 400)]
+    deg = torch.tensor(degs).flatten()
+    src = [torch.randint(100, n, (n // 2,), generator=gen), torch.randint(100, n, (int(deg.sum()),), generator=gen), n - 1 - torch.arange(n) % 100]
+    dst = [torch.randint(100, n, (n // 2,), generator=gen), 200 + torch.arange(deg.numel()).repeat_interleave(deg), torch.arange(n)]
+    src, dst = torch.cat(src).int(), torch.cat(dst).int()
+    both = torch.cat([src, dst]), torch.cat([dst, src])
+    p = Problem(n, both[0], both[1], H, F, 3, dtype=dtype, k=2, threshold=threshold, build_parts=True)
+    if masked:
+        off = torch.arange(n) < n // 2
+        p.host["er"][off.numpy()] = -np.inf
+        p.dev["er"][off.to(DEV)] = -float("inf")
+    with Launches() as ran:
+        _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
+    assert ran.only("_short"), set(ran.names)
+
+
 @pytest.mark.parametrize("H,F,dtype", [(1, 16, "f32"), (1, 32, "f32"), (2, 8, "bf16"), (4, 8, "bf16"), (4, 24, "bf16"), (8, 24, "bf16")])
 def test_an_infinity_on_the_last_edge_of_a_short_row(H, F, dtype):
     n = 33_000
