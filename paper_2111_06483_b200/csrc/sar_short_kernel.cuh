@@ -38,7 +38,8 @@ struct ShortItem {
     long long row, p;   // row, first edge
     int n, seg;         // edges (< 0: nothing to do); segment (< 0: a row)
 };
-// The rows of a block (or the segment, where it has one): one row per group of NG to a warp, or a segment per warp.
+// The rows of a block (or the segment, where it has one): one row per group of NG to a warp, or a segment per warp.  A row has no more edges
+// than there are (fewer than 2^30, see few_edges), whatever its pointers say, so that no position and no step beyond it overflows.
 template <int NG, bool SHARE>
 __device__ __forceinline__ ShortItem short_item(const RowArgs &a, unsigned block) {
     constexpr unsigned kAll = 0xffffffffu;
@@ -64,7 +65,7 @@ __device__ __forceinline__ ShortItem short_item(const RowArgs &a, unsigned block
         if (x.row < a.n_rows) {
             x.p = __ldg(a.indptr + x.row);
             const long long len = __ldg(a.indptr + x.row + 1) - x.p;
-            if (a.sp.threshold <= 0 || len <= a.sp.threshold) x.n = (int)min(len, 0x7fffffffLL);   // else its segments are items of their own
+            if (a.sp.threshold <= 0 || len <= a.sp.threshold) x.n = (int)min(len, a.nnz);   // else its segments are items of their own
         }
     }
     return x;

@@ -328,6 +328,23 @@ def test_sums_on_either_side_of_the_span_kernels_line(F, dtype, mb, deg, long):
     assert torch.equal(api.propagate(g, x, 0.5, 1, scale, scale), (0.5 * x.float() + 0.5 * want).to(tdt))
 
 
+def test_row_pointers_that_claim_more_edges_than_there_are():
+    """A row of 2^31 + 5 edges by its pointers has the graph's last edges again and again in the short-row kernel's sum, and the sum ends;
+    the other rows are what they were."""
+    n, row = 33_000, 1234
+    gen = torch.Generator(device=DEV).manual_seed(2)
+    src, dst = (torch.randint(0, n, (3 * n,), generator=gen, device=DEV, dtype=torch.int32) for _ in range(2))
+    g = api.Graph.from_coo(n, src, dst)
+    x = torch.randn(n, 16, generator=gen, device=DEV)
+    with Launches() as ran:
+        want = api.spmm_sum(g.whole, x)
+    assert ran.only("_short", ("spmm",)) and g.whole.split.n_long == 0
+    g.whole.indptr[row + 1] = g.whole.indptr[row] + 2 ** 31 + 5
+    got = api.spmm_sum(g.whole, x)
+    others = torch.arange(n, device=DEV) // 2 != row // 2   # (the next row's pointers end before they begin)
+    assert torch.equal(got[others], want[others])
+
+
 def test_ragged_shape_without_room_for_padded_copies():
     """No workspace in the forward call, one that holds the records alone in the backward call: the scalar kernels."""
     n, src, dst = hub_graph(n=500, e=6000, d_max=100.0, seed=3)
