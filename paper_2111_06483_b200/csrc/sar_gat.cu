@@ -273,7 +273,7 @@ static sar_status check_part(const sar_part *g, bool need_csc) {
 //    to 1.5 else.
 // With these lines the choice costs 1.1 % over the better kernel of each call in the mean, over shapes of up to 1 KB; with lines drawn
 // by the number of heads alone it was 2.8 %.
-constexpr unsigned long long kSpanBytes = 128ull << 20, kSpanSumBytes = 12ull << 20;
+constexpr unsigned long long kSpanBytes = 128ull << 20;
 static bool takes_span(const Shape &s, const RowGeo &geo, long long n_gathered, long long n_rows, long long nnz, bool backward, bool part) {
     if (!s.fast) return false;
     if ((unsigned long long)n_gathered * s.row_bytes > kSpanBytes) return true;
@@ -296,6 +296,8 @@ static bool takes_span(const Shape &s, const RowGeo &geo, long long n_gathered, 
 //  * NV <= 8, HP = 4: forward 0.9 to 3.2 / 1.1 to 2.0 with up to 24; backward 1.1 to 4.4 / 1.2 to 2.7 with up to 60.
 //  * HP = 8: backward 1.3 to 5.7 / 1.1 to 4.0; forward 0.96 to 3.5 / 1.0 to 2.6 with up to 30 (NV = 32, in arrays of up to 32 MB:
 //    0.96 to 1.5 / 0.9 to 1.2 with up to 14; else 0.73 to 1.2).
+//    In launches of up to 10,000 rows with some of 60 and more edges among them, HP >= 4, backward: 1.0 to 2.1, and in 20 of 600 calls 0.78 to
+//    0.95, NV = 4 with rows of 100 to 160 edges (0.81 to 0.92) and NV = 32 with ones of 60 to 100 in 1,200 to 1,600 rows (0.78 to 0.93).
 //  * NV = 16, HP = 4: forward 1.0 to 1.75 / 0.95 to 1.07 with up to 10, backward 1.1 to 2.2 / 0.95 to 1.4 with up to 16.
 // The rest is decided by rows of up to 100 or 240 edges, too short for segments, among ones of 2 to 20: a group waits for the longest
 // row of its warp, and the plan doesn't tell such graphs from uniform ones.
@@ -305,15 +307,6 @@ static bool takes_span(const Shape &s, const RowGeo &geo, long long n_gathered, 
 //  * Few rows do not fill the chip with groups.  HP >= 4, backward: 8,000 rows as above with half of these edges (1.05 to 1.9).  Else
 //    16,000 rows with half (1.0 to 1.9; with as many 0.8 to 1.1), 8,000 with a quarter (1.0 to 1.24), with NV >= 8, HP = 1 or
 //    NV = 16, HP = 2 not (0.89 to 1.07).
-static double short_edges(const RowGeo &geo, bool backward, unsigned long long bytes) {
-    const int NV = geo.NV, HP = geo.HP;
-    if (NV > 32) return 0;
-    if (HP == 8) return backward ? 100 : NV <= 16 ? 40 : bytes <= (32ull << 20) ? 14 : 0;
-    if (NV == 32) return HP == 4 && backward && bytes <= (8ull << 20) ? 10 : 0;
-    if (NV == 16) return HP == 4 ? (backward ? 16 : 10) : HP == 2 && backward ? 6 : 0;
-    if (HP == 4) return backward ? 100 : 24;
-    return NV == 4 ? (backward ? 28 : 20) : backward ? 16 : 14;
-}
 // `filled`: rows with which the limit holds in full
 static bool few_edges(double limit, long long filled, long long n_rows, long long nnz) {
     const double fill = n_rows < filled ? (double)n_rows / (double)filled : 1.0;
@@ -321,14 +314,14 @@ static bool few_edges(double limit, long long filled, long long n_rows, long lon
 }
 static bool takes_short(const RowGeo &geo, long long n_gathered, unsigned row_bytes, long long n_rows, long long nnz, bool backward) {
     if (n_rows < 12000 && ((geo.HP == 1 && geo.NV >= 8) || (geo.HP == 2 && geo.NV >= 16))) return false;
-    return few_edges(short_edges(geo, backward, (unsigned long long)n_gathered * row_bytes), geo.HP >= 4 && backward ? 16000 : 32000, n_rows, nnz);
+    return few_edges(short_edges(geo.NV, geo.HP, backward, (unsigned long long)n_gathered * row_bytes), geo.HP >= 4 && backward ? 16000 : 32000, n_rows, nnz);
 }
 // Sums, likewise, from 12,000 rows on (8,000: 0.83 to 1.06): rows of 64 bytes 1.0 to 4.1 / 1.0 to 2.4 with up to 20 edges per row; of 128
 // bytes, in arrays of up to 12 MB 1.1 to 2.4 / 1.0 to 1.4 with up to 14, up to 64 MB 1.1 to 1.9 / 1.0 to 1.3 with up to 8, beyond 1.1 to
 // 1.6 / 1.0 to 1.2 with up to 3; of 256 bytes 0.91 to 1.2 (uniform up to 1.5): not taken.
 static bool sum_takes_short(const RowGeo &geo, long long n_gathered, unsigned row_bytes, long long n_rows, long long nnz) {
     const unsigned long long bytes = (unsigned long long)n_gathered * row_bytes;
-    const double limit = geo.tiles > 1 || n_rows < 12000 ? 0 : geo.NV == 4 ? 20 : geo.NV == 8 ? (bytes <= kSpanSumBytes ? 14 : bytes <= (64ull << 20) ? 8 : 3) : 0;
+    const double limit = geo.tiles > 1 || n_rows < 12000 ? 0 : sum_short_edges(geo.NV, bytes);
     return few_edges(limit, 32000, n_rows, nnz);
 }
 // A sum has nothing between its ids and its rows.  Where the L2 doesn't hold the array the span kernels' ring keeps more loads in

@@ -52,6 +52,21 @@ struct RowGeo {
     int NV, HP, tiles;
 };
 
+// The most edges per row with which the kernel for short rows (sar_short_kernel.cuh) takes a call, by its tile and the bytes of the gathered
+// array; 0: it doesn't, and the kernel of that tile isn't compiled.  What the lines were drawn from is with takes_short in sar_gat.cu.
+constexpr double short_edges(int NV, int HP, bool backward, unsigned long long bytes) {
+    if (NV > 32) return 0;
+    if (HP == 8) return backward ? 100 : NV <= 16 ? 40 : bytes <= (32ull << 20) ? 14 : 0;
+    if (NV == 32) return HP == 4 && backward && bytes <= (8ull << 20) ? 10 : 0;
+    if (NV == 16) return HP == 4 ? (backward ? 16 : 10) : HP == 2 && backward ? 6 : 0;
+    if (HP == 4) return backward ? 100 : 24;
+    return NV == 4 ? (backward ? 28 : 20) : backward ? 16 : 14;
+}
+constexpr unsigned long long kSpanSumBytes = 12ull << 20;   // sums over larger arrays are the span kernels' where the short-row kernel does not take them
+constexpr double sum_short_edges(int NV, unsigned long long bytes) {
+    return NV == 4 ? 20 : NV == 8 ? (bytes <= kSpanSumBytes ? 14 : bytes <= (64ull << 20) ? 8 : 3) : 0;
+}
+
 // One launch over the segments of the long rows and the other rows.
 #define SAR_ROWS_DECL(PASS) \
     sar_status rows_##PASS##_f32(const RowArgs &a, RowGeo g, long long nnz, cudaStream_t st); \
@@ -65,7 +80,7 @@ SAR_ROWS_DECL(src)
 sar_status rows_sum_f32(const RowArgs &a, RowGeo g, long long nnz, bool weighted, cudaStream_t st);
 sar_status rows_sum_bf16(const RowArgs &a, RowGeo g, long long nnz, bool weighted, cudaStream_t st);
 
-// The long rows, from their segments' records (one block per long row).
+// The long rows, from their segments' records.
 sar_status rows_fwd_merge(const RowArgs &a, sar_dtype t, cudaStream_t st);
 // The end of Algorithm 1 on its own: out = numerator / d for every row.
 sar_status rows_fwd_finalize(const RowArgs &a, sar_dtype t, cudaStream_t st);

@@ -64,11 +64,16 @@ static sar_status launch_short_kernel(RowArgs a, RowGeo g, long long nnz, cudaSt
     return go(short_kernel<T, NV, HP, MODE, MINB, false>);
 }
 
+template <int MODE>
+constexpr bool has_short(int NV, int HP) {
+    return MODE == kRowSum || MODE == kRowSumW ? sum_short_edges(NV, 0) > 0 : short_edges(NV, HP, MODE != kRowFwd && MODE != kRowFwdPart, 0) > 0;
+}
+
 template <typename T, int MODE>
 static sar_status dispatch_rows(const RowArgs &a, RowGeo g, long long nnz, const char *name, cudaStream_t st) {
 #define SAR_ROW_CASE(NV_, HP_) \
     if (g.NV == NV_ && g.HP == HP_) { \
-        if constexpr (NV_ <= 32) \
+        if constexpr (has_short<MODE>(NV_, HP_)) \
             if (a.lone) return launch_short_kernel<T, NV_, HP_, MODE>(a, g, nnz, st); \
         return launch_row_kernel<T, NV_, HP_, MODE>(a, g, nnz, name, st); \
     }
