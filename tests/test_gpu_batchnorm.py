@@ -66,6 +66,39 @@ def test_batchnorm_forward_and_backward(C, dt, n, offset):
     assert torch.equal(x2, y)
 
 
+@pytest.mark.parametrize("C,dt,n", [(128, "f32", 250_001), (128, "bf16", 250_001), (128, "bf16", 120_003), (256, "f32", 120_003), (256, "bf16", 120_003), (64, "f32", 600_001)])
+def test_batchnorm_of_more_rows_than_the_grid(C, dt, n):
+    """Lane groups that take several rows, two or four of which they ask for at once, and a remainder one by one; results over x and over gy
+    in place.  The reference is float64 on the GPU."""
+    from paper_2111_06483_b200 import api, binding as B
+    gen = torch.Generator(device="cuda").manual_seed(C + n)
+    x, gy = ((torch.randn(n, C, generator=gen, device="cuda") + shift).to(DT[dt]) for shift in (3.0, 0.0))
+    gamma, beta = (torch.randn(C, generator=gen, device="cuda") for _ in range(2))
+    x64, g64 = x.double(), gy.double()
+    mean64, var64 = x64.mean(0), x64.var(0, unbiased=False)
+    xh = (x64 - mean64) / (var64 + 1e-5).sqrt()
+    y, (mean, rstd, n_all) = api.bn_forward(x, 1e-5, gamma, beta)
+    gx, dgamma, dbeta = api.bn_backward(x, gy, (mean, rstd, n_all), gamma)
+    s0, s1 = g64.sum(0), (g64 * xh).sum(0)
+    want_gx = gamma.double() * (g64 - s0 / n - xh * (s1 / n)) / (var64 + 1e-5).sqrt()
+    # the bounds of the test above: x - mean loses |offset| / std digits of a float32 input
+    lost = 4.0 * 2.0 ** -23 * 8
+    tol = (2e-2, 2e-2) if dt == "bf16" else (1e-4, 1e-5 + lost)
+    allclose_report(_np(y), (xh * gamma.double() + beta.double()).cpu().numpy(), *tol, "y")
+    allclose_report(_np(gx), want_gx.cpu().numpy(), *((2e-2, 2e-2 * max(1.0, float(want_gx.abs().max()) * 0.1)) if dt == "bf16" else
+                                                     (1e-3, (1e-5 + lost) * max(1.0, float(want_gx.abs().max())))), "gx")
+    scale_g = float(np.sqrt(n))
+    allclose_report(_np(dbeta), s0.cpu().numpy(), 1e-4, 1e-5 * scale_g, "dbeta")
+    allclose_report(_np(dgamma), s1.cpu().numpy(), 1e-3, (1e-5 + lost) * scale_g * 4, "dgamma")
+    over_x = x.clone()
+    B.sar_bn_apply(over_x, mean, rstd, gamma, beta, over_x)
+    assert torch.equal(over_x, y)
+    for target in (x.clone(), gy.clone()):   # the gradient over x, and over gy
+        xin, gin = (target, gy) if torch.equal(target, x) else (x, target)
+        B.sar_bn_bwd_apply(xin, mean, rstd, gamma, gin, dbeta, dgamma, 1.0 / n, target)
+        assert torch.equal(target, gx)
+
+
 def test_batchnorm_empty_input_and_errors():
     from paper_2111_06483_b200 import binding as B
     C = 16

@@ -58,20 +58,25 @@ def test_attention_on_arrays_larger_than_the_l2(H, F, dtype, n):
                                                    (5, 24, "f32", 20_000, 16, 300.0), (4, 24, "bf16", 20_000, 15, 300.0), (6, 128, "bf16", 900, 6, 100.0),
                                                    (3, 128, "f32", 1_500, 6, 100.0)])
 def test_attention_on_short_rows(H, F, dtype, n, deg, d_max):
-    """Few edges per row: the span kernels on small arrays, whole and step by step, with long rows among them."""
+    """Few edges per row: shapes on either side of the lines between the row, the span and the short-row kernels on small arrays, whole and
+    step by step, with long rows among them."""
     n, src, dst = hub_graph(n=n, e=deg * n, d_max=d_max, seed=H + F)
     p = Problem(n, src, dst, H, F, 31, dtype=dtype, k=2, threshold=100, build_parts=True)
     _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
 
 
 @pytest.mark.parametrize("H,F,dtype", [(1, 5, "f32"), (1, 32, "bf16"), (2, 12, "bf16"), (4, 8, "f32"), (3, 16, "bf16"), (1, 47, "bf16"), (8, 8, "bf16"),
-                                       (2, 32, "f32"), (4, 24, "bf16"), (7, 8, "f32"), (8, 24, "bf16"), (3, 24, "f32")])
+                                       (2, 32, "f32"), (4, 24, "bf16"), (7, 8, "f32"), (8, 24, "bf16"), (3, 24, "f32"),
+                                       (2, 32, "bf16"), (2, 16, "f32"), (4, 8, "bf16"), (3, 4, "f32"), (2, 64, "bf16"), (3, 32, "f32")])
 @pytest.mark.parametrize("scale", [1.0, 60.0])
 def test_attention_of_a_row_per_lane_group(H, F, dtype, scale):
     """Enough rows with few enough edges for the kernel for short rows: rows of 0, 1, 3 to 5, 23 to 25 and 95 to 97 edges (the ends of its
     steps of four, and of what one group keeps to itself), segments of 100 and of 1, and scores that lead a row's first by more than 60."""
     n, gen = 16_100, torch.Generator().manual_seed(H * F)
-    src, dst = [torch.randint(0, n, (3 * n,), generator=gen)], [torch.randint(500, n, (3 * n,), generator=gen)]
+    # tiles of 16 vectors and two heads, or 32 and four: three edges per row are too many, and the forward pass is another kernel's
+    backward_only = (H, F, dtype) in ((2, 32, "f32"), (2, 64, "bf16"), (3, 24, "f32"), (3, 32, "f32"))
+    many = 1 if backward_only or (H, F) == (4, 24) else 3
+    src, dst = [torch.randint(0, n, (many * n,), generator=gen)], [torch.randint(500, n, (many * n,), generator=gen)]
     for row, deg in enumerate([1, 3, 4, 5, 23, 24, 25, 95, 96, 97, 100, 101, 350]):
         src.append(torch.randint(0, n, (2 * deg,), generator=gen))
         dst.append(torch.tensor([7 * row, 7 * row + 3]).repeat_interleave(deg))
@@ -79,7 +84,11 @@ def test_attention_of_a_row_per_lane_group(H, F, dtype, scale):
     both = torch.cat([src, dst]), torch.cat([dst, src])   # the same lengths among the columns, which the source-major pass walks
     p = Problem(n, both[0], both[1], H, F, 3, dtype=dtype, k=2, threshold=100, build_parts=True, scale=scale)
     if scale == 1.0:
-        return _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
+        with Launches() as ran:
+            _full_check(p, dtype=dtype, modes=("fused", "stateful"), grad_floor=10.0)
+        # (a step has half of the sources, for some tiles too few rows for the source-major pass)
+        assert ran.only("_short", ("gat_bwd_dst",) if backward_only else ("gat_fwd", "gat_bwd_dst")) and "gat_bwd_src_short" in ran.names, set(ran.names)
+        return
     # d = sum exp(e - m) with |e| up to 500: an ulp of e is 2^-15, and that is the relative error of its exponential
     d, f = p.dev, p.oracle_fwd()
     for mode in ("fused", "stateful"):
@@ -88,7 +97,9 @@ def test_attention_of_a_row_per_lane_group(H, F, dtype, scale):
         assert np.array_equal(np.isfinite(m.cpu().numpy()), has)
         allclose_report(m.cpu().numpy()[has], f.m[has], 2.0 ** -23, 0.0, "m")
         allclose_report(dd.cpu().numpy(), f.d, 2.0 ** -14, 0.0, "d")
-        allclose_report(out.float().cpu().numpy(), f.out, 2.0 ** -7, 2.0 ** -9, "out")
+        # out is a mean of features of up to 5 with those weights: 2 x 2^-15 x 5, besides the rounding of a stored bf16
+        bf16 = dtype == "bf16"
+        allclose_report(out.float().cpu().numpy(), f.out, 2.0 ** -7 if bf16 else 1e-5, 2.0 ** -9 if bf16 else 10 * 2.0 ** -15, "out")
 
 
 def _masked_problem(H, F, dtype, which, threshold, long_rows=()):
@@ -162,6 +173,19 @@ def test_large_features_of_short_rows(H, F, dtype, lead, power):
         check_grad(dfeat.float() * 2.0 ** power, b.dfeat, dtype, "dfeat", stored=True)
         check_grad(del_, b.del_, dtype, "del", 10.0)
         check_grad(der, b.der, dtype, "der", 10.0)
+
+
+@pytest.mark.parametrize("H,F,dtype,n,deg,d_max,passes", [(2, 64, "bf16", 61_000, 2, 400.0, ("gat_fwd",)), (6, 48, "bf16", 21_000, 9, 300.0, ("gat_fwd", "gat_bwd_dst", "gat_bwd_src")),
+                                                          (12, 16, "f32", 900, 8, 100.0, ("gat_bwd_dst", "gat_bwd_src")), (8, 24, "bf16", 700, 11, 200.0, ("gat_bwd_dst", "gat_bwd_src")),
+                                                          (5, 24, "f32", 20_000, 16, 300.0, ("gat_bwd_dst", "gat_bwd_src")), (16, 8, "f32", 1_100, 9, 100.0, ("gat_bwd_dst", "gat_bwd_src")),
+                                                          (3, 32, "f32", 40_000, 13, 300.0, ("gat_bwd_dst", "gat_bwd_src"))])
+def test_span_kernels_on_small_arrays(H, F, dtype, n, deg, d_max, passes):
+    n, src, dst = hub_graph(n=n, e=deg * n, d_max=d_max, seed=H + F)
+    p = Problem(n, src, dst, H, F, 31, dtype=dtype, k=2, threshold=100, build_parts=True)
+    with Launches() as ran:
+        _full_check(p, dtype=dtype, modes=("fused",), grad_floor=10.0)
+    assert ran.only("_span", passes), set(ran.names)
+    _full_check(p, dtype=dtype, modes=("stateful",), grad_floor=10.0)
 
 
 def _infinite_last_sources(n):
@@ -304,6 +328,40 @@ def test_sums_of_ragged_rows(F, dtype, n):
     out = x.clone()
     api.spmm_scaled(g.whole, x, src_scale=scale, dst_scale=scale, out=out, first=False)   # += 4 * sum
     assert torch.equal(out, (x.float() + 4.0 * want).to(x.dtype))
+
+
+@pytest.mark.parametrize("F,dtype", [(3, "f32"), (16, "f32"), (32, "f32"), (47, "bf16")])
+@pytest.mark.parametrize("k", [1, 3])
+@pytest.mark.parametrize("scaled", [False, True])
+def test_means_and_propagation_over_short_rows(F, dtype, k, scaled):
+    """The ends of the short-row kernel's sum: the mean, factors of sources and rows, what earlier partitions left, the propagation's mix with and
+    without the next step's factor; rows without edges, of 25 and more, and split ones."""
+    n, tdt = 40_000, torch.bfloat16 if dtype == "bf16" else torch.float32
+    gen = torch.Generator().manual_seed(F + k)
+    src, dst = [torch.randint(0, n - 5, (2 * n,), generator=gen)], [torch.randint(100, n - 5, (2 * n,), generator=gen)]   # the last five: no edges
+    for row, deg in enumerate([1, 4, 24, 25, 26, 63, 64, 65, 200]):
+        src.append(torch.randint(0, n - 5, (deg,), generator=gen))
+        dst.append(torch.full((deg,), 3 * row))
+    src, dst = torch.cat(src), torch.cat(dst)
+    e = src.numel()
+    g = api.Graph.from_coo(n, src.int().to(DEV), dst.int().to(DEV), k=k, build_parts=k > 1, threshold=64)
+    adj = torch.sparse_coo_tensor(torch.stack([dst, src]), torch.ones(e, dtype=torch.float64), (n, n)).to_sparse_csr()
+    x0 = torch.randn((n, F), generator=gen).to(tdt)
+    deg = torch.bincount(dst, minlength=n)
+    s = torch.rand(n, generator=gen) + 0.5 if scaled else None
+    d = 1.0 / deg.clamp(min=1).float()
+    # sums of up to 200 float32 terms of size 1; a stored bf16 rounds by 2^-9 of its value in every step
+    tol = dict(rtol=1e-5, atol=1e-5) if dtype == "f32" else dict(rtol=2e-2, atol=2e-2)
+    with Launches() as ran:
+        mean = api.spmm_sum(g.whole, x0.to(DEV), mean=True, deg_total=deg.to(DEV))
+        got = api.propagate(g, x0.to(DEV), 0.7, 2, s.to(DEV) if scaled else None, d.to(DEV))
+    assert ran.only("_short", ("spmm",)), set(ran.names)
+    allclose_report(mean.double().cpu().numpy(), ((adj @ x0.double()) * d.double()[:, None]).numpy(), what="mean", **tol)
+    want = x0.double()
+    for _ in range(2):
+        y = want * s.double()[:, None] if scaled else want
+        want = 0.3 * x0.double() + 0.7 * d.double()[:, None] * (adj @ y)
+    allclose_report(got.double().cpu().numpy(), want.numpy(), what="propagation", **tol)
 
 
 @pytest.mark.parametrize("F,dtype", [(32, "f32"), (36, "f32"), (47, "f32"), (64, "f32"), (101, "f32"), (128, "f32"), (160, "f32"), (193, "f32"),
