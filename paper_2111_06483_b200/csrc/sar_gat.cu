@@ -335,6 +335,9 @@ static bool sum_takes_short(const RowGeo &geo, long long n_gathered, unsigned ro
 //  * rows of 528 to 768 bytes, no long rows, in up to 40 MB: float32 1.12 to 1.70 / 1.4, bf16 weighted 1.08 to 1.30.
 //  * rows of 128 and 256 bytes, full lanes in either: half the MB, from 20 edges on, 0.97 to 1.41 / 1.1 to 1.25, no mix (12 edges 0.87 to 1.0).
 // Beyond the line 0.55 to 1.1.
+// The numbers are where the measured curves cross and no model's.  What moves them, as far as the counters show: the ring costs a span kernel
+// its instructions for every slot (82 % of the issue slots busy at 42 an edge of 512 bytes), while a row kernel waits for memory once in four slots, which
+// costs the more the fewer gathers the L2 answers and the more a row reads besides (the mix: x0's row and a factor).
 static bool sum_takes_rows(const RowArgs &a, sar_dtype t, long long n_gathered, long long nnz, bool weighted) {
     const int vecs = (int)(a.row_bytes / 16);
     const bool hubs = a.sp.n_long > 0, mix = a.mix.x0 != nullptr, f32 = t == SAR_F32;

@@ -48,7 +48,7 @@ constexpr int kLeanCap = 256;   // edges a chunk stages; rows and segments must 
 // Both cover these shapes; measured on them, lean against row kernels, bf16, 4 heads of 32, forward / destination-major /
 // source-major: large workload 15.2 / 15.2 / 16.8 against 20.2 / 20.1 / 32.7 ms, 100,000 nodes and 2 million edges
 // 117 / 116 / 120 against 115 / 111 / 181 us; a partition step of the large workload 3.0 / 2.2 / 1.0 against
-// 3.9 / 2.8 / 2.1 ms.
+// 3.9 / 2.8 / 2.1 ms.  (The short-row kernel, sar_short_kernel.cuh, has not been compared with them on these shapes.)
 
 // Do the lean kernels cover this shape?  Slope >= 0, heads in groups of four, rows of
 // exactly G*V vectors with V <= 2, the vectors of a head a power of two within one lane group, and a long-row
