@@ -38,6 +38,7 @@ constexpr long long kShortBlock = 96, kShortFew = 4 * 32 * kRowSMs;   // edges (
 template <typename T, int NV, int HP, int MODE>
 static sar_status launch_short_kernel(RowArgs a, RowGeo g, long long nnz, cudaStream_t st) {
     constexpr int NG = 32 / NV;
+    if (a.n_rows <= 0) return SAR_OK;   // a partition without sources
     // 32 warps an SM at 64 registers; the backward passes over bf16 rows need 70 and more (24 warps at 80)
     constexpr int MINB = sizeof(T) == 2 && (MODE == kRowSrc || MODE == kRowDst || MODE == kRowDstPart) ? 6 : 8;
     a.nnz = nnz;
@@ -45,7 +46,6 @@ static sar_status launch_short_kernel(RowArgs a, RowGeo g, long long nnz, cudaSt
                                  : MODE == kRowSrc ? "gat_bwd_src_short" : "spmm_short";
     auto go = [&](auto kernel) {
         const long long warps = (a.wide ? a.sp.n_seg * kShortWarps : a.sp.n_seg) + (a.n_rows + NG - 1) / NG;
-        if (warps <= 0) return SAR_OK;
         SAR_LAUNCH(name, st, launch(kernel, dim3((unsigned)((warps + kShortWarps - 1) / kShortWarps), (unsigned)g.tiles), kShortThreads, 0, st, a));
         return sar_after_launch();
     };

@@ -245,6 +245,16 @@ def test_long_rows_that_the_warps_of_a_block_share(H, F, dtype, threshold, maske
     assert ran.only("_short"), set(ran.names)
 
 
+@pytest.mark.parametrize("H,F,dtype", [(8, 24, "bf16"), (6, 12, "f32"), (8, 8, "f32"), (3, 16, "bf16"), (1, 16, "f32")])
+def test_partitions_without_sources(H, F, dtype):
+    """More partitions than nodes: steps whose source-major pass has no rows."""
+    n, gen = 40, torch.Generator().manual_seed(H)
+    src, dst = (torch.randint(0, n, (90,), generator=gen).int() for _ in range(2))
+    p = Problem(n, src, dst, H, F, 5, dtype=dtype, k=64, build_parts=True)
+    assert any(part.n_src == 0 for part in p.graph.parts)
+    _full_check(p, dtype=dtype, modes=("stateful",), grad_floor=1.0)
+
+
 @pytest.mark.parametrize("H,F,dtype", [(1, 16, "f32"), (1, 32, "f32"), (2, 8, "bf16"), (4, 8, "bf16"), (4, 24, "bf16"), (8, 24, "bf16")])
 def test_an_infinity_on_the_last_edge_of_a_short_row(H, F, dtype):
     n = 33_000
